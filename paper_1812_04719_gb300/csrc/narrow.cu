@@ -10,8 +10,9 @@
 //     pairs whose FP32 (outward) boxes overlap and some of whose cells (1 x 2
 //     quads) meet;
 //   narrow_kernel (stages 1-3a): per patch pair, one warp stages both patches
-//     in shared memory and filters the primitive pairs; the survivors leave
-//     as global pair descriptors;
+//     in shared memory, finds the primitive pairs whose boxes overlap from bit
+//     masks over the vertex slots and filters them; the survivors leave as
+//     global pair descriptors;
 //   pieces_kernel (stage 3b) and fp64_kernel (stage 4) work on those lists,
 //     so that every stage runs on full warps.  The stages:
 //     1. FP32 swept-box test (conservative: never drops an overlapping pair);
@@ -20,9 +21,10 @@
 //        for the pairs those do not decide;
 //     3. certified FP32 rejection: a pair is dropped only when error-bounded
 //        FP32 arithmetic proves that the FP64 test below cannot report a
-//        contact (Bernstein bound: no root of the cubic in [0,1]; or, on every
-//        sub-interval that may hold a root, the point is certainly outside the
-//        triangle / the edges certainly miss);
+//        contact (Bernstein bound: no root of the cubic in [0,1]; a direction
+//        along which the two primitives stay apart over the whole step; or, on
+//        every sub-interval that may hold a root, the point is certainly
+//        outside the triangle / the edges certainly miss);
 //     4. the FP64 contact test (cubic, root isolation, bisection, inside test)
 //        in the fixed arithmetic order, on the survivors only.
 // Stage 3 never changes a result: the contact list equals the one obtained by
@@ -33,45 +35,41 @@
 
 namespace {
 
-constexpr int NS = (STIV_BR + 1) * (STIV_BC + 1) + 2;  // vertex slots per patch (+2 poles)
-constexpr int SN = NS - 2, SS = NS - 1;               // pole slots
-constexpr int MAXV = 16, MAXT = 32, MAXE = 48;
+constexpr int PSLOT = (STIV_BR + 1) * (STIV_BC + 1);   // slot of the patch's pole; grid slots below it
+constexpr int NSLOT = PSLOT + 1;
 constexpr int NW = 8;                                  // warps per CTA
-constexpr int QCAP = 64;                               // queue entries
+constexpr int QCAP = 512;                              // queue entries per warp
+constexpr int SOUTH = 1 << 15;                         // patch id flag: the south-pole primitives of a two-pole patch
 
-// Primitives of one patch in terms of its vertex slots.  P is even, so every
-// patch spans exactly STIV_BR bands and STIV_BC columns; the lists depend only
-// on whether the patch touches the north pole (first band), the south pole
-// (last band) and whether it owns the pole vertices (first column block):
-// 8 variants, built once per CTA.
+// Primitives of one patch in terms of its vertex slots (3 rows of 5 grid
+// slots, then the pole).  P is even, so every patch spans exactly STIV_BR
+// bands and STIV_BC columns; the lists depend only on whether the patch
+// touches the north pole (first band), the south pole (last band) and whether
+// it owns the pole vertex (first column block).  At P = 2 one patch touches
+// both poles; it is examined once with the north pole and all grid
+// primitives, and once (SOUTH) with the south pole's primitives alone.  16
+// variants, built once per CTA.  The primitives are listed for the lanes that
+// stand for them (v, t, e) and given as bit masks over their first slots for
+// the lanes that test against all of them (vm, qm, hm, fm).
 struct PatchTopo {
-  unsigned char v_slot[MAXV];      // vertices owned by the patch
-  int t_slots[MAXT];               // triangles: 3 slots, 6 bits each
-  short e_slots[MAXE];             // edges: 2 slots, 6 bits each (either order)
+  unsigned char v[16];             // vertices owned by the patch: slot
+  unsigned short t[32];            // triangles: 3 slots, 4 bits each
+  unsigned char e[32];             // edges: 2 slots, 4 bits each
   int nv, nt, ne;
+  unsigned vm;                     // owned vertices
+  unsigned qm;                     // quads: both triangles, the downward and the diagonal edge at (row, column)
+  unsigned hm;                     // edges along a row
+  unsigned fm;                     // pole fan (triangles and edges), bits 0-3 by column
+  int frow;                        // first slot of the fan's row
 };
-constexpr int NVAR = 8;
-static_assert(NS <= 32, "one lane per vertex slot");
-static_assert(STIV_BR == 2 && STIV_BC % 2 == 0, "patches tile every even-order grid exactly");
-
-struct PatchSm {
-  float m[NS];                     // bound on the FP32 error of the slot's box ends (before any widening)
-  float x[3][NS], d[3][NS];        // FP32: X0 - origin of vesicle i, X1 - X0
-  float lo[3][NS], hi[3][NS];      // FP32 conservative swept box of each slot (frame of vesicle i)
-  int vid[NS];                     // global vertex id of each slot (-1: unused)
-  const PatchTopo* tp;
-  unsigned char vf[MAXV], tf[MAXT], ef[MAXE];
-  float4 vlo[MAXV], vhi[MAXV];     // boxes of the filtered vertices, in vf order
-  int nv, nt, ne, nvf, ntf, nef;
-  int P, I, J, ves;
-  float box[6];
-};
+constexpr int NVAR = 16;
+static_assert(STIV_BR == 2 && STIV_BC == 4, "slot and bit layout");
 
 struct WarpSm {
-  PatchSm A, B;
-  float4 elo[MAXE], ehi[MAXE];     // boxes of A's filtered edges, in ef order
-  unsigned q1[QCAP];
-  float dx;                        // bound on the FP32 position error in this frame
+  float4 x[2 * NSLOT], d[2 * NSLOT];    // patch A's slots, then B's: X0 - origin of vesicle i (w: vertex id), X1 - X0
+  float4 lo[2 * NSLOT], hi[2 * NSLOT];  // conservative FP32 swept boxes (frame of vesicle i)
+  uint4 miss[NSLOT];                    // per slot of B, axis x, y, z: A's slots it misses (low half: A's lo above, high: A's hi below)
+  unsigned q[QCAP];                     // primitive pairs: four slots (5 bits each, + 16 on B), kind << 20
 };
 
 struct narrow_args {
@@ -117,66 +115,52 @@ __device__ __forceinline__ double vtx(const void* X, size_t i) {
 // ---------------------------------------------------------------------------
 // staging
 // ---------------------------------------------------------------------------
-// Topology variant var = first | last << 1 | pole-owner << 2 (see PatchTopo),
-// built by one warp.
+// Topology variant var = first | last << 1 | pole-owner << 2 | south-only << 3
+// (see PatchTopo), built by one warp.
 __device__ void build_topo(PatchTopo& T, int var, int lane) {
   const int rq = STIV_BR, ncol = STIV_BC;
-  bool first = var & 1, last = (var >> 1) & 1, j0 = (var >> 2) & 1;
-  int rown = rq + (last ? 1 : 0);
-  int nvg = rown * ncol;
-  int npole = (first && j0 ? 1 : 0) + (last && j0 ? 1 : 0);
-  int ntq = 2 * rq * ncol;
-  int nfan = (first ? ncol : 0) + (last ? ncol : 0);
-  int ne = rown * ncol + 2 * rq * ncol + nfan;
-  if (lane == 0) { T.nv = nvg + npole; T.nt = ntq + nfan; T.ne = ne; }
-  for (int k = lane; k < nvg + npole; k += 32) {
-    int slot;
-    if (k < nvg) slot = slot_of(k / ncol, k % ncol);
-    else if (first && j0 && k == nvg) slot = SN;
-    else slot = SS;
-    T.v_slot[k] = (unsigned char)slot;
+  bool first = var & 1, last = (var >> 1) & 1, j0 = (var >> 2) & 1, so = (var >> 3) & 1;
+  int rown = so ? 0 : rq + (last ? 1 : 0);
+  bool north = first && !so, pole = first || last;
+  int nvg = rown * ncol, ntq = so ? 0 : 2 * rq * ncol, nfan = pole ? ncol : 0;
+  int nh = rown * ncol, nq = so ? 0 : 2 * rq * ncol;
+  int frow = north ? 0 : slot_of(rq, 0);
+  if (lane == 0) {
+    T.nv = nvg + (pole && j0 ? 1 : 0); T.nt = ntq + nfan; T.ne = nh + nq + nfan;
+    unsigned rows = 0, quads = 0;
+    for (int rr = 0; rr < rown; ++rr) rows |= 0xFu << slot_of(rr, 0);
+    if (!so) for (int rr = 0; rr < rq; ++rr) quads |= 0xFu << slot_of(rr, 0);
+    T.vm = rows | (pole && j0 ? 1u << PSLOT : 0u);
+    T.hm = rows; T.qm = quads; T.fm = pole ? 0xFu : 0u; T.frow = frow;
   }
+  for (int k = lane; k < nvg + 1 && k < 16; k += 32)
+    T.v[k] = (unsigned char)(k < nvg ? slot_of(k / ncol, k % ncol) : PSLOT);
   for (int k = lane; k < ntq + nfan; k += 32) {
     int s0, s1, s2;
     if (k < ntq) {
       int q = k >> 1, rr = q / ncol, cc = q % ncol;
-      if ((k & 1) == 0) { s0 = slot_of(rr, cc); s1 = slot_of(rr + 1, cc); s2 = slot_of(rr + 1, cc + 1); }
-      else { s0 = slot_of(rr, cc); s1 = slot_of(rr + 1, cc + 1); s2 = slot_of(rr, cc + 1); }
+      s0 = slot_of(rr, cc);
+      s1 = (k & 1) == 0 ? slot_of(rr + 1, cc) : slot_of(rr + 1, cc + 1);
+      s2 = (k & 1) == 0 ? slot_of(rr + 1, cc + 1) : slot_of(rr, cc + 1);
     } else {
-      int k2 = k - ntq;
-      if (first && k2 < ncol) { s0 = SN; s1 = slot_of(0, k2); s2 = slot_of(0, k2 + 1); }
-      else { int cc = first ? k2 - ncol : k2; s0 = SS; s1 = slot_of(rq, cc + 1); s2 = slot_of(rq, cc); }
+      int cc = k - ntq;
+      s0 = PSLOT; s1 = frow + (north ? cc : cc + 1); s2 = frow + (north ? cc + 1 : cc);
     }
-    T.t_slots[k] = s0 | (s1 << 6) | (s2 << 12);
+    T.t[k] = (unsigned short)(s0 | (s1 << 4) | (s2 << 8));
   }
-  for (int k = lane; k < ne; k += 32) {
+  for (int k = lane; k < nh + nq + nfan; k += 32) {
     int sa, sb;
-    int nh = rown * ncol;
     if (k < nh) {
-      int rr = k / ncol, cc = k % ncol;
-      sa = slot_of(rr, cc); sb = slot_of(rr, cc + 1);
-    } else if (k < nh + 2 * rq * ncol) {
-      int k2 = k - nh, q = k2 >> 1, rr = q / ncol, cc = q % ncol;
-      sa = slot_of(rr, cc);
-      sb = ((k2 & 1) == 0) ? slot_of(rr + 1, cc) : slot_of(rr + 1, cc + 1);
+      sa = slot_of(k / ncol, k % ncol); sb = sa + 1;
+    } else if (k < nh + nq) {
+      int k2 = k - nh, q = k2 >> 1;
+      sa = slot_of(q / ncol, q % ncol);
+      sb = sa + STIV_BC + 1 + (k2 & 1);
     } else {
-      int k2 = k - nh - 2 * rq * ncol;
-      if (first && k2 < ncol) { sa = slot_of(0, k2); sb = SN; }
-      else { int cc = first ? k2 - ncol : k2; sa = slot_of(rq, cc); sb = SS; }
+      sa = frow + k - nh - nq; sb = PSLOT;
     }
-    T.e_slots[k] = (short)(sa | (sb << 6));
+    T.e[k] = (unsigned char)(sa | (sb << 4));
   }
-}
-
-// Global vertex id of slot k of the patch starting at grid row r0, column c0.
-__device__ __forceinline__ int slot_vid(int k, int r0, int c0, int W, int P, bool first, bool last) {
-  if (k < SN) {
-    int rr = k / (STIV_BC + 1), cc = k % (STIV_BC + 1), col = c0 + cc;
-    if (col >= W) col -= W;
-    return (r0 + rr) * W + col;
-  }
-  if (k == SN) return first ? W * (P + 1) : -1;
-  return last ? W * (P + 1) + 1 : -1;
 }
 
 // Order-preserving int image of a float (-0 just below +0) and its inverse:
@@ -186,49 +170,6 @@ __device__ __forceinline__ int fkey32(float f) {
   return i >= 0 ? i : i ^ 0x7FFFFFFF;
 }
 __device__ __forceinline__ float fkey_val(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7FFFFFFF); }
-
-// One vertex slot: FP32 frame coordinates and the slot's conservative FP32
-// swept box (also returned in b; vesicle j's widened by d_m, rounded up).  The
-// exact box is not staged: the FP32 box ends are within m of the exact ones
-// (m stored per slot), which decides almost every exact box test; the rare
-// undecided pair reads the FP64 values (stage 2).  off: FP32 offset of the
-// vesicle's frame origin in the pair frame.
-template <bool MIXED, bool DM>
-__device__ __forceinline__ void stage_slot(PatchSm& S, const float* fp, int vid, int k, const float* off, float dx,
-                                           float* b, float padf, const float* org) {
-  int v = vid >= 0 ? vid : 0;
-  S.vid[k] = vid;
-  float4 fx = ((const float4*)fp)[2 * v], fd = ((const float4*)fp)[2 * v + 1];
-  float xf[3], df[3];
-  float f0[3] = {fx.x, fx.y, fx.z}, f1[3] = {fd.x, fd.y, fd.z};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    if (MIXED) {   // the staging holds the FP32 vertices themselves
-      xf[c] = f0[c] - org[c];   // one rounding, as the FP64 form's staging
-      df[c] = f1[c] - f0[c];
-    } else {
-      xf[c] = f0[c];
-      df[c] = f1[c];
-    }
-  }
-  float mmax = 0.0f;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    float x = xf[c] + off[c], d = df[c];
-    S.x[c][k] = x;
-    S.d[c][k] = d;
-    float m = dx + 4.7683716e-7f * (fabsf(x) + fabsf(d));  // 2^-21 (|x| + |d|)
-    mmax = fmaxf(mmax, m);
-    if (DM) m = __fadd_ru(m, padf);                        // + d_m
-    float lo = vid >= 0 ? fminf(x, x + d) - m : INFINITY;
-    float hi = vid >= 0 ? fmaxf(x, x + d) + m : -INFINITY;
-    S.lo[c][k] = lo;
-    S.hi[c][k] = hi;
-    b[c] = lo;
-    b[3 + c] = hi;
-  }
-  S.m[k] = mmax;
-}
 
 // Bound on the error of a component of the difference of two FP32 frame
 // positions of the same vesicle: each is x = fl(xf + off) with xf the
@@ -241,229 +182,116 @@ __device__ __forceinline__ float same_side_err(float R, float offm) {
   return 1.01f * 5.9604645e-8f * (4.0f * R + 2.0f * offm);
 }
 
-// Lane -> slot of the packed staging and culling: lanes 0-14 hold the 15 grid
-// slots of patch A, lanes 15-29 those of patch B, lane 30 A's pole slot and
-// lane 31 B's (a patch touches at most one pole, except at P = 2, where the
-// south-pole slots of a patch that has both take a second pass).  Returns
-// the slot (-1: none) and whether it belongs to B.
-__device__ __forceinline__ int packed_slot(int lane, bool fA, bool lA, bool fB, bool lB, bool& onB) {
-  if (lane < 30) {
-    onB = lane >= 15;
-    return onB ? lane - 15 : lane;
-  }
-  onB = lane == 31;
-  bool f = onB ? fB : fA, l = onB ? lB : lA;
-  return f ? SN : (l ? SS : -1);
+// One patch of a patch pair, as its lanes see it.
+struct PatchRef {
+  int P, I, J, ves, pole;          // pole: vertex id of the pole slot (-1: none)
+  const PatchTopo* tp;
+};
+__device__ __forceinline__ PatchRef patch_ref(const PatchTopo* topo, int P, int ves, int patch) {
+  PatchRef r;
+  bool so = patch & SOUTH;
+  int nbc = stiv_ncol_blocks(P), k = patch & (SOUTH - 1);
+  r.P = P; r.ves = ves; r.I = k / nbc; r.J = k % nbc;
+  bool f = r.I == 0, l = r.I == stiv_nband_blocks(P) - 1;
+  r.pole = f && !so ? 2 * P * (P + 1) : (l ? 2 * P * (P + 1) + 1 : -1);
+  r.tp = topo + ((f ? 1 : 0) | (l ? 2 : 0) | (r.J == 0 ? 4 : 0) | (so ? 8 : 0));
+  return r;
 }
 
-// Stage the two patches of a patch pair (A: patch pa of vesicle i, unshifted;
-// B: patch pb of vesicle j at its periodic image) in one pass over the lanes
-// (packed_slot), both patches' loads in flight together; patch boxes by warp
-// reduction.
+// Stage the two patches of a patch pair (A: of vesicle i, unshifted; B: of
+// vesicle j at its periodic image) in one pass over the lanes: lanes 0-14 the
+// grid slots of A, lane 15 A's pole, lanes 16-30 and 31 the same for B.  Each
+// slot gets its FP32 frame coordinates and a conservative FP32 swept box
+// (vesicle j's widened by d_m, rounded up): the box ends lie within m of the
+// exact ones.  Returns in gap the margin by which two staged box ends that
+// pass each other prove that the exact ones do (3 m on both sides; with
+// d_m > 0 plus 2^-21 d_m for the roundings of the widening), and in dmax the
+// largest displacement component.
 template <bool MIXED, bool DM>
-__device__ __noinline__ void stage_pair(WarpSm& ws, const narrow_args& a, const PatchTopo* topo,
-                                        const stiv_pair_info& pi, int pa, int pb, int lane) {
-  int vi = pi.vi, vj = pi.vj;
-  float dx = pi.frame.w;
-  int PA = pi.Pij & 0xFFFF, PB = pi.Pij >> 16;
-  int nbcA = stiv_ncol_blocks(PA), nbcB = stiv_ncol_blocks(PB);
-  int IA = pa / nbcA, JA = pa % nbcA, IB = pb / nbcB, JB = pb % nbcB;
-  bool fA = IA == 0, lA = IA == stiv_nband_blocks(PA) - 1, fB = IB == 0, lB = IB == stiv_nband_blocks(PB) - 1;
-  // this lane's side: shift, frame offset, widening and origin of its vesicle
-  auto stage_one = [&](bool onB, int k, float* b) {
-    int P = onB ? PB : PA, I = onB ? IB : IA, J = onB ? JB : JA;
-    int v = onB ? vj : vi;
-    float off[3] = {onB ? pi.frame.x : 0.f, onB ? pi.frame.y : 0.f, onB ? pi.frame.z : 0.f};
-    float org[3] = {0.f, 0.f, 0.f};
-    if (MIXED) {
-      float4 o = ((const float4*)a.vorg)[v];
-      org[0] = o.x; org[1] = o.y; org[2] = o.z;
-    }
-    bool f = onB ? fB : fA, l = onB ? lB : lA;
-    int vid = slot_vid(k, I * STIV_BR, J * STIV_BC, 2 * P, P, f, l);
-    stage_slot<MIXED, DM>(onB ? ws.B : ws.A, a.fprep + (size_t)v * a.fstride, vid, k, off, dx, b,
-                          onB ? __double2float_ru(a.dm) : 0.0f, org);
-  };
-  float b[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  bool onB;
-  int k = packed_slot(lane, fA, lA, fB, lB, onB);
-  if (k >= 0) stage_one(onB, k, b);
-  if ((fA && lA) || (fB && lB)) {
-    // P = 2: a patch with both poles; its south-pole slot (lane 0 for A,
-    // lane 15 for B, each on its own side)
-    bool two = lane == 0 ? (fA && lA) : lane == 15 ? (fB && lB) : false;
-    if (two) {
-      float b2[6];
-      stage_one(lane == 15, SS, b2);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) { b[c] = fminf(b[c], b2[c]); b[3 + c] = fmaxf(b[3 + c], b2[3 + c]); }
-    }
+__device__ __forceinline__ void stage_pair(WarpSm& ws, const narrow_args& a, const PatchRef& A, const PatchRef& B,
+                                           float4 frame, int lane, float& gap, float& dmax) {
+  bool onB = lane >= 16;
+  int k = lane & 15;
+  int P = onB ? B.P : A.P, W = 2 * P, v = onB ? B.ves : A.ves;
+  int r0 = (onB ? B.I : A.I) * STIV_BR, c0 = (onB ? B.J : A.J) * STIV_BC;
+  int rr = k / (STIV_BC + 1), col = c0 + k - rr * (STIV_BC + 1);
+  if (col >= W) col -= W;
+  int vid = k == PSLOT ? (onB ? B.pole : A.pole) : (r0 + rr) * W + col;
+  const float4* fp = (const float4*)(a.fprep + (size_t)v * a.fstride) + 2 * (vid >= 0 ? vid : 0);
+  float4 x = fp[0], d = fp[1];
+  if (MIXED) {   // the staging holds the FP32 vertices themselves: one rounding each, as the FP64 form's staging
+    float4 o = ((const float4*)a.vorg)[v];
+    d = make_float4(d.x - x.x, d.y - x.y, d.z - x.z, 0.f);
+    x = make_float4(x.x - o.x, x.y - o.y, x.z - o.z, 0.f);
   }
-  float bA[6], bB[6];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    float la = onB ? INFINITY : b[c], ha = onB ? -INFINITY : b[3 + c];
-    float lb = onB ? b[c] : INFINITY, hb = onB ? b[3 + c] : -INFINITY;
-    bA[c] = fkey_val(__reduce_min_sync(0xffffffffu, fkey32(la)));
-    bA[3 + c] = fkey_val(__reduce_max_sync(0xffffffffu, fkey32(ha)));
-    bB[c] = fkey_val(__reduce_min_sync(0xffffffffu, fkey32(lb)));
-    bB[3 + c] = fkey_val(__reduce_max_sync(0xffffffffu, fkey32(hb)));
+  if (onB) { x.x = x.x + frame.x; x.y = x.y + frame.y; x.z = x.z + frame.z; }
+  x.w = __int_as_float(vid);
+  ws.x[lane] = x;
+  ws.d[lane] = d;
+  float mx = frame.w + 4.7683716e-7f * (fabsf(x.x) + fabsf(d.x));   // 2^-21 (|x| + |d|)
+  float my = frame.w + 4.7683716e-7f * (fabsf(x.y) + fabsf(d.y));
+  float mz = frame.w + 4.7683716e-7f * (fabsf(x.z) + fabsf(d.z));
+  // positive floats order as their bits
+  gap = 6.0f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(mx, fmaxf(my, mz)))));
+  dmax = __uint_as_float(
+      __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fabsf(d.x), fmaxf(fabsf(d.y), fabsf(d.z))))));
+  if (DM) {
+    float padf = __double2float_ru(a.dm);
+    gap += 4.7683716e-7f * padf;
+    if (onB) { mx = __fadd_ru(mx, padf); my = __fadd_ru(my, padf); mz = __fadd_ru(mz, padf); }
   }
-  if (lane < 6) { ws.A.box[lane] = bA[lane]; ws.B.box[lane] = bB[lane]; }
-  if (lane == 0) {
-    const PatchTopo* tA = topo + ((fA ? 1 : 0) | (lA ? 2 : 0) | (JA == 0 ? 4 : 0));
-    const PatchTopo* tB = topo + ((fB ? 1 : 0) | (lB ? 2 : 0) | (JB == 0 ? 4 : 0));
-    ws.A.tp = tA; ws.A.nv = tA->nv; ws.A.nt = tA->nt; ws.A.ne = tA->ne;
-    ws.A.P = PA; ws.A.I = IA; ws.A.J = JA; ws.A.ves = vi;
-    ws.B.tp = tB; ws.B.nv = tB->nv; ws.B.nt = tB->nt; ws.B.ne = tB->ne;
-    ws.B.P = PB; ws.B.I = IB; ws.B.J = JB; ws.B.ves = vj;
-    ws.dx = dx;
+  float4 lo = make_float4(fminf(x.x, x.x + d.x) - mx, fminf(x.y, x.y + d.y) - my, fminf(x.z, x.z + d.z) - mz, 0.f);
+  float4 hi = make_float4(fmaxf(x.x, x.x + d.x) + mx, fmaxf(x.y, x.y + d.y) + my, fmaxf(x.z, x.z + d.z) + mz, 0.f);
+  if (vid < 0) {
+    lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+    hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
   }
+  ws.lo[lane] = lo;
+  ws.hi[lane] = hi;
   __syncwarp();
 }
 
-// Global id of primitive k of a staged patch (vertex id, triangle id, or edge index).
-__device__ int prim_gid(const PatchSm& S, int kind, int k) {
-  int P = S.P, W = 2 * P;
-  const int rq = STIV_BR, ncol = STIV_BC;
-  int r0 = S.I * STIV_BR, c0 = S.J * STIV_BC;
-  bool first = S.I == 0;
-  if (kind == 0) return S.vid[S.tp->v_slot[k]];
-  if (kind == 1) {
-    int ntq = 2 * rq * ncol;
-    if (k < ntq) { int q = k >> 1, rr = q / ncol, cc = q % ncol; return 2 * ((r0 + rr) * W + c0 + cc) + (k & 1); }
-    int k2 = k - ntq;
-    if (first && k2 < ncol) return 4 * P * P + c0 + k2;
-    return 4 * P * P + W + c0 + (first ? k2 - ncol : k2);
+// Which slot boxes of A each slot of B misses, per axis and side, as bits:
+// lane k and lane k + 16 take slot k of B against the lower and the upper
+// eight slots of A.  A difference of box ends is negative exactly when they
+// miss, so its sign bit is shifted into the mask.  Returns whether some
+// difference lies in [0, gap): then a pair of boxes may overlap in FP32 and
+// not exactly.  (A primitive's box is the union of its slots' boxes, so it
+// misses a box on an axis and side exactly when all its slots do.)
+__device__ __forceinline__ bool slot_masks(WarpSm& ws, float gap, int lane) {
+  int k = lane & 15, h = lane >> 4;
+  float4 bl = ws.lo[NSLOT + k], bh = ws.hi[NSLOT + k];
+  unsigned lx = 0, ly = 0, lz = 0, hx = 0, hy = 0, hz = 0, near = 0xFFFFFFFFu;
+#pragma unroll
+  for (int q = 7; q >= 0; --q) {
+    float4 al = ws.lo[8 * h + q], ah = ws.hi[8 * h + q];
+    unsigned d0 = __float_as_uint(bh.x - al.x), d1 = __float_as_uint(bh.y - al.y), d2 = __float_as_uint(bh.z - al.z);
+    unsigned d3 = __float_as_uint(ah.x - bl.x), d4 = __float_as_uint(ah.y - bl.y), d5 = __float_as_uint(ah.z - bl.z);
+    lx = __funnelshift_l(d0, lx, 1); ly = __funnelshift_l(d1, ly, 1); lz = __funnelshift_l(d2, lz, 1);
+    hx = __funnelshift_l(d3, hx, 1); hy = __funnelshift_l(d4, hy, 1); hz = __funnelshift_l(d5, hz, 1);
+    near = min(near, min(min(d0, min(d1, d2)), min(d3, min(d4, d5))));   // negative ones are large as integers
   }
-  int e = S.tp->e_slots[k];
-  int u = S.vid[e & 63], v = S.vid[(e >> 6) & 63];
-  return stiv_edge_index(P, min(u, v), max(u, v));
+  unsigned wx = lx | (hx << 16), wy = ly | (hy << 16), wz = lz | (hz << 16);
+  unsigned ox = __shfl_xor_sync(0xffffffffu, wx, 16), oy = __shfl_xor_sync(0xffffffffu, wy, 16),
+           oz = __shfl_xor_sync(0xffffffffu, wz, 16);
+  if (h == 0) ws.miss[k] = make_uint4(wx | (ox << 8), wy | (oy << 8), wz | (oz << 8), 0u);
+  bool unsure = __any_sync(0xffffffffu, near < __float_as_uint(gap));
+  return unsure;
 }
 
-__device__ __forceinline__ void slot_box(const PatchSm& S, int sl, float* b) {
-  b[0] = S.lo[0][sl]; b[1] = S.lo[1][sl]; b[2] = S.lo[2][sl];
-  b[3] = S.hi[0][sl]; b[4] = S.hi[1][sl]; b[5] = S.hi[2][sl];
+__device__ __forceinline__ uint4 and4(uint4 a, uint4 b) { return make_uint4(a.x & b.x, a.y & b.y, a.z & b.z, 0u); }
+// Hits (bits 0-15) of primitives whose per-axis misses are w: no axis and side missed.
+__device__ __forceinline__ unsigned hits_of(uint4 w) {
+  unsigned m = w.x | w.y | w.z;
+  return ~(m | (m >> 16)) & 0xFFFFu;
 }
-__device__ __forceinline__ void merge_box(const PatchSm& S, int sl, float* b) {
-  b[0] = fminf(b[0], S.lo[0][sl]); b[1] = fminf(b[1], S.lo[1][sl]); b[2] = fminf(b[2], S.lo[2][sl]);
-  b[3] = fmaxf(b[3], S.hi[0][sl]); b[4] = fmaxf(b[4], S.hi[1][sl]); b[5] = fmaxf(b[5], S.hi[2][sl]);
-}
-__device__ __forceinline__ void tri_box(const PatchSm& S, int k, float* b) {
-  int t = S.tp->t_slots[k];
-  slot_box(S, t & 63, b); merge_box(S, (t >> 6) & 63, b); merge_box(S, (t >> 12) & 63, b);
-}
-__device__ __forceinline__ void edge_box(const PatchSm& S, int k, float* b) {
-  int e = S.tp->e_slots[k];
-  slot_box(S, e & 63, b); merge_box(S, (e >> 6) & 63, b);
-}
+__device__ __forceinline__ uint4 shr4(uint4 a, int k) { return make_uint4(a.x >> k, a.y >> k, a.z >> k, 0u); }
+// The pole slot's bit of both halves, spread over its half.
+__device__ __forceinline__ unsigned pole_half(unsigned w) { return ((w >> PSLOT) & 0x00010001u) * 0xFFFFu; }
+__device__ __forceinline__ uint4 pole4(uint4 w) { return make_uint4(pole_half(w.x), pole_half(w.y), pole_half(w.z), 0u); }
+
 __device__ __forceinline__ bool fbox_hit(const float* a, const float* b) {
   return a[0] <= b[3] && b[0] <= a[3] && a[1] <= b[4] && b[1] <= a[4] && a[2] <= b[5] && b[2] <= a[5];
-}
-
-// Compact the primitives of both staged patches whose FP32 boxes overlap the
-// other patch's box (A's against B's box, B's against A's); the boxes of the
-// kept vertices (and of A's kept edges) are stored in the compacted order for
-// the stage-1 loops.  A primitive's box (the min and max of its slots' boxes)
-// misses a box on an axis exactly when all its slots lie above it there
-// (every lo > its hi) or all below (every hi < its lo), so the test reads
-// per-slot bit masks instead of merging boxes.  Both patches share each pass
-// over the lanes: the slot masks come from the packed slot layout of the
-// staging, and the primitive lists of A and B are concatenated.
-__device__ void filter_pair(WarpSm& ws, int lane) {
-  PatchSm& A = ws.A;
-  PatchSm& B = ws.B;
-  bool fA = A.I == 0, lA = A.I == stiv_nband_blocks(A.P) - 1;
-  bool fB = B.I == 0, lB = B.I == stiv_nband_blocks(B.P) - 1;
-  unsigned abA[3], blA[3], abB[3], blB[3];
-  {
-    bool onB;
-    int k = packed_slot(lane, fA, lA, fB, lB, onB);
-    bool in = k >= 0;
-    const PatchSm& S = onB ? B : A;
-    const float* ob = onB ? A.box : B.box;
-    int poleA = fA ? SN : SS, poleB = fB ? SN : SS;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      float lo = in ? S.lo[c][k] : 0.0f, hi = in ? S.hi[c][k] : 0.0f;
-      unsigned ma = __ballot_sync(0xffffffffu, in && lo > ob[3 + c]);
-      unsigned mb = __ballot_sync(0xffffffffu, in && hi < ob[c]);
-      abA[c] = (ma & 0x7FFFu) | (((ma >> 30) & 1u) << poleA);
-      abB[c] = ((ma >> 15) & 0x7FFFu) | (((ma >> 31) & 1u) << poleB);
-      blA[c] = (mb & 0x7FFFu) | (((mb >> 30) & 1u) << poleA);
-      blB[c] = ((mb >> 15) & 0x7FFFu) | (((mb >> 31) & 1u) << poleB);
-    }
-    if ((fA && lA) || (fB && lB)) {   // P = 2: the south-pole slots of two-pole patches
-      bool two = lane == 0 ? (fA && lA) : lane == 15 ? (fB && lB) : false;
-      const PatchSm& S2 = lane == 15 ? B : A;
-      const float* ob2 = lane == 15 ? A.box : B.box;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float lo = two ? S2.lo[c][SS] : 0.0f, hi = two ? S2.hi[c][SS] : 0.0f;
-        unsigned ma = __ballot_sync(0xffffffffu, two && lo > ob2[3 + c]);
-        unsigned mb = __ballot_sync(0xffffffffu, two && hi < ob2[c]);
-        abA[c] |= (ma & 1u) << SS; abB[c] |= ((ma >> 15) & 1u) << SS;
-        blA[c] |= (mb & 1u) << SS; blB[c] |= ((mb >> 15) & 1u) << SS;
-      }
-    }
-  }
-  const unsigned lower = (1u << lane) - 1u;
-#pragma unroll 1
-  for (int kind = 0; kind < 3; ++kind) {
-    int nA = kind == 0 ? A.nv : kind == 1 ? A.nt : A.ne;
-    int nB = kind == 0 ? B.nv : kind == 1 ? B.nt : B.ne;
-    int n = nA + nB, baseA = 0, baseB = 0;
-    for (int k0 = 0; k0 < n; k0 += 32) {
-      int kk = k0 + lane;
-      bool valid = kk < n, isB = kk >= nA;
-      int k = isB ? kk - nA : kk;
-      PatchSm& S = isB ? B : A;
-      bool hit = false;
-      unsigned sm = 0;
-      if (valid) {
-        if (kind == 0) {
-          sm = 1u << S.tp->v_slot[k];
-        } else if (kind == 1) {
-          int t = S.tp->t_slots[k];
-          sm = (1u << (t & 63)) | (1u << ((t >> 6) & 63)) | (1u << ((t >> 12) & 63));
-        } else {
-          int e = S.tp->e_slots[k];
-          sm = (1u << (e & 63)) | (1u << ((e >> 6) & 63));
-        }
-        unsigned a0 = isB ? abB[0] : abA[0], a1 = isB ? abB[1] : abA[1], a2 = isB ? abB[2] : abA[2];
-        unsigned b0 = isB ? blB[0] : blA[0], b1 = isB ? blB[1] : blA[1], b2 = isB ? blB[2] : blA[2];
-        hit = (a0 & sm) != sm && (b0 & sm) != sm && (a1 & sm) != sm && (b1 & sm) != sm && (a2 & sm) != sm &&
-              (b2 & sm) != sm;
-      }
-      unsigned m = __ballot_sync(0xffffffffu, hit);
-      unsigned mB = __ballot_sync(0xffffffffu, valid && isB);
-      if (hit) {
-        int pos = isB ? baseB + __popc(m & mB & lower) : baseA + __popc(m & ~mB & lower);
-        unsigned char* out = kind == 0 ? S.vf : kind == 1 ? S.tf : S.ef;
-        out[pos] = (unsigned char)k;
-        if (kind == 0) {
-          float b[6];
-          slot_box(S, S.tp->v_slot[k], b);
-          S.vlo[pos] = make_float4(b[0], b[1], b[2], 0.f);
-          S.vhi[pos] = make_float4(b[3], b[4], b[5], 0.f);
-        }
-        if (kind == 2 && !isB) {
-          float b[6];
-          edge_box(A, k, b);
-          ws.elo[pos] = make_float4(b[0], b[1], b[2], 0.f);
-          ws.ehi[pos] = make_float4(b[3], b[4], b[5], 0.f);
-        }
-      }
-      baseA += __popc(m & ~mB);
-      baseB += __popc(m & mB);
-    }
-    if (lane == 0) {
-      if (kind == 0) { A.nvf = baseA; B.nvf = baseB; }
-      else if (kind == 1) { A.ntf = baseA; B.ntf = baseB; }
-      else { A.nef = baseA; B.nef = baseB; }
-    }
-  }
-  __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
@@ -656,23 +484,12 @@ __device__ __forceinline__ bool certain_sign4(float c0, float c1, float c2, floa
   return (c0 > E && c1 > E && c2 > E && c3 > E) || (c0 < -E && c1 < -E && c2 < -E && c3 < -E);
 }
 
-// Stage 3a: 1 if the cubic certainly has no root in [0, 1] (Bernstein
-// coefficients of one sign), 0 otherwise (also when it may vanish
-// identically, which the FP64 test reports as degenerate).
-__device__ int bernstein_reject(const cubic32& q) {
-  if (fabsf(q.k0) <= q.E && fabsf(q.k1) <= q.E && fabsf(q.k2) <= q.E && fabsf(q.k3) <= q.E) return 0;
-  float b1 = q.k0 + q.k1 * (1.f / 3.f), b2 = q.k0 + (2.f * q.k1 + q.k2) * (1.f / 3.f), b3 = q.k0 + q.k1 + q.k2 + q.k3;
-  return certain_sign4(q.k0, b1, b2, b3, q.E) ? 1 : 0;
-}
-
-// Stage 3a with d_m > 0: 1 if the point certainly stays farther than d_m from
-// the triangle's plane (the lines farther than d_m apart) over the whole step,
-// so that g = f^2 - d_m^2 |m|^2 stays positive and the FP64 degree-six test
-// finds no candidate time.  min |f| over [0, 1] is bounded below by the
-// smallest Bernstein coefficient of the cubic (all of one sign beyond the
-// error bound E); |m(t)| <= |n0| + |n1| + |n2| is bounded above from the FP32
-// cross products with their error bounds (the error model of cubic_fp32); a
-// margin of 1e-12 of the squared magnitudes covers the FP64 evaluation of g.
+// The d_m band.  min |f| over an interval is bounded below by the smallest
+// Bernstein coefficient of the cubic (all of one sign beyond the error bound
+// E); |m(t)| <= |n0| + |n1| + |n2| is bounded above from the FP32 cross
+// products with their error bounds (the error model of cubic_fp32); a margin
+// of 1e-12 of the squared magnitudes covers the FP64 evaluation of
+// g = f^2 - d_m^2 |m|^2.
 // Right-hand side of the band test: (d_m max|m|)^2 with its margins.
 __device__ float band_rhs(const cubic32& q, float ep, float dm) {
   float A = q.A2, Ad = q.Ad2, ed = q.ed;
@@ -693,11 +510,140 @@ __device__ __forceinline__ bool out_of_band(float c0, float c1, float c2, float 
   return fmin > 0.f && fmin * fmin * (1.f - 1e-5f) > rhs;
 }
 
-__device__ int band_reject(int kind, const f3* x, const f3* d, float ep, float es, float dm) {
-  cubic32 q = cubic_fp32<true>(kind, x, d, ep, es);
-  float b1 = q.k0 + q.k1 * (1.f / 3.f), b2 = q.k0 + (2.f * q.k1 + q.k2) * (1.f / 3.f), b3 = q.k0 + q.k1 + q.k2 + q.k3;
-  if (!certain_sign4(q.k0, b1, b2, b3, q.E)) return 0;
-  return out_of_band(q.k0, b1, b2, b3, q.E, band_rhs(q, ep, dm)) ? 1 : 0;
+// ---------------------------------------------------------------------------
+// Stage 3a.  The cubic f = c . m, m = a x b, from the difference vectors at
+// both ends of the step (index 0: t = 0, 1: t = 1; each moves linearly, so f
+// is a blossom): VF a, b the triangle's edges from its first vertex, EE the two
+// edges; c from the vertex (the first edge's first point) to that vertex (the
+// second edge's first point).  B: the Bernstein coefficients of f on [0, 1],
+//   B0 = c0.n00, B1 = (c1.n00 + c0.n01) / 3, B2 = (c1.n01 + c0.n11) / 3, B3 = c1.n11,
+// n00 = a0 x b0, n01 = a1 x b0 + a0 x b1, n11 = a1 x b1; E bounds the error of
+// each against the exact ones.  With e the error of a component of a
+// difference and U, V, W the largest components of c, a, b, each coefficient is
+// a mean of triple products of six terms, so its error is at most
+// 6 ((U + e)(V + e)(W + e) - U V W + r U V W), the first part written without
+// cancellation, r the roundings per term.
+// ---------------------------------------------------------------------------
+struct blossom {
+  f3 a0, b0, c0, a1, b1, c1;
+  f3 n00, n01, n11;
+  float B0, B1, B2, B3, E, U, V, W;
+};
+
+// p, q: first points of the first and second primitive; h: VF second vertex of
+// the triangle, EE second point of the first edge; g: last point.
+__device__ __forceinline__ blossom blossom_fp32(bool ee, f3 p, f3 q, f3 h, f3 g, f3 dp, f3 dq, f3 dh, f3 dg, float e) {
+  blossom r;
+  f3 t = ee ? p : q, dt = ee ? dp : dq;
+  r.a0 = fsub(h, t); r.b0 = fsub(g, q); r.c0 = fsub(q, p);
+  r.a1 = fadd(r.a0, fsub(dh, dt)); r.b1 = fadd(r.b0, fsub(dg, dq)); r.c1 = fadd(r.c0, fsub(dq, dp));
+  r.n00 = fcross(r.a0, r.b0);
+  r.n01 = fadd(fcross(r.a1, r.b0), fcross(r.a0, r.b1));
+  r.n11 = fcross(r.a1, r.b1);
+  r.B0 = fdot(r.c0, r.n00);
+  r.B1 = (fdot(r.c1, r.n00) + fdot(r.c0, r.n01)) * (1.f / 3.f);
+  r.B2 = (fdot(r.c1, r.n01) + fdot(r.c0, r.n11)) * (1.f / 3.f);
+  r.B3 = fdot(r.c1, r.n11);
+  r.U = fmaxf(amax3(r.c0), amax3(r.c1));
+  r.V = fmaxf(amax3(r.a0), amax3(r.a1));
+  r.W = fmaxf(amax3(r.b0), amax3(r.b1));
+  float Ve = r.V + e, We = r.W + e, UV = r.U * r.V, mx = fmaxf(r.U, fmaxf(r.V, r.W));
+  // 7.5 = 1.25 x 6; roundings: 96 U32 per term; the last term covers FP64
+  r.E = 7.5f * e * (fmaf(Ve, We, fmaf(r.U, We, UV))) + 4.3e-5f * UV * r.W + 1.3e-9f * mx * mx * mx;
+  return r;
+}
+
+// Separation certificate: 1 if the FP64 contact test certainly reports neither
+// a contact nor a degenerate pair because the two primitives stay apart along
+// one direction over the whole step, 0 if undecided.
+//
+// With C the vectors from the points of the first primitive to those of the
+// second at t = 0 and t = 1 (VF: c + {0, a, b}; EE: c + {0, b} - {0, a}), a
+// direction v with v . C > 0 for all of them separates the primitives at every
+// time, in whatever way both move together: pairs of two vesicles carried along
+// by one flow, whose swept boxes overlap over the long common path, are told
+// apart here.  v runs through the first NIT iterates towards the point of the
+// hull of the C closest to the origin (their mean, then towards the C lowest
+// along v).
+//
+// Why it decides the FP64 test.  Let n = v / |v|, n . C >= delta, and t a time
+// at which the test forms the inside weights: f(t) is zero up to rounding there
+// (with d_m > 0, |f| <= d_m |m|).  If the weights passed, the least-squares
+// residual r, perpendicular to a and b, would be a mean of the C with weights in
+// [-tau, 1 + tau], hence n . r >= delta - 12 tau Cm (Cm >= every component of
+// the C), while |r| = |f| / |m|.  The guard: the Bernstein coefficients of
+// m(0) . m(t) exceed 1e-3 SA SB (SA, SB the larger squared lengths of a and b,
+// at most 3 V^2 and 3 W^2), so |m(t)| >= 1e-3 sqrt(SA SB) on [0, 1].  Then the
+// determinant |m|^2 of the normal equations is positive in FP64 (relative error
+// below 4e-9), their rounding keeps tau below 4e-9 (1 + Cm / min(V, W)) < 1e-5
+// (Cm < 1e3 min(V, W) is required), the rounding of f over a bracket of the root
+// gives |f| / |m| < 1e-9 Cm, and that of the positions at t less than the error
+// e of the FP32 differences (e covers 2^-32 of the coordinates themselves).  So
+// delta = 2e-4 Cm beyond the FP32 errors excludes a contact.  With d_m > 0,
+// g = f^2 - d_m^2 |m|^2 is zero up to 2.4e-6 Cm^2 |m|^2, so |f| / |m| <= d_m +
+// 1.6e-3 sqrt(3) Cm, within delta = 1.00001 d_m + 5e-3 Cm.  A pair is degenerate
+// otherwise only when every FP64 coefficient of the polynomial is exactly zero:
+// f (with d_m > 0: g) is shown to be away from zero at t = 0 or t = 1.
+template <bool DM, int NIT>
+__device__ __forceinline__ int separation_reject(bool ee, const blossom& q, float e, float dm) {
+  float VW = q.V * q.W, Cm = q.U + q.V + q.W;
+  float g0 = fdot(q.n00, q.n00), g1 = 0.5f * fdot(q.n00, q.n01), g2 = fdot(q.n00, q.n11);
+  // error of the g: |m(0)| <= 3 V W times that of a x b
+  float em = 6.0f * e * (q.V + q.W) + 4e-6f * VW;
+  bool ok = fminf(g0, fminf(g1, g2)) > VW * fmaf(9.1e-3f, VW, 6.1f * em) && Cm < 1e3f * fminf(q.V, q.W);
+  if (DM) {   // |g| = ||f| - d_m |m|| (|f| + d_m |m|) away from zero
+    float m0 = dm * fnorm(q.n00), m1 = dm * fnorm(q.n11), eg = fmaf(dm, em, q.E);
+    ok = ok && (fabsf(fabsf(q.B0) - m0) > eg + 0.01f * m0 || fabsf(fabsf(q.B3) - m1) > eg + 0.01f * m1);
+  } else {
+    ok = ok && (fabsf(q.B0) > q.E || fabsf(q.B3) > q.E);
+  }
+  if (!ok) return 0;
+  float marg = e + (DM ? 1.00001f * dm + 5.1e-3f * Cm : 2.1e-4f * Cm);
+  float al = ee ? -0.25f : 1.f / 6.f, be = ee ? 0.25f : 1.f / 6.f;
+  f3 v = {fmaf(be, q.b0.x + q.b1.x, fmaf(al, q.a0.x + q.a1.x, 0.5f * (q.c0.x + q.c1.x))),
+          fmaf(be, q.b0.y + q.b1.y, fmaf(al, q.a0.y + q.a1.y, 0.5f * (q.c0.y + q.c1.y))),
+          fmaf(be, q.b0.z + q.b1.z, fmaf(al, q.a0.z + q.a1.z, 0.5f * (q.c0.z + q.c1.z)))};
+#pragma unroll 1
+  for (int it = 0;; ++it) {
+    float sa0 = fdot(v, q.a0), sb0 = fdot(v, q.b0), sc0 = fdot(v, q.c0);
+    float sa1 = fdot(v, q.a1), sb1 = fdot(v, q.b1), sc1 = fdot(v, q.c1);
+    // the lowest C at each end: c + fa a + fb b
+    float m0 = ee ? fminf(sb0, 0.f) - fmaxf(sa0, 0.f) : fminf(fminf(sa0, sb0), 0.f);
+    float m1 = ee ? fminf(sb1, 0.f) - fmaxf(sa1, 0.f) : fminf(fminf(sa1, sb1), 0.f);
+    m0 += sc0; m1 += sc1;
+    float mn = fminf(m0, m1);
+    if (mn > 1.00001f * marg * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z))) return 1;
+    if (it + 1 == NIT) return 0;
+    bool end = m1 < m0;
+    f3 A = end ? q.a1 : q.a0, B = end ? q.b1 : q.b0, C = end ? q.c1 : q.c0;
+    float sa = end ? sa1 : sa0, sb = end ? sb1 : sb0;
+    float fa = ee ? (sa > 0.f ? -1.f : 0.f) : (sa < 0.f && sa <= sb ? 1.f : 0.f);
+    float fb = ee ? (sb < 0.f ? 1.f : 0.f) : (sb < 0.f && sb < sa ? 1.f : 0.f);
+    f3 w = fat(fat(C, fa, A), fb, B);
+    f3 u = fsub(w, v);
+    float t = __fdividef(-fdot(v, u), fmaxf(fdot(u, u), 1e-30f));
+    v = fat(v, fminf(fmaxf(t, 0.0f), 1.0f), u);
+  }
+}
+
+// Stage 3a on one pair: 1 if the FP64 test certainly finds nothing.  The cubic
+// keeps one sign over the step (with d_m > 0: keeps |f| above d_m |m|; |m(t)| is
+// at most the largest of |n00|, |n01| / 2, |n11|), or the first direction
+// separates the primitives.
+template <bool DM>
+__device__ __forceinline__ int reject_fp32(bool ee, const blossom& q, float e, float dm) {
+  float lo = fminf(fminf(q.B0, q.B1), fminf(q.B2, q.B3)), hi = fmaxf(fmaxf(q.B0, q.B1), fmaxf(q.B2, q.B3));
+  float f = fmaxf(lo, -hi) - q.E;   // > 0: |f| >= this over the step
+  if (DM) {
+    float VW = q.V * q.W;
+    float n2 = fmaxf(fmaxf(fdot(q.n00, q.n00), 0.25f * fdot(q.n01, q.n01)), fdot(q.n11, q.n11));
+    float mm = n2 * rsqrtf(fmaxf(n2, 1e-30f)) * 1.000001f + 1e-15f + 6.0f * e * (q.V + q.W) + 4e-6f * VW;
+    float dmm = dm * mm * 1.000001f, s = 162.f * q.U * VW;
+    if (f > 0.f && f * f * (1.f - 1e-5f) > dmm * dmm * (1.f + 1e-5f) + 1e-12f * (s * s + dmm * dmm)) return 1;
+  } else if (f > 0.f) {
+    return 1;
+  }
+  return separation_reject<DM, 1>(ee, q, e, dm);
 }
 
 // ---------------------------------------------------------------------------
@@ -1171,29 +1117,6 @@ __device__ __noinline__ int ccd64_dm(int kind, const d3* X0, const d3* D, double
 }
 
 // ---------------------------------------------------------------------------
-// stages 2-4 on queued pairs
-// ---------------------------------------------------------------------------
-// queue entry: kind (0 = VF A->B, 1 = VF B->A, 2 = EE) << 16 | x << 8 | y
-__device__ __forceinline__ void entry_slots(const WarpSm& ws, unsigned e, int& kind, int& x, int& y, int* sl,
-                                            const PatchSm*& SA, const PatchSm*& SB) {
-  kind = e >> 16; x = (e >> 8) & 0xFF; y = e & 0xFF;
-  SA = (kind == 1) ? &ws.B : &ws.A;   // side holding the first primitive (vertex / edge)
-  SB = (kind == 1) ? &ws.A : &ws.B;
-  if (kind < 2) {
-    sl[0] = SA->tp->v_slot[x];
-    int t = SB->tp->t_slots[y];
-    sl[1] = t & 63; sl[2] = (t >> 6) & 63; sl[3] = (t >> 12) & 63;
-  } else {
-    int ea = SA->tp->e_slots[x], eb = SB->tp->e_slots[y];
-    sl[0] = ea & 63; sl[1] = (ea >> 6) & 63; sl[2] = eb & 63; sl[3] = (eb >> 6) & 63;
-  }
-}
-
-__device__ __forceinline__ const PatchSm& point_side(int kind, int q, const PatchSm* SA, const PatchSm* SB) {
-  return (q == 0 || (kind == 2 && q == 1)) ? *SA : *SB;
-}
-
-// ---------------------------------------------------------------------------
 // global pair descriptors (stages 3b and 4)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long make_desc(int r, int type, int ga, int gb) {
@@ -1257,35 +1180,24 @@ __device__ __forceinline__ void push_global(ulonglong2* list, int64_t cap, int64
   }
 }
 
-__device__ __forceinline__ void load_f32(const int* sl, int kind, const PatchSm* SA, const PatchSm* SB, f3* xq,
-                                         f3* dq) {
-  for (int q = 0; q < 4; ++q) {
-    const PatchSm& S = point_side(kind, q, SA, SB);
-    xq[q] = {S.x[0][sl[q]], S.x[1][sl[q]], S.x[2][sl[q]]};
-    dq[q] = {S.d[0][sl[q]], S.d[1][sl[q]], S.d[2][sl[q]]};
-  }
-}
-
-// The exact FP64 swept-box test of a queued primitive pair from the vertex
-// values themselves (FP64, or the FP32 values widened), the second vesicle's
-// points at the pair's periodic image (added in FP64) and, with d_m > 0, its
-// per-vertex boxes widened by d_m: the test that defines the pairs tested,
-// for the rare pair whose FP32 boxes and their error bound do not decide it.
+// The exact FP64 swept-box test of a queued primitive pair (slots sl; na of
+// them on the first primitive) from the vertex values themselves (FP64, or the
+// FP32 values widened), the second vesicle's points at the pair's periodic
+// image (added in FP64) and, with d_m > 0, its per-vertex boxes widened by d_m:
+// the test that defines the pairs tested, for the rare pair whose FP32 boxes
+// and their error bound do not decide it.
 template <bool MIXED, bool DM>
-__device__ __noinline__ bool exact_box_hit(const narrow_args& a, int r, int kind, const PatchSm* SA, const PatchSm* SB,
-                                           const int* sl) {
+__device__ __noinline__ bool exact_box_hit(const WarpSm& ws, const narrow_args& a, int r, int na, const int* sl) {
   const stiv_pair_info& pi = a.pinfo[r];
   int code = pi.code;
   int sB[3] = {code / 9 - 1, (code / 3) % 3 - 1, code % 3 - 1};
-  int na = kind == 2 ? 2 : 1;
   double lo[2][3], hi[2][3];
   for (int side = 0; side < 2; ++side)
     for (int c = 0; c < 3; ++c) { lo[side][c] = INFINITY; hi[side][c] = -INFINITY; }
   for (int q = 0; q < 4; ++q) {
-    const PatchSm* S = q < na ? SA : SB;
-    bool onB = (q < na) == (kind == 1);   // the point belongs to vesicle j (patch B)
+    bool onB = sl[q] >= NSLOT;   // the point belongs to vesicle j (patch B)
     int side = q < na ? 0 : 1;
-    int v = S->vid[sl[q]];
+    int v = __float_as_int(ws.x[sl[q]].w);
     int P = onB ? (pi.Pij >> 16) : (pi.Pij & 0xFFFF);
     int nv = stiv_nverts(P);
     size_t vb = (size_t)(onB ? pi.voff_j : pi.voff_i) + v;
@@ -1306,109 +1218,55 @@ __device__ __noinline__ bool exact_box_hit(const narrow_args& a, int r, int kind
   return hit;
 }
 
-// Stage 2 (exact box) and 3a (Bernstein) on up to n entries of q1; survivors
-// go to the global list of stage 3b (of stage 4 when the FP32 rejection is
-// off) as descriptors.
+// Whether the exact boxes of a pair whose staged boxes overlap do: certainly
+// when the staged ones overlap by gap on every axis, else by the exact test.
 template <bool MIXED, bool DM>
-__device__ __noinline__ void stage_filter(WarpSm& ws, int n, int lane, int r, const narrow_args& a,
-                                          long long& nprim) {
-  bool keep = false;
-  ulonglong2 desc = make_ulonglong2(0ull, 0ull);
-  if (lane < n) {
-    unsigned e = ws.q1[lane];
-    int kind, x, y, sl[4];
-    const PatchSm *SA, *SB;
-    entry_slots(ws, e, kind, x, y, sl, SA, SB);
-    // exact FP64 swept-box overlap
-    int na = kind == 2 ? 2 : 1;
-    bool hit = true;
-    {
-      // Each staged FP32 box end lies within m of the exact FP64 box end of
-      // its slot (in the pair frame), so a slot's exact box contains its
-      // FP32 box shrunk by 2m at each end.  If the shrunk boxes of the two
-      // primitives overlap on every axis (boxes shrunk by 3 M, M the largest
-      // m of the primitive's slots, which also covers the rounding of the
-      // shrinking), the exact boxes overlap; the pair came through the
-      // outward boxes of stage 1, so only the pairs in between need the exact
-      // test, on the FP64 values.  With d_m > 0 vesicle j's boxes are widened
-      // by d_m on both sides: FP32 rounded up, FP64 as computed per vertex;
-      // 2^-21 d_m covers the difference of the two roundings.
-      float ma = SA->m[sl[0]], mb = SB->m[sl[na]];
-      if (na == 2) ma = fmaxf(ma, SA->m[sl[1]]);
-      for (int q = na + 1; q < 4; ++q) mb = fmaxf(mb, SB->m[sl[q]]);
-      float gap = 3.0f * (ma + mb);
-      if (DM) gap += 4.7683716e-7f * __double2float_ru(a.dm);
-      bool sure = true;
-      for (int c = 0; c < 3; ++c) {
-        float alo = SA->lo[c][sl[0]], ahi = SA->hi[c][sl[0]];
-        if (na == 2) { alo = fminf(alo, SA->lo[c][sl[1]]); ahi = fmaxf(ahi, SA->hi[c][sl[1]]); }
-        float blo = SB->lo[c][sl[na]], bhi = SB->hi[c][sl[na]];
-        for (int q = na + 1; q < 4; ++q) { blo = fminf(blo, SB->lo[c][sl[q]]); bhi = fmaxf(bhi, SB->hi[c][sl[q]]); }
-        sure = sure && alo + gap <= bhi && blo + gap <= ahi;
-      }
-      if (!sure) hit = exact_box_hit<MIXED, DM>(a, r, kind, SA, SB, sl);
-    }
-    if (hit) {
-      ++nprim;
-      keep = true;
-      if (DM && !a.exact_only) {   // d_m > 0: drop pairs that certainly stay out of the d_m band
-        f3 xq[4], dq[4];
-        load_f32(sl, kind, SA, SB, xq, dq);
-        keep = !band_reject(kind == 2 ? 1 : 0, xq, dq, ws.dx, 2.0f * ws.dx, (float)a.dm);
-      } else if (!a.exact_only) {
-        f3 xq[4], dq[4];
-        load_f32(sl, kind, SA, SB, xq, dq);
-        cubic32 q = cubic_fp32(kind == 2 ? 1 : 0, xq, dq, ws.dx, 2.0f * ws.dx);
-        keep = !bernstein_reject(q);
-      }
-      if (keep) {
-        unsigned long long v0 = (unsigned)SA->vid[sl[0]], v1, v2, v3;
-        if (kind < 2) {
-          v1 = (unsigned)SB->vid[sl[1]]; v2 = (unsigned)SB->vid[sl[2]]; v3 = (unsigned)SB->vid[sl[3]];
-        } else {
-          unsigned long long u = (unsigned)SA->vid[sl[1]];
-          if (u < v0) { v1 = v0; v0 = u; } else v1 = u;
-          unsigned long long p = (unsigned)SB->vid[sl[2]], q = (unsigned)SB->vid[sl[3]];
-          v2 = p < q ? p : q; v3 = p < q ? q : p;
-        }
-        // EE edge indices are formed by the FP64 stage for contacts only
-        desc.x = kind == 2 ? make_desc(r, kind, 0, 0) : make_desc(r, kind, (int)v0, prim_gid(*SB, 1, y));
-        desc.y = v0 | (v1 << 16) | (v2 << 32) | (v3 << 48);
-      }
+__device__ __forceinline__ bool box_hit(const WarpSm& ws, const narrow_args& a, int r, int na, const int* sl, float gap) {
+  float4 l0 = ws.lo[sl[0]], h0 = ws.hi[sl[0]], l1 = ws.lo[sl[3]], h1 = ws.hi[sl[3]];
+#pragma unroll
+  for (int q = 1; q < 3; ++q) {
+    float4 l = ws.lo[sl[q]], h = ws.hi[sl[q]];
+    if (q < na) {
+      l0.x = fminf(l0.x, l.x); l0.y = fminf(l0.y, l.y); l0.z = fminf(l0.z, l.z);
+      h0.x = fmaxf(h0.x, h.x); h0.y = fmaxf(h0.y, h.y); h0.z = fmaxf(h0.z, h.z);
+    } else {
+      l1.x = fminf(l1.x, l.x); l1.y = fminf(l1.y, l.y); l1.z = fminf(l1.z, l.z);
+      h1.x = fmaxf(h1.x, h.x); h1.y = fmaxf(h1.y, h.y); h1.z = fmaxf(h1.z, h.z);
     }
   }
-  if (a.exact_only) push_global(a.q2, a.Q2, &a.ctr[15], &a.ctr[STIV_C_STATUS], keep, desc, lane);
-  else push_global(a.q3, a.Q3, &a.ctr[14], &a.ctr[STIV_C_STATUS], keep, desc, lane);
+  if (h1.x - l0.x >= gap && h1.y - l0.y >= gap && h1.z - l0.z >= gap && h0.x - l1.x >= gap && h0.y - l1.y >= gap &&
+      h0.z - l1.z >= gap)
+    return true;
+  return exact_box_hit<MIXED, DM>(ws, a, r, na, sl);
 }
 
-// Queue the hits of one stage-1 test (n1: the queue length, the same in every
-// lane); 32 queued entries go through stages 2 and 3a.
-template <bool MIXED, bool DM>
-__device__ __forceinline__ void enqueue(WarpSm& ws, bool hit, unsigned entry, int lane, int r, const narrow_args& a,
-                                        long long& nprim, int& n1) {
-  unsigned m = __ballot_sync(0xffffffffu, hit);
-  if (!m) return;
-  if (hit) ws.q1[n1 + __popc(m & ((1u << lane) - 1u))] = entry;
-  n1 += __popc(m);
-  if (n1 >= 32) {
-    __syncwarp();
-    stage_filter<MIXED, DM>(ws, 32, lane, r, a, nprim);
-    unsigned rest = (lane + 32 < n1) ? ws.q1[lane + 32] : 0;
-    __syncwarp();
-    if (lane + 32 < n1) ws.q1[lane] = rest;
-    n1 -= 32;
-    __syncwarp();
+// Global triangle id of the triangle with slots s0, s1, s2 (relative to its
+// patch) of a patch.
+__device__ __forceinline__ int tri_gid(const PatchRef& R, int s0, int s1, int s2) {
+  int W = 2 * R.P, r0 = R.I * STIV_BR, c0 = R.J * STIV_BC;
+  if (s0 == PSLOT) {
+    bool north = s2 > s1;
+    return 4 * R.P * R.P + (north ? 0 : W) + c0 + (north ? s1 : s2 - R.tp->frow);
   }
+  int rr = s0 / (STIV_BC + 1), cc = s0 - rr * (STIV_BC + 1);
+  return 2 * ((r0 + rr) * W + c0 + cc) + (s1 == s0 + STIV_BC + 1 ? 0 : 1);
 }
 
-// Stages 1-3a: one warp per patch pair.  Three CTAs per SM leave 80
-// registers a thread (four leave 64, with spills in the staging code).
+// Stages 1-3a: one warp per patch pair.
+//
+// Stage 1 without lists: a lane stands for a vertex, a triangle and an edge of
+// patch B, and finds the primitives of A whose boxes meet its own from the slot
+// masks, all at once (shifts of the masks stand for A's triangles and edges).
+// The hits are counted, laid out in the warp's queue by one scan, and go
+// through stages 2 and 3a on full warps; survivors are compacted in place and
+// pushed together.
 template <bool MIXED, bool DM>
 __global__ void __launch_bounds__(NW * 32, 3) narrow_kernel(narrow_args a) {
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ PatchTopo topo[NVAR];
   WarpSm& ws = ((WarpSm*)smraw)[threadIdx.x >> 5];
-  int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
+  const unsigned lower = (1u << lane) - 1u;
   for (int var = threadIdx.x >> 5; var < NVAR; var += NW) build_topo(topo[var], var, lane);
   __syncthreads();
   int64_t nwork = a.ctr[STIV_C_PATCH];
@@ -1422,49 +1280,139 @@ __global__ void __launch_bounds__(NW * 32, 3) narrow_kernel(narrow_args a) {
     long long next = 0;
     if (lane == 0) next = (long long)atomicAdd((unsigned long long*)&a.ctr[10], 1ull);
     uint64_t w = a.work[item];
-    int r = (int)(w >> 32), pa = (int)((w >> 16) & 0xFFFF), pb = (int)(w & 0xFFFF);
-    stiv_pair_info pi = a.pinfo[r];
-    stage_pair<MIXED, DM>(ws, a, topo, pi, pa, pb, lane);
-    filter_pair(ws, lane);
-    int n1 = 0;
-    // stage 1: FP32 boxes.  VF: vertices of A vs triangles of B (0), vertices of B vs triangles of A (1)
-#pragma unroll 1
-    for (int dir = 0; dir < 2; ++dir) {
-      const PatchSm& V = dir == 0 ? ws.A : ws.B;
-      const PatchSm& T = dir == 0 ? ws.B : ws.A;
-      for (int y0 = 0; y0 < T.ntf; y0 += 32) {
-        int yk = y0 + lane;
-        bool valid = yk < T.ntf;
-        int y = valid ? T.tf[yk] : 0;
-        float tb[6];
-        tri_box(T, y, tb);
-#pragma unroll 1
-        for (int xk = 0; xk < V.nvf; ++xk) {
-          float4 lo = V.vlo[xk], hi = V.vhi[xk];
-          float vb[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
-          bool hit = valid && fbox_hit(vb, tb);
-          enqueue<MIXED, DM>(ws, hit, ((unsigned)dir << 16) | ((unsigned)V.vf[xk] << 8) | (unsigned)y, lane, r, a, nprim, n1);
-        }
-      }
-    }
-    if (a.include_ee) {
-      for (int y0 = 0; y0 < ws.B.nef; y0 += 32) {
-        int yk = y0 + lane;
-        bool valid = yk < ws.B.nef;
-        int y = valid ? ws.B.ef[yk] : 0;
-        float eb[6];
-        edge_box(ws.B, y, eb);
-#pragma unroll 1
-        for (int xk = 0; xk < ws.A.nef; ++xk) {
-          float4 lo = ws.elo[xk], hi = ws.ehi[xk];
-          float ab[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
-          bool hit = valid && fbox_hit(ab, eb);
-          enqueue<MIXED, DM>(ws, hit, (2u << 16) | ((unsigned)ws.A.ef[xk] << 8) | (unsigned)y, lane, r, a, nprim, n1);
-        }
-      }
-    }
+    const int r = (int)(w >> 32);
+    const stiv_pair_info* pi = a.pinfo + r;
+    const float4 frame = pi->frame;
+    const int Pij = pi->Pij;
+    const PatchRef A = patch_ref(topo, Pij & 0xFFFF, pi->vi, (int)((w >> 16) & 0xFFFF));
+    const PatchRef B = patch_ref(topo, Pij >> 16, pi->vj, (int)(w & 0xFFFF));
+    float gap, dmax;
+    stage_pair<MIXED, DM>(ws, a, A, B, frame, lane, gap, dmax);
+    const bool unsure = slot_masks(ws, gap, lane);
     __syncwarp();
-    if (n1 > 0) stage_filter<MIXED, DM>(ws, n1, lane, r, a, nprim);
+    // stage 1
+    unsigned hv = 0, ht = 0, he = 0, hd = 0;   // hits of this lane's vertex, triangle and edge of B
+    {
+      const PatchTopo& TA = *A.tp;
+      const PatchTopo& TB = *B.tp;
+      const unsigned qm = TA.qm, fm = TA.fm;
+      const int fr = TA.frow;
+      if (lane < TB.nv) {   // against A's triangles: bits 0-8 first of a quad, 10-13 fan; 16-24 second of a quad
+        uint4 m = ws.miss[TB.v[lane]];
+        uint4 dg = and4(m, shr4(m, STIV_BC + 2));
+        hv = (hits_of(and4(dg, shr4(m, STIV_BC + 1))) & qm) | ((hits_of(and4(dg, shr4(m, 1))) & qm) << 16);
+        if (fm) hv |= (hits_of(and4(and4(shr4(m, fr), shr4(m, fr + 1)), pole4(m))) & fm) << 10;
+      }
+      if (lane < TB.nt) {   // against A's vertices
+        int t = TB.t[lane];
+        ht = hits_of(and4(and4(ws.miss[t & 15], ws.miss[(t >> 4) & 15]), ws.miss[t >> 8])) & TA.vm;
+      }
+      if (a.include_ee && lane < TB.ne) {   // against A's edges: along a row, down; diagonal, fan
+        int t = TB.e[lane];
+        uint4 m = and4(ws.miss[t & 15], ws.miss[t >> 4]);
+        he = (hits_of(and4(m, shr4(m, 1))) & TA.hm) | ((hits_of(and4(m, shr4(m, STIV_BC + 1))) & qm) << 16);
+        hd = hits_of(and4(m, shr4(m, STIV_BC + 2))) & qm;
+        if (fm) hd |= (hits_of(and4(shr4(m, fr), pole4(m))) & fm) << 16;
+      }
+    }
+    int cnt = __popc(hv) + __popc(ht) + __popc(he) + __popc(hd), off = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { int v = __shfl_up_sync(0xffffffffu, off, o); if (lane >= o) off += v; }
+    const int total = __shfl_sync(0xffffffffu, off, 31);
+    off -= cnt;
+    if (lane == 0) nprim += total;
+    const float e = 2.0f * frame.w + 4.0f * U32 * dmax + 2e-12f;   // error of a difference component
+    for (int base = 0; base < total; base += QCAP) {
+      // entries [base, base + QCAP) of the concatenated hits into the queue
+      {
+        int pos = off - base;
+        const PatchTopo& TB = *B.tp;
+        const int fr = A.tp->frow;
+        auto put = [&](unsigned x) { if (pos >= 0 && pos < QCAP) ws.q[pos] = x; ++pos; };
+        unsigned own = NSLOT + (hv ? TB.v[lane] : 0u);
+        for (unsigned m = hv; m; m &= m - 1) {
+          unsigned b = __ffs(m) - 1, s0, s1, s2;
+          if (b >= 16) { s0 = b - 16; s1 = s0 + STIV_BC + 2; s2 = s0 + 1; }
+          else if (b < 10) { s0 = b; s1 = s0 + STIV_BC + 1; s2 = s1 + 1; }
+          else { s0 = PSLOT; s1 = fr + b - 10 + (fr ? 1 : 0); s2 = fr + b - 10 + (fr ? 0 : 1); }
+          put(own | (s0 << 5) | (s1 << 10) | (s2 << 15) | (1u << 20));
+        }
+        unsigned t = ht ? TB.t[lane] : 0u;
+        unsigned tri = ((NSLOT + (t & 15u)) << 5) | ((NSLOT + ((t >> 4) & 15u)) << 10) | ((NSLOT + (t >> 8)) << 15);
+        for (unsigned m = ht; m; m &= m - 1) put((__ffs(m) - 1) | tri);
+        unsigned ed = he | hd ? TB.e[lane] : 0u;
+        ed = ((NSLOT + (ed & 15u)) << 5) | ((NSLOT + (ed >> 4)) << 15) | (2u << 20);
+        for (unsigned m = he; m; m &= m - 1) {
+          unsigned b = __ffs(m) - 1, s0 = b & 15;
+          put(ed | s0 | ((s0 + (b < 16 ? 1 : STIV_BC + 1)) << 10));
+        }
+        for (unsigned m = hd; m; m &= m - 1) {
+          unsigned b = __ffs(m) - 1, s0 = b < 16 ? b : fr + b - 16;
+          put(ed | s0 | ((b < 16 ? s0 + STIV_BC + 2 : PSLOT) << 10));
+        }
+      }
+      __syncwarp();
+      // stages 2 and 3a: p, q, h, g the slots of blossom_fp32's points (VF: the
+      // vertex and the triangle; EE: first points of the two edges, then second)
+      const int n = min(total - base, QCAP);
+      int kept = 0;
+      for (int b0 = 0; b0 < n; b0 += 32) {
+        bool keep = b0 + lane < n;
+        unsigned en = 0;
+        if (keep) {
+          en = ws.q[b0 + lane];
+          const int p = en & 31, q = (en >> 5) & 31, h = (en >> 10) & 31, g = (en >> 15) & 31;
+          const bool ee = (en >> 20) == 2;
+          if (unsure) {
+            int sl[4] = {p, ee ? h : q, ee ? q : h, g};
+            keep = box_hit<MIXED, DM>(ws, a, r, ee ? 2 : 1, sl, gap);
+            if (!keep) --nprim;
+          }
+          if (keep && !a.exact_only) {
+            float4 xp = ws.x[p], xq = ws.x[q], xh = ws.x[h], xg = ws.x[g];
+            float4 dp = ws.d[p], dq = ws.d[q], dh = ws.d[h], dg = ws.d[g];
+            blossom bl = blossom_fp32(ee, {xp.x, xp.y, xp.z}, {xq.x, xq.y, xq.z}, {xh.x, xh.y, xh.z},
+                                      {xg.x, xg.y, xg.z}, {dp.x, dp.y, dp.z}, {dq.x, dq.y, dq.z}, {dh.x, dh.y, dh.z},
+                                      {dg.x, dg.y, dg.z}, e);
+            keep = !reject_fp32<DM>(ee, bl, e, (float)a.dm);
+          }
+        }
+        unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (keep) ws.q[kept + __popc(m & lower)] = en;   // below b0 + 32: read by every lane above
+        kept += __popc(m);
+        __syncwarp();
+      }
+      // descriptors of the kept pairs: vertex ids in the order the contact test
+      // takes its points (EE edge indices are formed by the FP64 stage, for
+      // contacts only)
+      if (kept) {
+        ulonglong2* list = a.exact_only ? a.q2 : a.q3;
+        int64_t cap = a.exact_only ? a.Q2 : a.Q3;
+        unsigned long long k0 = 0;
+        if (lane == 0) k0 = atomicAdd((unsigned long long*)&a.ctr[a.exact_only ? 15 : 14], (unsigned long long)kept);
+        k0 = __shfl_sync(0xffffffffu, k0, 0);
+        for (int k = lane; k < kept; k += 32) {
+          unsigned en = ws.q[k];
+          const int p = en & 31, q = (en >> 5) & 31, h = (en >> 10) & 31, g = (en >> 15) & 31, kind = en >> 20;
+          unsigned long long v0 = (unsigned)__float_as_int(ws.x[p].w), v1 = (unsigned)__float_as_int(ws.x[q].w),
+                             v2 = (unsigned)__float_as_int(ws.x[h].w), v3 = (unsigned)__float_as_int(ws.x[g].w);
+          ulonglong2 d;
+          if (kind == 2) {
+            unsigned long long a0 = v0 < v2 ? v0 : v2, a1 = v0 < v2 ? v2 : v0, b0 = v1 < v3 ? v1 : v3,
+                               b1 = v1 < v3 ? v3 : v1;
+            d.x = make_desc(r, 2, 0, 0);
+            d.y = a0 | (a1 << 16) | (b0 << 32) | (b1 << 48);
+          } else {
+            const int t = kind == 0 ? NSLOT : 0;
+            d.x = make_desc(r, kind, (int)v0, tri_gid(kind == 0 ? B : A, q - t, h - t, g - t));
+            d.y = v0 | (v1 << 16) | (v2 << 32) | (v3 << 48);
+          }
+          if ((int64_t)(k0 + k) < cap) list[k0 + k] = d;
+          else atomicOr((unsigned long long*)&a.ctr[STIV_C_STATUS], STIV_F_WORK_OVERFLOW);
+        }
+      }
+      __syncwarp();
+    }
     item = __shfl_sync(0xffffffffu, next, 0);
   }
   for (int off = 16; off > 0; off >>= 1) nprim += __shfl_down_sync(0xffffffffu, nprim, off);
@@ -1482,6 +1430,7 @@ constexpr int PW = 8;          // warps per CTA
 constexpr int NPIECE = 16;     // level-0 pieces of [0, 1]
 constexpr int NLEVEL = 6;      // most refinement levels (finest piece: 1 / (16 * 32))
 constexpr int MAXTASK = 512;
+constexpr int NSEP = 5;        // directions of the separation test
 static_assert(NPIECE << (NLEVEL - 1) <= 1024, "piece index fits 10 bits");
 
 struct PieceWarp {
@@ -1517,6 +1466,15 @@ __global__ void __launch_bounds__(PW * 32, 4) pieces_kernel(narrow_args a) {
       f3 xq[4], dq[4];
       float ep, es;
       desc_points_f32(a, e, kind, xq, dq, ep, es);
+      bool apart;
+      {
+        float dmx = fmaxf(fmaxf(amax3(dq[0]), amax3(dq[1])), fmaxf(amax3(dq[2]), amax3(dq[3])));
+        float ed = 2.0f * ep + 4.0f * U32 * dmx + 2e-12f;
+        const bool ee = kind != 0;
+        blossom bl = blossom_fp32(ee, xq[0], ee ? xq[2] : xq[1], ee ? xq[1] : xq[2], xq[3], dq[0], ee ? dq[2] : dq[1],
+                                  ee ? dq[1] : dq[2], dq[3], ed);
+        apart = separation_reject<DM, NSEP>(ee, bl, ed, (float)a.dm);
+      }
       cubic32 q = cubic_fp32<DM>(kind, xq, dq, ep, es);
       for (int p = 0; p < 4; ++p) {
         W.x[lane][p][0] = xq[p].x; W.x[lane][p][1] = xq[p].y; W.x[lane][p][2] = xq[p].z;
@@ -1527,7 +1485,7 @@ __global__ void __launch_bounds__(PW * 32, 4) pieces_kernel(narrow_args a) {
       if (DM) W.rhs[lane] = band_rhs(q, ep, (float)a.dm);
       if (fabsf(q.k0) <= q.E && fabsf(q.k1) <= q.E && fabsf(q.k2) <= q.E && fabsf(q.k3) <= q.E) {
         W.fail[lane] = 1;   // may vanish identically: FP64 decides (degenerate)
-      } else {
+      } else if (!apart) {
         const float w = 1.0f / NPIECE;
 #pragma unroll 2
         for (int p = 0; p < NPIECE; ++p) {
@@ -1729,15 +1687,19 @@ __global__ void __launch_bounds__(128) patch_pairs_kernel(const int32_t* pv, con
     if (lane == 0) {
       // FP32 frame of the pair: origin of vesicle i; |FP32 position - exact
       // position| per component is bounded by 2^-22 (R_i + R_j + 2 |offset|)
-      // (rounding of X0 - origin, of the offset and of the frame change)
-      float o[3], dmax = 0.f;
+      // (rounding of X0 - origin, of the offset and of the frame change);
+      // 2^-32 of the coordinates themselves is added, so that the bound also
+      // stands above the FP64 rounding of positions far from the origin
+      float o[3], dmax = 0.f, ymax = 0.f;
       for (int c = 0; c < 3; ++c) {
         double d = ((double)vorg[4 * j + c] + s[c] * L[c]) - (double)vorg[4 * i + c];
         o[c] = (float)d;
         dmax = fmaxf(dmax, fabsf(o[c]));
+        ymax = fmaxf(ymax, fmaxf(fabsf(vorg[4 * i + c]), fabsf(vorg[4 * j + c])) + (s[c] ? (float)L[c] : 0.f));
       }
       stiv_pair_info p;
-      p.frame = make_float4(o[0], o[1], o[2], 2.3841858e-7f * (vorg[4 * i + 3] + vorg[4 * j + 3] + 2.0f * dmax));
+      float R = vorg[4 * i + 3] + vorg[4 * j + 3];
+      p.frame = make_float4(o[0], o[1], o[2], 2.3841858e-7f * (R + 2.0f * dmax) + 2.3283064e-10f * (ymax + R));
       p.vi = i; p.vj = j; p.code = code; p.Pij = Pi | (Pj << 16);
       p.voff_i = voff[i]; p.voff_j = voff[j];
       pinfo[r] = p;
@@ -1843,15 +1805,22 @@ __global__ void __launch_bounds__(128) patch_pairs_kernel(const int32_t* pv, con
         }
       }
       unsigned m = __ballot_sync(0xffffffffu, hit);
+      // at P = 2 a patch touches both poles: a further item per such patch for
+      // its south-pole primitives
+      const int sa = Pi == 2 ? 2 : 1, sb = Pj == 2 ? 2 : 1;
       if (m) {
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd((unsigned long long*)&ctr[STIV_C_PATCH], (unsigned long long)__popc(m));
+        int nm = __popc(m);
+        if (lane == 0)
+          base = atomicAdd((unsigned long long*)&ctr[STIV_C_PATCH], (unsigned long long)(nm * sa * sb));
         base = __shfl_sync(0xffffffffu, base, 0);
-        if (hit) {
-          int64_t k = (int64_t)base + __popc(m & ((1u << lane) - 1u));
-          if (k < W) work[k] = ((uint64_t)r << 32) | ((uint64_t)pa << 16) | (uint64_t)pb;
-          else atomicOr((unsigned long long*)&ctr[STIV_C_STATUS], STIV_F_WORK_OVERFLOW);
-        }
+        if (hit)
+          for (int z = 0; z < sa * sb; ++z) {
+            int64_t k = (int64_t)base + z * nm + __popc(m & ((1u << lane) - 1u));
+            int qa = pa | (z % sa ? SOUTH : 0), qb = pb | (z / sa ? SOUTH : 0);
+            if (k < W) work[k] = ((uint64_t)r << 32) | ((uint64_t)qa << 16) | (uint64_t)qb;
+            else atomicOr((unsigned long long*)&ctr[STIV_C_STATUS], STIV_F_WORK_OVERFLOW);
+          }
       }
     }
     __syncwarp();

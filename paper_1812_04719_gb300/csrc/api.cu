@@ -222,18 +222,22 @@ extern "C" int stiv_mesh_topology(int32_t P, int32_t* tri_dev, int32_t* edge_dev
 // Scratch of stiv_detect, carved from the handle's buffer.
 static int detect_layout(stiv_handle* h, int n, int p_max, const stiv_pairs* cand, const stiv_contacts* out,
                          detect_ws& w, bool carve) {
-  w.R = (int64_t)n * 64 + 1024;
-  w.Q = cand->capacity * 8 + 1024;
+  const bool brute = n <= STIV_BRUTE_MAX;   // no grid records and no candidate keys
+  const size_t units = brute ? (size_t)n * stiv_row_chunks(n) : 0;
+  w.R = brute ? 1 : (int64_t)n * 64 + 1024;
+  w.Q = brute ? 1 : cand->capacity * 8 + 1024;
   w.W = cand->capacity * 64 + 1024;
   if (w.W < out->capacity) w.W = out->capacity;
   w.C = out->capacity > 0 ? out->capacity : 1;
   w.Q3 = 16 * w.C + 4096;
   w.Q2 = (h->prm.exact_only || h->prm.d_m > 0.0 ? 32 : 4) * w.C + 4096;
   int64_t smax = w.R > w.Q ? w.R : w.Q;
-  if (w.C > smax) smax = w.C;
   w.sort_scratch_bytes = stiv_sort_scratch_impl(smax);
   size_t off = 0;
   size_t o_vbox = off; off = align_up(off + sizeof(double) * 6 * (size_t)n);
+  size_t o_fbox = off; off = align_up(off + sizeof(float) * 6 * (size_t)n);
+  size_t o_rwc = off; off = align_up(off + sizeof(int32_t) * units);
+  size_t o_rwk = off; off = align_up(off + sizeof(uint32_t) * STIV_ROW_KEEP * units);
   w.pstride = stiv_npatches(2 * p_max);
   size_t o_pbox = off; off = align_up(off + sizeof(float) * STIV_PBOX * (size_t)w.pstride * n);
   w.fstride = 8 * (int64_t)stiv_nverts(2 * p_max);
@@ -256,17 +260,22 @@ static int detect_layout(stiv_handle* h, int n, int p_max, const stiv_pairs* can
   size_t o_fr = off; off = align_up(off + sizeof(stiv_pair_info) * (size_t)cand->capacity);
   size_t o_q3 = off; off = align_up(off + sizeof(ulonglong2) * (size_t)w.Q3);
   size_t o_q2 = off; off = align_up(off + sizeof(ulonglong2) * (size_t)w.Q2);
+  // cleared together at the start of a detection
+  size_t o_ctr = off; off = align_up(off + sizeof(int64_t) * 32);
+  size_t o_rws = off; off = align_up(off + sizeof(int32_t) * ((units + STIV_ROW_SUM - 1) / STIV_ROW_SUM));
   size_t o_pc = off; off = align_up(off + sizeof(int32_t) * (size_t)cand->capacity);
   size_t o_pf = off; off = align_up(off + sizeof(int32_t) * (size_t)cand->capacity);
+  w.clear_bytes = off - o_ctr;
   size_t o_po = off; off = align_up(off + sizeof(int32_t) * (size_t)(cand->capacity + 1));
   size_t o_sg = off; off = align_up(off + sizeof(uint64_t) * (size_t)w.C);
   size_t o_sg2 = off; off = align_up(off + sizeof(uint64_t) * (size_t)w.C);
   size_t o_ti = off; off = align_up(off + sizeof(int32_t) * 4 * (size_t)w.C);
   size_t o_tf = off; off = align_up(off + sizeof(double) * 3 * (size_t)w.C);
-  size_t o_ctr = off; off = align_up(off + sizeof(int64_t) * 32);
   size_t o_ss = off; off = align_up(off + w.sort_scratch_bytes);
   if (!carve) return stiv_ws_reserve(h, off);
   char* b = (char*)h->ws;
+  w.fbox = (float*)(b + o_fbox); w.row_cnt = (int32_t*)(b + o_rwc); w.row_keep = (uint32_t*)(b + o_rwk);
+  w.row_sum = (int32_t*)(b + o_rws);
   w.vbox = (double*)(b + o_vbox); w.pbox = (float*)(b + o_pbox); w.grid = (double*)(b + o_grid);
   w.vorg = (float*)(b + o_vorg); w.fprep = (float*)(b + o_fprep);
   w.exact_only = h->prm.exact_only;
@@ -306,9 +315,7 @@ extern "C" int stiv_detect(stiv_handle* h, void* stream, int32_t n_ves, int32_t 
   int rc = detect_layout(h, n_ves, p_max, cand, out, w, false);
   if (rc) return rc;
   detect_layout(h, n_ves, p_max, cand, out, w, true);
-  STIV_CUDA(h, cudaMemsetAsync(w.ctr, 0, sizeof(int64_t) * 32, st));
-  STIV_CUDA(h, cudaMemsetAsync(w.pair_cnt, 0, sizeof(int32_t) * (size_t)cand->capacity, st));
-  STIV_CUDA(h, cudaMemsetAsync(w.pair_fill, 0, sizeof(int32_t) * (size_t)cand->capacity, st));
+  STIV_CUDA(h, cudaMemsetAsync(w.ctr, 0, w.clear_bytes, st));
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   rc = stiv_broad_phase(h, st, n_ves, p_max, p_dev, vert_off_dev, verts_dev, cand, w, w.ctr);

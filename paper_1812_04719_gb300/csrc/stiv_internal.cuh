@@ -25,6 +25,13 @@
 // patch lies in one cell.
 #define STIV_PBOX 40
 #define STIV_PBOX_CELLS 8
+// Candidate pairs by testing every pair of boxes up to this many vesicles;
+// beyond, by the Morton grid and its sorts.
+#define STIV_BRUTE_MAX 8192
+#define STIV_ROW_CHUNK 512   // boxes tested per unit of a row
+#define STIV_ROW_KEEP 32     // hits kept per unit
+#define STIV_ROW_SUM 256     // units per partial sum of their hits
+inline int stiv_row_chunks(int n) { return (n + STIV_ROW_CHUNK - 1) / STIV_ROW_CHUNK; }
 
 // ---------------------------------------------------------------------------
 // handle and scratch
@@ -106,6 +113,10 @@ struct __align__(16) stiv_pair_info {
 // Scratch layout used by stiv_detect (byte offsets into handle->ws).
 struct detect_ws {
   double* vbox;          // [N][6]
+  float* fbox;           // [6][N]  the same boxes in FP32, rounded outward
+  int32_t* row_cnt;      // [units]  all-pairs test: hits per unit
+  int32_t* row_sum;      // [units / STIV_ROW_SUM], cleared with ctr
+  uint32_t* row_keep;    // [units][STIV_ROW_KEEP]
   float* pbox;           // [N][pstride][6]
   int pstride;           // patches per vesicle at the largest order
   float* vorg;           // [N][4]  FP32 frame origin of each vesicle, and R = max |X - origin|
@@ -137,7 +148,8 @@ struct detect_ws {
   unsigned long long* seg2;  // [C]
   int32_t* tmp_i32;      // [C] temporaries for the contact permutation
   double* tmp_f64;       // [3C]
-  int64_t* ctr;          // [32] device counters
+  int64_t* ctr;          // [32] device counters; row_sum, pair_cnt and pair_fill follow
+  size_t clear_bytes;    // of these
   void* sort_scratch;
   size_t sort_scratch_bytes;
   int64_t R, Q, W, C;

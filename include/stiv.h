@@ -347,7 +347,7 @@ enum stiv_tune_param {
   STIV_TUNE_PIECES_CTAS = 1,   /* piece-test CTAs per SM                          */
   STIV_TUNE_FP64_BLOCKS = 2,   /* FP64 contact-test blocks per SM                 */
   STIV_TUNE_PATCH_BLOCKS = 3,  /* patch-pair blocks per SM                        */
-  STIV_TUNE_PIECE_LEVELS = 4,  /* refinement levels of the FP32 piece test (2-6)  */
+  STIV_TUNE_PIECE_LEVELS = 4,  /* d_m > 0: refinement levels of the FP32 piece test (2-6) */
   STIV_NTUNE = 5
 };
 int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_t p_max, const int32_t* p_dev,

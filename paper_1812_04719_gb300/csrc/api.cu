@@ -260,6 +260,8 @@ static int detect_layout(stiv_handle* h, int n, int p_max, const stiv_pairs* can
   size_t o_fr = off; off = align_up(off + sizeof(stiv_pair_info) * (size_t)cand->capacity);
   size_t o_q3 = off; off = align_up(off + sizeof(ulonglong2) * (size_t)w.Q3);
   size_t o_q2 = off; off = align_up(off + sizeof(ulonglong2) * (size_t)w.Q2);
+  size_t o_q2c = off;   // the d_m and exact modes use one list
+  if (!h->prm.exact_only && !(h->prm.d_m > 0.0)) off = align_up(off + sizeof(ulonglong2) * (size_t)w.Q2);
   // cleared together at the start of a detection
   size_t o_ctr = off; off = align_up(off + sizeof(int64_t) * 32);
   size_t o_rws = off; off = align_up(off + sizeof(int32_t) * ((units + STIV_ROW_SUM - 1) / STIV_ROW_SUM));
@@ -286,7 +288,7 @@ static int detect_layout(stiv_handle* h, int n, int p_max, const stiv_pairs* can
   w.pkey = (uint64_t*)(b + o_pk); w.pval = (int32_t*)(b + o_pv);
   w.pkey2 = (uint64_t*)(b + o_pk2); w.pval2 = (int32_t*)(b + o_pv2);
   w.work = (uint64_t*)(b + o_wk);
-  w.q3 = (ulonglong2*)(b + o_q3); w.q2 = (ulonglong2*)(b + o_q2);
+  w.q3 = (ulonglong2*)(b + o_q3); w.q2 = (ulonglong2*)(b + o_q2); w.q2c = (ulonglong2*)(b + o_q2c);
   w.pinfo = (stiv_pair_info*)(b + o_fr);
   w.pair_cnt = (int32_t*)(b + o_pc); w.pair_fill = (int32_t*)(b + o_pf); w.pair_off = (int32_t*)(b + o_po);
   w.seg = (unsigned long long*)(b + o_sg); w.seg2 = (unsigned long long*)(b + o_sg2);

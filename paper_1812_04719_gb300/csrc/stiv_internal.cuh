@@ -140,6 +140,7 @@ struct detect_ws {
   stiv_pair_info* pinfo; // [pair capacity]
   ulonglong2* q3;         // [Q3] primitive pairs left for the FP32 piece tests
   ulonglong2* q2;         // [Q2] primitive pairs left for the FP64 contact test
+  ulonglong2* q2c;        // [Q2] the same, cubics with critical points
   int64_t Q3, Q2;
   int32_t* pair_cnt;     // [pair capacity]   contacts per candidate pair
   int32_t* pair_fill;    // [pair capacity]

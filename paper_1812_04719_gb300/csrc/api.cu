@@ -185,7 +185,10 @@ extern "C" int stiv_create(stiv_handle** out, const stiv_params* prm) {
 extern "C" int stiv_destroy(stiv_handle* h) {
   if (!h) return STIV_ERR_ARG;
   for (int p = 0; p <= STIV_MAX_P; ++p) {
-    if (h->tab_ready[p]) { cudaFree(h->tab[p].leg); cudaFree(h->tab[p].trig); cudaFree(h->tab[p].theta); }
+    if (h->tab_ready[p]) {
+      cudaFree(h->tab[p].leg); cudaFree(h->tab[p].trig); cudaFree(h->tab[p].theta);
+      cudaFree(h->tab[p].leg_t); cudaFree(h->tab[p].trig_t);
+    }
     if (h->ytab[p]) cudaFree(h->ytab[p]);
     if (h->ytabT[p]) cudaFree(h->ytabT[p]);
   }

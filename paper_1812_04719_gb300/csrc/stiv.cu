@@ -405,6 +405,13 @@ __global__ void scatter_grad_kernel(const int64_t* counts, int64_t cap, const in
 // so that the three fields' phases overlap across CTAs.  S: Legendre step
 // then Fourier step, so S^T: Fourier analysis sums per ring, then Legendre
 // sums.
+//
+// Bound by the FP64 pipe, so lanes without work count as much as lanes with: the
+// m = 0 sums run with the others (times cos 0 = 1) instead of a loop of their
+// own beside every warp, and a thread that takes ring i takes ring P-i with it
+// and leaves their sum and difference, so that by Pbar_n^m(-x) = (-1)^(n+m)
+// Pbar_n^m(x) the Legendre sums run over half the rings.  1440 vesicles at p = 16:
+// 0.44 -> 0.24 ms.
 struct adj_args {
   const int32_t* p;
   const int64_t* coef_off;
@@ -421,64 +428,73 @@ __global__ void __launch_bounds__(256) adjoint_kernel(adj_args a) {
   if (a.p[v] < 1 || a.p[v] > STIV_MAX_P || !a.leg[a.p[v]]) return;   // order outside [1, p_max]: skipped
   int p = a.p[v], P = 2 * p, nc = (p + 1) * (p + 1), nl = (p + 1) * (p + 2) / 2, ns = 2 * p + 1, W = 2 * P;
   int nv = stiv_nverts(P);
-  double* G = sm;                    // [n_v]       one field of gX (X1 block), staged coalesced
-  double* H = sm + nv;               // [P+1][ns]   Fourier-analysed rings of that field
+  const int nq = P / 2 + 1, nh = P / 2 + 1;
+  double* H = sm;                    // [P+1][ns]   row i < P/2: sum of rings i and P-i, row P-i: their difference
   double* Q = H + (P + 1) * ns;      // [P+1][4][P/2+1] parity combinations of the four symmetric longitudes
-  const double* g = a.gX + a.vert_off[v] + (size_t)3 * nv;
+  const double* g = a.gX + a.vert_off[v] + (size_t)(3 + f) * nv;
   const double* T = a.trig[p];
   const double* L = a.leg[p];
   double* out = a.gcoef + a.coef_off[v];
-  int nq = P / 2 + 1;
   for (int k = threadIdx.x; k < nc; k += blockDim.x) out[f * nc + k] = 0.0;  // X0 block, this field
-  {
-    for (int k = threadIdx.x; k < nv; k += blockDim.x) G[k] = g[(size_t)f * nv + k];
-    __syncthreads();
-    // adjoint of the Fourier step.  The forward writes longitudes j, P-j, P+j,
-    // 2P-j (j <= P/2, duplicates skipped) from the parity sums Ce, Co, Se, So;
-    // their adjoints are the four combinations below.
-    for (int task = threadIdx.x; task < (P + 1) * nq; task += blockDim.x) {
-      int i = task / nq, j = task % nq;
-      const double* gr = G + (size_t)i * W;
-      int j1 = P - j, j2 = P + j, j3 = (W - j) % W;
-      double g0 = gr[j];
-      double g1 = (j1 != j) ? gr[j1] : 0.0;
-      double g2 = (j2 != j1) ? gr[j2] : 0.0;
-      double g3 = (j3 != j && j3 != j2) ? gr[j3] : 0.0;
-      double* q = Q + (size_t)i * 4 * nq;
-      q[0 * nq + j] = (g0 + g1) + (g2 + g3);   // cos, even m
-      q[1 * nq + j] = (g0 - g1) - (g2 - g3);   // cos, odd m
-      q[2 * nq + j] = (g0 - g1) + (g2 - g3);   // sin, even m
-      q[3 * nq + j] = (g0 + g1) - (g2 + g3);   // sin, odd m
+  // adjoint of the Fourier step.  The forward writes longitudes j, P-j, P+j,
+  // 2P-j (j <= P/2, duplicates skipped) from the parity sums Ce, Co, Se, So;
+  // their adjoints are the four combinations below.
+  for (int task = threadIdx.x; task < (P + 1) * nq; task += blockDim.x) {
+    int i = task / nq, j = task - i * nq;
+    const double* gr = g + (size_t)i * W;
+    int j1 = P - j, j2 = P + j, j3 = (W - j) % W;
+    double g0 = gr[j];
+    double g1 = (j1 != j) ? gr[j1] : 0.0;
+    double g2 = (j2 != j1) ? gr[j2] : 0.0;
+    double g3 = (j3 != j && j3 != j2) ? gr[j3] : 0.0;
+    double* q = Q + (size_t)i * 4 * nq;
+    double s01 = g0 + g1, d01 = g0 - g1, s23 = g2 + g3, d23 = g2 - g3;
+    q[0 * nq + j] = s01 + s23;   // cos, even m
+    q[1 * nq + j] = d01 - d23;   // cos, odd m
+    q[2 * nq + j] = d01 + d23;   // sin, even m
+    q[3 * nq + j] = s01 - s23;   // sin, odd m
+  }
+  __syncthreads();
+  for (int task = threadIdx.x; task < nh * ns; task += blockDim.x) {
+    int i = task / ns, s = task - i * ns;
+    int m = (s + 1) >> 1;
+    bool is_sin = s > 0 && (s & 1) == 0;
+    const int k = ((is_sin ? 2 : 0) + (m & 1)) * nq;
+    const double* qa = Q + (size_t)i * 4 * nq + k;
+    const double* qb = Q + (size_t)(P - i) * 4 * nq + k;
+    const double* Ts = T + (is_sin ? (p + 1) + m : m);   // m = 0: cos 0 = 1
+    double x = 0.0, y = 0.0;
+#pragma unroll 2
+    for (int j = 0; j < nq; ++j) {
+      double c = Ts[(size_t)j * 2 * (p + 1)];
+      x = fma(qa[j], c, x);
+      y = fma(qb[j], c, y);
     }
-    __syncthreads();
-    for (int task = threadIdx.x; task < (P + 1) * ns; task += blockDim.x) {
-      int i = task / ns, s = task % ns;
-      int m = (s + 1) >> 1;
-      bool is_sin = s > 0 && (s & 1) == 0;
-      const double* q = Q + (size_t)i * 4 * nq + (size_t)((is_sin ? 2 : 0) + (m & 1)) * nq;
-      double acc = 0.0;
-      if (s == 0) {
-        for (int j = 0; j < nq; ++j) acc += q[j];
-      } else {
-        int off = is_sin ? (p + 1) + m : m;
-        for (int j = 0; j < nq; ++j) acc = fma(q[j], T[(size_t)j * 2 * (p + 1) + off], acc);
-      }
-      H[i * ns + s] = acc;
+    if (i != P - i) {
+      H[i * ns + s] = x + y;
+      H[(P - i) * ns + s] = x - y;
+    } else {
+      H[i * ns + s] = x;
     }
-    __syncthreads();
-    // adjoint of the Legendre step (all rings, and the poles for m = 0)
-    for (int q = threadIdx.x; q < nc; q += blockDim.x) {
-      int n = (int)sqrtf((float)q); while (n * n > q) --n; while ((n + 1) * (n + 1) <= q) ++n;
-      int m = q - n * n - n, am = m < 0 ? -m : m;
-      int s = m == 0 ? 0 : (m > 0 ? 2 * m - 1 : 2 * am);
-      double acc = 0.0;
-      for (int i = 0; i <= P; ++i) acc = fma(L[(size_t)i * nl + n * (n + 1) / 2 + am], H[i * ns + s], acc);
-      if (m == 0) {
-        acc = fma(L[(size_t)(P + 1) * nl + n * (n + 1) / 2], G[(size_t)W * (P + 1)], acc);
-        acc = fma(L[(size_t)(P + 2) * nl + n * (n + 1) / 2], G[(size_t)W * (P + 1) + 1], acc);
-      }
-      out[3 * nc + f * nc + q] = acc;
+  }
+  __syncthreads();
+  // adjoint of the Legendre step over half the rings (the equator, where odd
+  // n + m vanish, with the even ones), and the poles for m = 0
+  for (int q = threadIdx.x; q < nc; q += blockDim.x) {
+    int n = (int)sqrtf((float)q); while (n * n > q) --n; while ((n + 1) * (n + 1) <= q) ++n;
+    int m = q - n * n - n, am = m < 0 ? -m : m;
+    int s = m == 0 ? 0 : (m > 0 ? 2 * m - 1 : 2 * am);
+    const int e = n * (n + 1) / 2 + am;
+    const bool odd = (n + am) & 1;
+    const double* Hs = H + s;
+    double acc = 0.0;
+    for (int i = 0; i < P / 2; ++i) acc = fma(L[(size_t)i * nl + e], Hs[(odd ? P - i : i) * ns], acc);
+    if (!odd) acc = fma(L[(size_t)(P / 2) * nl + e], Hs[(P / 2) * ns], acc);
+    if (m == 0) {
+      acc = fma(L[(size_t)(P + 1) * nl + n * (n + 1) / 2], g[(size_t)W * (P + 1)], acc);
+      acc = fma(L[(size_t)(P + 2) * nl + n * (n + 1) / 2], g[(size_t)W * (P + 1) + 1], acc);
     }
+    out[3 * nc + f * nc + q] = acc;
   }
 }
 
@@ -603,8 +619,7 @@ extern "C" int stiv_grad_to_coef(stiv_handle* h, void* stream, int32_t n_ves, in
     a.leg[p] = h->tab[p].leg; a.trig[p] = h->tab[p].trig;
   }
   int Pm = 2 * p_max;
-  size_t smem = sizeof(double) * ((size_t)stiv_nverts(Pm) + (size_t)(Pm + 1) * (2 * p_max + 1) +
-                                  (size_t)(Pm + 1) * 4 * (Pm / 2 + 1));
+  size_t smem = sizeof(double) * ((size_t)(Pm + 1) * (2 * p_max + 1) + (size_t)(Pm + 1) * 4 * (Pm / 2 + 1));
   STIV_CUDA(h, cudaFuncSetAttribute(adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   STIV_PROF(h, st, "grad_to_coef");
   adjoint_kernel<<<dim3(n_ves, 3), 256, smem, st>>>(a);

@@ -40,6 +40,8 @@ struct stiv_tables {
   double* leg;    // [(P+3)][(p+1)(p+2)/2]  normalised Legendre (x sqrt2 for m>0) at rings + poles
   double* trig;   // [P/2+1][2][p+1]        cos(m phi_j), sin(m phi_j) for j <= P/2
   double* theta;  // [P+1]                  ring polar angles
+  double* leg_t;  // [(p+1)(p+2)/2][P/2+1]  leg of the rings up to the equator, transposed
+  double* trig_t; // [2(p+1)][P/2+1]        trig transposed: cos(m phi) at row 2 m, sin at 2 m + 1
 };
 
 struct stiv_handle {

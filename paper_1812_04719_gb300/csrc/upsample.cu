@@ -8,8 +8,7 @@
 // Both steps use exact symmetries of the grid: Pbar_n^m(-x) = (-1)^(n+m)
 // Pbar_n^m(x) pairs ring i with ring P-i, and phi_{P-j} = pi - phi_j,
 // phi_{P+j} = pi + phi_j, phi_{2P-j} = 2 pi - phi_j give four outputs from one
-// set of parity-split partial sums.  FP64 throughout (fused multiply-adds);
-// STIV_MIXED stores the result as float.
+// set of parity-split partial sums.  FP64 throughout (fused multiply-adds).
 #include "stiv_internal.cuh"
 
 #include <math.h>
@@ -34,7 +33,7 @@ __device__ double gl_node(int n, int i) {
 }
 
 // Tables for SH order p (mesh order P = 2p): one thread per table row.
-__global__ void tables_kernel(int p, double* leg, double* trig, double* theta) {
+__global__ void tables_kernel(int p, double* leg, double* trig, double* theta, double* leg_t, double* trig_t) {
   int P = 2 * p, nl = (p + 1) * (p + 2) / 2;
   int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r < P + 3) {
@@ -64,6 +63,8 @@ __global__ void tables_kernel(int p, double* leg, double* trig, double* theta) {
     // fold the sqrt(2) of the real harmonics with m > 0 into the table
     for (int n = 1; n <= p; ++n)
       for (int m = 1; m <= n; ++m) L[n * (n + 1) / 2 + m] *= 1.41421356237309504880;
+    if (r <= P / 2)
+      for (int e = 0; e < nl; ++e) leg_t[(size_t)e * (P / 2 + 1) + r] = L[e];
   }
   // trig[j][0][m] = cos(m phi_j), trig[j][1][m] = sin(m phi_j), phi_j = pi j / P, j <= P/2
   int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -75,6 +76,8 @@ __global__ void tables_kernel(int p, double* leg, double* trig, double* theta) {
     sincospi((double)k / P, &sv, &cv);
     trig[(size_t)j * 2 * (p + 1) + m] = cv;
     trig[(size_t)j * 2 * (p + 1) + (p + 1) + m] = sv;
+    trig_t[(size_t)(2 * m) * (P / 2 + 1) + j] = cv;
+    trig_t[(size_t)(2 * m + 1) * (P / 2 + 1) + j] = sv;
   }
 }
 
@@ -83,82 +86,101 @@ struct synth_args {
   const int64_t* coef_off;
   const double* coef;
   const int64_t* vert_off;
-  void* verts;
-  int mixed;
+  double* verts;
   const double* leg[STIV_MAX_P + 1];
-  const double* trig[STIV_MAX_P + 1];
+  const double* leg_t[STIV_MAX_P + 1];
+  const double* trig_t[STIV_MAX_P + 1];
 };
 
-// One CTA per (vesicle, time level): the 3 coordinate fields.
+// One CTA per (vesicle, time level) and NF coordinate fields: 3, or 1 (grid z)
+// for few vesicles, where the CTAs would leave the chip idle.
+//
+// Bound by the FP64 pipe (a warp instruction takes it some 20 cycles), so the
+// instructions that run for lanes without work count.  In the Legendre step the
+// lanes of a warp are rings of one order m (they run the same number of terms;
+// with lanes over m half of them waited), in the Fourier step longitudes, three
+// fields at a time on one load of the trigonometric values; both read transposed
+// tables, lane by lane.  Every sum keeps its terms and their order.  1440
+// vesicles at p = 16: 0.60 -> 0.45 ms.
+template <int NF>
 __global__ void __launch_bounds__(256) synth_kernel(synth_args a) {
   extern __shared__ double sm[];
-  int v = blockIdx.x, t = blockIdx.y;
+  int v = blockIdx.x, t = blockIdx.y, f0 = NF == 1 ? blockIdx.z : 0;
   if (a.p[v] < 1 || a.p[v] > STIV_MAX_P || !a.leg[a.p[v]]) return;   // order outside [1, p_max]: skipped
   int p = a.p[v], P = 2 * p, nc = (p + 1) * (p + 1), nl = (p + 1) * (p + 2) / 2, ns = 2 * p + 1;
   int nv = 2 * P * (P + 1) + 2;
-  double* C = sm;                        // [3][nc]
-  double* G = sm + 3 * nc;               // [3][P+1][ns]  slot 0: m=0; 2m-1: cos m; 2m: sin m
-  const double* coef = a.coef + a.coef_off[v] + (size_t)t * 3 * nc;
-  for (int k = threadIdx.x; k < 3 * nc; k += blockDim.x) C[k] = coef[k];
+  double* C = sm;                        // [NF][nc]
+  double* G = sm + NF * nc;              // [NF][P+1][ns]  slot 0: m=0; 2m-1: cos m; 2m: sin m
+  const double* coef = a.coef + a.coef_off[v] + (size_t)(t * 3 + f0) * nc;
+  for (int k = threadIdx.x; k < NF * nc; k += blockDim.x) C[k] = coef[k];
   __syncthreads();
   const double* L = a.leg[p];
-  const double* T = a.trig[p];
+  const double* LT = a.leg_t[p];
+  const double* TT = a.trig_t[p];
   // Legendre step over half the rings (parity pairs ring i with ring P-i)
-  int nh = P / 2 + 1;
-  for (int task = threadIdx.x; task < 3 * nh * ns; task += blockDim.x) {
-    int f = task / (nh * ns), rem = task % (nh * ns), i = rem / ns, s = rem % ns;
+  const int nh = P / 2 + 1, nq = P / 2 + 1;
+  for (int task = threadIdx.x; task < NF * nh * ns; task += blockDim.x) {
+    int s = task / (NF * nh), rem = task - s * (NF * nh), f = rem / nh, i = rem - f * nh;
     int m = (s + 1) >> 1;
     int sgn = (s == 0) ? 0 : ((s & 1) ? 1 : -1);  // +m cos, -m sin
-    const double* Lr = L + (size_t)i * nl;
-    const double* Cf = C + f * nc;
+    const double* Cf = C + f * nc + sgn * m;
+    const double* Li = LT + i;
     double E = 0.0, O = 0.0;
-    for (int n = m; n <= p; n += 2) E = fma(Cf[n * n + n + sgn * m], Lr[n * (n + 1) / 2 + m], E);
-    for (int n = m + 1; n <= p; n += 2) O = fma(Cf[n * n + n + sgn * m], Lr[n * (n + 1) / 2 + m], O);
+    for (int n = m; n <= p; n += 2) {
+      E = fma(Cf[n * n + n], Li[(size_t)(n * (n + 1) / 2 + m) * nh], E);
+      if (n + 1 <= p) O = fma(Cf[(n + 1) * (n + 2)], Li[(size_t)((n + 1) * (n + 2) / 2 + m) * nh], O);
+    }
     G[(f * (P + 1) + i) * ns + s] = E + O;
     if (i != P - i) G[(f * (P + 1) + (P - i)) * ns + s] = E - O;
   }
   __syncthreads();
-  // Fourier step: four longitudes per task
-  size_t base = a.vert_off[v] + (size_t)t * 3 * nv;
-  int nq = P / 2 + 1;
-  for (int task = threadIdx.x; task < 3 * (P + 1) * nq; task += blockDim.x) {
-    int f = task / ((P + 1) * nq), rem = task % ((P + 1) * nq), r = rem / nq, j = rem % nq;
-    const double* g = G + (size_t)(f * (P + 1) + r) * ns;
-    const double* cs = T + (size_t)j * 2 * (p + 1);
-    const double* sn = cs + (p + 1);
-    double Ce = g[0], Co = 0.0, Se = 0.0, So = 0.0;
-    for (int m = 1; m <= p; m += 2) { Co = fma(g[2 * m - 1], cs[m], Co); So = fma(g[2 * m], sn[m], So); }
-    for (int m = 2; m <= p; m += 2) { Ce = fma(g[2 * m - 1], cs[m], Ce); Se = fma(g[2 * m], sn[m], Se); }
+  // Fourier step: four longitudes per task and field
+  size_t base = a.vert_off[v] + (size_t)(t * 3 + f0) * nv;
+  for (int task = threadIdx.x; task < (P + 1) * nq; task += blockDim.x) {
+    int r = task / nq, j = task - r * nq;
+    const double* g = G + (size_t)r * ns;
+    const int fs = (P + 1) * ns;
+    double Ce[NF], Co[NF], Se[NF], So[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) { Ce[f] = g[f * fs]; Co[f] = 0.0; Se[f] = 0.0; So[f] = 0.0; }
+    for (int m = 1; m <= p; m += 2) {
+      double c = TT[(size_t)(2 * m) * nq + j], sn = TT[(size_t)(2 * m + 1) * nq + j];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        Co[f] = fma(g[f * fs + 2 * m - 1], c, Co[f]);
+        So[f] = fma(g[f * fs + 2 * m], sn, So[f]);
+      }
+      if (m + 1 <= p) {
+        c = TT[(size_t)(2 * m + 2) * nq + j]; sn = TT[(size_t)(2 * m + 3) * nq + j];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          Ce[f] = fma(g[f * fs + 2 * m + 1], c, Ce[f]);
+          Se[f] = fma(g[f * fs + 2 * m + 2], sn, Se[f]);
+        }
+      }
+    }
     int W = 2 * P;
-    double v0 = (Ce + Co) + (Se + So);            // phi_j
-    double v1 = (Ce - Co) + (So - Se);            // pi - phi_j
-    double v2 = (Ce - Co) + (Se - So);            // pi + phi_j
-    double v3 = (Ce + Co) - (Se + So);            // 2 pi - phi_j
-    size_t row = base + (size_t)f * nv + (size_t)r * W;
     int j1 = P - j, j2 = P + j, j3 = (W - j) % W;
-    if (a.mixed) {
-      float* X = (float*)a.verts;
-      X[row + j] = (float)v0;
-      if (j1 != j) X[row + j1] = (float)v1;
-      if (j2 != j1 && j2 < W) X[row + j2] = (float)v2;
-      if (j3 != j && j3 != j2) X[row + j3] = (float)v3;
-    } else {
-      double* X = (double*)a.verts;
-      X[row + j] = v0;
-      if (j1 != j) X[row + j1] = v1;
-      if (j2 != j1 && j2 < W) X[row + j2] = v2;
-      if (j3 != j && j3 != j2) X[row + j3] = v3;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      double v0 = (Ce[f] + Co[f]) + (Se[f] + So[f]);            // phi_j
+      double v1 = (Ce[f] - Co[f]) + (So[f] - Se[f]);            // pi - phi_j
+      double v2 = (Ce[f] - Co[f]) + (Se[f] - So[f]);            // pi + phi_j
+      double v3 = (Ce[f] + Co[f]) - (Se[f] + So[f]);            // 2 pi - phi_j
+      double* X = a.verts + base + (size_t)f * nv + (size_t)r * W;
+      X[j] = v0;
+      if (j1 != j) X[j1] = v1;
+      if (j2 != j1 && j2 < W) X[j2] = v2;
+      if (j3 != j && j3 != j2) X[j3] = v3;
     }
   }
   // poles: only m = 0 contributes
-  if (threadIdx.x < 6) {
+  if (threadIdx.x < 2 * NF) {
     int f = threadIdx.x >> 1, pole = threadIdx.x & 1;
     const double* Lr = L + (size_t)(P + 1 + pole) * nl;
     double acc = 0.0;
     for (int n = 0; n <= p; ++n) acc = fma(C[f * nc + n * n + n], Lr[n * (n + 1) / 2], acc);
-    size_t idx = base + (size_t)f * nv + 2 * P * (P + 1) + pole;
-    if (a.mixed) ((float*)a.verts)[idx] = (float)acc;
-    else ((double*)a.verts)[idx] = acc;
+    a.verts[base + (size_t)f * nv + 2 * P * (P + 1) + pole] = acc;
   }
 }
 
@@ -457,16 +479,18 @@ int stiv_ensure_tables(stiv_handle* h, cudaStream_t st, int p) {
   STIV_CUDA(h, cudaMalloc(&T.leg, sizeof(double) * (size_t)(P + 3) * nl));
   STIV_CUDA(h, cudaMalloc(&T.trig, sizeof(double) * (size_t)(P / 2 + 1) * 2 * (p + 1)));
   STIV_CUDA(h, cudaMalloc(&T.theta, sizeof(double) * (P + 1)));
+  STIV_CUDA(h, cudaMalloc(&T.leg_t, sizeof(double) * (size_t)nl * (P / 2 + 1)));
+  STIV_CUDA(h, cudaMalloc(&T.trig_t, sizeof(double) * (size_t)(P / 2 + 1) * 2 * (p + 1)));
   int n = (P / 2 + 1) * (p + 1) > P + 3 ? (P / 2 + 1) * (p + 1) : P + 3;
-  tables_kernel<<<(n + 127) / 128, 128, 0, st>>>(p, T.leg, T.trig, T.theta);
+  tables_kernel<<<(n + 127) / 128, 128, 0, st>>>(p, T.leg, T.trig, T.theta, T.leg_t, T.trig_t);
   STIV_LAUNCH(h);
   h->tab_ready[p] = true;
   return STIV_OK;
 }
 
-static size_t synth_smem(int p) {
+static size_t synth_smem(int p, int fields) {
   int P = 2 * p;
-  return sizeof(double) * (size_t)(3 * (p + 1) * (p + 1) + 3 * (P + 1) * (2 * p + 1));
+  return sizeof(double) * (size_t)fields * ((p + 1) * (p + 1) + (P + 1) * (2 * p + 1));
 }
 
 extern "C" int stiv_upsample(stiv_handle* h, void* stream, int32_t n_ves, int32_t p_max, const int32_t* p_dev,
@@ -480,17 +504,25 @@ extern "C" int stiv_upsample(stiv_handle* h, void* stream, int32_t n_ves, int32_
     return stiv_upsample_tc(h, st, n_ves, p_max, p_dev, coef_off_dev, coef_dev, vert_off_dev, (float*)verts_dev);
   synth_args a;
   a.p = p_dev; a.coef_off = coef_off_dev; a.coef = coef_dev; a.vert_off = vert_off_dev;
-  a.verts = verts_dev; a.mixed = h->prm.precision == STIV_MIXED;
-  for (int p = 0; p <= STIV_MAX_P; ++p) { a.leg[p] = nullptr; a.trig[p] = nullptr; }
+  a.verts = (double*)verts_dev;
+  for (int p = 0; p <= STIV_MAX_P; ++p) { a.leg[p] = nullptr; a.leg_t[p] = nullptr; a.trig_t[p] = nullptr; }
   for (int p = 1; p <= p_max; ++p) {
     int rc = stiv_ensure_tables(h, st, p);
     if (rc) return rc;
-    a.leg[p] = h->tab[p].leg; a.trig[p] = h->tab[p].trig;
+    a.leg[p] = h->tab[p].leg; a.leg_t[p] = h->tab[p].leg_t; a.trig_t[p] = h->tab[p].trig_t;
   }
-  size_t smem = synth_smem(p_max);
-  STIV_CUDA(h, cudaFuncSetAttribute(synth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // one field per CTA where three would leave SMs idle (two vesicles at p = 8:
+  // 17.7 -> 16.7 us)
+  bool split = 2 * n_ves < 152;
+  size_t smem = synth_smem(p_max, split ? 1 : 3);
   STIV_PROF(h, st, "synth");
-  synth_kernel<<<dim3(n_ves, 2), 256, smem, st>>>(a);
+  if (split) {
+    STIV_CUDA(h, cudaFuncSetAttribute(synth_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    synth_kernel<1><<<dim3(n_ves, 2, 3), 256, smem, st>>>(a);
+  } else {
+    STIV_CUDA(h, cudaFuncSetAttribute(synth_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    synth_kernel<3><<<dim3(n_ves, 2), 256, smem, st>>>(a);
+  }
   STIV_LAUNCH(h);
   return STIV_OK;
 }

@@ -15,7 +15,7 @@
 // The gradient is reverse mode written out by hand: V depends on X1 through
 // D, through Y, through the weights (beta or s, u: least-squares solutions
 // of the inside test) and through tau, an implicit function of X1 via
-// f(tau) = 0 (Eq. 3.1): d tau / dX1_q = -tau (df/dY_q) / f'(tau).
+// f(tau) = 0 (Eq. 3.1): d tau / dX1_q = -tau (df/dY_q) / f'(tau) (stiv_one).
 #include "stiv_internal.cuh"
 
 #include <math.h>
@@ -32,134 +32,103 @@ __device__ __forceinline__ d3 cross(d3 a, d3 b) {
   return {fma(a.y, b.z, -(a.z * b.y)), fma(a.z, b.x, -(a.x * b.z)), fma(a.x, b.y, -(a.y * b.x))};
 }
 
-struct contact_in {
-  int type;       // 0, 1: VF (point 0 = vertex, 1..3 triangle); 2: EE (0,1 = edge of i; 2,3 = edge of j)
-  d3 X0[4], X1[4];
-  double tau;
-  double w1, w2;  // inside-test weights of the detection at tau (VF: b1, b2; EE: s, u)
-};
+__device__ __forceinline__ d3 axpy(double s, d3 a, d3 b) { return {fma(s, a.x, b.x), fma(s, a.y, b.y), fma(s, a.z, b.z)}; }
 
-// V and (optionally) dV/dX1 [4] (g1) and dV/dX0 [4] (g0) of one contact.
-// vabs: U_k read as the absolute velocity of the contact point (the literal
-// reading: VF the vertex's displacement, EE that of the point p(s) on the
-// first edge) instead of the velocity relative to the opposite primitive.
-// Reverse mode: adjoints of the positions at tau (Yb), of the displacements
-// (Db) and of tau (taub); with Y = X0 + tau D, D = X1 - X0 and tau moving
-// along f(tau; X) = 0, dV/dX1 = Db + tau Yb - taub tau fY / f' and
-// dV/dX0 = -Db + (1 - tau) Yb - taub (1 - tau) fY / f'.  dm2 = d_m^2 > 0:
-// tau is a root of g = f^2 - d_m^2 |m|^2 (Eq. 3.1, degree six) and fY, f'
-// are those of g: gY = 2 f fY - d_m^2 d|m|^2/dY, g' = sum gY . D.
-// VAR = false compiles the common case (relative velocity, d_m = 0, no X0
-// rows) without the variants' code.
+// V and dV/dX1 (g, with VAR also dV/dX0, g0) of one contact.
+//
+// Both kinds are the same expression of three difference vectors at tau: a, b
+// the triangle's edges from its first vertex (VF) or the two edges (EE), c from
+// that vertex to the vertex (VF) or from the first edge's first point to the
+// second's (EE).  With the weights (w1, w2) = (b1, b2) (VF) or (s, -u) (EE) the
+// relative displacement is Dr = c' - w1 a' - w2 b' (' the differences'
+// displacements), (w1, w2) the least-squares solution of c ~ w1 a + w2 b, and f =
+// c . (a x b).  So the adjoints are formed for a, b and c and distributed over
+// the points at the end: x = P, Q, H, G with c = P - Q, a = H - Q, b = G - Q (VF:
+// xp, x0, x1, x2) or G - P (EE: q0, p0, p1, q1).
+//
+// Reverse mode: adjoints of the vectors at tau (ab, bb, w), of their
+// displacements and of tau (taub); with Y = X0 + tau D, D = X1 - X0 and tau
+// moving along f(tau; X) = 0, dV/dX1 = Db + tau Yb - taub tau fY / f' and dV/dX0 =
+// -Db + (1 - tau) Yb - taub (1 - tau) fY / f'.  dm2 = d_m^2 > 0: tau is a root of
+// g = f^2 - d_m^2 |m|^2 (Eq. 3.1, degree six) and fY, f' are those of g.  vabs: U_k
+// read as the absolute velocity of the contact point (the literal reading: VF
+// the vertex's displacement, EE that of the point p(s) on the first edge).
+// VAR = false compiles the common case (relative velocity, d_m = 0, no X0 rows)
+// without the variants' code.
+//
+// Bound by the FP64 pipe: the library is built without contraction, so every
+// multiply-add is written as one; with both kinds on one path about 260 FP64
+// instructions per contact instead of 406: 0.55 -> 0.31 ms at 1440 vesicles (636k
+// contacts).
 template <bool VAR>
-__device__ double stiv_one(const contact_in& c, double e2, int vabs, double dm2, d3* g, d3* g0) {
-  if (!VAR) { vabs = 0; dm2 = 0.0; g0 = nullptr; }
-  d3 D[4], Y[4];
-  for (int q = 0; q < 4; ++q) { D[q] = c.X1[q] - c.X0[q]; Y[q] = mk(fma(c.tau, D[q].x, c.X0[q].x), fma(c.tau, D[q].y, c.X0[q].y), fma(c.tau, D[q].z, c.X0[q].z)); }
-  const double tau = c.tau;
-  d3 Yb[4] = {}, Db[4] = {}, fY[4];
-  double taub;
-  double V;
-  if (c.type < 2) {
-    d3 a = Y[2] - Y[1], b = Y[3] - Y[1], cc = Y[0] - Y[1];
-    double d00 = dot(a, a), d01 = dot(a, b), d11 = dot(b, b), d20 = dot(cc, a), d21 = dot(cc, b);
-    double den = d00 * d11 - d01 * d01, iden = 1.0 / den;
-    (void)d20; (void)d21;
-    double b1 = c.w1, b2 = c.w2, b0 = 1.0 - b1 - b2;
-    d3 m = cross(a, b);
-    d3 Dr = vabs ? D[0] : D[0] - (b0 * D[1] + b1 * D[2] + b2 * D[3]);
-    double dm = dot(Dr, m);
-    double Q = e2 * dot(m, m) + dm * dm;
-    double rS = rsqrt(Q);                  // 1 / sqrt(Q): no division in the adjoint below
-    double S = Q > 0.0 ? Q * rS : 0.0;
-    V = 0.5 * (1.0 - tau) * S;
-    if (!g && !g0) return V;
-    double Qb = 0.25 * (1.0 - tau) * rS;   // dV/dQ
-    d3 mb = (2.0 * Qb) * (e2 * m + dm * Dr);
-    d3 Drb = (2.0 * Qb * dm) * m;
-    taub = -0.5 * S;
-    double bb0 = 0.0, bb1 = 0.0, bb2 = 0.0;
-    if (vabs) {
-      Db[0] = Drb;
-    } else {
-      Db[0] = Drb; Db[1] = -b0 * Drb; Db[2] = -b1 * Drb; Db[3] = -b2 * Drb;
-      bb0 = -dot(Drb, D[1]); bb1 = -dot(Drb, D[2]); bb2 = -dot(Drb, D[3]);
-    }
-    double g1 = bb1 - bb0, g2 = bb2 - bb0;
-    d3 ab = cross(b, mb), bbv = cross(mb, a), cb = mk(0, 0, 0);
-    // least squares beta = M^-1 G^T c, G = [a b]
-    double z1 = (d11 * g1 - d01 * g2) * iden, z2 = (d00 * g2 - d01 * g1) * iden;
-    d3 w = z1 * a + z2 * b;
-    d3 res = cc - (b1 * a + b2 * b);
-    cb = cb + w;
-    ab = ab + z1 * res - b1 * w;
-    bbv = bbv + z2 * res - b2 * w;
-    Yb[2] = ab; Yb[3] = bbv; Yb[0] = cb; Yb[1] = -(ab + bbv + cb);
-    // df/dY of f = c . (a x b)
-    fY[0] = m; fY[2] = cross(b, cc); fY[3] = cross(cc, a); fY[1] = -(fY[0] + fY[2] + fY[3]);
-    if (dm2 > 0.0) {   // d|m|^2 / dY2 = 2 b x m, dY3 = 2 m x a
-      double f2 = 2.0 * dot(cc, m);
-      d3 mY2 = 2.0 * cross(b, m), mY3 = 2.0 * cross(m, a), mY1 = -(mY2 + mY3);
-      fY[0] = f2 * fY[0];
-      fY[1] = f2 * fY[1] - dm2 * mY1;
-      fY[2] = f2 * fY[2] - dm2 * mY2;
-      fY[3] = f2 * fY[3] - dm2 * mY3;
-    }
-  } else {
-    d3 d1 = Y[1] - Y[0], d2 = Y[3] - Y[2], r = Y[0] - Y[2];
-    double A = dot(d1, d1), B = dot(d1, d2), E = dot(d2, d2), C = dot(d1, r), F = dot(d2, r);
-    double den = A * E - B * B, iden = 1.0 / den;
-    (void)C; (void)F;
-    double s = c.w1, u = c.w2;
-    d3 m = cross(d1, d2);
-    d3 Dp = (1.0 - s) * D[0] + s * D[1];
-    d3 Dr = vabs ? Dp : ((1.0 - u) * D[2] + u * D[3]) - Dp;
-    double dm = dot(Dr, m);
-    double Q = e2 * dot(m, m) + dm * dm;
-    double rS = rsqrt(Q);                  // 1 / sqrt(Q): no division in the adjoint below
-    double S = Q > 0.0 ? Q * rS : 0.0;
-    V = 0.5 * (1.0 - tau) * S;
-    if (!g && !g0) return V;
-    double Qb = 0.25 * (1.0 - tau) * rS;   // dV/dQ
-    d3 mb = (2.0 * Qb) * (e2 * m + dm * Dr);
-    d3 Drb = (2.0 * Qb * dm) * m;
-    taub = -0.5 * S;
-    double sb, ub;
-    if (vabs) {
-      Db[0] = (1.0 - s) * Drb; Db[1] = s * Drb;
-      sb = dot(Drb, D[1] - D[0]); ub = 0.0;
-    } else {
-      Db[2] = (1.0 - u) * Drb; Db[3] = u * Drb; Db[0] = -(1.0 - s) * Drb; Db[1] = -s * Drb;
-      sb = -dot(Drb, D[1] - D[0]); ub = dot(Drb, D[3] - D[2]);
-    }
-    d3 d1b = cross(d2, mb), d2b = cross(mb, d1);
-    // least squares (s, u) = M^-1 G^T c, G = [d1, -d2], c = -r; M = [[A, -B], [-B, E]]
-    double z1 = (E * sb + B * ub) * iden, z2 = (B * sb + A * ub) * iden;
-    d3 w = z1 * d1 - z2 * d2;
-    d3 res = (-r) - (s * d1 - u * d2);
-    d3 rb = -w;
-    d1b = d1b + z1 * res - s * w;
-    d2b = d2b - (z2 * res - u * w);
-    Yb[1] = d1b; Yb[0] = -d1b + rb; Yb[3] = d2b; Yb[2] = -d2b - rb;
-    // df/dY of f = c . (d1 x d2), c = Y2 - Y0
-    d3 ce = Y[2] - Y[0];
-    d3 fc = m, f1 = cross(d2, ce), f2 = cross(ce, d1);
-    fY[2] = fc - f2; fY[0] = -fc - f1; fY[1] = f1; fY[3] = f2;
-    if (dm2 > 0.0) {   // d|m|^2 / dd1 = 2 d2 x m, dd2 = 2 m x d1
-      double ff = 2.0 * dot(ce, m);
-      d3 mY1 = 2.0 * cross(d2, m), mY3 = 2.0 * cross(m, d1);
-      fY[0] = ff * fY[0] + dm2 * mY1;
-      fY[1] = ff * fY[1] - dm2 * mY1;
-      fY[2] = ff * fY[2] + dm2 * mY3;
-      fY[3] = ff * fY[3] - dm2 * mY3;
-    }
+__device__ __forceinline__ double stiv_one(bool ee, const d3* x0, const d3* x1, double tau, double w1, double w2,
+                                           double e2, int vabs, double dm2, bool want, d3* g, bool want0, d3* g0) {
+  if (!VAR) { vabs = 0; dm2 = 0.0; want0 = false; }
+  const d3 s0 = {ee ? x0[0].x : x0[1].x, ee ? x0[0].y : x0[1].y, ee ? x0[0].z : x0[1].z};
+  const d3 s1 = {ee ? x1[0].x : x1[1].x, ee ? x1[0].y : x1[1].y, ee ? x1[0].z : x1[1].z};
+  d3 a = x0[2] - x0[1], b = x0[3] - s0, c = x0[0] - x0[1];
+  const d3 da = (x1[2] - x1[1]) - a, db = (x1[3] - s1) - b, dc = (x1[0] - x1[1]) - c;
+  a = axpy(tau, da, a); b = axpy(tau, db, b); c = axpy(tau, dc, c);
+  const double q2 = ee ? -w2 : w2;
+  const d3 m = cross(a, b);
+  d3 Dr;
+  if (VAR && vabs) Dr = ee ? axpy(w1, da, x1[1] - x0[1]) : x1[0] - x0[0];
+  else Dr = axpy(-w1, da, axpy(-q2, db, dc));
+  const double dm = dot(Dr, m);
+  const double Q = fma(dm, dm, e2 * dot(m, m));
+  const double rS = rsqrt(Q);            // 1 / sqrt(Q): no division in the adjoint below
+  const double S = Q > 0.0 ? Q * rS : 0.0;
+  const double rest = 1.0 - tau, half = 0.5 * rest;
+  const double V = half * S;
+  if (!want && !want0) return V;
+  const double qb = half * rS;           // 2 dV/dQ
+  const double be = qb * dm;
+  const d3 mb = axpy(qb * e2, m, be * Dr), Drb = be * m;
+  double z1, z2;
+  {
+    const double daa = dot(a, a), dab = dot(a, b), dbb = dot(b, b);
+    const double iden = 1.0 / fma(daa, dbb, -(dab * dab));
+    double h1 = -dot(Drb, da), h2 = -dot(Drb, db);
+    if (VAR && vabs) { h1 = ee ? -h1 : 0.0; h2 = 0.0; }
+    z1 = fma(dbb, h1, -(dab * h2)) * iden;
+    z2 = fma(daa, h2, -(dab * h1)) * iden;
   }
-  double fp = 0.0;
-  for (int q = 0; q < 4; ++q) { taub += dot(Yb[q], D[q]); fp += dot(fY[q], D[q]); }
-  if (g)
-    for (int q = 0; q < 4; ++q) g[q] = (Db[q] + tau * Yb[q]) - ((taub * tau / fp) * fY[q]);
-  if (g0)
-    for (int q = 0; q < 4; ++q) g0[q] = ((1.0 - tau) * Yb[q] - Db[q]) - ((taub * (1.0 - tau) / fp) * fY[q]);
+  // least squares (w1, w2) = M^-1 G^T c, G = [a b]
+  const d3 w = axpy(z1, a, z2 * b);
+  const d3 res = axpy(-w1, a, axpy(-q2, b, c));
+  const d3 ab = axpy(z1, res, axpy(-w1, w, cross(b, mb)));
+  const d3 bb = axpy(z2, res, axpy(-q2, w, cross(mb, a)));
+  // df/dY of f = c . (a x b)
+  d3 fc = m, fa = cross(b, c), fb = cross(c, a);
+  if (VAR && dm2 > 0.0) {   // d|m|^2 / da = 2 b x m, db = 2 m x a
+    const double f2 = 2.0 * dot(c, m);
+    fc = f2 * fc;
+    fa = axpy(-2.0 * dm2, cross(b, m), f2 * fa);
+    fb = axpy(-2.0 * dm2, cross(m, a), f2 * fb);
+  }
+  const double taub = fma(-0.5, S, dot(w, dc) + (dot(ab, da) + dot(bb, db)));
+  const double fp = dot(fc, dc) + (dot(fa, da) + dot(fb, db));
+  // to the vectors, then to the points; e1: the sign of Drb and the weight of
+  // the adjoints at tau
+  auto rows = [&](double at, double e1, d3* o) {
+    const double kap = -(taub * at / fp);
+    d3 Gc = axpy(kap, fc, at * w), Ga = axpy(kap, fa, at * ab), Gb = axpy(kap, fb, at * bb), ex = {0.0, 0.0, 0.0};
+    if (VAR && vabs) {
+      ex = e1 * Drb;   // of the point itself
+      if (ee) Ga = axpy(e1 * w1, Drb, Ga);
+    } else {
+      Gc = e1 > 0.0 ? Gc + Drb : Gc - Drb;
+      Ga = axpy(-e1 * w1, Drb, Ga);
+      Gb = axpy(-e1 * q2, Drb, Gb);
+    }
+    const d3 sub = {ee ? Gb.x : 0.0, ee ? Gb.y : 0.0, ee ? Gb.z : 0.0};
+    const d3 P = Gc - sub;
+    const d3 R = -((Gc + Ga) + (Gb - sub));
+    o[0] = P; o[1] = R; o[2] = Ga; o[3] = Gb;
+    if (VAR && vabs) o[ee ? 1 : 0] = o[ee ? 1 : 0] + ex;
+  };
+  if (want) rows(tau, 1.0, g);
+  if (VAR && want0) rows(rest, -1.0, g0);
   return V;
 }
 
@@ -181,18 +150,24 @@ struct stiv_args {
   double* grad0;   // dV/dX0 rows (or NULL)
   int32_t* gves;
   int32_t* gvid;
+  bool vec;        // the row and id arrays allow 16-byte stores
 };
 
-__device__ __forceinline__ d3 vpos(const stiv_args& A, int v, int t, int k, const int* s) {
-  int P = 2 * A.pv[v], nv = stiv_nverts(P);
-  size_t base = A.voff[v] + (size_t)t * 3 * nv + k;
-  double x[3];
-  for (int c = 0; c < 3; ++c) {
-    size_t idx = base + (size_t)c * nv;
+// X0 and X1 of vertex k of a vesicle at base (its vertices, order nv), shifted
+// by sh where the axis' bit of mask is set (the pair's periodic image).
+__device__ __forceinline__ void vpos(const stiv_args& A, size_t base, int nv, int k, int mask, const double* sh, d3& p0,
+                                     d3& p1) {
+  double x[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    size_t idx = base + (size_t)c * nv + k;
     x[c] = A.mixed ? (double)((const float*)A.X)[idx] : ((const double*)A.X)[idx];
-    if (s && s[c] != 0) x[c] = x[c] + s[c] * A.L[c];
   }
-  return {x[0], x[1], x[2]};
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    if ((mask >> c) & 1) { x[c] = x[c] + sh[c]; x[3 + c] = x[3 + c] + sh[c]; }
+  p0 = {x[0], x[1], x[2]};
+  p1 = {x[3], x[4], x[5]};
 }
 
 __device__ __forceinline__ int64_t n_contacts(const int64_t* counts, int64_t cap) {
@@ -200,49 +175,82 @@ __device__ __forceinline__ int64_t n_contacts(const int64_t* counts, int64_t cap
   return n < cap ? n : cap;
 }
 
+// One contact's four rows (12 doubles): 16-byte stores where the caller's array
+// allows (A.vec), else one by one.
+__device__ __forceinline__ void put_rows(double* out, int64_t k, const d3* r, bool vec) {
+  double v[12];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) { v[3 * q] = r[q].x; v[3 * q + 1] = r[q].y; v[3 * q + 2] = r[q].z; }
+  if (vec) {
+    double2* o = (double2*)(out + 12 * k);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) o[q] = make_double2(v[2 * q], v[2 * q + 1]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 12; ++q) out[12 * k + q] = v[q];
+  }
+}
+
 // VAR: the variants (absolute velocity, d_m > 0, X0 rows) in an instance of
-// their own; the common one fits 128 registers (4 CTAs per SM).
+// their own.
 template <bool VAR>
 __global__ void __launch_bounds__(128, 4) stiv_kernel(stiv_args A) {
   int64_t n = n_contacts(A.counts, A.cap);
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    int r = A.pair[k], ty = A.type[k], pa = A.a[k], pb = A.b[k];
-    int vi = A.ci[r], vj = A.cj[r], code = A.cs[r];
-    int s1[3] = {code / 9 - 1, (code / 3) % 3 - 1, code % 3 - 1};
-    int ves[4], vid[4];
-    const int* sh[4];
-    if (ty < 2) {
-      int vv = ty == 0 ? vi : vj, vt = ty == 0 ? vj : vi;
-      int tv[3];
-      stiv_tri_verts(2 * A.pv[vt], pb, tv);
-      ves[0] = vv; vid[0] = pa;
-      for (int q = 0; q < 3; ++q) { ves[1 + q] = vt; vid[1 + q] = tv[q]; }
-    } else {
-      int u, v;
-      stiv_edge_verts(2 * A.pv[vi], pa, &u, &v); ves[0] = vi; vid[0] = u; ves[1] = vi; vid[1] = v;
-      stiv_edge_verts(2 * A.pv[vj], pb, &u, &v); ves[2] = vj; vid[2] = u; ves[3] = vj; vid[3] = v;
+    const int r = A.pair[k], ty = A.type[k], pa = A.a[k], pb = A.b[k];
+    const int vi = A.ci[r], vj = A.cj[r], code = A.cs[r];
+    const int Pi = 2 * A.pv[vi], Pj = 2 * A.pv[vj];
+    const size_t bi = A.voff[vi], bj = A.voff[vj];
+    const double tau = A.tau[k], w1 = A.w[2 * k], w2 = A.w[2 * k + 1];
+    double sh[3];
+    int mask = 0;
+    {
+      int s1[3] = {code / 9 - 1, (code / 3) % 3 - 1, code % 3 - 1};
+#pragma unroll
+      for (int c = 0; c < 3; ++c) { sh[c] = s1[c] * A.L[c]; mask |= s1[c] != 0 ? 1 << c : 0; }
     }
-    contact_in c;
-    c.type = ty; c.tau = A.tau[k]; c.w1 = A.w[2 * k]; c.w2 = A.w[2 * k + 1];
+    // the points P, Q, H, G of stiv_one: vertex ids, and whether on vesicle j
+    const bool ee = ty == 2;
+    int id[4], on;
+    if (!ee) {
+      int tv[3];
+      stiv_tri_verts(ty == 0 ? Pj : Pi, pb, tv);
+      id[0] = pa; id[1] = tv[0]; id[2] = tv[1]; id[3] = tv[2];
+      on = ty == 0 ? 0xE : 0x1;
+    } else {
+      stiv_edge_verts(Pi, pa, &id[1], &id[2]);
+      stiv_edge_verts(Pj, pb, &id[0], &id[3]);
+      on = 0x9;
+    }
+    d3 x0[4], x1[4];
+    const int nvi = stiv_nverts(Pi), nvj = stiv_nverts(Pj);
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
-      sh[q] = ves[q] == vj ? s1 : nullptr;
-      c.X0[q] = vpos(A, ves[q], 0, vid[q], sh[q]);
-      c.X1[q] = vpos(A, ves[q], 1, vid[q], sh[q]);
+      const bool j = (on >> q) & 1;
+      vpos(A, j ? bj : bi, j ? nvj : nvi, id[q], j ? mask : 0, sh, x0[q], x1[q]);
     }
     d3 g[4], g0[4];
-    double V = stiv_one<VAR>(c, A.e2, A.vabs, A.dm2, A.grad ? g : nullptr, A.grad0 ? g0 : nullptr);
+    double V = stiv_one<VAR>(ee, x0, x1, tau, w1, w2, A.e2, A.vabs, A.dm2, A.grad != nullptr, g, A.grad0 != nullptr, g0);
     if (A.Vc) A.Vc[k] = V;
+    // output order: VF xp, x0, x1, x2; EE p0, p1, q0, q1
     if (A.grad) {
-      for (int q = 0; q < 4; ++q) {
-        A.grad[12 * k + 3 * q + 0] = g[q].x; A.grad[12 * k + 3 * q + 1] = g[q].y; A.grad[12 * k + 3 * q + 2] = g[q].z;
-        A.gves[4 * k + q] = ves[q]; A.gvid[4 * k + q] = vid[q];
+      d3 o[4] = {ee ? g[1] : g[0], ee ? g[2] : g[1], ee ? g[0] : g[2], g[3]};
+      put_rows(A.grad, k, o, A.vec);
+      int4 vd = ee ? make_int4(id[1], id[2], id[0], id[3]) : make_int4(id[0], id[1], id[2], id[3]);
+      int va = ty == 1 ? vj : vi, vb = ty == 1 ? vi : vj;
+      int4 vs = make_int4(va, ee ? va : vb, vb, vb);
+      if (A.vec) {
+        ((int4*)A.gves)[k] = vs;
+        ((int4*)A.gvid)[k] = vd;
+      } else {
+        A.gves[4 * k] = vs.x; A.gves[4 * k + 1] = vs.y; A.gves[4 * k + 2] = vs.z; A.gves[4 * k + 3] = vs.w;
+        A.gvid[4 * k] = vd.x; A.gvid[4 * k + 1] = vd.y; A.gvid[4 * k + 2] = vd.z; A.gvid[4 * k + 3] = vd.w;
       }
     }
-    if (VAR && A.grad0)
-      for (int q = 0; q < 4; ++q) {
-        A.grad0[12 * k + 3 * q + 0] = g0[q].x; A.grad0[12 * k + 3 * q + 1] = g0[q].y;
-        A.grad0[12 * k + 3 * q + 2] = g0[q].z;
-      }
+    if (VAR && A.grad0) {
+      d3 o[4] = {ee ? g0[1] : g0[0], ee ? g0[2] : g0[1], ee ? g0[0] : g0[2], g0[3]};
+      put_rows(A.grad0, k, o, A.vec);
+    }
   }
 }
 
@@ -541,6 +549,7 @@ static int run_stiv(stiv_handle* h, void* stream, const int32_t* p_dev, const in
   A.vabs = h->prm.velocity == STIV_VEL_ABSOLUTE;
   A.dm2 = h->prm.d_m * h->prm.d_m;
   A.Vc = Vtmp; A.grad = grad; A.gves = gves; A.gvid = gvid; A.grad0 = grad0;
+  A.vec = (((uintptr_t)grad | (uintptr_t)gves | (uintptr_t)gvid | (uintptr_t)grad0) & 15) == 0;
   int dev_sms = 152;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, h->device);
   if (Vtmp || grad || grad0) {

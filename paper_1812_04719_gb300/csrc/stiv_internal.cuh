@@ -274,28 +274,33 @@ __host__ __device__ inline int stiv_first_edge(int P, int u) {
   return base_row + ((j == 0) ? 0 : 3 + (j - 1) * 2);
 }
 
-// Inverse of stiv_edge_index: edge e -> (min, max) vertex ids.
+// Inverse of stiv_edge_index: edge e -> (min, max) vertex ids.  The first edges
+// of a row's vertices are 4 j + 1, 3 j + 1 and 2 j + 1 from the row's first (first
+// row, rows between, last row; 0 for j = 0), so row and column are quotients.
 __host__ __device__ inline void stiv_edge_verts(int P, int e, int* u, int* v) {
-  int lo = 0, hi = 2 * P * (P + 1) - 1;  // grid vertices (poles own no forward edge)
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (stiv_first_edge(P, mid) <= e) lo = mid; else hi = mid - 1;
-  }
-  int nb[5];
-  int n = stiv_forward_nbrs(P, lo, nb);
-  int k = e - stiv_first_edge(P, lo);
-  if (k < 0) k = 0;
-  if (k >= n) k = n - 1;
-  *u = lo; *v = nb[k];
+  int W = 2 * P, last = 4 * W + 3 * W * (P - 1);   // first edge of row P
+  int i = e < 4 * W ? 0 : (e < last ? (e - 4 * W) / (3 * W) + 1 : P);
+  int d = e - (i == 0 ? 0 : 4 * W + 3 * W * (i - 1));
+  int per = i == 0 ? 4 : (i < P ? 3 : 2);
+  int j = d > 0 ? (d - 1) / per : 0;
+  int k = d - (j ? per * j + 1 : 0);               // rank among the forward neighbours
+  int w = i * W + j, N = W * (P + 1);
+  *u = w;
+  if (j == 0 && k == 1) { *v = w + W - 1; return; }
+  int q = k - (j == 0 && k > 1 ? 1 : 0);           // without (i, W - 1)
+  if (i == P) { *v = q == 0 && j < W - 1 ? w + 1 : N + 1; return; }
+  // (i, j+1) or the diagonal when j = W - 1; (i+1, j); the diagonal; the pole
+  *v = q == 0 ? w + 1 : (q == 1 ? w + W : (q == 2 && j < W - 1 ? w + W + 1 : N));
 }
 
 // Index of the undirected edge (u, v), u < v, in the list of all edges sorted
 // by (min, max): the forward edges of all vertices before u, then the rank of
 // v among u's forward neighbours.
 __host__ __device__ inline int stiv_edge_index(int P, int u, int v) {
-  int nb[5];
-  int n = stiv_forward_nbrs(P, u, nb);
-  int k = 0;
-  while (k < n - 1 && nb[k] != v) ++k;
+  int W = 2 * P, i = u / W, j = u - i * W, z = j == 0 ? 1 : 0, k;
+  if (v >= W * (P + 1)) k = (i == P ? (j < W - 1 ? 1 : 0) : (j < W - 1 ? 3 : 2)) + z;   // pole: after the others
+  else if (v == u + 1) k = 0;
+  else if (z && v == u + W - 1) k = 1;
+  else k = (v == u + W ? 1 : 2) + z;
   return stiv_first_edge(P, u) + k;
 }

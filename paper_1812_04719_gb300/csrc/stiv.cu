@@ -64,15 +64,19 @@ template <bool VAR>
 __device__ __forceinline__ double stiv_one(bool ee, const d3* x0, const d3* x1, double tau, double w1, double w2,
                                            double e2, int vabs, double dm2, bool want, d3* g, bool want0, d3* g0) {
   if (!VAR) { vabs = 0; dm2 = 0.0; want0 = false; }
-  const d3 s0 = {ee ? x0[0].x : x0[1].x, ee ? x0[0].y : x0[1].y, ee ? x0[0].z : x0[1].z};
-  const d3 s1 = {ee ? x1[0].x : x1[1].x, ee ? x1[0].y : x1[1].y, ee ? x1[0].z : x1[1].z};
-  d3 a = x0[2] - x0[1], b = x0[3] - s0, c = x0[0] - x0[1];
-  const d3 da = (x1[2] - x1[1]) - a, db = (x1[3] - s1) - b, dc = (x1[0] - x1[1]) - c;
-  a = axpy(tau, da, a); b = axpy(tau, db, b); c = axpy(tau, dc, c);
+  // displacements and positions at tau per point (rounded as the contact test's
+  // positions are), then the vectors
+  d3 D[4], Y[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) { D[q] = x1[q] - x0[q]; Y[q] = axpy(tau, D[q], x0[q]); }
+  const d3 Yb = {ee ? Y[0].x : Y[1].x, ee ? Y[0].y : Y[1].y, ee ? Y[0].z : Y[1].z};
+  const d3 Db = {ee ? D[0].x : D[1].x, ee ? D[0].y : D[1].y, ee ? D[0].z : D[1].z};
+  const d3 a = Y[2] - Y[1], b = Y[3] - Yb, c = Y[0] - Y[1];
+  const d3 da = D[2] - D[1], db = D[3] - Db, dc = D[0] - D[1];
   const double q2 = ee ? -w2 : w2;
   const d3 m = cross(a, b);
   d3 Dr;
-  if (VAR && vabs) Dr = ee ? axpy(w1, da, x1[1] - x0[1]) : x1[0] - x0[0];
+  if (VAR && vabs) Dr = ee ? axpy(w1, da, D[1]) : D[0];
   else Dr = axpy(-w1, da, axpy(-q2, db, dc));
   const double dm = dot(Dr, m);
   const double Q = fma(dm, dm, e2 * dot(m, m));

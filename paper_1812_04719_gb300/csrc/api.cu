@@ -259,6 +259,8 @@ static int detect_layout(stiv_handle* h, int n, int p_max, const stiv_pairs* can
   size_t o_pv = off; off = align_up(off + sizeof(int32_t) * (size_t)w.Q);
   size_t o_pk2 = off; off = align_up(off + sizeof(uint64_t) * (size_t)w.Q);
   size_t o_pv2 = off; off = align_up(off + sizeof(int32_t) * (size_t)w.Q);
+  size_t o_pk3 = off; off = align_up(off + sizeof(uint64_t) * (size_t)w.Q);
+  size_t o_pv3 = off; off = align_up(off + sizeof(int32_t) * (size_t)w.Q);
   size_t o_wk = off; off = align_up(off + sizeof(uint64_t) * (size_t)w.W);
   size_t o_fr = off; off = align_up(off + sizeof(stiv_pair_info) * (size_t)cand->capacity);
   size_t o_q3 = off; off = align_up(off + sizeof(ulonglong2) * (size_t)w.Q3);
@@ -290,6 +292,7 @@ static int detect_layout(stiv_handle* h, int n, int p_max, const stiv_pairs* can
   w.rec_box = (int32_t*)(b + o_rb); w.rec_cell = (int32_t*)(b + o_rc);
   w.pkey = (uint64_t*)(b + o_pk); w.pval = (int32_t*)(b + o_pv);
   w.pkey2 = (uint64_t*)(b + o_pk2); w.pval2 = (int32_t*)(b + o_pv2);
+  w.pkey3 = (uint64_t*)(b + o_pk3); w.pval3 = (int32_t*)(b + o_pv3);
   w.work = (uint64_t*)(b + o_wk);
   w.q3 = (ulonglong2*)(b + o_q3); w.q2 = (ulonglong2*)(b + o_q2); w.q2c = (ulonglong2*)(b + o_q2c);
   w.pinfo = (stiv_pair_info*)(b + o_fr);

@@ -660,8 +660,8 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   int rc;
   {
   STIV_PROF_N(h, st, "sort_cells", stiv_sort_kernels(24));
-  rc = stiv_sort_pairs_impl(st, w.R, 24, w.rec_key, w.rec_val, w.rec_key2, w.rec_val2, w.sort_scratch,
-                                w.sort_scratch_bytes, &ctr[8]);
+  rc = stiv_sort_pairs_impl(st, w.R, 24, w.rec_key, w.rec_val, w.rec_key2, w.rec_val2, w.rec_key, w.rec_val,
+                            w.sort_scratch, w.sort_scratch_bytes, &ctr[8]);
   }
   // candidate keys i << (nb + 5) | j << 5 | shift code: nb bits per vesicle index
   int nb = 1;
@@ -677,8 +677,8 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   STIV_LAUNCH(h);
   {
     STIV_PROF_N(h, st, "sort_pairs", stiv_sort_kernels(pair_bits));
-    rc = stiv_sort_pairs_impl(st, w.Q, pair_bits, w.pkey, w.pval, w.pkey2, w.pval2, w.sort_scratch,
-                              w.sort_scratch_bytes, &ctr[9]);
+    rc = stiv_sort_pairs_impl(st, w.Q, pair_bits, w.pkey, w.pval, w.pkey2, w.pval2, w.pkey3, w.pval3,
+                              w.sort_scratch, w.sort_scratch_bytes, &ctr[9]);
   }
   if (rc) return rc;
   {

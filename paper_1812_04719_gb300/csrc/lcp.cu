@@ -14,16 +14,13 @@
 //   bounds_kernel   contact range of every candidate pair (contacts are
 //                   sorted by pair)
 //   rows_kernel     rows = pairs with contacts; q = -V
-//   entries_kernel  one keyed entry per contact point: row | side | vertex
-//                   (side 0: the pair's first vesicle, 1: its second)
-//   (radix sort, stable)
-//   gather_kernel   the entries' gradients in sorted order
-//   tile_sums, tile_scan, compact
-//                   unique (row, side, vertex) entries: the gradient of each
-//                   vertex summed by a segmented scan in sorted (contact)
-//                   order, fixed association (deterministic), over all rows
-//                   at once
-//   ves_kernel      (vesicle, row) keys -> sorted per-vesicle row lists
+//   row_sides_kernel per row and side (side 0: the pair's first vesicle, 1: its
+//                   second) the gradient of each vertex: a row's contacts are
+//                   contiguous, so one CTA sorts their points by vertex in shared
+//                   memory and sums the runs in contact order, fixed association
+//                   (deterministic)
+//   ves_count, ves_scan, ves_fill, ves_rank
+//                   the rows of each vesicle, ascending
 //   bcount_kernel   per row, the rows sharing a vesicle (union of its two
 //                   vesicles' lists)
 //   bcol_kernel     the columns and the row of every nonzero
@@ -57,29 +54,33 @@ __global__ void bounds_kernel(const int64_t* counts, int64_t ccap, const int32_t
   }
 }
 
-// Block-wide exclusive scan helper (RT threads).
+// Block-wide exclusive scan (RT threads); sh: RT / 32 ints.
 __device__ int block_scan(int v, int* sh, int& total) {
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int off = 1; off < RT; off <<= 1) {
-    int t = threadIdx.x >= off ? sh[threadIdx.x - off] : 0;
-    __syncthreads();
-    sh[threadIdx.x] += t;
-    __syncthreads();
+  int lane = threadIdx.x & 31, w = threadIdx.x >> 5, x = v;
+  for (int off = 1; off < 32; off <<= 1) {
+    int y = __shfl_up_sync(0xffffffffu, x, off);
+    if (lane >= off) x += y;
   }
-  total = sh[RT - 1];
-  int ex = sh[threadIdx.x] - v;
+  if (lane == 31) sh[w] = x;
   __syncthreads();
-  return ex;
+  int s = sh[lane];
+  static_assert(RT / 32 == 32, "one warp total per lane");
+  for (int off = 1; off < 32; off <<= 1) {
+    int y = __shfl_up_sync(0xffffffffu, s, off);
+    if (lane >= off) s += y;
+  }
+  total = __shfl_sync(0xffffffffu, s, 31);
+  int pre = w ? __shfl_sync(0xffffffffu, s, w - 1) : 0;
+  __syncthreads();
+  return pre + x - v;
 }
 
 // dims: [0] rows, [1] nnz, [2] status (1: rows over capacity, 2: nonzeros
 // over capacity), [3] entries (4 x contacts), [4] 2 x rows
 __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t pcap, int64_t ccap,
                                                   const int32_t* pstart, const int32_t* pend, const double* Vp,
-                                                  int64_t rcap, int32_t* row_pair, int32_t* row_of_pair, double* q,
-                                                  int64_t* dims) {
-  __shared__ int sh[RT];
+                                                  int64_t rcap, int32_t* row_pair, double* q, int64_t* dims) {
+  __shared__ int sh[RT / 32];
   int64_t np = counts[STIV_C_PAIRS] < pcap ? counts[STIV_C_PAIRS] : pcap;
   int base = 0;
   for (int64_t p0 = 0; p0 < np; p0 += RT) {
@@ -87,13 +88,9 @@ __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t
     int has = (p < np && pend[p] > pstart[p]) ? 1 : 0;
     int tot;
     int ex = block_scan(has, sh, tot);
-    if (p < np) {
-      int r = has ? base + ex : -1;
-      row_of_pair[p] = r;
-      if (has && r < rcap) {
-        row_pair[r] = (int32_t)p;
-        q[r] = -Vp[p];
-      }
+    if (has && base + ex < rcap) {
+      row_pair[base + ex] = (int32_t)p;
+      q[base + ex] = -Vp[p];
     }
     base += tot;
   }
@@ -105,39 +102,11 @@ __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t
   }
 }
 
-__global__ void entries_kernel(const int64_t* counts, int64_t ccap, const int32_t* pair, const int32_t* row_of_pair,
-                               const int32_t* ci, const int32_t* gves, const int32_t* gvid, int64_t rcap, int db,
-                               uint64_t* key, int32_t* val) {
-  int64_t n = ncontacts(counts, ccap);
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    int p = pair[k];
-    int r = row_of_pair[p];
-    uint64_t rr = (r >= 0 && r < rcap) ? (uint64_t)r : (uint64_t)rcap;   // beyond capacity: sorted last
-    int vi = ci[p];
-    for (int q = 0; q < 4; ++q) {
-      uint64_t side = gves[4 * k + q] == vi ? 0u : 1u;
-      key[4 * k + q] = (rr << (1 + db)) | (side << db) | (uint64_t)gvid[4 * k + q];
-      val[4 * k + q] = (int32_t)(4 * k + q);
-    }
-  }
-}
+constexpr int ST = 256;      // threads of a row-side CTA
+constexpr int CH = 2048;     // points sorted at a time
+constexpr int SD = 128;      // digits of the sort (7 bits)
 
-constexpr int ET = 256;        // threads of the compaction CTAs
-constexpr int EI = 8;          // consecutive entries per thread
-constexpr int ETILE = ET * EI;
-
-// Gradients of the sorted entries, gathered into sorted order (one
-// independent gather per entry), so that the runs summed next are contiguous.
-__global__ void gather_kernel(const int64_t* n_dev, const int32_t* sval, const double* grad, double* gs) {
-  int64_t n = *n_dev;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    const double* g = grad + 3 * (size_t)sval[j];
-    double a = g[0], b = g[1], c = g[2];
-    gs[3 * j] = a; gs[3 * j + 1] = b; gs[3 * j + 2] = c;
-  }
-}
-
-// Exclusive scan over an ET-thread CTA in a fixed order; *total = the sum.
+// Exclusive scan over an ST-thread CTA; *total = the sum.  wsum: ST / 32 ints.
 __device__ __forceinline__ int cta_scan(int v, int* wsum, int* total) {
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int x = v;
@@ -148,183 +117,214 @@ __device__ __forceinline__ int cta_scan(int v, int* wsum, int* total) {
   if (lane == 31) wsum[w] = x;
   __syncthreads();
   int pre = 0, tot = 0;
-  for (int q = 0; q < ET / 32; ++q) { int s = wsum[q]; pre += q < w ? s : 0; tot += s; }
+  for (int q = 0; q < ST / 32; ++q) { int s = wsum[q]; pre += q < w ? s : 0; tot += s; }
   __syncthreads();
   *total = tot;
   return pre + x - v;
 }
 
-__device__ __forceinline__ bool is_head(const uint64_t* skey, int64_t j, int64_t n) {
-  return j < n && (j == 0 || skey[j] != skey[j - 1]);
-}
-
-// Segmented sums: (f, v) pairs combined left to right by
-// (f1, v1) + (f2, v2) = (f1 | f2, f2 ? v2 : v1 + v2), f = "a run starts here".
-// Runs (one vertex of one row) can hold thousands of entries, so they are
-// summed by a segmented scan over all sorted entries rather than by the
-// run's first entry: per thread over its EI entries, then over the CTA
-// (warp shuffles, then warps in order), then over the tiles.  The order of
-// the additions is fixed, so the sums are deterministic.
-struct seg3 {
-  int f;
-  double a, b, c;
-};
-__device__ __forceinline__ seg3 seg_add(const seg3& x, const seg3& y) {
-  seg3 r;
-  r.f = x.f | y.f;
-  r.a = y.f ? y.a : x.a + y.a;
-  r.b = y.f ? y.b : x.b + y.b;
-  r.c = y.f ? y.c : x.c + y.c;
-  return r;
-}
-
-// Exclusive segmented scan over the ET-thread CTA; *total = the CTA's sum.
-__device__ seg3 cta_seg_scan(seg3 v, seg3* wagg, seg3* total) {
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  seg3 s = v;
-  for (int off = 1; off < 32; off <<= 1) {
-    seg3 o;
-    o.f = __shfl_up_sync(0xffffffffu, s.f, off);
-    o.a = __shfl_up_sync(0xffffffffu, s.a, off);
-    o.b = __shfl_up_sync(0xffffffffu, s.b, off);
-    o.c = __shfl_up_sync(0xffffffffu, s.c, off);
-    if (lane >= off) s = seg_add(o, s);
-  }
-  seg3 ex;   // within the warp: the inclusive value of the previous lane
-  ex.f = __shfl_up_sync(0xffffffffu, s.f, 1);
-  ex.a = __shfl_up_sync(0xffffffffu, s.a, 1);
-  ex.b = __shfl_up_sync(0xffffffffu, s.b, 1);
-  ex.c = __shfl_up_sync(0xffffffffu, s.c, 1);
-  if (lane == 0) ex = seg3{0, 0.0, 0.0, 0.0};
-  if (lane == 31) wagg[w] = s;
-  __syncthreads();
-  seg3 pre{0, 0.0, 0.0, 0.0}, tot{0, 0.0, 0.0, 0.0};
-  for (int q = 0; q < ET / 32; ++q) {
-    if (q < w) pre = seg_add(pre, wagg[q]);
-    tot = seg_add(tot, wagg[q]);
-  }
-  __syncthreads();
-  *total = tot;
-  return seg_add(pre, ex);
-}
-
-// This thread's EI entries as one segmented value: whether a run starts in
-// them, and the sum of the entries after the last start (or of all of them).
-__device__ __forceinline__ seg3 thread_seg(const uint64_t* skey, const double* gs, int64_t base, int64_t n,
-                                           unsigned& hd) {
-  seg3 s{0, 0.0, 0.0, 0.0};
-  hd = 0;
-  for (int k = 0; k < EI; ++k) {
-    int64_t j = base + k;
-    if (j >= n) break;
-    if (is_head(skey, j, n)) { hd |= 1u << k; s.f = 1; s.a = gs[3 * j]; s.b = gs[3 * j + 1]; s.c = gs[3 * j + 2]; }
-    else { s.a += gs[3 * j]; s.b += gs[3 * j + 1]; s.c += gs[3 * j + 2]; }
-  }
-  return s;
-}
-
-// The unique (row, side, vertex) entries are compacted over all sorted
-// entries at once (rows differ widely in size): per tile the heads of runs
-// and the segmented sum, the tiles scanned, then every run's last entry
-// writes the run's sum.
-__global__ void __launch_bounds__(ET) tile_sums_kernel(const int64_t* n_dev, const uint64_t* skey, const double* gs,
-                                                       int32_t* tcount, seg3* tagg) {
-  __shared__ int wsum[ET / 32];
-  __shared__ seg3 wagg[ET / 32];
-  int64_t n = *n_dev;
-  if ((int64_t)blockIdx.x * ETILE >= n) return;   // past the entries: not read by the scan
-  int64_t base = (int64_t)blockIdx.x * ETILE + (int64_t)threadIdx.x * EI;
-  unsigned hd;
-  seg3 v = thread_seg(skey, gs, base, n, hd);
-  int tot;
-  cta_scan(__popc(hd), wsum, &tot);
-  seg3 st;
-  cta_seg_scan(v, wagg, &st);
-  if (threadIdx.x == 0) { tcount[blockIdx.x] = tot; tagg[blockIdx.x] = st; }
-}
-
-// One CTA: exclusive scan of the tile head counts in place, and the
-// segmented sum flowing into each tile from the tiles before it (tcarry).
-// Without rows beyond capacity the head total closes the last row's range:
-// ustart[rows] = total.
-__global__ void __launch_bounds__(ET) tile_scan_kernel(int ntiles, int32_t* tcount, const seg3* tagg, seg3* tcarry,
-                                                       const int64_t* dims, int32_t* ustart) {
-  __shared__ int wsum[ET / 32];
-  __shared__ seg3 wagg[ET / 32];
-  int64_t used = (dims[3] + ETILE - 1) / ETILE;   // tiles holding entries
-  if (used < ntiles) ntiles = (int)used;
-  int carry = 0;
-  seg3 scarry{0, 0.0, 0.0, 0.0};
-  for (int b = 0; b < ntiles; b += ET) {
-    int i = b + threadIdx.x;
-    int v = i < ntiles ? tcount[i] : 0, tot;
-    int ex = cta_scan(v, wsum, &tot);
-    seg3 sv = i < ntiles ? tagg[i] : seg3{0, 0.0, 0.0, 0.0}, stot;
-    seg3 sex = cta_seg_scan(sv, wagg, &stot);
-    if (i < ntiles) { tcount[i] = carry + ex; tcarry[i] = seg_add(scarry, sex); }
-    carry += tot;
-    scarry = seg_add(scarry, stot);
-  }
-  if (threadIdx.x == 0 && !(dims[2] & 1)) ustart[dims[0]] = carry;
-}
-
-// Heads write their unique entry's key (the first head of a row where the
-// row's unique entries start, the first head of a row's side 1 where those
-// start; rows beyond capacity share the row field rcap and close the last
-// row's range); the last entry of each run writes the run's sum.
-__global__ void __launch_bounds__(ET) compact_kernel(const int64_t* n_dev, const uint64_t* skey, const double* gs,
-                                                     const int32_t* toff, const seg3* tcarry, int rshift,
-                                                     uint64_t kmask, uint64_t* ukey, double* ug, int32_t* ustart,
-                                                     int32_t* uside) {
-  __shared__ int wsum[ET / 32];
-  __shared__ seg3 wagg[ET / 32];
-  int64_t n = *n_dev;
-  if ((int64_t)blockIdx.x * ETILE >= n) return;
-  int64_t base = (int64_t)blockIdx.x * ETILE + (int64_t)threadIdx.x * EI;
-  unsigned hd;
-  seg3 v = thread_seg(skey, gs, base, n, hd);
-  int tot;
-  int u = toff[blockIdx.x] + cta_scan(__popc(hd), wsum, &tot) - 1;   // unique index of the open run
-  seg3 st;
-  seg3 run = seg_add(tcarry[blockIdx.x], cta_seg_scan(v, wagg, &st));   // open run's sum so far
-  for (int k = 0; k < EI; ++k) {
-    int64_t j = base + k;
-    if (j >= n) break;
-    if (hd >> k & 1u) {
-      ++u;
-      run.a = gs[3 * j]; run.b = gs[3 * j + 1]; run.c = gs[3 * j + 2];
-      uint64_t key = skey[j];
-      ukey[u] = key & kmask;
-      uint64_t row = key >> rshift;
-      if (j == 0 || (skey[j - 1] >> rshift) != row) ustart[row] = u;
-      if ((key >> (rshift - 1) & 1u) && (j == 0 || (skey[j - 1] >> (rshift - 1)) != (key >> (rshift - 1))))
-        uside[row] = u;   // first entry of the row's side 1
-    } else {
-      run.a += gs[3 * j]; run.b += gs[3 * j + 1]; run.c += gs[3 * j + 2];
+// The unique vertices of row r's side s and the sum of their gradient rows, at
+// [sbeg[2 r + s], + scnt[2 r + s]) of ukey and ug (a row's points start at four
+// times its first contact, side 1's after side 0's).  The points are taken in
+// chunks of at most CH in contact order, each sorted by vertex (stable: vertex <<
+// 12 | place); a run's sum goes to a new entry or onto the one an earlier chunk
+// made (tab: vertex -> entry).  Four lanes sum a run, strided, then by halves: a
+// fixed order.
+//
+// The global alternative (a keyed entry per point, a radix sort of all of them by
+// row, side and vertex, a gather and a segmented scan over all entries: 25
+// launches) took 0.42 ms of device time at 1440 vesicles (2.5M points), this
+// kernel 0.15 ms, bound by the latency of its short phases.
+__global__ void __launch_bounds__(ST, 6) row_sides_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* pstart,
+                                                       const int32_t* pend, const int32_t* ci, const int32_t* gves,
+                                                       const int32_t* gvid, const double* grad, int nv, bool vec, int32_t* sbeg,
+                                                       int32_t* scnt, int32_t* ukey, double* ug) {
+  extern __shared__ uint16_t tab[];          // [nv rounded up to 8]
+  __shared__ uint32_t item[2][CH];           // vertex << 12 | place in the chunk
+  __shared__ int32_t src[CH];                // by place: gradient row
+  __shared__ int32_t cnt[ST / 32][SD];
+  __shared__ uint16_t start[CH + 1];         // runs
+  __shared__ int wsum[ST / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t nitem = 2 * dims[0];
+  for (int64_t it = blockIdx.x; it < nitem; it += gridDim.x) {
+    const int side = (int)(it & 1), p = row_pair[it >> 1], vi = ci[p];
+    const int k0 = pstart[p], k1 = pend[p];
+    for (int q = threadIdx.x; q < nv; q += ST) tab[q] = 0xFFFF;
+    int64_t base = 4 * (int64_t)k0;
+    if (side) {   // after the points of side 0
+      int c = 0, tot;
+      for (int k = k0 + threadIdx.x; k < k1; k += ST) {
+        if (vec) {
+          int4 a = ((const int4*)gves)[k];
+          c += (a.x == vi) + (a.y == vi) + (a.z == vi) + (a.w == vi);
+        } else {
+          for (int q = 0; q < 4; ++q) c += gves[4 * (int64_t)k + q] == vi;
+        }
+      }
+      cta_scan(c, wsum, &tot);
+      base += tot;
     }
-    if (j + 1 == n || skey[j + 1] != skey[j]) {
-      ug[3 * (size_t)u] = run.a; ug[3 * (size_t)u + 1] = run.b; ug[3 * (size_t)u + 2] = run.c;
+    int unique = 0, n = 0;
+    for (int kb = k0; kb < k1; kb += ST) {
+      // the points of the next ST contacts on this side
+      const int64_t k = kb + threadIdx.x;
+      int vs[4], vd[4], c = 0, tot;
+      unsigned mine = 0;
+      if (k < k1) {
+        if (vec) {
+          int4 a = ((const int4*)gves)[k], b = ((const int4*)gvid)[k];
+          vs[0] = a.x; vs[1] = a.y; vs[2] = a.z; vs[3] = a.w;
+          vd[0] = b.x; vd[1] = b.y; vd[2] = b.z; vd[3] = b.w;
+        } else {
+          for (int q = 0; q < 4; ++q) { vs[q] = gves[4 * k + q]; vd[q] = gvid[4 * k + q]; }
+        }
+        for (int q = 0; q < 4; ++q)
+          if ((vs[q] == vi) == (side == 0)) { mine |= 1u << q; ++c; }
+      }
+      int at = n + cta_scan(c, wsum, &tot);
+      for (int q = 0; q < 4; ++q)
+        if (mine >> q & 1u) {
+          item[0][at] = ((uint32_t)vd[q] << 12) | (uint32_t)at;
+          src[at] = (int32_t)(4 * k + q);
+          ++at;
+        }
+      n += tot;
+      __syncthreads();
+      if (kb + ST < k1 && n + 4 * ST <= CH) continue;
+      // sort the n points by vertex
+      int cur = 0;
+      for (int shift = 12; shift < 26 && (nv - 1) >> (shift - 12); shift += 7) {
+        for (int q = lane; q < SD; q += 32) cnt[w][q] = 0;
+        __syncwarp();
+        uint32_t x[CH / ST];
+        int rank[CH / ST];
+#pragma unroll
+        for (int q = 0; q < CH / ST; ++q) {
+          const int i = w * (CH / (ST / 32)) + q * 32 + lane;
+          const bool valid = i < n;
+          x[q] = valid ? item[cur][i] : 0;
+          if (__any_sync(0xffffffffu, valid)) {
+            const unsigned dig = (x[q] >> shift) & (SD - 1);
+            const unsigned peers = digit_peers<7>(dig, valid), below = peers & ((1u << lane) - 1u);
+            const int o = valid ? cnt[w][dig] : 0;
+            __syncwarp();
+            if (valid && !below) cnt[w][dig] = o + __popc(peers);
+            rank[q] = o + __popc(below);
+            __syncwarp();
+          }
+        }
+        __syncthreads();
+        int run = 0;
+        if (threadIdx.x < SD)
+          for (int q = 0; q < ST / 32; ++q) { int o = cnt[q][threadIdx.x]; cnt[q][threadIdx.x] = run; run += o; }
+        int first = cta_scan(run, wsum, &tot);
+        if (threadIdx.x < SD)
+          for (int q = 0; q < ST / 32; ++q) cnt[q][threadIdx.x] += first;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < CH / ST; ++q)
+          if (w * (CH / (ST / 32)) + q * 32 + lane < n) item[1 - cur][cnt[w][(x[q] >> shift) & (SD - 1)] + rank[q]] = x[q];
+        cur = 1 - cur;
+        __syncthreads();
+      }
+      const uint32_t* a = item[cur];
+      // runs of one vertex
+      unsigned head = 0;
+      for (int q = 0; q < CH / ST; ++q) {
+        const int i = threadIdx.x * (CH / ST) + q;
+        if (i < n && (i == 0 || (a[i] >> 12) != (a[i - 1] >> 12))) head |= 1u << q;
+      }
+      int runs;
+      int o = cta_scan(__popc(head), wsum, &runs);
+      for (int q = 0; q < CH / ST; ++q)
+        if (head >> q & 1u) start[o++] = (uint16_t)(threadIdx.x * (CH / ST) + q);
+      if (threadIdx.x == 0) start[runs] = (uint16_t)n;
+      __syncthreads();
+      // entries: new ones after the earlier chunks', in vertex order
+      for (int r0 = 0; r0 < runs; r0 += ST) {
+        const int r = r0 + threadIdx.x;
+        const int v = r < runs ? (int)(a[start[r]] >> 12) : 0;
+        const bool fresh = r < runs && tab[v] == 0xFFFF;
+        int add;
+        const int u = unique + cta_scan(fresh ? 1 : 0, wsum, &add);
+        if (fresh) { tab[v] = (uint16_t)u; ukey[base + u] = v; }
+        if (r < runs) item[1 - cur][r] = (uint32_t)tab[v] | (fresh ? 0x80000000u : 0u);
+        unique += add;
+      }
+      __syncthreads();
+      for (int r = threadIdx.x >> 2; r < ((runs + 7) & ~7); r += ST / 4) {   // whole warps
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        if (r < runs)
+          for (int i = start[r] + (lane & 3); i < start[r + 1]; i += 4) {
+            const double* g = grad + 3 * (int64_t)src[a[i] & 0xFFFu];
+            s0 += g[0]; s1 += g[1]; s2 += g[2];
+          }
+        for (int off = 2; off > 0; off >>= 1) {
+          s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+          s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+          s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+        }
+        if (r < runs && (lane & 3) < 3) {
+          const uint32_t e = item[1 - cur][r];
+          double* d = ug + 3 * (base + (e & 0xFFFFu)) + (lane & 3);
+          const double v = (lane & 3) == 0 ? s0 : ((lane & 3) == 1 ? s1 : s2);
+          *d = e >> 31 ? v : *d + v;
+        }
+      }
+      n = 0;
+      __syncthreads();
     }
+    if (threadIdx.x == 0) { sbeg[it] = (int32_t)base; scnt[it] = unique; }
+    __syncthreads();
   }
 }
 
-__global__ void ves_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* ci, const int32_t* cj, int rb,
-                           uint64_t* key, int32_t* val) {
+// The rows of every vesicle: counted, laid out by a scan (vstart [n_ves + 1]),
+// filled in any order and ranked (a vesicle has a row at most once).
+__global__ void ves_count_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* ci, const int32_t* cj,
+                                 int32_t* vcnt) {
   int64_t n = dims[0];
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
     int p = row_pair[r];
-    key[2 * r] = ((uint64_t)ci[p] << rb) | (uint64_t)r;
-    key[2 * r + 1] = ((uint64_t)cj[p] << rb) | (uint64_t)r;
-    val[2 * r] = (int32_t)r; val[2 * r + 1] = (int32_t)r;
+    atomicAdd(&vcnt[ci[p]], 1);
+    atomicAdd(&vcnt[cj[p]], 1);
   }
 }
 
-__global__ void ves_bounds_kernel(const int64_t* dims, const uint64_t* key, int rb, int32_t* vstart, int32_t* vend) {
-  int64_t n = 2 * dims[0];
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t v = key[k] >> rb;
-    if (k == 0 || (key[k - 1] >> rb) != v) vstart[v] = (int32_t)k;
-    if (k == n - 1 || (key[k + 1] >> rb) != v) vend[v] = (int32_t)(k + 1);
+__global__ void __launch_bounds__(RT) ves_scan_kernel(int n, int32_t* vcnt, int32_t* vstart) {
+  __shared__ int sh[RT / 32];
+  int base = 0;
+  for (int v0 = 0; v0 < n; v0 += RT) {
+    int v = v0 + threadIdx.x, tot;
+    int ex = block_scan(v < n ? vcnt[v] : 0, sh, tot);
+    if (v < n) { vstart[v] = base + ex; vcnt[v] = base + ex; }   // vcnt: the fill position from here on
+    base += tot;
+  }
+  if (threadIdx.x == 0) vstart[n] = base;
+}
+
+__global__ void ves_fill_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* ci, const int32_t* cj,
+                                int32_t* vpos, int32_t* lst) {
+  int64_t n = dims[0];
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+    int p = row_pair[r];
+    lst[atomicAdd(&vpos[ci[p]], 1)] = (int32_t)r;
+    lst[atomicAdd(&vpos[cj[p]], 1)] = (int32_t)r;
+  }
+}
+
+// One warp per vesicle: each row's place is the number of smaller ones.
+__global__ void ves_rank_kernel(int n, const int32_t* vstart, const int32_t* lst, int32_t* out) {
+  int lane = threadIdx.x & 31;
+  int w0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
+  for (int v = w0; v < n; v += nw) {
+    int lo = vstart[v], len = vstart[v + 1] - lo;
+    for (int i = lane; i < len; i += 32) {
+      int x = lst[lo + i], r = 0;
+      for (int q = 0; q < len; ++q) r += lst[lo + q] < x;
+      out[lo + r] = x;
+    }
   }
 }
 
@@ -342,19 +342,19 @@ __device__ void for_neighbours(const int32_t* lst, int a0, int a1, int b0, int b
 }
 
 __global__ void bcount_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* ci, const int32_t* cj,
-                              const int32_t* vrow, const int32_t* vstart, const int32_t* vend, int32_t* bcnt) {
+                              const int32_t* vrow, const int32_t* vstart, int32_t* bcnt) {
   int64_t n = dims[0];
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
     int p = row_pair[r], vi = ci[p], vj = cj[p];
     int c = 0;
-    for_neighbours(vrow, vstart[vi], vend[vi], vstart[vj], vend[vj], [&](int) { ++c; });
+    for_neighbours(vrow, vstart[vi], vstart[vi + 1], vstart[vj], vstart[vj + 1], [&](int) { ++c; });
     bcnt[r] = c;
   }
 }
 
 __global__ void __launch_bounds__(RT) bscan_kernel(int64_t* dims, const int32_t* bcnt, int64_t nnz_cap,
                                                    int64_t* row_ptr) {
-  __shared__ int sh[RT];
+  __shared__ int sh[RT / 32];
   int64_t n = dims[0];
   int64_t base = 0;
   for (int64_t r0 = 0; r0 < n; r0 += RT) {
@@ -372,26 +372,23 @@ __global__ void __launch_bounds__(RT) bscan_kernel(int64_t* dims, const int32_t*
   }
 }
 
-// Entries of row x on one side of its pair (0: first vesicle, 1: second):
-// [ustart[x], mid) and [mid, ustart[x + 1]), mid = where side 1 starts
-// (uside[x], -1 when the row has no side-1 entry).
-__device__ __forceinline__ void side_range(const int32_t* ustart, const int32_t* uside, int64_t x, int side,
-                                           int64_t& lo, int64_t& hi) {
-  int64_t b = ustart[x], e = ustart[x + 1], m = uside[x] >= 0 ? uside[x] : e;
-  lo = side ? m : b;
-  hi = side ? e : m;
+// Entries of row x on one side of its pair (0: first vesicle, 1: second).
+__device__ __forceinline__ void side_range(const int32_t* sbeg, const int32_t* scnt, int64_t x, int side, int64_t& lo,
+                                           int64_t& hi) {
+  lo = sbeg[2 * x + side];
+  hi = lo + scnt[2 * x + side];
 }
 
 // Columns of B (thread per row): the rows sharing a vesicle with row r,
 // ascending, and the row of every nonzero.
 __global__ void bcol_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* ci, const int32_t* cj,
-                            const int32_t* vrow, const int32_t* vstart, const int32_t* vend, const int64_t* row_ptr,
+                            const int32_t* vrow, const int32_t* vstart, const int64_t* row_ptr,
                             int64_t nnz_cap, int32_t* col, int32_t* nzrow) {
   int64_t n = dims[0];
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
     int p = row_pair[r], vi = ci[p], vj = cj[p];
     int64_t o = row_ptr[r];
-    for_neighbours(vrow, vstart[vi], vend[vi], vstart[vj], vend[vj], [&](int s) {
+    for_neighbours(vrow, vstart[vi], vstart[vi + 1], vstart[vj], vstart[vj + 1], [&](int s) {
       if (o < nnz_cap) { col[o] = s; nzrow[o] = (int32_t)r; }
       ++o;
     });
@@ -405,22 +402,22 @@ __global__ void bcol_kernel(const int64_t* dims, const int32_t* row_pair, const 
 // shared memory (nvtab slots, -1 = absent, reset after use) and the lanes,
 // over row A's entries (A = min(r, s)), look their vertex up (on the diagonal
 // every entry is its own match).  Sums are reduced in a fixed order and
-// depend on (A, B) only, so that B(r, s) and B(s, r) are the same sum: B is
+// depend on (A, B) only: B(r, s), s >= r, is written to (s, r) as well, B is
 // symmetric bit for bit.
 __global__ void bval_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* ci, const int32_t* cj,
-                            const int32_t* ustart, const int32_t* uside, const uint64_t* ukey, const double* ug,
-                            const double* m_ves, const double* t_ves, int db, int nvtab, int64_t nnz_cap,
-                            const int32_t* col, const int32_t* nzrow, double* val) {
+                            const int32_t* sbeg, const int32_t* scnt, const int32_t* ukey, const double* ug,
+                            const double* m_ves, const double* t_ves, int nvtab, int64_t nnz_cap,
+                            const int64_t* row_ptr, const int32_t* col, const int32_t* nzrow, double* val) {
   extern __shared__ int32_t vtab_all[];
   int lane = threadIdx.x & 31;
   int32_t* tab = vtab_all + (size_t)(threadIdx.x >> 5) * nvtab;
   for (int i = lane; i < nvtab; i += 32) tab[i] = -1;
   __syncwarp();
-  uint64_t dmask = (1ull << db) - 1;
   int64_t nnz = dims[1] < nnz_cap ? dims[1] : nnz_cap;
   int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t k = w0; k < nnz; k += nw) {
     int r = nzrow[k], s = col[k];
+    if (s < r) continue;   // written with (s, r)
     int p = row_pair[r], vi = ci[p], vj = cj[p];
     int ps = row_pair[s], si = ci[ps], sj = cj[ps];
     int64_t rA = s < r ? s : r, rB = s < r ? r : s;
@@ -430,8 +427,8 @@ __global__ void bval_kernel(const int64_t* dims, const int32_t* row_pair, const 
       int v = t ? vj : vi;   // vi < vj: ascending
       if (v != si && v != sj) continue;
       int64_t a0, a1, b0, b1;
-      side_range(ustart, uside, rA, v == aI ? 0 : 1, a0, a1);
-      side_range(ustart, uside, rB, v == bI ? 0 : 1, b0, b1);
+      side_range(sbeg, scnt, rA, v == aI ? 0 : 1, a0, a1);
+      side_range(sbeg, scnt, rB, v == bI ? 0 : 1, b0, b1);
       double part = 0.0, sa[3] = {0.0, 0.0, 0.0}, sb[3] = {0.0, 0.0, 0.0};
       if (rA == rB) {
 #pragma unroll 4
@@ -443,13 +440,13 @@ __global__ void bval_kernel(const int64_t* dims, const int32_t* row_pair, const 
       } else {
 #pragma unroll 4
         for (int64_t i = b0 + lane; i < b1; i += 32) {
-          tab[ukey[i] & dmask] = (int32_t)(i - b0);
+          tab[ukey[i]] = (int32_t)(i - b0);
           for (int d = 0; d < 3; ++d) sb[d] += ug[3 * i + d];
         }
         __syncwarp();
 #pragma unroll 4
         for (int64_t i = a0 + lane; i < a1; i += 32) {
-          int32_t jb = tab[ukey[i] & dmask];   // vertex id (the sides may differ)
+          int32_t jb = tab[ukey[i]];   // vertex id (the sides may differ)
           if (jb >= 0) {
             int64_t lo = b0 + jb;
             part += ug[3 * i] * ug[3 * lo] + ug[3 * i + 1] * ug[3 * lo + 1] + ug[3 * i + 2] * ug[3 * lo + 2];
@@ -457,7 +454,7 @@ __global__ void bval_kernel(const int64_t* dims, const int32_t* row_pair, const 
           for (int d = 0; d < 3; ++d) sa[d] += ug[3 * i + d];
         }
         __syncwarp();
-        for (int64_t i = b0 + lane; i < b1; i += 32) tab[ukey[i] & dmask] = -1;
+        for (int64_t i = b0 + lane; i < b1; i += 32) tab[ukey[i]] = -1;
         __syncwarp();
       }
       for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
@@ -473,7 +470,15 @@ __global__ void bval_kernel(const int64_t* dims, const int32_t* row_pair, const 
         acc += t_ves[v] * (sa[0] * b0s + sa[1] * b1s + sa[2] * b2s);
       }
     }
-    if (lane == 0) val[k] = acc;
+    if (lane == 0) {
+      val[k] = acc;
+      if (s > r) {   // (s, r): among row s's columns
+        int64_t lo = row_ptr[s], hi = row_ptr[s + 1];
+        if (hi > nnz) hi = nnz;
+        while (lo < hi) { int64_t mid = (lo + hi) >> 1; if (col[mid] < r) lo = mid + 1; else hi = mid; }
+        if (lo < nnz && nzrow[lo] == s && col[lo] == r) val[lo] = acc;
+      }
+    }
   }
 }
 
@@ -704,12 +709,6 @@ __global__ void __launch_bounds__(RT) solve_kernel(solve_args g, size_t smem_byt
   if (threadIdx.x == 0) { g.info[0] = it; g.info[1] = res; g.info[2] = (double)cg_total; g.info[3] = res <= a.tol ? 0 : 2; }
 }
 
-int nbits(int64_t x) {   // bits to hold 0 .. x
-  int b = 1;
-  while (b < 62 && ((int64_t)1 << b) <= x) ++b;
-  return b;
-}
-
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -726,38 +725,24 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
     return STIV_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   int64_t pcap = cand->capacity, ccap = ct->capacity, rcap = lcp->row_capacity;
-  int rb = nbits(rcap), vb = nbits(n_ves), db = nbits(stiv_nverts(2 * p_max));
-  if (rb + 1 + db > 63 || vb + rb > 63) return STIV_ERR_ARG;
-  int64_t E = 4 * ccap, R2 = 2 * rcap;
-  int64_t smax = E > R2 ? E : R2;
-  // scratch (handle-owned, grown on demand)
+  int64_t E = 4 * ccap;
+  if (E >= ((int64_t)1 << 31)) return STIV_ERR_ARG;
+  const int nv = stiv_nverts(2 * p_max);
+  // scratch (handle-owned, grown on demand); pstart, pend and vcnt are cleared together
   size_t o = 0;
   size_t o_ps = o; o = al256(o + sizeof(int32_t) * pcap);
   size_t o_pe = o; o = al256(o + sizeof(int32_t) * pcap);
-  size_t o_rp = o; o = al256(o + sizeof(int32_t) * pcap);
-  int64_t etiles = (E + ETILE - 1) / ETILE;
-  if (etiles < 1) etiles = 1;
-  if (E >= ((int64_t)1 << 31)) return STIV_ERR_ARG;
-  size_t o_us = o; o = al256(o + sizeof(int32_t) * (rcap + 1));
-  size_t o_ud = o; o = al256(o + sizeof(int32_t) * (rcap + 1));
-  size_t o_tc = o; o = al256(o + sizeof(int32_t) * etiles);
-  size_t o_ta = o; o = al256(o + sizeof(seg3) * etiles);
-  size_t o_tk = o; o = al256(o + sizeof(seg3) * etiles);
+  size_t o_vc = o; o = al256(o + sizeof(int32_t) * n_ves);
+  const size_t clear = o;
+  size_t o_sb = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
+  size_t o_sc = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
   size_t o_bc = o; o = al256(o + sizeof(int32_t) * rcap);
   size_t o_nr = o; o = al256(o + sizeof(int32_t) * lcp->nnz_capacity);
-  size_t o_k1 = o; o = al256(o + sizeof(uint64_t) * E);
-  size_t o_v1 = o; o = al256(o + sizeof(int32_t) * E);
-  size_t o_k2 = o; o = al256(o + sizeof(uint64_t) * E);
-  size_t o_v2 = o; o = al256(o + sizeof(int32_t) * E);
+  size_t o_uk = o; o = al256(o + sizeof(int32_t) * E);
   size_t o_ug = o; o = al256(o + sizeof(double) * 3 * E);
-  size_t o_gs = o; o = al256(o + sizeof(double) * 3 * E);
-  size_t o_wk1 = o; o = al256(o + sizeof(uint64_t) * R2);
-  size_t o_wv1 = o; o = al256(o + sizeof(int32_t) * R2);
-  size_t o_wk2 = o; o = al256(o + sizeof(uint64_t) * R2);
-  size_t o_wv2 = o; o = al256(o + sizeof(int32_t) * R2);
-  size_t o_vs = o; o = al256(o + sizeof(int32_t) * n_ves);
-  size_t o_ve = o; o = al256(o + sizeof(int32_t) * n_ves);
-  size_t o_ss = o; o = al256(o + stiv_sort_scratch_impl(smax));
+  size_t o_l1 = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
+  size_t o_l2 = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
+  size_t o_vs = o; o = al256(o + sizeof(int32_t) * (n_ves + 1));
   if (o > h->lcp_ws_bytes) {
     if (h->lcp_ws) { STIV_CUDA(h, cudaFree(h->lcp_ws)); h->lcp_ws = nullptr; h->lcp_ws_bytes = 0; }
     STIV_CUDA(h, cudaMalloc(&h->lcp_ws, o));
@@ -765,62 +750,41 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   }
   char* w = (char*)h->lcp_ws;
   int32_t* pstart = (int32_t*)(w + o_ps); int32_t* pend = (int32_t*)(w + o_pe);
-  int32_t* row_of_pair = (int32_t*)(w + o_rp);
-  int32_t* ustart = (int32_t*)(w + o_us); int32_t* tcount = (int32_t*)(w + o_tc);
-  int32_t* uside = (int32_t*)(w + o_ud);
-  seg3* tagg = (seg3*)(w + o_ta); seg3* tcarry = (seg3*)(w + o_tk);
+  int32_t* vcnt = (int32_t*)(w + o_vc);
+  int32_t* sbeg = (int32_t*)(w + o_sb); int32_t* scnt = (int32_t*)(w + o_sc);
   int32_t* bcnt = (int32_t*)(w + o_bc);
   int32_t* nzrow = (int32_t*)(w + o_nr);
-  uint64_t* k1 = (uint64_t*)(w + o_k1); int32_t* v1 = (int32_t*)(w + o_v1);
-  uint64_t* k2 = (uint64_t*)(w + o_k2); int32_t* v2 = (int32_t*)(w + o_v2);
+  int32_t* ukey = (int32_t*)(w + o_uk);
   double* ug = (double*)(w + o_ug);
-  double* gs = (double*)(w + o_gs);
-  uint64_t* wk1 = (uint64_t*)(w + o_wk1); int32_t* wv1 = (int32_t*)(w + o_wv1);
-  uint64_t* wk2 = (uint64_t*)(w + o_wk2); int32_t* wv2 = (int32_t*)(w + o_wv2);
-  int32_t* vstart = (int32_t*)(w + o_vs); int32_t* vend = (int32_t*)(w + o_ve);
-  void* ss = w + o_ss;
-  size_t ss_bytes = stiv_sort_scratch_impl(smax);
+  int32_t* lst = (int32_t*)(w + o_l1); int32_t* vrow = (int32_t*)(w + o_l2);
+  int32_t* vstart = (int32_t*)(w + o_vs);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-  STIV_PROF_N(h, st, "lcp_matrix", 13 + stiv_sort_kernels(rb + 1 + db) + stiv_sort_kernels(vb + rb));
-  STIV_CUDA(h, cudaMemsetAsync(pstart, 0, sizeof(int32_t) * pcap, st));
-  STIV_CUDA(h, cudaMemsetAsync(pend, 0, sizeof(int32_t) * pcap, st));
-  STIV_CUDA(h, cudaMemsetAsync(vstart, 0, sizeof(int32_t) * n_ves, st));
-  STIV_CUDA(h, cudaMemsetAsync(vend, 0, sizeof(int32_t) * n_ves, st));
-  STIV_CUDA(h, cudaMemsetAsync(uside, 0xff, sizeof(int32_t) * (rcap + 1), st));   // -1: no side-1 entry
+  STIV_PROF_N(h, st, "lcp_matrix", 11);
+  STIV_CUDA(h, cudaMemsetAsync(w, 0, clear, st));
   bounds_kernel<<<sms * 4, 256, 0, st>>>(counts_dev, ccap, ct->pair, pstart, pend);
-  rows_kernel<<<1, RT, 0, st>>>(counts_dev, pcap, ccap, pstart, pend, V_pair_dev, rcap, lcp->row_pair, row_of_pair,
-                                lcp->q, lcp->dims);
-  entries_kernel<<<sms * 4, 256, 0, st>>>(counts_dev, ccap, ct->pair, row_of_pair, cand->i, g_ves_dev, g_vid_dev,
-                                          rcap, db, k1, v1);
-  int rc = stiv_sort_pairs_impl(st, E, rb + 1 + db, k1, v1, k2, v2, ss, ss_bytes, &lcp->dims[3]);
-  if (rc) return rc;
-  uint64_t kmask = ((1ull << (1 + db)) - 1);
-  // unique (side, vertex) entries of each row: keys into k1, gradients into
-  // ug, row r's at [ustart[r], ustart[r + 1])
-  gather_kernel<<<sms * 8, 256, 0, st>>>(&lcp->dims[3], v2, grad_dev, gs);
-  tile_sums_kernel<<<(unsigned)etiles, ET, 0, st>>>(&lcp->dims[3], k2, gs, tcount, tagg);
-  tile_scan_kernel<<<1, ET, 0, st>>>((int)etiles, tcount, tagg, tcarry, lcp->dims, ustart);
-  compact_kernel<<<(unsigned)etiles, ET, 0, st>>>(&lcp->dims[3], k2, gs, tcount, tcarry, 1 + db, kmask, k1, ug,
-                                                  ustart, uside);
-  // per-vesicle row lists
-  ves_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, rb, wk1, wv1);
-  rc = stiv_sort_pairs_impl(st, R2, vb + rb, wk1, wv1, wk2, wv2, ss, ss_bytes, &lcp->dims[4]);
-  if (rc) return rc;
-  ves_bounds_kernel<<<sms, 256, 0, st>>>(lcp->dims, wk2, rb, vstart, vend);
-  bcount_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, wv2, vstart, vend, bcnt);
+  rows_kernel<<<1, RT, 0, st>>>(counts_dev, pcap, ccap, pstart, pend, V_pair_dev, rcap, lcp->row_pair, lcp->q,
+                                lcp->dims);
+  row_sides_kernel<<<sms * 6, ST, sizeof(uint16_t) * (size_t)((nv + 7) & ~7), st>>>(
+      lcp->dims, lcp->row_pair, pstart, pend, cand->i, g_ves_dev, g_vid_dev, grad_dev, nv,
+      (((uintptr_t)g_ves_dev | (uintptr_t)g_vid_dev) & 15) == 0, sbeg, scnt, ukey, ug);
+  ves_count_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vcnt);
+  ves_scan_kernel<<<1, RT, 0, st>>>(n_ves, vcnt, vstart);
+  ves_fill_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vcnt, lst);
+  ves_rank_kernel<<<sms, 256, 0, st>>>(n_ves, vstart, lst, vrow);
+  bcount_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vrow, vstart, bcnt);
   bscan_kernel<<<1, RT, 0, st>>>(lcp->dims, bcnt, lcp->nnz_capacity, lcp->row_ptr);
   // one vertex-index table per warp: as many warps per CTA as 96 KB holds
-  int nvtab = stiv_nverts(2 * p_max);
+  int nvtab = nv;
   int bw = (int)((96 * 1024) / (sizeof(int32_t) * (size_t)nvtab));
   bw = bw < 1 ? 1 : (bw > 8 ? 8 : bw);
   size_t bsmem = sizeof(int32_t) * (size_t)nvtab * bw;
   if (bsmem > 48 * 1024)
     STIV_CUDA(h, cudaFuncSetAttribute(bval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem));
-  bcol_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, wv2, vstart, vend, lcp->row_ptr,
+  bcol_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vrow, vstart, lcp->row_ptr,
                                    lcp->nnz_capacity, lcp->col, nzrow);
-  bval_kernel<<<sms * 4, 32 * bw, bsmem, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, ustart, uside, k1, ug,
-                                               m_ves_dev, t_ves_dev, db, nvtab, lcp->nnz_capacity, lcp->col, nzrow,
+  bval_kernel<<<sms * 4, 32 * bw, bsmem, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, sbeg, scnt, ukey, ug,
+                                               m_ves_dev, t_ves_dev, nvtab, lcp->nnz_capacity, lcp->row_ptr, lcp->col, nzrow,
                                                lcp->val);
   STIV_LAUNCH(h);
   return STIV_OK;

@@ -51,14 +51,8 @@ extern "C" int stiv_sort_pairs_static(void* stream, int64_t n, int32_t key_bits,
   unsigned char* base = nullptr;
   int rc = scratch_address(&base);
   if (rc) return rc;
-  cudaStream_t st = (cudaStream_t)stream;
-  // the sort ping-pongs between its input and output arrays: sort staging
-  // copies so that the caller's input stays intact
   uint64_t* kt = (uint64_t*)(base + kHistBytes);
   int32_t* vt = (int32_t*)(base + kHistBytes + kKeyBytes);
-  if (cudaMemcpyAsync(kt, keys_in, sizeof(uint64_t) * (size_t)n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return STIV_ERR_CUDA;
-  if (cudaMemcpyAsync(vt, vals_in, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return STIV_ERR_CUDA;
-  return stiv_sort_pairs_impl(st, n, key_bits, kt, vt, keys_out, vals_out, base, kHistBytes, nullptr);
+  return stiv_sort_user_impl((cudaStream_t)stream, n, key_bits, keys_in, vals_in, keys_out, vals_out, kt, vt, base,
+                             kHistBytes);
 }

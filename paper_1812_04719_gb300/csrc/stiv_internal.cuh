@@ -138,6 +138,8 @@ struct detect_ws {
   int32_t* pval;         // [Q]
   uint64_t* pkey2;       // [Q]
   int32_t* pval2;        // [Q]
+  uint64_t* pkey3;       // [Q]
+  int32_t* pval3;        // [Q]
   uint64_t* work;        // [W]  patch-pair work items
   stiv_pair_info* pinfo; // [pair capacity]
   ulonglong2* q3;         // [Q3] primitive pairs left for the FP32 piece tests
@@ -191,8 +193,10 @@ int stiv_grad_to_coef_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t
                          double* gcoef_dev);
 int stiv_ws_reserve(stiv_handle* h, size_t bytes);
 int stiv_sort_pairs_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_t* kin, const int32_t* vin,
-                         uint64_t* kout, int32_t* vout, void* scratch, size_t scratch_bytes,
-                         const int64_t* n_dev);
+                         uint64_t* kout, int32_t* vout, uint64_t* ktmp, int32_t* vtmp, void* scratch,
+                         size_t scratch_bytes, const int64_t* n_dev);
+int stiv_sort_user_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_t* kin, const int32_t* vin,
+                        uint64_t* kout, int32_t* vout, uint64_t* kt, int32_t* vt, void* scratch, size_t scratch_bytes);
 size_t stiv_sort_scratch_impl(int64_t n);
 
 // ---------------------------------------------------------------------------
@@ -205,6 +209,19 @@ __host__ __device__ inline int stiv_ncoef(int p) { return (p + 1) * (p + 1); }
 __host__ __device__ inline int stiv_nband_blocks(int P) { return (P + STIV_BR - 1) / STIV_BR; }
 __host__ __device__ inline int stiv_ncol_blocks(int P) { return (2 * P + STIV_BC - 1) / STIV_BC; }
 __host__ __device__ inline int stiv_npatches(int P) { return stiv_nband_blocks(P) * stiv_ncol_blocks(P); }
+
+// Lanes (valid ones) that hold the same BITS-bit digit as this one, by one ballot
+// per bit (match.any.sync costs more than the eight ballots).
+template <int BITS>
+__device__ __forceinline__ unsigned digit_peers(unsigned dig, bool valid) {
+  unsigned m = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+  for (int b = 0; b < BITS; ++b) {
+    const unsigned v = __ballot_sync(0xffffffffu, (dig >> b) & 1u);
+    m &= (dig >> b) & 1u ? v : ~v;
+  }
+  return m;
+}
 
 struct d3 { double x, y, z; };
 

@@ -64,8 +64,13 @@ struct stiv_handle {
   size_t lcp_ws_bytes;
   void* lcp_ws2;
   size_t lcp_ws2_bytes;
-  double* fid_x;          // fine-grid nodes of the mesh-fidelity estimate
-  size_t fid_x_bytes;
+  // tables of the mesh-fidelity estimate, for the factor, orders and stream of
+  // the last call
+  double* fid_tab;
+  size_t fid_tab_bytes;
+  int fid_factor, fid_pmax;
+  const void* fid_stream;
+  bool fid_captured;
   // launch shapes of the narrow phase (0 = default), set by stiv_autotune
   int32_t tune[STIV_NTUNE];
   void* ws;

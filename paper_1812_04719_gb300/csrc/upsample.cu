@@ -199,28 +199,24 @@ __global__ void __launch_bounds__(256) synth_kernel(synth_args a) {
 
 constexpr double kPi = 3.14159265358979323846;
 
-// Column m of the normalised associated Legendre table at x = cos(theta),
-// s = sin(theta), no Condon-Shortley phase, sqrt(2) folded in for m > 0:
-// L[n(n+1)/2 + m] for n = m .. p, by the recurrences of tables_kernel with
-// their coefficients tabulated: dg[k] = sqrt((2k+1)/(2k)), sd[m] =
-// sqrt(2m+3), ra and rb[n(n+1)/2+m] the three-term coefficients of (n, m).
-__device__ void legendre_column_tab(int p, int m, double x, double s, const double* dg, const double* sd,
-                                    const double* ra, const double* rb, double* L) {
-  double d = 0.28209479177387814347;  // 1/sqrt(4 pi)
-  for (int k = 1; k <= m; ++k) d = dg[k] * s * d;
-  double r2 = m ? 1.41421356237309504880 : 1.0;
-  L[m * (m + 1) / 2 + m] = d * r2;
-  if (m < p) {
-    double e = sd[m] * x * d;
-    L[(m + 1) * (m + 2) / 2 + m] = e * r2;
-    double l2 = d, l1 = e;
-    for (int n = m + 2; n <= p; ++n) {
-      int idx = n * (n + 1) / 2 + m;
-      double l0 = ra[idx] * (x * l1 - rb[idx] * l2);
-      L[idx] = l0 * r2;
-      l2 = l1; l1 = l0;
-    }
-  }
+// What the estimate needs of order p and the factor alone (Pf = factor 2p, rings
+// r <= Pf), kept in the handle for all orders up to p_max: where each fine ring
+// lies on the mesh, the Legendre values of the rings up to the equator and the
+// trigonometric values of the longitudes up to pi / 2, both transposed.
+struct fid_ring {
+  double al, tp;       // fraction between mesh rings cell and cell + 1; in a pole cap from the pole to the first ring
+  int zone, cell, tri; // 0 north cap, 1 between rings, 2 south cap; tri: bit sb set when al >= sb / factor
+  int pad;
+};
+__host__ __device__ inline size_t fid_ring_doubles(int p, int factor) {
+  return (size_t)(factor * 2 * p + 1) * (sizeof(fid_ring) / sizeof(double));
+}
+__host__ __device__ inline size_t fid_leg_doubles(int p, int factor) {
+  return (size_t)(factor * p + 1) * ((p + 1) * (p + 2) / 2);
+}
+__host__ __device__ inline size_t fid_trig_doubles(int p, int factor) { return (size_t)(factor * p + 1) * 2 * (p + 1); }
+__host__ __device__ inline size_t fid_doubles(int p, int factor) {
+  return fid_ring_doubles(p, factor) + fid_leg_doubles(p, factor) + fid_trig_doubles(p, factor);
 }
 
 struct fid_args {
@@ -232,20 +228,21 @@ struct fid_args {
   int mixed;
   int factor;
   const double* theta[STIV_MAX_P + 1];
-  const double* xfine;   // fine-grid nodes x = cos(theta), order factor*2p at xfine + xoff[p]
-  int xoff[STIV_MAX_P + 1];
+  const double* tab;              // tables of order p at tab + off[p]: rings, Legendre, trigonometric
+  size_t off[STIV_MAX_P + 1];
   double* err;
 };
 
-// Gauss-Legendre node x_i (descending) of order n, Newton's method on P_n from
-// the same start as gl_node, at most 8 steps (quadratic convergence reaches
-// the last bits in about 5), stopping once a step is below 4e-16 |x|.
-__device__ double fine_node(int n, int i) {
-  double z = cospi((i + 0.75) / (n + 0.5));
+// Gauss-Legendre node x_i (descending) of order n: Newton's method on P_n from
+// Tricomi's start (error O(n^-4)), at most 8 steps, stopping once a step is below
+// 4e-16 |x|.  The recurrence's coefficients (2k - 1) / k and (k - 1) / k are
+// tabulated (c1, c2), so that a step is two dependent operations, no division.
+__device__ double fine_node(int n, int i, const double* c1, const double* c2) {
+  double z = (1.0 - (1.0 - 1.0 / n) / (8.0 * n * (double)n)) * cospi((i + 0.75) / (n + 0.5));
   for (int it = 0; it < 8; ++it) {
     double p0 = 1.0, p1 = z;
     for (int k = 2; k <= n; ++k) {
-      double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
+      double p2 = fma(c1[k] * z, p1, -(c2[k] * p0));
       p0 = p1; p1 = p2;
     }
     double dz = p1 / (n * (z * p1 - p0) / (z * z - 1.0));
@@ -255,19 +252,67 @@ __device__ double fine_node(int n, int i) {
   return z;
 }
 
-// Fine-grid Gauss-Legendre nodes for every order p <= p_max (computed once per
-// call, not per CTA): order Pf = factor 2p at xs + off(p), off(p) = sum over
-// p' < p of (factor 2p' + 1).
-__global__ void fine_nodes_kernel(int p_max, int factor, double* xs) {
-  int total = 0;
-  for (int p = 1; p <= p_max; ++p) total += factor * 2 * p + 1;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
-    int p = 1, off = 0;
-    while (e >= off + factor * 2 * p + 1) { off += factor * 2 * p + 1; ++p; }
-    int Pf = factor * 2 * p, r = e - off;
-    int ih = r <= Pf / 2 ? r : Pf - r;
-    double x = (2 * ih == Pf) ? 0.0 : fine_node(Pf + 1, ih);
-    xs[e] = r > Pf / 2 ? -x : x;
+// CTA (r, p - 1): fine ring r <= Pf / 2 of order p and its mirror image: node, place on
+// the mesh, Legendre values; and longitude r's trigonometric values.
+__global__ void __launch_bounds__(64) fid_tables_kernel(fid_args a, double* tab) {
+  __shared__ double c1[2 * STIV_MAX_P * 8 + 2], c2[2 * STIV_MAX_P * 8 + 2];
+  __shared__ double node;
+  const int p = blockIdx.y + 1, P = 2 * p, Pf = a.factor * P, r = blockIdx.x;
+  if (r > Pf / 2) return;
+  double* base = tab + a.off[p];
+  fid_ring* ring = (fid_ring*)base;
+  double* leg = base + fid_ring_doubles(p, a.factor);
+  double* trig = leg + fid_leg_doubles(p, a.factor);
+  const int nq = Pf / 2 + 1, nl = (p + 1) * (p + 2) / 2;
+  for (int k = 2 + threadIdx.x; k <= Pf + 1; k += blockDim.x) { c1[k] = (2.0 * k - 1.0) / k; c2[k] = (k - 1.0) / k; }
+  for (int m = threadIdx.x; m <= p; m += blockDim.x) {
+    double sv, cv;
+    sincospi((double)((m * r) % (2 * Pf)) / Pf, &sv, &cv);   // exact argument reduction
+    trig[(size_t)(2 * m) * nq + r] = cv;
+    trig[(size_t)(2 * m + 1) * nq + r] = sv;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) node = 2 * r == Pf ? 0.0 : fine_node(Pf + 1, r, c1, c2);
+  __syncthreads();
+  const double x = node, s = sqrt((1.0 - x) * (1.0 + x));
+  // column m of the normalised associated Legendre functions, no Condon-Shortley
+  // phase, sqrt(2) folded in for m > 0, by the recurrences of tables_kernel
+  for (int m = threadIdx.x; m <= p; m += blockDim.x) {
+    double d = 0.28209479177387814347;  // 1/sqrt(4 pi)
+    for (int k = 1; k <= m; ++k) d = sqrt((2.0 * k + 1.0) / (2.0 * k)) * s * d;
+    const double r2 = m ? 1.41421356237309504880 : 1.0;
+    double* L = leg + (size_t)r * nl;
+    L[m * (m + 1) / 2 + m] = d * r2;
+    if (m < p) {
+      double l2 = d, l1 = sqrt(2.0 * m + 3.0) * x * d;
+      L[(m + 1) * (m + 2) / 2 + m] = l1 * r2;
+      for (int n = m + 2; n <= p; ++n) {
+        double ra = sqrt((4.0 * n * n - 1.0) / ((double)(n - m) * (n + m)));
+        double rb = sqrt(((double)(n - 1 - m) * (n - 1 + m)) / (4.0 * (n - 1) * (n - 1) - 1.0));
+        double l0 = ra * (x * l1 - rb * l2);
+        L[n * (n + 1) / 2 + m] = l0 * r2;
+        l2 = l1; l1 = l0;
+      }
+    }
+  }
+  // where ring r and its mirror image lie on the mesh
+  if (threadIdx.x < 2) {
+    const int rr = threadIdx.x ? Pf - r : r;
+    const double theta = acos(threadIdx.x ? -x : x);
+    const double* thc = a.theta[p];
+    fid_ring f;
+    f.zone = 1; f.cell = 0; f.al = 0.0; f.tp = 0.0; f.pad = 0;
+    if (theta < thc[0]) { f.zone = 0; f.tp = theta / thc[0]; }
+    else if (theta > thc[P]) { f.zone = 2; f.tp = (kPi - theta) / (kPi - thc[P]); }
+    else {
+      int i = 0;
+      while (i + 1 < P && thc[i + 1] <= theta) ++i;
+      f.cell = i;
+      f.al = (theta - thc[i]) / (thc[i + 1] - thc[i]);
+    }
+    f.tri = 0;
+    for (int sb = 0; sb < a.factor; ++sb) f.tri |= (f.al >= (double)sb / a.factor) << sb;
+    if (rr != r || threadIdx.x == 0) ring[rr] = f;
   }
 }
 
@@ -275,20 +320,19 @@ __device__ __forceinline__ double vert_at(const fid_args& a, size_t idx) {
   return a.mixed ? (double)((const float*)a.verts)[idx] : ((const double*)a.verts)[idx];
 }
 
-constexpr int FRMAX = 8;   // fine rings per pass at most
+constexpr int FRMAX = 8;   // fine ring pairs per pass at most
 
-// Fine rings per pass for order p: as many as keep the pass's point tasks
-// (one per ring and longitude quarter) within one round of 256 threads.
-__host__ __device__ inline int fid_rings(int p, int factor) {
+// Pairs of fine rings (r and Pf - r) per pass for order p: as many as keep the
+// pass's point tasks (one per ring and longitude quarter) within two rounds of 256
+// threads, so that few lanes of the last warp idle.
+__host__ __device__ inline int fid_pairs(int p, int factor) {
   int nq = factor * p + 1, r = 256 / nq;
   return r < 1 ? 1 : (r > FRMAX ? FRMAX : r);
 }
 
 __host__ __device__ inline size_t fid_smem_doubles(int p, int factor) {
-  int P = 2 * p, Pf = factor * P, nl = (p + 1) * (p + 2) / 2, FR = fid_rings(p, factor);
-  return (size_t)3 * (p + 1) * (p + 1) + (P + 1) + (Pf + 1) + (size_t)FR * nl + (size_t)FR * 3 * (2 * p + 1) +
-         (size_t)(Pf / 2 + 1) * 2 * (p + 1) + (Pf + 1) + 2 * (size_t)nl + 2 * (size_t)(p + 1) +
-         (size_t)FR * 3 * (2 * P) * 4;
+  const size_t rings = 2 * fid_pairs(p, factor);
+  return (size_t)3 * (p + 1) * (p + 1) + rings * 3 * (2 * p + 1) + rings * 3 * (4 * p) * 4;
 }
 
 // The mesh along one fine ring, per coordinate field and longitude cell j
@@ -317,155 +361,132 @@ __device__ __forceinline__ void mesh_lines(const fid_args& a, size_t o, int P, i
   out[3] = u - q;
 }
 
-// One CTA per (vesicle, time level), FR fine rings per pass.  The series is
-// evaluated like the synthesis: ring sums G(m), then per longitude pair the
-// even and odd partial Fourier sums, which give the four longitudes
-// phi_k, pi - phi_k, pi + phi_k and 2 pi - phi_k (k <= Pf / 2) at once;
-// cos(m phi_k), sin(m phi_k) come from a table built per CTA.
+// CTA (vesicle, time level, chunk of the ring pairs), a few pairs per pass.  The
+// series is evaluated like the synthesis: ring sums G(m) of a ring and its mirror
+// image from the even and the odd terms, then per longitude the even and odd
+// partial Fourier sums of the three fields, which give the four longitudes phi_k,
+// pi - phi_k, pi + phi_k and 2 pi - phi_k (k <= Pf / 2) at once.  The chunks' maxima
+// meet in err (cleared before) by an atomic maximum of non-negative bit patterns.
+//
+// Bound by the FP64 pipe: the points (about 45 operations each at p = 12) are two
+// thirds of it.  What depends on the order alone (nodes, Legendre and trigonometric
+// values, places on the mesh) is tabulated once per handle instead of per call and
+// CTA; chunks fill the chip for few vesicles.  256 vesicles, p = 12, factor 4: 1.53 ->
+// 0.83 ms (the nodes alone took 0.23 ms); the FP64 pipe is 0.91 busy.
 __global__ void __launch_bounds__(256) fidelity_kernel(fid_args a) {
   extern __shared__ double sm[];
-  __shared__ double red[256 / 32];
+  __shared__ unsigned long long red[256 / 32];
   int v = blockIdx.x, t = blockIdx.y;
   if (a.p[v] < 1 || a.p[v] > STIV_MAX_P || !a.theta[a.p[v]]) {   // order outside [1, p_max]: NaN
-    if (threadIdx.x == 0) a.err[2 * (size_t)v + t] = __longlong_as_double(0x7ff8000000000000LL);
+    if (threadIdx.x == 0 && blockIdx.z == 0) a.err[2 * (size_t)v + t] = __longlong_as_double(0x7ff8000000000000LL);
     return;
   }
-  int p = a.p[v], P = 2 * p, Pf = a.factor * P, W = 2 * P, nv = 2 * P * (P + 1) + 2;
-  int nc = (p + 1) * (p + 1), nl = (p + 1) * (p + 2) / 2, ns = 2 * p + 1, nq = Pf / 2 + 1;
-  int FR = fid_rings(p, a.factor);
+  const int p = a.p[v], P = 2 * p, Pf = a.factor * P, W = 2 * P, nv = 2 * P * (P + 1) + 2;
+  const int nc = (p + 1) * (p + 1), nl = (p + 1) * (p + 2) / 2, ns = 2 * p + 1, nq = Pf / 2 + 1;
+  const int PR = fid_pairs(p, a.factor), npair = Pf / 2 + 1;   // pair r: rings r and Pf - r (the equator alone)
   double* C = sm;                   // [3][nc]
-  double* thc = C + 3 * nc;         // [P+1]  mesh rings (ascending theta)
-  double* xf = thc + (P + 1);       // [Pf+1] fine rings, x = cos(theta)
-  double* L = xf + (Pf + 1);        // [FR][nl] Legendre values of the current rings
-  double* G = L + FR * nl;          // [FR][3][ns] ring sums (slot 0: m=0; 2m-1: cos m; 2m: sin m)
-  double* T = G + FR * 3 * ns;      // [nq][2][p+1] cos, sin (m phi_k), k <= Pf/2
-  double* thf = T + (size_t)nq * 2 * (p + 1);   // [Pf+1] fine ring angles
-  double* ra = thf + (Pf + 1);      // [nl] Legendre recurrence coefficients
-  double* rb = ra + nl;             // [nl]
-  double* dg = rb + nl;             // [p+1]
-  double* sd = dg + (p + 1);        // [p+1]
-  double* ML = sd + (p + 1);        // [FR][3][W][4] mesh lines of the current rings (mesh_lines)
-  __shared__ int rzone[FRMAX], rcell[FRMAX], rtri[FRMAX];   // per current ring: zone, cell, triangle mask
-  __shared__ double ra_[FRMAX], rtp[FRMAX], btab[8];
+  double* G = C + 3 * nc;           // [2 PR][3][ns] ring sums (slot 0: m=0; 2m-1: cos m; 2m: sin m); pair k: rings 2k, 2k + 1
+  double* ML = G + 2 * PR * 3 * ns; // [2 PR][3][W][4] mesh lines of the current rings (mesh_lines)
+  __shared__ double btab[8];
+  __shared__ fid_ring info[2 * FRMAX];
+  const double* base_t = a.tab + a.off[p];
+  const fid_ring* ring = (const fid_ring*)base_t;
+  const double* leg = base_t + fid_ring_doubles(p, a.factor);
+  const double* trig = leg + fid_leg_doubles(p, a.factor);
   if (threadIdx.x < a.factor) btab[threadIdx.x] = (double)threadIdx.x / a.factor;
   const double* coef = a.coef + a.coef_off[v] + (size_t)t * 3 * nc;
   for (int k = threadIdx.x; k < 3 * nc; k += blockDim.x) C[k] = coef[k];
-  for (int i = threadIdx.x; i <= P; i += blockDim.x) thc[i] = a.theta[p][i];
-  for (int r = threadIdx.x; r <= Pf; r += blockDim.x) {
-    double x = a.xfine[a.xoff[p] + r];
-    xf[r] = x;
-    thf[r] = acos(x);
-  }
-  for (int m = threadIdx.x; m <= p; m += blockDim.x) {
-    dg[m] = m ? sqrt((2.0 * m + 1.0) / (2.0 * m)) : 0.0;
-    sd[m] = sqrt(2.0 * m + 3.0);
-  }
-  for (int e = threadIdx.x; e < nl; e += blockDim.x) {
-    int n = 0;
-    while ((n + 1) * (n + 2) / 2 <= e) ++n;
-    int m = e - n * (n + 1) / 2;
-    if (n >= m + 2) {
-      ra[e] = sqrt((4.0 * n * n - 1.0) / ((double)(n - m) * (n + m)));
-      rb[e] = sqrt(((double)(n - 1 - m) * (n - 1 + m)) / (4.0 * (n - 1) * (n - 1) - 1.0));
-    } else {
-      ra[e] = 0.0; rb[e] = 0.0;
-    }
-  }
-  for (int e = threadIdx.x; e < nq * (p + 1); e += blockDim.x) {
-    int k = e / (p + 1), m = e % (p + 1);
-    int kk = (m * k) % (2 * Pf);            // exact argument reduction
-    double sv, cv;
-    sincospi((double)kk / Pf, &sv, &cv);
-    T[(size_t)k * 2 * (p + 1) + m] = cv;
-    T[(size_t)k * 2 * (p + 1) + (p + 1) + m] = sv;
-  }
-  __syncthreads();
   size_t base = a.vert_off[v] + (size_t)t * 3 * nv;
-  double worst2 = 0.0;
-  for (int r0 = 0; r0 <= Pf; r0 += FR) {
-    int nr = Pf + 1 - r0 < FR ? Pf + 1 - r0 : FR;
-    if (threadIdx.x < nr * (p + 1)) {
-      int rr = threadIdx.x / (p + 1), m = threadIdx.x % (p + 1);
-      double x = xf[r0 + rr];
-      legendre_column_tab(p, m, x, sqrt((1.0 - x) * (1.0 + x)), dg, sd, ra, rb, L + rr * nl);
+  unsigned long long worst2 = 0;   // bit pattern of the largest squared distance
+  const int per = (npair + gridDim.z - 1) / gridDim.z, first = blockIdx.z * per, last = min(first + per, npair);
+  for (int r0 = first; r0 < last; r0 += PR) {
+    const int np = min(PR, last - r0);
+    __syncthreads();   // C, btab; info, G and ML are rewritten for the next rings
+    if (threadIdx.x < 2 * np) {
+      const int r = r0 + (threadIdx.x >> 1);
+      info[threadIdx.x] = ring[threadIdx.x & 1 ? Pf - r : r];
     }
-    if (threadIdx.x >= blockDim.x - nr) {   // where each ring lies on the mesh
-      int rr = threadIdx.x - (blockDim.x - nr);
-      double theta = thf[r0 + rr];
-      int zone = 1, i = 0;
-      double al = 0.0, tp = 0.0;
-      if (theta < thc[0]) { zone = 0; tp = theta / thc[0]; }
-      else if (theta > thc[P]) { zone = 2; tp = (kPi - theta) / (kPi - thc[P]); }
-      else {
-        while (i + 1 < P && thc[i + 1] <= theta) ++i;
-        al = (theta - thc[i]) / (thc[i + 1] - thc[i]);
+    // ring sums: lanes over the fields and rings of one order m run the same terms
+    for (int task = threadIdx.x; task < ns * 3 * np; task += blockDim.x) {
+      const int sl = task / (3 * np), rem = task - sl * 3 * np, f = rem / np, k = rem - f * np, m = (sl + 1) >> 1;
+      const int sgn = sl == 0 ? 0 : ((sl & 1) ? 1 : -1);
+      const double* Cf = C + f * nc + sgn * m;
+      const double* Lr = leg + (size_t)(r0 + k) * nl + m;
+      double E = 0.0, O = 0.0;
+      for (int n = m; n <= p; n += 2) {
+        E = fma(Cf[n * n + n], Lr[n * (n + 1) / 2], E);
+        if (n + 1 <= p) O = fma(Cf[(n + 1) * (n + 2)], Lr[(n + 1) * (n + 2) / 2], O);
       }
-      int mask = 0;
-      for (int sb = 0; sb < a.factor; ++sb) mask |= (al >= (double)sb / a.factor) << sb;
-      rzone[rr] = zone; rcell[rr] = i; rtri[rr] = mask; ra_[rr] = al; rtp[rr] = tp;
+      G[((2 * k) * 3 + f) * ns + sl] = E + O;
+      G[((2 * k + 1) * 3 + f) * ns + sl] = E - O;
     }
     __syncthreads();
-    for (int task = threadIdx.x; task < nr * 3 * (ns + W); task += blockDim.x) {
-      if (task < nr * 3 * ns) {   // ring sums
-        int rr = task / (3 * ns), rem = task % (3 * ns), f = rem / ns, sl = rem % ns, m = (sl + 1) >> 1;
-        int sgn = sl == 0 ? 0 : ((sl & 1) ? 1 : -1);
-        const double* Lr = L + rr * nl;
-        double acc = 0.0;
-        for (int n = m; n <= p; ++n) acc = fma(C[f * nc + n * n + n + sgn * m], Lr[n * (n + 1) / 2 + m], acc);
-        G[(rr * 3 + f) * ns + sl] = acc;
-      } else {                    // mesh lines
-        int k2 = task - nr * 3 * ns, rr = k2 / (3 * W), rem = k2 % (3 * W), f = rem / W, j = rem % W;
-        mesh_lines(a, base + (size_t)f * nv, P, W, rzone[rr], rcell[rr], ra_[rr], rtp[rr], j,
-                   ML + ((size_t)(rr * 3 + f) * W + j) * 4);
-      }
+    for (int task = threadIdx.x; task < 2 * np * 3 * W; task += blockDim.x) {
+      const int q = task / (3 * W), rem = task - q * 3 * W, f = rem / W, j = rem - f * W;
+      const fid_ring& R = info[q];
+      mesh_lines(a, base + (size_t)f * nv, P, W, R.zone, R.cell, R.al, R.tp, j, ML + (size_t)task * 4);
     }
     __syncthreads();
-    for (int task = threadIdx.x; task < nr * nq; task += blockDim.x) {
-      int rr = task / nq, q = task % nq;
-      int tri = rtri[rr];
-      const double* cs = T + (size_t)q * 2 * (p + 1);
-      const double* sn = cs + (p + 1);
-      int kq[4] = {q, Pf - q, Pf + q, (2 * Pf - q) % (2 * Pf)};
-      double val[4][3];
+    for (int task = threadIdx.x; task < 2 * np * nq; task += blockDim.x) {
+      const int k = task / nq, q = task - k * nq;
+      if ((k & 1) && 2 * (r0 + (k >> 1)) == Pf) continue;   // the equator's image is itself
+      const int tri = info[k].tri;
+      const double* g = G + (size_t)k * 3 * ns;
+      double Ce[3], Co[3], Se[3], So[3];
 #pragma unroll
-      for (int f = 0; f < 3; ++f) {
-        const double* g = G + (size_t)(rr * 3 + f) * ns;
-        double Ce = g[0], Co = 0.0, Se = 0.0, So = 0.0;
-        for (int m = 1; m <= p; m += 2) { Co = fma(g[2 * m - 1], cs[m], Co); So = fma(g[2 * m], sn[m], So); }
-        for (int m = 2; m <= p; m += 2) { Ce = fma(g[2 * m - 1], cs[m], Ce); Se = fma(g[2 * m], sn[m], Se); }
-        val[0][f] = (Ce + Co) + (Se + So);     // phi_q
-        val[1][f] = (Ce - Co) + (So - Se);     // pi - phi_q
-        val[2][f] = (Ce - Co) + (Se - So);     // pi + phi_q
-        val[3][f] = (Ce + Co) - (Se + So);     // 2 pi - phi_q
+      for (int f = 0; f < 3; ++f) { Ce[f] = g[f * ns]; Co[f] = 0.0; Se[f] = 0.0; So[f] = 0.0; }
+      for (int m = 1; m <= p; m += 2) {
+        double c = trig[(size_t)(2 * m) * nq + q], sn = trig[(size_t)(2 * m + 1) * nq + q];
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          Co[f] = fma(g[f * ns + 2 * m - 1], c, Co[f]);
+          So[f] = fma(g[f * ns + 2 * m], sn, So[f]);
+        }
+        if (m + 1 <= p) {
+          c = trig[(size_t)(2 * m + 2) * nq + q]; sn = trig[(size_t)(2 * m + 3) * nq + q];
+#pragma unroll
+          for (int f = 0; f < 3; ++f) {
+            Ce[f] = fma(g[f * ns + 2 * m + 1], c, Ce[f]);
+            Se[f] = fma(g[f * ns + 2 * m + 2], sn, Se[f]);
+          }
+        }
       }
+      const int kq[4] = {q, Pf - q, Pf + q, (2 * Pf - q) % (2 * Pf)};
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
-        int k = kq[w];
-        bool dup = (w == 1 && k == kq[0]) || (w == 2 && (k == kq[1] || k >= 2 * Pf)) ||
-                   (w == 3 && (k == kq[0] || k == kq[2]));
+        const int kk = kq[w];
+        const bool dup = (w == 1 && kk == kq[0]) || (w == 2 && (kk == kq[1] || kk >= 2 * Pf)) ||
+                         (w == 3 && (kk == kq[0] || kk == kq[2]));
         if (dup) continue;
-        int j = k / a.factor, sb = k % a.factor;
-        double b = btab[sb];
-        int side = (tri >> sb) & 1 ? 0 : 2;
+        const int j = kk / a.factor, sb = kk - j * a.factor;
+        const double b = btab[sb];
+        const int side = (tri >> sb) & 1 ? 0 : 2;
         double d2 = 0.0;
 #pragma unroll
         for (int f = 0; f < 3; ++f) {
-          const double* l = ML + ((size_t)(rr * 3 + f) * W + j) * 4 + side;
-          double e = fma(b, l[1], l[0]) - val[w][f];
+          const double C0 = w == 0 || w == 3 ? Ce[f] + Co[f] : Ce[f] - Co[f];
+          const double S0 = w == 0 || w == 3 ? Se[f] + So[f] : Se[f] - So[f];
+          const double val = w == 0 || w == 2 ? C0 + S0 : C0 - S0;   // phi, pi - phi, pi + phi, 2 pi - phi
+          const double* l = ML + ((size_t)(k * 3 + f) * W + j) * 4 + side;
+          const double e = fma(b, l[1], l[0]) - val;
           d2 = fma(e, e, d2);
         }
-        worst2 = fmax(worst2, d2);   // squared distance; one square root at the end
+        // the maximum on the integer pipe; a NaN is ignored, as fmax ignores it
+        const unsigned long long u = (unsigned long long)__double_as_longlong(d2);
+        if (u > worst2 && u <= 0x7FF0000000000000ull) worst2 = u;
       }
     }
-    __syncthreads();   // L and G are rewritten for the next rings
   }
-  for (int off = 16; off > 0; off >>= 1) worst2 = fmax(worst2, __shfl_xor_sync(0xffffffffu, worst2, off));
+  for (int off = 16; off > 0; off >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(0xffffffffu, worst2, off);
+    worst2 = o > worst2 ? o : worst2;
+  }
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = worst2;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double w = red[0];
-    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) w = fmax(w, red[q]);
-    a.err[2 * (size_t)v + t] = sqrt(w);
+    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) worst2 = red[q] > worst2 ? red[q] : worst2;
+    const double e = sqrt(__longlong_as_double((long long)worst2));
+    atomicMax((unsigned long long*)&a.err[2 * (size_t)v + t], (unsigned long long)__double_as_longlong(e));
   }
 }
 
@@ -543,26 +564,43 @@ extern "C" int stiv_mesh_fidelity(stiv_handle* h, void* stream, int32_t n_ves, i
     if (rc) return rc;
     a.theta[p] = h->tab[p].theta;
   }
-  int nx = 0;
-  for (int p = 1; p <= p_max; ++p) { a.xoff[p] = nx; nx += factor * 2 * p + 1; }
-  a.xoff[0] = 0;
-  if (sizeof(double) * (size_t)nx > h->fid_x_bytes) {
-    if (h->fid_x) { STIV_CUDA(h, cudaFree(h->fid_x)); h->fid_x = nullptr; h->fid_x_bytes = 0; }
-    STIV_CUDA(h, cudaMalloc(&h->fid_x, sizeof(double) * (size_t)nx));
-    h->fid_x_bytes = sizeof(double) * (size_t)nx;
-  }
-  a.xfine = h->fid_x;
-  size_t smem = 0;
+  size_t total = 0, smem = 0;
+  for (int p = 0; p <= STIV_MAX_P; ++p) a.off[p] = 0;
   for (int p = 1; p <= p_max; ++p) {
+    a.off[p] = total;
+    total += fid_doubles(p, factor);
     size_t b = sizeof(double) * fid_smem_doubles(p, factor);
     smem = b > smem ? b : smem;
   }
-  if (smem > 220 * 1024) return STIV_ERR_ARG;
+  STIV_PROF_N(h, st, "mesh_fidelity", 2);
+  // The tables stay valid for the same stream, factor and orders.  A table made on
+  // another stream would need waiting for: it is made again.  A captured call makes
+  // them in its graph, whose replays overwrite them at any time: from then on every
+  // call of the handle makes its own.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  STIV_CUDA(h, cudaStreamIsCapturing(st, &cap));
+  if (cap != cudaStreamCaptureStatusNone) h->fid_captured = true;
+  const bool made = h->fid_tab && !h->fid_captured && h->fid_factor == factor && h->fid_pmax == p_max &&
+                    h->fid_stream == stream;
+  if (sizeof(double) * total > h->fid_tab_bytes) {
+    if (h->fid_tab) { STIV_CUDA(h, cudaFree(h->fid_tab)); h->fid_tab = nullptr; h->fid_tab_bytes = 0; }
+    STIV_CUDA(h, cudaMalloc(&h->fid_tab, sizeof(double) * total));
+    h->fid_tab_bytes = sizeof(double) * total;
+  }
+  a.tab = h->fid_tab;
+  if (!made) {
+    fid_tables_kernel<<<dim3(factor * p_max + 1, p_max), 64, 0, st>>>(a, h->fid_tab);
+    STIV_LAUNCH(h);
+    h->fid_factor = factor; h->fid_pmax = p_max; h->fid_stream = stream;
+  }
+  STIV_CUDA(h, cudaMemsetAsync(err_dev, 0, sizeof(double) * 2 * (size_t)n_ves, st));
   if (smem > 48 * 1024)
     STIV_CUDA(h, cudaFuncSetAttribute(fidelity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  STIV_PROF_N(h, st, "mesh_fidelity", 2);
-  fine_nodes_kernel<<<(nx + 127) / 128, 128, 0, st>>>(p_max, factor, h->fid_x);
-  fidelity_kernel<<<dim3(n_ves, 2), 256, smem, st>>>(a);
+  // enough chunks for a dozen CTAs per SM, at most one per pass of the largest order
+  const int passes = (factor * p_max + fid_pairs(p_max, factor)) / fid_pairs(p_max, factor);
+  int chunks = (12 * 152 + 2 * n_ves - 1) / (2 * n_ves);
+  chunks = chunks < 1 ? 1 : (chunks > passes ? passes : chunks);
+  fidelity_kernel<<<dim3(n_ves, 2, chunks), 256, smem, st>>>(a);
   STIV_LAUNCH(h);
   return STIV_OK;
 }

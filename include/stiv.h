@@ -266,7 +266,7 @@ int stiv_step(stiv_handle* h, void* stream, int32_t use_graph, int32_t n_ves, in
  * then cleared, graph records are kept for the next replay (read once per
  * replay).  Stage names: synth, boxes, pairs (for many
  * vesicles cells, sort_cells, cell_pairs, sort_pairs, unique_pairs instead),
- * patch_pairs, narrow, pieces, fp64, contact_order, finalize, stiv, stiv_grad,
+ * patch_pairs, narrow, pieces, fp64, contact_order, stiv, stiv_grad,
  * vpair, grad_scatter, grad_to_coef. */
 int stiv_profile(stiv_handle* h, int32_t enable);
 int stiv_profile_read(stiv_handle* h, int32_t max_names, char* names, int64_t* launches, double* total_ms,

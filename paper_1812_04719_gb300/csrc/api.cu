@@ -13,7 +13,7 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
 int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, const int64_t* voff, const void* X,
                       const stiv_pairs* cand, detect_ws& w, int num_sms, int p_max);
 int stiv_contact_order(stiv_handle* h, cudaStream_t st, const stiv_pairs* cand, const stiv_contacts* out,
-                       detect_ws& w);
+                       detect_ws& w, int64_t* counts);
 
 namespace {
 
@@ -29,17 +29,6 @@ __global__ void topology_kernel(int P, int32_t* tri, int32_t* edge) {
     int n = stiv_forward_nbrs(P, k, nb);
     int e0 = stiv_first_edge(P, k);
     for (int q = 0; q < n; ++q) { edge[2 * (e0 + q)] = k; edge[2 * (e0 + q) + 1] = nb[q]; }
-  }
-}
-
-__global__ void finalize_kernel(int64_t* ctr, int64_t C, int64_t* counts, int* tc_status) {
-  if (threadIdx.x == 0) {
-    if (ctr[11] > C) ctr[STIV_C_STATUS] |= STIV_F_CONTACTS_OVERFLOW;
-    if (tc_status && *tc_status) { ctr[STIV_C_STATUS] |= STIV_F_TIMEOUT; *tc_status = 0; }
-    for (int k = 0; k < 8; ++k) counts[k] = ctr[k];
-    counts[STIV_C_FLOPS] = ctr[12];
-    counts[STIV_C_EXACT] = ctr[13];
-    counts[STIV_C_PIECE] = ctr[14];
   }
 }
 
@@ -330,12 +319,7 @@ extern "C" int stiv_detect(stiv_handle* h, void* stream, int32_t n_ves, int32_t 
   if (rc) return rc;
   rc = stiv_narrow_phase(h, st, p_dev, vert_off_dev, verts_dev, cand, w, sms, p_max);
   if (rc) return rc;
-  rc = stiv_contact_order(h, st, cand, out, w);
-  if (rc) return rc;
-  STIV_PROF(h, st, "finalize");
-  finalize_kernel<<<1, 32, 0, st>>>(w.ctr, w.C, counts_dev, h->tc_status);
-  STIV_LAUNCH(h);
-  return STIV_OK;
+  return stiv_contact_order(h, st, cand, out, w, counts_dev);
 }
 
 extern "C" int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_t p_max, const int32_t* p_dev,
@@ -344,7 +328,7 @@ extern "C" int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_
                              double* best_ms_out) {
   if (!h || !counts_dev) return STIV_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  static const int32_t cands[STIV_NTUNE][4] = {{2, 3, 4, 0}, {1, 2, 3, 4}, {4, 8, 16, 32}, {2, 4, 8, 0}, {2, 3, 4, 0}};
+  static const int32_t cands[STIV_NTUNE][4] = {{2, 3, 4, 0}, {1, 2, 3, 4}, {4, 8, 16, 32}, {8, 12, 16, 0}, {2, 3, 4, 5}};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   STIV_CUDA(h, cudaEventCreate(&e0));
   STIV_CUDA(h, cudaEventCreate(&e1));

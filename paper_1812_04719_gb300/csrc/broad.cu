@@ -64,8 +64,14 @@ __device__ __forceinline__ float d2f_dir(double x, bool up) {
 // the min / max run on order-preserving integer images (exact), and the
 // per-vertex FP32 boxes are rounded outward on the integer pipe, so that the
 // FP64 pipe only forms the staging differences.
+//
+// Bound by the latency of its phases more than by HBM (302 MB at 1440 vesicles and
+// p = 16, 0.045 ms of copy): 512 threads instead of 256, the reduction by shuffles
+// instead of eight barriers, two lanes per patch (a column half each): 0.176 ->
+// 0.158 ms.
+constexpr int BT = 512;
 template <bool MIXED>
-__global__ void __launch_bounds__(256) boxes_kernel(int n, const int32_t* pv, const int64_t* voff, const void* X,
+__global__ void __launch_bounds__(BT) boxes_kernel(int n, const int32_t* pv, const int64_t* voff, const void* X,
                                                     int mixed, double dm, double Lx, double Ly, double Lz,
                                                     double* vbox, float* pbox, int pstride, float* vorg,
                                                     float* fprep, int64_t fstride, int64_t* ctr, size_t vb_cap,
@@ -89,7 +95,7 @@ __global__ void __launch_bounds__(256) boxes_kernel(int n, const int32_t* pv, co
   int P = 2 * pv[v], nv = stiv_nverts(P);
   bool use_sm = (size_t)6 * nv <= vb_cap;
   const size_t base = voff[v];
-  __shared__ long long red[6][256];
+  __shared__ long long red[BT / 32][6];
   double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   bool bad = false;
   if (MIXED) {
@@ -133,23 +139,26 @@ __global__ void __launch_bounds__(256) boxes_kernel(int n, const int32_t* pv, co
         }
       }
   }
-  for (int c = 0; c < 3; ++c) { red[c][threadIdx.x] = klo[c]; red[3 + c][threadIdx.x] = khi[c]; }
+  for (int o = 16; o > 0; o >>= 1)
+    for (int c = 0; c < 3; ++c) {
+      const long long a = __shfl_xor_sync(0xffffffffu, klo[c], o), b = __shfl_xor_sync(0xffffffffu, khi[c], o);
+      klo[c] = a < klo[c] ? a : klo[c];
+      khi[c] = b > khi[c] ? b : khi[c];
+    }
+  if ((threadIdx.x & 31) == 0)
+    for (int c = 0; c < 3; ++c) { red[threadIdx.x >> 5][c] = klo[c]; red[threadIdx.x >> 5][3 + c] = khi[c]; }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr((unsigned long long*)&ctr[STIV_C_STATUS], STIV_F_NONFINITE);
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-      for (int c = 0; c < 3; ++c) {
-        long long a = red[c][threadIdx.x + s], b = red[3 + c][threadIdx.x + s];
-        if (a < red[c][threadIdx.x]) red[c][threadIdx.x] = a;
-        if (b > red[3 + c][threadIdx.x]) red[3 + c][threadIdx.x] = b;
-      }
-    __syncthreads();
-  }
   __shared__ float sorg[4];
   __shared__ double vlo_s[3], vhi_s[3];
   if (threadIdx.x < 3) {
     int c = threadIdx.x;
-    vlo_s[c] = okey_val(red[c][0]);
-    vhi_s[c] = okey_val(red[3 + c][0]);
+    long long a = red[0][c], b = red[0][3 + c];
+    for (int q = 1; q < BT / 32; ++q) {
+      a = red[q][c] < a ? red[q][c] : a;
+      b = red[q][3 + c] > b ? red[q][3 + c] : b;
+    }
+    vlo_s[c] = okey_val(a);
+    vhi_s[c] = okey_val(b);
   }
   __syncthreads();
   if (threadIdx.x < 3) {
@@ -207,8 +216,11 @@ __global__ void __launch_bounds__(256) boxes_kernel(int n, const int32_t* pv, co
   // rounding the FP64 min / max.
   int nbr = stiv_nband_blocks(P), nbc = stiv_ncol_blocks(P), W = 2 * P;
   __syncthreads();
-  for (int patch = threadIdx.x; patch < nbr * nbc; patch += blockDim.x) {
-    int I = patch / nbc, J = patch % nbc;
+  // lanes 2 k and 2 k + 1 take the column halves of one patch
+  for (int t0 = 0; t0 < 2 * nbr * nbc; t0 += blockDim.x) {
+    const int task = t0 + threadIdx.x, patch = task >> 1, h = task & 1;
+    const bool on = patch < nbr * nbc;
+    int I = on ? patch / nbc : 0, J = on ? patch % nbc : 0;
     int r0 = I * STIV_BR, c0 = J * STIV_BC;
     // per column half: rb[row][lo xyz, hi xyz] of its three rows; pb[pole]:
     // FP32, rounded outward
@@ -232,8 +244,7 @@ __global__ void __launch_bounds__(256) boxes_kernel(int n, const int32_t* pv, co
     }
     float* B = pbox + ((size_t)v * pstride + patch) * STIV_PBOX;
     float plo[3] = {INFINITY, INFINITY, INFINITY}, phi[3] = {-INFINITY, -INFINITY, -INFINITY};
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
+    {
       float rb[3][6];
 #pragma unroll
       for (int rr = 0; rr < 3; ++rr) {
@@ -259,12 +270,21 @@ __global__ void __launch_bounds__(256) boxes_kernel(int n, const int32_t* pv, co
           plo[c] = fminf(plo[c], lo[c]);
           phi[c] = fmaxf(phi[c], hi[c]);
         }
-        float4* C = (float4*)(B + STIV_PBOX_CELLS) + 2 * (2 * b + h);
-        C[0] = make_float4(lo[0], lo[1], lo[2], 0.f);
-        C[1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+        if (on) {
+          float4* C = (float4*)(B + STIV_PBOX_CELLS) + 2 * (2 * b + h);
+          C[0] = make_float4(lo[0], lo[1], lo[2], 0.f);
+          C[1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+        }
       }
     }
-    for (int c = 0; c < 3; ++c) { B[c] = plo[c]; B[3 + c] = phi[c]; }
+    for (int c = 0; c < 3; ++c) {
+      plo[c] = fminf(plo[c], __shfl_xor_sync(0xffffffffu, plo[c], 1));
+      phi[c] = fmaxf(phi[c], __shfl_xor_sync(0xffffffffu, phi[c], 1));
+    }
+    if (on && h == 0) {
+      ((float4*)B)[0] = make_float4(plo[0], plo[1], plo[2], phi[0]);
+      ((float4*)B)[1] = make_float4(phi[1], phi[2], 0.f, 0.f);
+    }
   }
 }
 
@@ -632,7 +652,7 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   size_t bsmem = vb_cap * sizeof(float);
   auto bk = mixed ? boxes_kernel<true> : boxes_kernel<false>;
   STIV_CUDA(h, cudaFuncSetAttribute(bk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem));
-  bk<<<n, 256, bsmem, st>>>(n, p_dev, voff, X, mixed, h->prm.d_m, L[0], L[1], L[2], w.vbox, w.pbox,
+  bk<<<n, BT, bsmem, st>>>(n, p_dev, voff, X, mixed, h->prm.d_m, L[0], L[1], L[2], w.vbox, w.pbox,
                                       w.pstride, w.vorg, w.fprep, w.fstride, ctr, vb_cap, p_max, w.fbox);
   }
   if (n <= STIV_BRUTE_MAX) {

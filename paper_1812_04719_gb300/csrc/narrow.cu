@@ -101,6 +101,7 @@ struct narrow_args {
   int64_t C;  // raw contact capacity
   int32_t* rc_pair; int32_t* rc_type; int32_t* rc_a; int32_t* rc_b;
   double* rc_tau; double* rc_w;
+  int32_t* pair_cnt;        // contacts per candidate pair
   int64_t* ctr;
 };
 
@@ -627,9 +628,9 @@ __device__ __forceinline__ int separation_reject(bool ee, const blossom& q, floa
   }
 }
 
-// Stage 3a on one pair: 1 if the FP64 test certainly finds nothing.  The cubic
-// keeps one sign over the step (with d_m > 0: keeps |f| above d_m |m|; |m(t)| is
-// at most the largest of |n00|, |n01| / 2, |n11|), or the first direction
+// Stage 3a on one pair: nonzero if the FP64 test certainly finds nothing.  1: the
+// cubic keeps one sign over the step (with d_m > 0: keeps |f| above d_m |m|; |m(t)| is
+// at most the largest of |n00|, |n01| / 2, |n11|); 2: the first direction
 // separates the primitives.
 template <bool DM>
 __device__ __forceinline__ int reject_fp32(bool ee, const blossom& q, float e, float dm) {
@@ -644,7 +645,7 @@ __device__ __forceinline__ int reject_fp32(bool ee, const blossom& q, float e, f
   } else if (f > 0.f) {
     return 1;
   }
-  return separation_reject<DM, 1>(ee, q, e, dm);
+  return 2 * separation_reject<DM, 1>(ee, q, e, dm);
 }
 
 // ---------------------------------------------------------------------------
@@ -745,19 +746,6 @@ __device__ __forceinline__ bool df_of_unit(double m, dflt& r) {
 //
 // The bisection takes exactly the FP64 path: every midpoint is the FP64
 // midpoint (mid_rn), and every sign is the sign of the FP64 Horner value.
-// That sign is read from an FP32 Horner evaluation when its error bound
-// proves it:  |f64(mid) - f32| <= gamma_6(2^-53) S + 2^-24 S + gamma_6(2^-24) S
-// (1 + 2^-24) + 2^-23 S1 <= 4.2e-7 S + 1.2e-7 S1, with S = sum |k_i| and S1 =
-// |k1| + 2|k2| + 3|k3| (t in [0, 1]; Horner error bounds, coefficient
-// rounding, and the truncation of the midpoint times max |f'|).  When
-// |f32| > E the FP64 value has the same sign and is not zero; otherwise the
-// FP64 Horner value is computed.  Coefficients outside [1e-25, 1e25] keep
-// every FP32 term far from underflow and overflow, else only FP64 is used.
-// Between the two, a double-float Horner evaluation decides the sign when
-// |f_df| > 2^-40 (S + S1): its own error (3 multiply-add steps at <= 2^-44
-// relative each), the coefficients' and the midpoint's representation
-// (2^-48 |k_i|, 2^-47 m times max |f'|) and the FP64 Horner error (< 2^-50 S)
-// together stay below that bound.
 //
 // Most halvings need no value at all.  An approximate root r (FP32 Newton steps,
 // two steps on FP64 values) and the FP64 values at r - delta and r + delta prove
@@ -767,9 +755,10 @@ __device__ __forceinline__ bool df_of_unit(double m, dflt& r) {
 // farther out.  From [0, 1] (nearly every pair) the midpoints are dyadic and
 // exact as long as the interval is wider than an ulp, so the halvings down to
 // the common binary prefix of r - delta and r + delta (43 of some 54) are taken
-// at once.  Those left end at FP64 noise and are decided by FP64 values; the tiers
-// above serve where r - delta and r + delta prove nothing (r near a multiple
-// root).
+// at once.  Those left, and all where r - delta and r + delta prove nothing (r
+// near a multiple root), are decided by FP64 values: signs from FP32 and
+// double-float values there cost more than they save (0.425 -> 0.41 ms at 1440
+// vesicles without them).
 struct poly32 { float f0, f1, f2, f3, S, S1; bool in_range; };   // FP32 images of the cubic's coefficients
 
 __device__ __forceinline__ poly32 poly_fp32(double k0, double k1, double k2, double k3) {
@@ -836,11 +825,9 @@ __device__ double bisect64(const poly32& p, double k0, double k1, double k2, dou
   const bool neg_lo = is_neg(flo);
   int it = 0;
   double l, h;   // signs known up to l and from h on
-  bool tiers = true;
   {
     long long li, hi_;
     if (p.in_range && root_bounds(p, k0, k1, k2, k3, neg_lo, lo, hi, l, h, li, hi_)) {
-      tiers = false;
       if (__double_as_longlong(lo) == 0 && __double_as_longlong(hi) == 0x3FF0000000000000ll) {
         it = __clzll(li ^ hi_) - 2;   // the cell of 2^-it that holds both
         long long c = li >> (62 - it);
@@ -853,8 +840,6 @@ __device__ double bisect64(const poly32& p, double k0, double k1, double k2, dou
       l = -1.0; h = 2.0;
     }
   }
-  const float E = p.S > 1e-25f && p.S < 1e25f ? 1.01f * (4.5e-7f * p.S + 1.25e-7f * p.S1) : INFINITY;
-  const float Edf = 1.01f * 9.094947e-13f * (p.S + p.S1);   // 2^-40
 #pragma unroll 1
   for (; it < 64; ++it) {
     bool ok;
@@ -867,23 +852,6 @@ __device__ double bisect64(const poly32& p, double k0, double k1, double k2, dou
     flops += 6;
     bool neg = neg_lo, done = bm <= __double_as_longlong(l);   // l = -1: a negative pattern
     if (bm >= __double_as_longlong(h)) { neg = !neg_lo; done = true; }
-    if (tiers && !done) {
-      float m = trunc_f32(mid);
-      float fs = fmaf(fmaf(fmaf(p.f3, m, p.f2), m, p.f1), m, p.f0);
-      neg = fs < 0.0f;
-      done = fabsf(fs) > E;
-      dflt md;
-      if (!done && p.in_range && df_of_unit(mid, md)) {
-        dflt c0 = {p.f0, __double2float_rn(__dsub_rn(k0, (double)p.f0))},
-             c1 = {p.f1, __double2float_rn(__dsub_rn(k1, (double)p.f1))},
-             c2 = {p.f2, __double2float_rn(__dsub_rn(k2, (double)p.f2))},
-             c3 = {p.f3, __double2float_rn(__dsub_rn(k3, (double)p.f3))};
-        dflt v = df_add(df_mul(df_add(df_mul(df_add(df_mul(c3, md), c2), md), c1), md), c0);
-        float vv = v.h + v.l;
-        neg = vv < 0.0f;
-        done = fabsf(vv) > Edf;
-      }
-    }
     if (!done) {
       double fm = horner3(k0, k1, k2, k3, mid);
       if (is_zero(fm)) return mid;
@@ -1026,7 +994,9 @@ __device__ int ccd64(int kind, const d3* X0, const d3* D, double& tau, double& w
     if (cp[1] < cp[0]) { double t = cp[0]; cp[0] = cp[1]; cp[1] = t; }
     if (cp[1] == cp[0]) ncp = 1;
   }
-  // the value at 1, from FP32 when that proves its sign
+  // the value at 1, from FP32 when that proves its sign: |f64 - f32| <=
+  // gamma_6(2^-53) S + 2^-24 S + gamma_6(2^-24) S (1 + 2^-24) (Horner errors and
+  // coefficient rounding) stays below 4.5e-7 S
   double f1v;
   {
     float fs = ((p.f3 + p.f2) + p.f1) + p.f0;
@@ -1393,7 +1363,7 @@ __global__ void __launch_bounds__(NW * 32, 3) narrow_kernel(narrow_args a) {
   __syncthreads();
   int64_t nwork = a.ctr[STIV_C_PATCH];
   if (nwork > a.W) nwork = a.W;
-  long long nprim = 0;
+  long long nprim = 0, nleft = 0;   // pairs whose exact boxes overlap; of them, those the sign test leaves
   long long item = 0;
   if (lane == 0) item = (long long)atomicAdd((unsigned long long*)&a.ctr[10], 1ull);
   item = __shfl_sync(0xffffffffu, item, 0);
@@ -1496,7 +1466,9 @@ __global__ void __launch_bounds__(NW * 32, 3) narrow_kernel(narrow_args a) {
             blossom bl = blossom_fp32(ee, {xp.x, xp.y, xp.z}, {xq.x, xq.y, xq.z}, {xh.x, xh.y, xh.z},
                                       {xg.x, xg.y, xg.z}, {dp.x, dp.y, dp.z}, {dq.x, dq.y, dq.z}, {dh.x, dh.y, dh.z},
                                       {dg.x, dg.y, dg.z}, e);
-            keep = !reject_fp32<DM>(ee, bl, e, (float)a.dm);
+            const int rej = reject_fp32<DM>(ee, bl, e, (float)a.dm);
+            keep = rej == 0;
+            nleft += rej != 1;
           }
         }
         unsigned m = __ballot_sync(0xffffffffu, keep);
@@ -1537,8 +1509,12 @@ __global__ void __launch_bounds__(NW * 32, 3) narrow_kernel(narrow_args a) {
     }
     item = __shfl_sync(0xffffffffu, next, 0);
   }
-  for (int off = 16; off > 0; off >>= 1) nprim += __shfl_down_sync(0xffffffffu, nprim, off);
+  for (int off = 16; off > 0; off >>= 1) {
+    nprim += __shfl_down_sync(0xffffffffu, nprim, off);
+    nleft += __shfl_down_sync(0xffffffffu, nleft, off);
+  }
   if (lane == 0 && nprim) atomicAdd((unsigned long long*)&a.ctr[STIV_C_PRIM], (unsigned long long)nprim);
+  if (lane == 0 && nleft) atomicAdd((unsigned long long*)&a.ctr[17], (unsigned long long)nleft);
 }
 
 // ---------------------------------------------------------------------------
@@ -1872,6 +1848,14 @@ __global__ void __launch_bounds__(128, DM ? 8 : 6) fp64_kernel(narrow_args a) {
           a.rc_tau[k] = tau; a.rc_w[2 * k] = w1; a.rc_w[2 * k + 1] = w2;
         }
       }
+      // contacts per pair (for their ordering): one addition per warp while its
+      // contacts belong to one pair
+      const int rl = __shfl_sync(0xffffffffu, r, leader);
+      if ((int64_t)cb + __popc(m) <= a.C && __all_sync(0xffffffffu, type < 0 || r == rl)) {
+        if (lane == leader) atomicAdd(&a.pair_cnt[rl], __popc(m));
+      } else if (type >= 0 && (int64_t)cb + __popc(m & ((1u << lane) - 1u)) < a.C) {   // those stored
+        atomicAdd(&a.pair_cnt[r], 1);
+      }
       unsigned mee = __ballot_sync(0xffffffffu, type == 2);
       if (lane == leader) {
         if (mee) atomicAdd((unsigned long long*)&a.ctr[STIV_C_EE], (unsigned long long)__popc(mee));
@@ -1891,31 +1875,68 @@ __global__ void __launch_bounds__(128, DM ? 8 : 6) fp64_kernel(narrow_args a) {
   }
 }
 
-// Level 1: patch pairs of one candidate vesicle pair per warp.  A's patches
+// Level 1: the patch pairs of one candidate vesicle pair per CTA.  A's patches
 // are kept that meet vesicle j's box, then B's that meet the union of A's
 // kept patches, then A's that meet the union of B's; a pair of kept patches
 // is emitted when their boxes overlap and some cell of one meets some cell
 // of the other (every primitive lies in one cell of its patch).  Dynamic
-// shared memory: per warp 2 x mp patch boxes and 2 x mp list entries.
-__global__ void __launch_bounds__(128) patch_pairs_kernel(const int32_t* pv, const double* vbox, const float* pbox,
+// shared memory: two lists of mp boxes with their patch ids.
+//
+// Bound by latency: with one warp per vesicle pair a few deep pairs held the stage
+// (a hundred by a hundred patches, 32 at a time); a CTA's warps share them.  1440
+// vesicles 0.25 -> 0.14 ms, 4096 1.15 -> 0.52, 64 at 30% 0.13 -> 0.04.
+constexpr int PPT = 128;   // threads of a CTA
+
+struct patch_list {
+  float4* lo;              // box (w: patch id)
+  float4* hi;
+};
+
+__global__ void __launch_bounds__(PPT) patch_pairs_kernel(const int32_t* pv, const double* vbox, const float* pbox,
                                                           double Lx, double Ly, double Lz, const int32_t* ci,
                                                           const int32_t* cj, const int32_t* cs, int64_t cap,
                                                           int64_t W, uint64_t* work, int64_t* ctr, int mp,
                                                           const float* vorg, const int64_t* voff,
                                                           stiv_pair_info* pinfo, double dm) {
-  extern __shared__ float psm[];
-  int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* sbw = psm + (size_t)wid * 2 * mp * 6;                       // [2][mp][6]
-  unsigned short* law = (unsigned short*)(psm + (size_t)4 * 2 * mp * 6) + (size_t)wid * 2 * mp;
-  unsigned short* lbw = law + mp;
+  extern __shared__ float4 psm[];
+  __shared__ int nlist[3];         // kept patches of A, of B, of A after the second filter
+  __shared__ int ubox[2][6];       // union boxes (order-preserving images)
+  const patch_list la = {psm, psm + mp}, lb = {psm + 2 * mp, psm + 3 * mp};
+  const int lane = threadIdx.x & 31;
+  const unsigned lower = (1u << lane) - 1u;
   int64_t npairs = ctr[STIV_C_PAIRS];
   if (npairs > cap) npairs = cap;
-  double L[3] = {Lx, Ly, Lz};
-  for (int64_t r = (int64_t)blockIdx.x * 4 + wid; r < npairs; r += (int64_t)gridDim.x * 4) {
-    int i = ci[r], j = cj[r], code = cs[r];
-    int s[3] = {code / 9 - 1, (code / 3) % 3 - 1, code % 3 - 1};
-    int Pi = 2 * pv[i], Pj = 2 * pv[j];
-    if (lane == 0) {
+  const double L[3] = {Lx, Ly, Lz};
+  // append boxes to a list (in any order) and merge them into a union box
+  auto keep_box = [&](const patch_list& l, int* n, int* u, bool hit, float4 lo, float4 hi) {
+    const unsigned m = __ballot_sync(0xffffffffu, hit);
+    if (!m) return;
+    int base = 0;
+    const int leader = __ffs(m) - 1;
+    if (lane == leader) base = atomicAdd(n, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (hit) {
+      const int k = base + __popc(m & lower);
+      l.lo[k] = lo;
+      l.hi[k] = hi;
+    }
+    if (!u) return;
+    const float v[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const int key = fkey32(hit ? v[c] : (c < 3 ? INFINITY : -INFINITY));
+      const int e = c < 3 ? __reduce_min_sync(0xffffffffu, key) : __reduce_max_sync(0xffffffffu, key);
+      if (lane == c) { if (c < 3) atomicMin(&u[c], e); else atomicMax(&u[c], e); }
+    }
+  };
+  for (int64_t r = blockIdx.x; r < npairs; r += gridDim.x) {
+    const int i = ci[r], j = cj[r], code = cs[r];
+    const int s[3] = {code / 9 - 1, (code / 3) % 3 - 1, code % 3 - 1};
+    const int Pi = 2 * pv[i], Pj = 2 * pv[j];
+    __syncthreads();   // the previous pair's lists are read
+    if (threadIdx.x < 3) nlist[threadIdx.x] = 0;
+    if (threadIdx.x < 12) ubox[threadIdx.x / 6][threadIdx.x % 6] = fkey32(threadIdx.x % 6 < 3 ? INFINITY : -INFINITY);
+    if (threadIdx.x == 0) {
       // FP32 frame of the pair: origin of vesicle i; |FP32 position - exact
       // position| per component is bounded by 2^-22 (R_i + R_j + 2 |offset|)
       // (rounding of X0 - origin, of the offset and of the frame change);
@@ -1935,82 +1956,83 @@ __global__ void __launch_bounds__(128) patch_pairs_kernel(const int32_t* pv, con
       p.voff_i = voff[i]; p.voff_j = voff[j];
       pinfo[r] = p;
     }
-    int ni = stiv_npatches(Pi), nj = stiv_npatches(Pj);
+    const int ni = stiv_npatches(Pi), nj = stiv_npatches(Pj);
     float shlo[3], shhi[3];
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
       double sh = s[c] * L[c];
       // d_m > 0: vesicle j's patch boxes widened by d_m (rounded outward)
       shlo[c] = __double2float_rd(__dsub_rd(sh, dm)); shhi[c] = __double2float_ru(__dadd_ru(sh, dm));
     }
     float bj[6];   // vesicle j's box at its image (A's patches are filtered against it)
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
       bj[c] = __fadd_rd(__double2float_rd(vbox[6 * j + c]), shlo[c]);
       bj[3 + c] = __fadd_ru(__double2float_ru(vbox[6 * j + 3 + c]), shhi[c]);
     }
-    for (int k = lane; k < ni; k += 32)
-      for (int c = 0; c < 6; ++c) sbw[(0 * mp + k) * 6 + c] = pbox[((size_t)i * mp + k) * STIV_PBOX + c];
-    for (int k = lane; k < nj; k += 32)
-      for (int c = 0; c < 3; ++c) {
-        sbw[(1 * mp + k) * 6 + c] = __fadd_rd(pbox[((size_t)j * mp + k) * STIV_PBOX + c], shlo[c]);
-        sbw[(1 * mp + k) * 6 + 3 + c] = __fadd_ru(pbox[((size_t)j * mp + k) * STIV_PBOX + 3 + c], shhi[c]);
+    __syncthreads();
+    for (int k0 = 0; k0 < ni; k0 += PPT) {
+      const int k = k0 + threadIdx.x;
+      float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+      bool hit = false;
+      if (k < ni) {
+        const float4* b = (const float4*)(pbox + ((size_t)i * mp + k) * STIV_PBOX);
+        float4 b0 = b[0], b1 = b[1];   // lo xyz, hi x; hi yz
+        lo = make_float4(b0.x, b0.y, b0.z, __int_as_float(k));
+        hi = make_float4(b0.w, b1.x, b1.y, 0.f);
+        const float box[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+        hit = fbox_hit(box, bj);
       }
-    __syncwarp();
-    int na = 0, nb = 0;
-    for (int k0 = 0; k0 < ni; k0 += 32) {
-      int k = k0 + lane;
-      bool hit = k < ni && fbox_hit(&sbw[(0 * mp + k) * 6], bj);
-      unsigned m = __ballot_sync(0xffffffffu, hit);
-      if (hit) law[na + __popc(m & ((1u << lane) - 1u))] = (unsigned short)k;
-      na += __popc(m);
+      keep_box(la, &nlist[0], ubox[0], hit, lo, hi);
     }
-    // union box of a list of staged patch boxes (side 0: A, 1: B)
-    auto list_union = [&](const unsigned short* lst, int n, int side, float* u) {
-      float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-      for (int q = lane; q < n; q += 32) {
-        const float* bx = &sbw[(side * mp + lst[q]) * 6];
-        for (int c = 0; c < 3; ++c) { lo[c] = fminf(lo[c], bx[c]); hi[c] = fmaxf(hi[c], bx[3 + c]); }
-      }
-      for (int c = 0; c < 3; ++c) {
-        u[c] = fkey_val(__reduce_min_sync(0xffffffffu, fkey32(lo[c])));
-        u[3 + c] = fkey_val(__reduce_max_sync(0xffffffffu, fkey32(hi[c])));
-      }
-    };
+    __syncthreads();
+    float ua[6], ub[6];
+    for (int c = 0; c < 6; ++c) ua[c] = fkey_val(ubox[0][c]);
     // B's patches against the union of A's kept patches (a patch of B that
     // meets a kept patch of A meets their union), then A's kept patches
     // against the union of B's
-    __syncwarp();
-    float ua[6], ub[6];
-    list_union(law, na, 0, ua);
-    for (int k0 = 0; k0 < nj; k0 += 32) {
-      int k = k0 + lane;
-      bool hit = k < nj && fbox_hit(&sbw[(1 * mp + k) * 6], ua);
-      unsigned m = __ballot_sync(0xffffffffu, hit);
-      if (hit) lbw[nb + __popc(m & ((1u << lane) - 1u))] = (unsigned short)k;
-      nb += __popc(m);
-    }
-    __syncwarp();
-    list_union(lbw, nb, 1, ub);
-    {
-      int na2 = 0;
-      for (int q0 = 0; q0 < na; q0 += 32) {
-        int q = q0 + lane;
-        int k = q < na ? law[q] : 0;
-        bool hit = q < na && fbox_hit(&sbw[(0 * mp + k) * 6], ub);
-        unsigned m = __ballot_sync(0xffffffffu, hit);
-        __syncwarp();
-        if (hit) law[na2 + __popc(m & ((1u << lane) - 1u))] = (unsigned short)k;
-        na2 += __popc(m);
+    for (int k0 = 0; k0 < nj; k0 += PPT) {
+      const int k = k0 + threadIdx.x;
+      float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+      bool hit = false;
+      if (k < nj) {
+        const float4* b = (const float4*)(pbox + ((size_t)j * mp + k) * STIV_PBOX);
+        float4 b0 = b[0], b1 = b[1];
+        lo = make_float4(__fadd_rd(b0.x, shlo[0]), __fadd_rd(b0.y, shlo[1]), __fadd_rd(b0.z, shlo[2]), __int_as_float(k));
+        hi = make_float4(__fadd_ru(b0.w, shhi[0]), __fadd_ru(b1.x, shhi[1]), __fadd_ru(b1.y, shhi[2]), 0.f);
+        const float box[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+        hit = fbox_hit(box, ua);
       }
-      na = na2;
+      keep_box(lb, &nlist[1], ubox[1], hit, lo, hi);
     }
-    __syncwarp();
-    for (int e0 = 0; e0 < na * nb; e0 += 32) {
-      int e = e0 + lane;
+    __syncthreads();
+    const int na0 = nlist[0], nb = nlist[1];
+    if (na0 == 0 || nb == 0) continue;
+    for (int c = 0; c < 6; ++c) ub[c] = fkey_val(ubox[1][c]);
+    // in place: an entry moves to a place no later than its own, in rounds
+    for (int q0 = 0; q0 < na0; q0 += PPT) {
+      const int q = q0 + threadIdx.x;
+      float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+      bool hit = false;
+      if (q < na0) {
+        lo = la.lo[q]; hi = la.hi[q];
+        const float box[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+        hit = fbox_hit(box, ub);
+      }
+      __syncthreads();
+      keep_box(la, &nlist[2], nullptr, hit, lo, hi);
+      __syncthreads();
+    }
+    const int na = nlist[2];
+    for (int e0 = 0; e0 < na * nb; e0 += PPT) {
+      const int e = e0 + threadIdx.x;
       bool hit = false;
       int pa = 0, pb = 0;
       if (e < na * nb) {
-        pa = law[e / nb]; pb = lbw[e % nb];
-        hit = fbox_hit(&sbw[(0 * mp + pa) * 6], &sbw[(1 * mp + pb) * 6]);
+        const int qa = e / nb, qb = e - qa * nb;
+        const float4 al = la.lo[qa], ah = la.hi[qa], bl = lb.lo[qb], bh = lb.hi[qb];
+        pa = __float_as_int(al.w); pb = __float_as_int(bl.w);
+        hit = al.x <= bh.x && bl.x <= ah.x && al.y <= bh.y && bl.y <= ah.y && al.z <= bh.z && bl.z <= ah.z;
         if (hit) {
           // every primitive lies in one of its patch's four cells: some cell
           // of pa must meet some cell of pb (vesicle j's at its image,
@@ -2035,26 +2057,25 @@ __global__ void __launch_bounds__(128) patch_pairs_kernel(const int32_t* pv, con
           hit = any;
         }
       }
-      unsigned m = __ballot_sync(0xffffffffu, hit);
+      const unsigned m = __ballot_sync(0xffffffffu, hit);
       // at P = 2 a patch touches both poles: a further item per such patch for
       // its south-pole primitives
       const int sa = Pi == 2 ? 2 : 1, sb = Pj == 2 ? 2 : 1;
       if (m) {
         unsigned long long base = 0;
-        int nm = __popc(m);
+        const int nm = __popc(m);
         if (lane == 0)
           base = atomicAdd((unsigned long long*)&ctr[STIV_C_PATCH], (unsigned long long)(nm * sa * sb));
         base = __shfl_sync(0xffffffffu, base, 0);
         if (hit)
           for (int z = 0; z < sa * sb; ++z) {
-            int64_t k = (int64_t)base + z * nm + __popc(m & ((1u << lane) - 1u));
+            int64_t k = (int64_t)base + z * nm + __popc(m & lower);
             int qa = pa | (z % sa ? SOUTH : 0), qb = pb | (z / sa ? SOUTH : 0);
             if (k < W) work[k] = ((uint64_t)r << 32) | ((uint64_t)qa << 16) | (uint64_t)qb;
             else atomicOr((unsigned long long*)&ctr[STIV_C_STATUS], STIV_F_WORK_OVERFLOW);
           }
       }
     }
-    __syncwarp();
   }
 }
 
@@ -2065,16 +2086,17 @@ size_t stiv_narrow_smem() { return sizeof(WarpSm) * NW; }
 int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, const int64_t* voff, const void* X,
                       const stiv_pairs* cand, detect_ws& w, int num_sms, int p_max) {
   const double* L = h->prm.box_L;
-  int blocks = (int)((cand->capacity + 3) / 4);
-  int pp_mult = h->tune[STIV_TUNE_PATCH_BLOCKS] > 0 ? h->tune[STIV_TUNE_PATCH_BLOCKS] : 4;
-  if (blocks > pp_mult * num_sms) blocks = pp_mult * num_sms;
+  // CTAs per SM: enough to hide the phases of one pair behind those of others
+  int blocks = (int)cand->capacity;
+  int pp_mult = h->tune[STIV_TUNE_PATCH_BLOCKS] > 0 ? h->tune[STIV_TUNE_PATCH_BLOCKS] : 12;
+  if (cand->capacity > (int64_t)pp_mult * num_sms) blocks = pp_mult * num_sms;
   if (blocks < 1) blocks = 1;
   int mp = stiv_npatches(2 * p_max);
-  size_t psmem = (size_t)4 * 2 * mp * 6 * sizeof(float) + (size_t)4 * 2 * mp * sizeof(unsigned short);
+  size_t psmem = (size_t)4 * mp * sizeof(float4);
   STIV_CUDA(h, cudaFuncSetAttribute(patch_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
   {
     STIV_PROF(h, st, "patch_pairs");
-    patch_pairs_kernel<<<blocks, 128, psmem, st>>>(p_dev, w.vbox, w.pbox, L[0], L[1], L[2], cand->i, cand->j,
+    patch_pairs_kernel<<<blocks, PPT, psmem, st>>>(p_dev, w.vbox, w.pbox, L[0], L[1], L[2], cand->i, cand->j,
                                                    cand->shift, cand->capacity, w.W, w.work, w.ctr, mp, w.vorg,
                                                    voff, w.pinfo, h->prm.d_m);
   }
@@ -2097,6 +2119,7 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
   a.C = w.C;
   a.rc_pair = w.tmp_i32; a.rc_type = w.tmp_i32 + w.C; a.rc_a = w.tmp_i32 + 2 * w.C; a.rc_b = w.tmp_i32 + 3 * w.C;
   a.rc_tau = w.tmp_f64; a.rc_w = w.tmp_f64 + w.C;
+  a.pair_cnt = w.pair_cnt;
   a.ctr = w.ctr;
   // d_m > 0: widened boxes and the degree-six test, in kernels of their own
   bool dmk = h->prm.d_m > 0.0;

@@ -54,3 +54,22 @@ def test_one_row_sums(p, gap):
     assert abs(float(a["val"][0]) - want) <= 1e-12 * want
     b = S.ContactLCP().assemble(eng, ds, torch.as_tensor(m, device="cuda"), torch.as_tensor(t, device="cuda"))
     assert float(a["val"][0]) == float(b["val"][0])
+
+
+@pytest.mark.parametrize("p,gap", [(8, 0.05), (16, -0.9), (32, -0.9)])
+def test_long_contact_segments(orc, p, gap):
+    """The ordering of one pair's contacts, of a segment that fits the sorting
+    CTA's shared memory and of longer ones (2048 entries, merged): the oracle's list
+    on the same vertices."""
+    from tests.gpu_run import run_gpu_on, verts_list
+    from tests.oracle_pool import oracle_vertices
+    sc = G.two_vesicles(p=p, seed=1, gap=gap, approach=0.4)
+    X = oracle_vertices(sc)
+    g = run_gpu_on(sc, X, pair_cap=16, contact_cap=1 << 17)
+    c = orc.contacts(sc.P, verts_list(sc, X), np.zeros((1, 5), np.int32) + np.array([[0, 1, 0, 0, 0]], np.int32), sc.L,
+                     sc.eps * sc.dt, grad=False)
+    if p == 32:
+        assert len(c["pair"]) > 4096
+    for k in ("pair", "type", "a", "b"):
+        assert np.array_equal(g[k], c[k]), k
+    assert np.array_equal(g["tau"].view(np.int64), np.ascontiguousarray(c["tau"]).view(np.int64))

@@ -28,15 +28,19 @@
 // Kernels:
 //   ytab_kernel   Y blocks per order p (once per handle and order)
 //   group_kernel  vesicles bucketed by order, per-order tile counts and offsets
-//   bprep_kernel  coefficient blocks (FP64 -> FP32 split) and per-column
-//                 output address and degree-0 term
-//   gemm_kernel   persistent, warp-specialised: per tile (order, 128 rows,
-//                 128 columns) warp 0 streams the A and B blocks through a
-//                 3-stage shared-memory ring (bulk copies completing on
+//   prep_kernel   B blocks (FP64 -> FP32 split) and per-column output address
+//                 and degree-0 term
+//   gemm_kernel   persistent, warp-specialised: per tile unit (order, 128 rows,
+//                 128 or 256 columns) warp 0 streams the A and B blocks through
+//                 a shared-memory ring of 192 KB (bulk copies completing on
 //                 mbarriers), warp 1 issues tcgen05.mma (M = 128, N = 128,
 //                 K = 8, kind::tf32) into one of two TMEM accumulators, and
 //                 warps 2-5 read the other accumulator (tcgen05.ld 32x32b) and
 //                 write the FP32 vertices while the next tile accumulates.
+// 4096 vesicles of orders 8, 12 and 16: the synthesis products take 72 us (87
+// with every column's address and degree-0 term loaded and shuffled between
+// its stores), the adjoint's 58 us (71 with the tiles in ascending order,
+// whose last round held the longest).
 // Every wait on an mbarrier is bounded; a wait that gives up sets a status
 // word (reported as STIV_F_TIMEOUT) and the tile is abandoned.
 #include "stiv_internal.cuh"
@@ -145,12 +149,23 @@ __global__ void ytabT_kernel(int p, const double* leg, float* ytab) {
 struct tc_group {
   int cnt, list_off, ntn, mt, kb, tile_off;  // vesicles, list offset, column tiles, row tiles, k blocks, first tile
   int nrows;                                 // rows of the output (vertices, or coefficients for the adjoint)
-  int pad;
+  int ntu;                                   // tile units in the column direction (nb column tiles each)
   long long boff;                            // first B block of the group
   long long coff;                            // first column (of all groups' padded columns)
 };
 
-// tc_ws layout: [status int][ntiles int][pad][groups (STIV_MAX_P+1)][list n][colinfo][B blocks]
+// Column tiles per tile unit.  A unit of two goes as one N = 256 product: its A
+// blocks are copied and read from shared memory once for both (the products
+// are bound by shared memory's bandwidth: 8 KB read per N = 128 instruction
+// beside the copies into it).  It pays while the units still fill the SMs
+// evenly, from four rounds of single tiles on: synthesis of 4096 vesicles of
+// orders 8, 12 and 16 (13 rounds) 115 us in single tiles and 108 us in pairs,
+// of 1440 of order 16 (7.6 rounds) 78 and 73; but the adjoint of the same 4096
+// (1.3 rounds) 139 and 170, of the 1440 (0.7 rounds) 95 and 134.
+constexpr int WIDE_ROUNDS = 4;
+constexpr int GROUP_V = 4;              // vesicles per thread and round of the grouping
+
+// workspace: [groups (STIV_MAX_P+1)][list n][colinfo][B blocks]
 struct tc_colinfo {
   long long dst;  // element offset of row 0 of this field in the vertex array (-1: padding column)
   float bias;     // degree-0 term
@@ -159,136 +174,199 @@ struct tc_colinfo {
 
 // adjoint = 0: synthesis (6 fields per vesicle, rows = vertices, k = q - 1);
 // adjoint = 1: transposed synthesis of the X1 gradient (3 fields per vesicle,
-// rows = coefficients, k = vertices)
-__global__ void group_kernel(int n, int p_max, const int32_t* pv, tc_group* g, int* ntiles, int* list, int adjoint) {
+// rows = coefficients, k = vertices).  tiles = (tile units, column tiles per
+// unit).  Units are numbered from the highest order down: the longest first,
+// so that the persistent kernel's last round holds the short ones.  Lanes
+// with the same order share one atomic (a batch has few orders), and thread p
+// sums the groups beside its own.
+__global__ void group_kernel(int n, int p_max, const int32_t* pv, tc_group* g, int* tiles, int* list, int adjoint,
+                             int sms) {
   __shared__ int cnt[STIV_MAX_P + 1], fill[STIV_MAX_P + 1], off[STIV_MAX_P + 1];
-  for (int p = threadIdx.x; p <= STIV_MAX_P; p += blockDim.x) { cnt[p] = 0; fill[p] = 0; }
+  int tid = threadIdx.x, lane = tid & 31;
+  for (int p = tid; p <= STIV_MAX_P; p += blockDim.x) { cnt[p] = 0; fill[p] = 0; }
   __syncthreads();
-  for (int v = threadIdx.x; v < n; v += blockDim.x) {
-    int p = pv[v];
-    if (p >= 1 && p <= p_max) atomicAdd(&cnt[p], 1);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int lo = 0, to = 0;
-    long long bo = 0, co = 0;
-    for (int p = 0; p <= STIV_MAX_P; ++p) {
-      tc_group G;
-      G.cnt = (p >= 1 && p <= p_max) ? cnt[p] : 0;
-      G.list_off = lo;
-      G.ntn = ((adjoint ? 3 : 6) * G.cnt + TN - 1) / TN;
-      G.mt = p < 1 ? 0 : adjoint ? tcA_mtiles(p) : tc_mtiles(p);
-      G.kb = p < 1 ? 0 : adjoint ? tcA_kblocks(p) : tc_kblocks(p);
-      G.nrows = p < 1 ? 0 : adjoint ? (p + 1) * (p + 1) : stiv_nverts(2 * p);
-      G.pad = 0;
-      G.tile_off = to;
-      G.boff = bo;
-      G.coff = co;
-      off[p] = lo;
-      lo += G.cnt;
-      to += G.mt * G.ntn;
-      bo += (long long)G.ntn * G.kb;
-      co += (long long)G.ntn * TN;
-      g[p] = G;
+  // the orders of GROUP_V vesicles a thread and round; 0 = outside [1, p_max]
+  auto orders = [&](int v0, int* q) {
+#pragma unroll
+    for (int u = 0; u < GROUP_V; ++u) {
+      int v = v0 + u * blockDim.x + tid;
+      q[u] = v < n ? pv[v] : 0;
     }
-    *ntiles = to;
+#pragma unroll
+    for (int u = 0; u < GROUP_V; ++u)
+      if (q[u] < 1 || q[u] > p_max) q[u] = 0;
+  };
+  for (int v0 = 0; v0 < n; v0 += GROUP_V * blockDim.x) {
+    int q[GROUP_V];
+    orders(v0, q);
+#pragma unroll
+    for (int u = 0; u < GROUP_V; ++u) {
+      unsigned peers = __match_any_sync(0xffffffffu, q[u]);
+      if (q[u] && lane == __ffs(peers) - 1) atomicAdd(&cnt[q[u]], __popc(peers));
+    }
   }
   __syncthreads();
-  for (int v = threadIdx.x; v < n; v += blockDim.x) {
-    int p = pv[v];
-    if (p >= 1 && p <= p_max) list[off[p] + atomicAdd(&fill[p], 1)] = v;
+  if (tid <= STIV_MAX_P) {
+    auto ntn = [&](int p) { return ((adjoint ? 3 : 6) * cnt[p] + TN - 1) / TN; };
+    auto mt = [&](int p) { return adjoint ? tcA_mtiles(p) : tc_mtiles(p); };
+    auto kb = [&](int p) { return adjoint ? tcA_kblocks(p) : tc_kblocks(p); };
+    long long all = 0;
+    for (int p = 1; p <= p_max; ++p)
+      if (cnt[p]) all += (long long)mt(p) * ntn(p);
+    int nb = all >= (long long)WIDE_ROUNDS * sms ? 2 : 1;
+    tc_group G;
+    G.cnt = cnt[tid];
+    G.list_off = 0; G.tile_off = 0; G.boff = 0; G.coff = 0;
+    for (int p = 1; p <= p_max; ++p) {
+      if (!cnt[p]) continue;
+      if (p < tid) {
+        G.list_off += cnt[p];
+        G.boff += (long long)ntn(p) * kb(p);
+        G.coff += (long long)ntn(p) * TN;
+      }
+      if (p > tid) G.tile_off += mt(p) * ((ntn(p) + nb - 1) / nb);
+    }
+    G.ntn = tid ? ntn(tid) : 0;
+    G.mt = tid ? mt(tid) : 0;
+    G.kb = tid ? kb(tid) : 0;
+    G.nrows = tid ? (adjoint ? (tid + 1) * (tid + 1) : stiv_nverts(2 * tid)) : 0;
+    G.ntu = (G.ntn + nb - 1) / nb;
+    off[tid] = G.list_off;
+    g[tid] = G;
+    if (tid == 0) { tiles[0] = G.tile_off; tiles[1] = nb; }
+  }
+  __syncthreads();
+  for (int v0 = 0; v0 < n; v0 += GROUP_V * blockDim.x) {
+    int q[GROUP_V];
+    orders(v0, q);
+#pragma unroll
+    for (int u = 0; u < GROUP_V; ++u) {
+      unsigned peers = __match_any_sync(0xffffffffu, q[u]);
+      int lead = __ffs(peers) - 1, base = 0;
+      if (q[u] && lane == lead) base = atomicAdd(&fill[q[u]], __popc(peers));
+      base = __shfl_sync(0xffffffffu, base, lead);
+      if (q[u]) list[off[q[u]] + base + __popc(peers & ((1u << lane) - 1u))] = v0 + u * (int)blockDim.x + tid;
+    }
   }
 }
 
-// B blocks: column c of order group p is field (c % 6) of vesicle list[c / 6];
-// thread per (group, column, k block, k group of 4).
-__global__ void bprep_kernel(int p_max, const tc_group* g, const int* list, const int64_t* coef_off,
-                             const double* coef, const int64_t* vert_off, float* bblk, tc_colinfo* ci) {
-  for (int p = 1; p <= p_max; ++p) {
-    tc_group G = g[p];
-    if (G.cnt == 0) continue;
+// FP64 -> FP32, to nearest (ties to even), on the integer pipe: the FP64 pipe
+// takes a warp's conversion in about 20 SM cycles, which alone would hold the
+// block preparation to half of the memory's rate.  Right for zeros and for
+// 2^-126 <= |x| < 2^127; sets bad for anything else.
+__device__ __forceinline__ float d2f_normal(double x, bool& bad) {
+  unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  unsigned ab = hi & 0x7FFFFFFFu;
+  unsigned f = __funnelshift_l(lo, ab, 3) - 0xC0000000u;  // 20 + 3 mantissa bits, exponent rebased (mod 2^32)
+  f += (lo & 0x1FFFFFFFu) + (f & 1u) > 0x10000000u;
+  bool zero = (ab | lo) == 0u;
+  bad |= ab - 0x38100000u >= 0x47E00000u - 0x38100000u && !zero;
+  return __uint_as_float((zero ? 0u : f) | (hi & 0x80000000u));
+}
+
+// B blocks, one CTA per (column tile, k block).  Synthesis: column c of order
+// group p is field c % 6 of vesicle list[c / 6], k = q - 1.  Adjoint: column c
+// is coordinate c % 3 of the X1 block of vesicle list[c / 3] of the gradient
+// (FP64, vertex layout), k = vertex.
+//
+// 8 bytes read and 8 written per element.  A warp takes 16 columns and reads
+// 32 consecutive k of each (256 bytes in a row; one thread per 4 k of a
+// column, the order of the blocks, had the lanes of a load on 8-byte words of
+// different columns and the warp's values in as many sectors), turns them in
+// its own part of shared memory (k groups 4 words apart modulo the 32 banks:
+// no conflicts, no barrier of the CTA) and writes runs of 256 bytes.  4096
+// vesicles of orders 8, 12 and 16: 28 us for the coefficients (29 MB each
+// way) and 63 us for the gradient (126 MB each way, 4 TB/s), before 28 and 65
+// with zeroing of the X0 gradient in 7 more; about 50 instructions per
+// element and the loads' latency hold it there, at 12 warps a scheduler.
+constexpr int PREP_THREADS = 256;
+constexpr int PREP_KG = TM * 4 + 4;      // floats of a k group in shared memory
+
+template <bool ADJ>
+__global__ void __launch_bounds__(PREP_THREADS, 6)
+    prep_kernel(int p_max, const tc_group* g, const int* tiles, const int* list, const int64_t* coef_off,
+                const int64_t* vert_off, const double* src, float* bblk, tc_colinfo* ci) {
+  constexpr int NF = ADJ ? 3 : 6;
+  __shared__ float sh[2][8 * PREP_KG];
+  __shared__ __align__(16) const double* cb[TN];
+  __shared__ long long bend[STIV_MAX_P + 1];
+  int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid <= STIV_MAX_P) bend[tid] = tid <= p_max ? g[tid].boff + (long long)g[tid].ntn * g[tid].kb : 0;
+  __syncthreads();
+  // a run of consecutive blocks per CTA: mostly of one column tile, whose
+  // columns' addresses (two dependent loads) are then looked up once
+  const long long b0 = bend[p_max] * blockIdx.x / gridDim.x, b1 = bend[p_max] * (blockIdx.x + 1) / gridDim.x;
+  const bool pairs = tiles[1] == 2;
+  int p = 0, nt = 0, kb = 0;
+  tc_group G;
+  G.kb = 0;
+  for (long long blk = b0; blk < b1; ++blk) {
+    bool fresh = ++kb >= G.kb;           // first block of a column tile here
+    if (fresh) { kb = 0; ++nt; }
+    if (p == 0 || blk >= bend[p]) {      // orders ascend with the block number
+      do ++p; while (blk >= bend[p]);
+      G = g[p];
+      nt = (int)(blk - G.boff) / G.kb;
+      kb = (int)(blk - G.boff) % G.kb;
+      fresh = true;
+    }
     int nc = (p + 1) * (p + 1), nv = stiv_nverts(2 * p);
-    long long ncols = (long long)G.ntn * TN;
-    long long items = ncols * G.kb * (TK / 4);
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < items;
-         t += (long long)gridDim.x * blockDim.x) {
-      int kg = (int)(t % (TK / 4));
-      long long rest = t / (TK / 4);
-      long long c = rest % ncols;
-      int kb = (int)(rest / ncols);
-      int v = c / 6 < G.cnt ? list[G.list_off + c / 6] : -1;
-      int f = (int)(c % 6);
-      float hi[4], lo[4];
-      for (int e = 0; e < 4; ++e) {
-        int q = kb * TK + kg * 4 + e + 1;
-        float x = 0.f;
-        if (v >= 0 && q < nc) x = __double2float_rn(coef[coef_off[v] + (size_t)f * nc + q]);
-        hi[e] = tf32_rn(x);
-        lo[e] = tf32_rn(x - hi[e]);
+    if (fresh && lane < 16) {
+      int c = nt * TN + warp * 16 + lane;
+      const double* base = src;
+      tc_colinfo info;
+      info.dst = -1; info.bias = 0.f; info.pad = 0.f;
+      if (c / NF < G.cnt) {
+        int v = list[G.list_off + c / NF], f = c % NF;
+        long long vb = vert_off[v], qb = coef_off[v];
+        base = src + (ADJ ? vb + (long long)(3 + f) * nv : qb + (long long)f * nc);
+        info.dst = ADJ ? qb + (long long)(3 + f) * nc : vb + (long long)f * nv;
+        if (!ADJ && kb == 0) info.bias = (float)(Y00 * *base);
       }
-      int nt = (int)(c / TN), r = (int)(c % TN);
-      float* blk = bblk + ((size_t)G.boff + (size_t)nt * G.kb + kb) * (2 * BLK_FLOATS);
-      *(float4*)(blk + blk_index(r, kg * 4)) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-      *(float4*)(blk + BLK_FLOATS + blk_index(r, kg * 4)) = make_float4(lo[0], lo[1], lo[2], lo[3]);
-      if (kb == 0 && kg == 0) {
-        tc_colinfo info;
-        info.dst = v >= 0 ? (long long)vert_off[v] + (long long)f * nv : -1;
-        info.bias = v >= 0 ? (float)(Y00 * coef[coef_off[v] + (size_t)f * nc]) : 0.f;
-        info.pad = 0.f;
-        ci[(size_t)G.coff + c] = info;
+      if (kb == 0) ci[(size_t)G.coff + c] = info;
+      cb[warp * 16 + lane] = base;
+    }
+    __syncwarp();
+    int k = kb * TK + lane + (ADJ ? 0 : 1);
+    int ncol = NF * G.cnt - nt * TN;     // columns of this tile (the rest is padding)
+    if (k >= (ADJ ? nv : nc)) ncol = 0;
+    int at = (lane >> 2) * PREP_KG + (lane & 3);
+#pragma unroll
+    for (int c0 = warp * 16; c0 < warp * 16 + 16; c0 += 8) {
+      double x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const double* base = cb[c0 + u];
+        x[u] = c0 + u < ncol ? __ldg(base + k) : 0.0;
+      }
+      float xf[8];
+      bool bad = false;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) xf[u] = d2f_normal(x[u], bad);
+      if (bad) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) xf[u] = __double2float_rn(x[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        float hi = tf32_rn(xf[u]);
+        sh[0][at + (c0 + u) * 4] = hi;
+        sh[1][at + (c0 + u) * 4] = tf32_rn(xf[u] - hi);
       }
     }
-  }
-}
-
-// B blocks of the adjoint: column c of order group p is coordinate (c % 3) of
-// the X1 block of vesicle list[c / 3] of the gradient gX (FP64, vertex
-// layout); k = vertex.  Thread per (group, column, k block, 4 vertices).
-__global__ void gprep_kernel(int p_max, const tc_group* g, const int* list, const int64_t* coef_off,
-                             const int64_t* vert_off, const double* gX, float* bblk, tc_colinfo* ci) {
-  for (int p = 1; p <= p_max; ++p) {
-    tc_group G = g[p];
-    if (G.cnt == 0) continue;
-    int nc = (p + 1) * (p + 1), nv = stiv_nverts(2 * p);
-    long long ncols = (long long)G.ntn * TN;
-    long long items = ncols * G.kb * (TK / 4);
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < items;
-         t += (long long)gridDim.x * blockDim.x) {
-      int kg = (int)(t % (TK / 4));
-      long long rest = t / (TK / 4);
-      long long c = rest % ncols;
-      int kb = (int)(rest / ncols);
-      int v = c / 3 < G.cnt ? list[G.list_off + c / 3] : -1;
-      int f = (int)(c % 3);
-      float hi[4], lo[4];
-      for (int e = 0; e < 4; ++e) {
-        int row = kb * TK + kg * 4 + e;
-        float x = 0.f;
-        if (v >= 0 && row < nv) x = __double2float_rn(gX[vert_off[v] + (size_t)(3 + f) * nv + row]);
-        hi[e] = tf32_rn(x);
-        lo[e] = tf32_rn(x - hi[e]);
-      }
-      int nt = (int)(c / TN), r = (int)(c % TN);
-      float* blk = bblk + ((size_t)G.boff + (size_t)nt * G.kb + kb) * (2 * BLK_FLOATS);
-      *(float4*)(blk + blk_index(r, kg * 4)) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-      *(float4*)(blk + BLK_FLOATS + blk_index(r, kg * 4)) = make_float4(lo[0], lo[1], lo[2], lo[3]);
-      if (kb == 0 && kg == 0) {
-        tc_colinfo info;
-        info.dst = v >= 0 ? (long long)coef_off[v] + (long long)(3 + f) * nc : -1;
-        info.bias = 0.f;
-        info.pad = 0.f;
-        ci[(size_t)G.coff + c] = info;
-      }
+    __syncwarp();
+    // column tiles of a pair share blocks of 256 columns, [hi | lo][8][256][4]
+    int wide = pairs && (nt | 1) < G.ntn, rows = wide ? 2 * TN : TN;
+    long long dst = wide ? G.boff + (long long)(nt & ~1) * G.kb + 2 * kb : blk;
+    int r = warp * 16 + (lane & 15);
+    float4* out = (float4*)(bblk + (size_t)dst * (2 * BLK_FLOATS)) + (wide ? (nt & 1) * TN : 0) + r;
+#pragma unroll
+    for (int u = 0; u < 16; u += 2) {
+      int i = u + (lane >> 4);            // [hi | lo][kg]
+      out[i * rows] = *(const float4*)&sh[i >> 3][(i & 7) * PREP_KG + r * 4];
     }
+    __syncwarp();
   }
-}
-
-// X0 blocks of the coefficient gradient are zero (X0 is a constant of the step).
-__global__ void zero_x0_kernel(int n, int p_max, const int32_t* pv, const int64_t* coef_off, double* gcoef) {
-  int v = blockIdx.x;
-  if (v >= n || pv[v] < 1 || pv[v] > p_max) return;   // order outside [1, p_max]: skipped
-  int nc = (pv[v] + 1) * (pv[v] + 1);
-  for (int k = threadIdx.x; k < 3 * nc; k += blockDim.x) gcoef[coef_off[v] + k] = 0.0;
 }
 
 // ---------------------------------------------------------------------------
@@ -344,15 +422,16 @@ __device__ __forceinline__ unsigned long long smem_desc(unsigned addr, unsigned 
   return (unsigned long long)((addr & 0x3FFFFu) >> 4) | ((unsigned long long)((lbo >> 4) & 0x3FFFu) << 16) |
          ((unsigned long long)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
-// instruction descriptor: D f32, A and B tf32, both K-major, N = TN, M = TM
+// instruction descriptor: D f32, A and B tf32, both K-major, N = TN (a pair: 2 TN, added below), M = TM
 constexpr unsigned IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(TN >> 3) << 17) | ((unsigned)(TM >> 4) << 24);
 
-__device__ __forceinline__ void mma_tf32(unsigned tmem, unsigned long long ad, unsigned long long bd, unsigned acc) {
+__device__ __forceinline__ void mma_tf32(unsigned tmem, unsigned long long ad, unsigned long long bd, unsigned idesc,
+                                         unsigned acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-      "l"(ad), "l"(bd), "r"(IDESC), "r"(acc)
+      "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(unsigned bar) {
@@ -376,7 +455,7 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float* v) {
 
 struct gemm_args {
   const tc_group* g;
-  const int* ntiles;
+  const int* tiles;     // tile units, column tiles per unit
   const float* ytab[STIV_MAX_P + 1];
   const float* bblk;
   const tc_colinfo* ci;
@@ -385,23 +464,41 @@ struct gemm_args {
   int p_max;
 };
 
-constexpr int NSTAGE = 3;               // shared-memory ring of (A, B) blocks
+constexpr int NSTAGE = 3;               // shared-memory ring of (A, B) blocks: 3 x 64 KB, or 2 x 96 KB with two B
 constexpr int NACC = 2;                 // TMEM accumulators (MMA of tile t+1 overlaps the epilogue of tile t)
 constexpr int GEMM_THREADS = 192;       // warp 0 copies, warp 1 issues MMAs, warps 2-5 epilogue
 
-// Tile t of this CTA's sequence: order group, row tile, column tile.
-__device__ __forceinline__ bool tile_of(const tc_group* G, int p_max, int tile, int& p, int& mt, int& nt) {
-  p = 1;
-  while (p <= p_max && tile >= G[p].tile_off + G[p].mt * G[p].ntn) ++p;
-  if (p > p_max) return false;
-  int local = tile - G[p].tile_off;
-  mt = local / G[p].ntn;
-  nt = local % G[p].ntn;
+// A column in the epilogue: output address of row 0 (null: padding), degree-0 term.
+template <typename OUT>
+struct __align__(16) ep_col {
+  OUT* dst;
+  float bias, pad;
+};
+constexpr size_t GEMM_SMEM = (size_t)NSTAGE * STAGE_BYTES + 4 * 2 * TN * 16 + 1024;  // ring, 4 warps' columns, alignment
+
+// Unit i of this CTA's sequence.  Every other round runs backwards over the
+// CTAs: units come longest first, so the CTAs with the longest of one round
+// take the shortest of the next.
+__device__ __forceinline__ int unit_at(int i) {
+  return i * (int)gridDim.x + (i & 1 ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
+}
+
+// Tile unit u: order group, row tile, first column tile and column tiles.
+__device__ __forceinline__ bool tile_of(const tc_group* G, int p_max, int u, int nb, int& p, int& mt, int& nt, int& w) {
+  p = p_max;
+  while (p >= 1 && u >= G[p].tile_off + G[p].mt * G[p].ntu) --p;
+  if (p < 1) return false;
+  int local = u - G[p].tile_off;
+  mt = local / G[p].ntu;
+  nt = local % G[p].ntu * nb;
+  w = G[p].ntn - nt < nb ? G[p].ntn - nt : nb;
   return true;
 }
 
+// OUT float: synthesis; double: adjoint.
 template <typename OUT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(gemm_args a) {
+  constexpr bool ADJ = sizeof(OUT) == 8;
   extern __shared__ __align__(1024) unsigned char tc_smem[];
   __shared__ tc_group G[STIV_MAX_P + 1];
   // full[NSTAGE], empty[NSTAGE], acc_full[NACC], acc_empty[NACC], drain
@@ -422,7 +519,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(gemm_args a) {
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                 "r"((unsigned)(NACC * TN)));
+                 "r"((unsigned)(NACC * 2 * TN)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
@@ -434,62 +531,65 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(gemm_args a) {
   auto acc_full = [&](int b) { return smem_u32(&bars[2 * NSTAGE + b]); };
   auto acc_empty = [&](int b) { return smem_u32(&bars[2 * NSTAGE + NACC + b]); };
   const unsigned drain = smem_u32(&bars[2 * NSTAGE + 2 * NACC]);
-  int ntiles = *a.ntiles;
+  const int units = a.tiles[0], nb = a.tiles[1];
+  const int nst = nb == 2 ? 2 : NSTAGE;
+  const unsigned stage = (unsigned)(1 + nb) * BLK_BYTES;
   bool ok = true;
   if (warp == 0) {
     // producer: one lane streams the A and B blocks of every tile through the ring
     if (lane == 0) {
       unsigned it = 0;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        int p, mt, nt;
-        if (!tile_of(G, a.p_max, tile, p, mt, nt)) break;
+      for (int i = 0, u; (u = unit_at(i)) < units && ok; ++i) {
+        int p, mt, nt, w;
+        if (!tile_of(G, a.p_max, u, nb, p, mt, nt, w)) break;
         int KB = G[p].kb;
         const unsigned char* asrc = (const unsigned char*)(a.ytab[p] + (size_t)mt * KB * (2 * BLK_FLOATS));
         const unsigned char* bsrc =
             (const unsigned char*)(a.bblk + ((size_t)G[p].boff + (size_t)nt * KB) * (2 * BLK_FLOATS));
         for (int kb = 0; kb < KB; ++kb, ++it) {
-          int s = it % NSTAGE;
-          unsigned ph = (it / NSTAGE) & 1;
+          int s = it % nst;
+          unsigned ph = (it / nst) & 1;
           if (!mbar_wait(empty(s), ph ^ 1)) { ok = false; break; }
-          unsigned char* dst = sm + (size_t)s * STAGE_BYTES;
-          mbar_expect_tx(full(s), STAGE_BYTES);
+          unsigned char* dst = sm + (size_t)s * stage;
+          mbar_expect_tx(full(s), (unsigned)(1 + w) * BLK_BYTES);
           bulk_g2s(smem_u32(dst), asrc + (size_t)kb * BLK_BYTES, BLK_BYTES, full(s));
-          bulk_g2s(smem_u32(dst + BLK_BYTES), bsrc + (size_t)kb * BLK_BYTES, BLK_BYTES, full(s));
+          bulk_g2s(smem_u32(dst + BLK_BYTES), bsrc + (size_t)(w * kb) * BLK_BYTES, (unsigned)w * BLK_BYTES, full(s));
         }
       }
       // before the shared memory is left: the copies of the last stages
       // issued have landed (already true unless another warp gave up early;
       // the wait is bounded either way)
-      for (unsigned k = it > NSTAGE ? it - NSTAGE : 0; k < it; ++k)
-        if (!mbar_wait(full(k % NSTAGE), (k / NSTAGE) & 1, DRAIN_CYCLES)) ok = false;
+      for (unsigned k = it > (unsigned)nst ? it - nst : 0; k < it; ++k)
+        if (!mbar_wait(full(k % nst), (k / nst) & 1, DRAIN_CYCLES)) ok = false;
     }
   } else if (warp == 1) {
     // MMA issuer: one lane; accumulator b = (tile count) % NACC
     if (lane == 0) {
       unsigned it = 0, tc = 0;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++tc) {
-        int p, mt, nt;
-        if (!tile_of(G, a.p_max, tile, p, mt, nt)) break;
+      for (int u; (u = unit_at(tc)) < units && ok; ++tc) {
+        int p, mt, nt, w;
+        if (!tile_of(G, a.p_max, u, nb, p, mt, nt, w)) break;
         int KB = G[p].kb;
         int b = tc % NACC;
         if (!mbar_wait(acc_empty(b), ((tc / NACC) & 1) ^ 1)) { ok = false; break; }
         tc_fence_after();
-        unsigned dtm = tmem + (unsigned)(b * TN);
+        unsigned dtm = tmem + (unsigned)(b * 2 * TN), idesc = IDESC + ((unsigned)((w - 1) * (TN >> 3)) << 17);
         for (int kb = 0; kb < KB; ++kb, ++it) {
-          int s = it % NSTAGE;
-          if (!mbar_wait(full(s), (it / NSTAGE) & 1)) { ok = false; break; }
+          int s = it % nst;
+          if (!mbar_wait(full(s), (it / nst) & 1)) { ok = false; break; }
           tc_fence_after();
-          unsigned abase = smem_u32(sm + (size_t)s * STAGE_BYTES), bbase = abase + BLK_BYTES;
+          unsigned abase = smem_u32(sm + (size_t)s * stage);
+          unsigned bbase = abase + BLK_BYTES, ldb = (unsigned)w * (TN * 16);
 #pragma unroll
           for (int ks = 0; ks < TK / 8; ++ks) {
             unsigned off = ks * 2 * (TM * 16);   // two k groups of 2048 bytes per K = 8
             unsigned long long ahi = smem_desc(abase + off, TM * 16, 128);
             unsigned long long alo = smem_desc(abase + BLK_BYTES / 2 + off, TM * 16, 128);
-            unsigned long long bhi = smem_desc(bbase + off, TN * 16, 128);
-            unsigned long long blo = smem_desc(bbase + BLK_BYTES / 2 + off, TN * 16, 128);
-            mma_tf32(dtm, ahi, bhi, (kb | ks) != 0);
-            mma_tf32(dtm, ahi, blo, 1u);
-            mma_tf32(dtm, alo, bhi, 1u);
+            unsigned long long bhi = smem_desc(bbase + w * off, ldb, 128);
+            unsigned long long blo = smem_desc(bbase + w * (BLK_BYTES / 2 + off), ldb, 128);
+            mma_tf32(dtm, ahi, bhi, idesc, (kb | ks) != 0);
+            mma_tf32(dtm, ahi, blo, idesc, 1u);
+            mma_tf32(dtm, alo, bhi, idesc, 1u);
           }
           mma_commit(empty(s));      // the stage is free once these MMAs have read it
         }
@@ -506,28 +606,43 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(gemm_args a) {
   } else {
     // epilogue warps 2-5: TMEM lanes 32 (w % 4) .. + 31 are tile rows
     int q = warp & 3;
+    ep_col<OUT>* col = (ep_col<OUT>*)(sm + NSTAGE * STAGE_BYTES) + q * 2 * TN;
     unsigned tc = 0;
-    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++tc) {
-      int p, mt, nt;
-      if (!tile_of(G, a.p_max, tile, p, mt, nt)) break;
+    for (int u; (u = unit_at(tc)) < units && ok; ++tc) {
+      int p, mt, nt, w;
+      if (!tile_of(G, a.p_max, u, nb, p, mt, nt, w)) break;
       int b = tc % NACC;
+      int row = mt * TM + q * 32 + lane;
+      bool in = row < G[p].nrows;
+      int x0 = 3 * G[p].nrows;         // adjoint: X0 is a constant of the step, its gradient zero
+      // the unit's columns, fetched while its MMAs run; every lane reads them
+      // all, so they wait in the warp's own part of shared memory (one 16-byte
+      // broadcast a column)
+      const tc_colinfo* cinfo = a.ci + (size_t)G[p].coff + (size_t)nt * TN;
+      for (int c = lane; c < w * TN; c += 32) {
+        tc_colinfo mine = cinfo[c];
+        ep_col<OUT> e;
+        e.dst = mine.dst >= 0 ? (OUT*)a.X + mine.dst : nullptr;
+        e.bias = mine.bias;
+        e.pad = 0.f;
+        col[c] = e;
+      }
+      __syncwarp();
       if (!mbar_wait(acc_full(b), (tc / NACC) & 1)) { ok = false; break; }
       tc_fence_after();
-      int row = mt * TM + q * 32 + lane;
-      int nrows = G[p].nrows;
-      OUT* X = (OUT*)a.X;
-      const tc_colinfo* cinfo = a.ci + (size_t)G[p].coff + (size_t)nt * TN;
 #pragma unroll 1
-      for (int c0 = 0; c0 < TN; c0 += 16) {
+      for (int c0 = 0; c0 < w * TN; c0 += 16) {
         float v[16];
-        tmem_ld16(tmem + ((unsigned)(q * 32) << 16) + (unsigned)(b * TN + c0), v);
-        tc_colinfo mine = cinfo[c0 + (lane & 15)];
+        ep_col<OUT> e[16];               // all read before the first store, which they could alias
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          long long dst = __shfl_sync(0xffffffffu, mine.dst, i);
-          float bias = __shfl_sync(0xffffffffu, mine.bias, i);
-          if (dst >= 0 && row < nrows) X[dst + row] = (OUT)(v[i] + bias);
-        }
+        for (int i = 0; i < 16; ++i) e[i] = col[c0 + i];
+        tmem_ld16(tmem + ((unsigned)(q * 32) << 16) + (unsigned)(b * 2 * TN + c0), v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (e[i].dst && in) {
+            e[i].dst[row] = (OUT)(v[i] + e[i].bias);
+            if (ADJ) e[i].dst[row - x0] = (OUT)0;
+          }
       }
       tc_fence_before();
       __syncwarp();
@@ -539,7 +654,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(gemm_args a) {
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((unsigned)(NACC * TN)));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((unsigned)(NACC * 2 * TN)));
   }
 }
 
@@ -557,10 +672,16 @@ static int ensure_ytab(stiv_handle* h, cudaStream_t st, int p) {
   return STIV_OK;
 }
 
+// CTAs of the block preparation: six fit an SM (36 KB of shared memory each).
+static int prep_grid(int sms, long long max_blocks) {
+  return (int)(max_blocks < 6LL * sms ? max_blocks : 6LL * sms);
+}
+
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Device status word of the bounded waits (word 0) and the tile count of the
-// synthesis (word 1) and of the adjoint (word 2); allocated once per handle.
+// Device status word of the bounded waits (word 0) and the tile units and their
+// width of the synthesis (words 1, 2) and of the adjoint (words 3, 4);
+// allocated once per handle.
 static int ensure_status(stiv_handle* h, cudaStream_t st) {
   if (h->tc_status) return STIV_OK;
   STIV_CUDA(h, cudaMalloc(&h->tc_status, 256));
@@ -604,7 +725,7 @@ int stiv_upsample_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t p_m
   }
   char* w = (char*)h->tc_ws;
   int* status = h->tc_status;
-  int* ntiles = status + 1;
+  int* tiles = status + 1;
   tc_group* g = (tc_group*)(w + o_g);
   int* list = (int*)(w + o_list);
   tc_colinfo* ci = (tc_colinfo*)(w + o_ci);
@@ -612,16 +733,16 @@ int stiv_upsample_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t p_m
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   STIV_PROF_N(h, st, "synth", 3);
-  group_kernel<<<1, 1024, 0, st>>>(n_ves, p_max, p_dev, g, ntiles, list, 0);
-  bprep_kernel<<<sms * 8, 256, 0, st>>>(p_max, g, list, coef_off_dev, coef_dev, vert_off_dev, bblk, ci);
+  group_kernel<<<1, 1024, 0, st>>>(n_ves, p_max, p_dev, g, tiles, list, 0, sms);
+  prep_kernel<false><<<prep_grid(sms, max_blocks), PREP_THREADS, 0, st>>>(p_max, g, tiles, list, coef_off_dev, vert_off_dev,
+                                                                         coef_dev, bblk, ci);
   gemm_args A;
-  A.g = g; A.ntiles = ntiles; A.bblk = bblk; A.ci = ci; A.X = verts_dev; A.status = status; A.p_max = p_max;
+  A.g = g; A.tiles = tiles; A.bblk = bblk; A.ci = ci; A.X = verts_dev; A.status = status; A.p_max = p_max;
   for (int p = 0; p <= STIV_MAX_P; ++p) A.ytab[p] = p >= 1 && p <= p_max ? h->ytab[p] : nullptr;
-  size_t smem = (size_t)NSTAGE * STAGE_BYTES + 1024;
-  STIV_CUDA(h, cudaFuncSetAttribute(gemm_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  STIV_CUDA(h, cudaFuncSetAttribute(gemm_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
   long long tiles_bound = max_ntn * tc_mtiles(p_max);
   int grid = (int)(tiles_bound < sms ? tiles_bound : sms);
-  gemm_kernel<float><<<grid, GEMM_THREADS, smem, st>>>(A);
+  gemm_kernel<float><<<grid, GEMM_THREADS, GEMM_SMEM, st>>>(A);
   STIV_LAUNCH(h);
   return STIV_OK;
 }
@@ -651,25 +772,24 @@ int stiv_grad_to_coef_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t
   }
   char* w = (char*)h->tc_ws2;
   int* status = h->tc_status;
-  int* ntiles = status + 2;
+  int* tiles = status + 3;
   tc_group* g = (tc_group*)(w + o_g);
   int* list = (int*)(w + o_list);
   tc_colinfo* ci = (tc_colinfo*)(w + o_ci);
   float* bblk = (float*)(w + o_b);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-  STIV_PROF_N(h, st, "grad_to_coef", 4);
-  zero_x0_kernel<<<n_ves, 256, 0, st>>>(n_ves, p_max, p_dev, coef_off_dev, gcoef_dev);
-  group_kernel<<<1, 1024, 0, st>>>(n_ves, p_max, p_dev, g, ntiles, list, 1);
-  gprep_kernel<<<sms * 8, 256, 0, st>>>(p_max, g, list, coef_off_dev, vert_off_dev, gX_dev, bblk, ci);
+  STIV_PROF_N(h, st, "grad_to_coef", 3);
+  group_kernel<<<1, 1024, 0, st>>>(n_ves, p_max, p_dev, g, tiles, list, 1, sms);
+  prep_kernel<true><<<prep_grid(sms, max_blocks), PREP_THREADS, 0, st>>>(p_max, g, tiles, list, coef_off_dev, vert_off_dev,
+                                                                        gX_dev, bblk, ci);
   gemm_args A;
-  A.g = g; A.ntiles = ntiles; A.bblk = bblk; A.ci = ci; A.X = gcoef_dev; A.status = status; A.p_max = p_max;
+  A.g = g; A.tiles = tiles; A.bblk = bblk; A.ci = ci; A.X = gcoef_dev; A.status = status; A.p_max = p_max;
   for (int p = 0; p <= STIV_MAX_P; ++p) A.ytab[p] = p >= 1 && p <= p_max ? h->ytabT[p] : nullptr;
-  size_t smem = (size_t)NSTAGE * STAGE_BYTES + 1024;
-  STIV_CUDA(h, cudaFuncSetAttribute(gemm_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  STIV_CUDA(h, cudaFuncSetAttribute(gemm_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
   long long tiles_bound = max_ntn * tcA_mtiles(p_max);
   int grid = (int)(tiles_bound < sms ? tiles_bound : sms);
-  gemm_kernel<double><<<grid, GEMM_THREADS, smem, st>>>(A);
+  gemm_kernel<double><<<grid, GEMM_THREADS, GEMM_SMEM, st>>>(A);
   STIV_LAUNCH(h);
   return STIV_OK;
 }

@@ -1352,8 +1352,12 @@ __device__ __forceinline__ int tri_gid(const PatchRef& R, int s0, int s1, int s2
 // The hits are counted, laid out in the warp's queue by one scan, and go
 // through stages 2 and 3a on full warps; survivors are compacted in place and
 // pushed together.
+//
+// Four CTAs of 4 warps an SM (139 KB of staging): bound by issue slots at 70 %
+// of them.  4096 vesicles 7.7 ms, with three CTAs 8.3, with five (registers
+// spill) 8.0; 1440 of order 16 0.58, 0.62 and 0.62 ms.
 template <bool MIXED, bool DM>
-__global__ void __launch_bounds__(NW * 32, 3) narrow_kernel(narrow_args a) {
+__global__ void __launch_bounds__(NW * 32, 4) narrow_kernel(narrow_args a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ PatchTopo topo[NVAR];
   WarpSm& ws = ((WarpSm*)smraw)[threadIdx.x >> 5];

@@ -42,18 +42,18 @@ NARROW_SRC = os.path.join(ROOT, "paper_1812_04719_gb300", "csrc", "narrow.cu")
 
 # ncu figures of narrow_kernel (stages 1-3a), per patch pair it processes:
 # smsp__inst_executed.sum (warp instructions) and dram__bytes_read.sum +
-# dram__bytes_write.sum, from one capture of one launch per form on the
-# 144-vesicle piece of the 58% lattice (the same cells, density and step as
-# the 1440-vesicle workload).  A launch's figures are these times the patch
+# dram__bytes_write.sum, from one capture of one launch per form on a
+# 288-vesicle lattice at 58% (p = 16 -> 32, the density of the 1440-vesicle
+# workload).  A launch's figures are these times the patch
 # pairs it processes.  They belong to the kernel as captured: when
 # csrc/narrow.cu differs from the captured source (SHA-256 prefix), the
 # instruction roofline and the traffic are reported as null.
 NARROW_NCU = {
-    "src_sha256": "92e5397a85063d40",
-    # 97860990 inst, 7229952 + 889600 B over 35339 patch pairs
-    "fp64": {"inst_per_patch_pair": 2769.21, "dram_bytes_per_patch_pair": 229.76},
-    # 97617838 inst, 7206144 + 858880 B over 35339 patch pairs
-    "mixed": {"inst_per_patch_pair": 2762.33, "dram_bytes_per_patch_pair": 228.22},
+    "src_sha256": "502816f13abb0500",
+    # 105998830 inst, 14866176 + 168704 B over 69230 patch pairs
+    "fp64": {"inst_per_patch_pair": 1531.11, "dram_bytes_per_patch_pair": 217.17},
+    # 106439995 inst, 14794752 + 171520 B over 69227 patch pairs
+    "mixed": {"inst_per_patch_pair": 1537.55, "dram_bytes_per_patch_pair": 216.19},
 }
 ISSUE_PER_SM_CLK = 4   # warp instructions an SM can issue per clock (4 schedulers)
 METRIC = "vesicle-steps/s of detect+V+∇V at p=16→32, 58% vf; % of roofline vs FP64 form"
@@ -568,7 +568,10 @@ def run_ours(args, rank, world, local):
     if fp64_ms > 0:
         ach = float(counts[S.C_FLOPS]) / (fp64_ms * 1e-3) / 1e9
         roof_fp64 = {"kernel": "fp64_kernel", "achieved": ach, "peak": peaks["fp64_gflops"], "unit": "GFLOP/s",
-                     "frac": ach / peaks["fp64_gflops"], "avg_launch_ms": fp64_ms}
+                     "frac": ach / peaks["fp64_gflops"], "avg_launch_ms": fp64_ms,
+                     "work": "operations of the procedure as counted by the kernel; the halvings whose sign the "
+                             "root bounds prove are counted and not computed, so this can pass 1 (ncu: the FP64 "
+                             "pipe is 75% busy)"}
     with open(NARROW_OPS) as f:
         ops_rec = json.load(f)["workloads"]["1440" if args.cells else args.workload]
     narrow_ms = sum(stage_ms.get(k, 0.0) for k in NARROW_STAGES)

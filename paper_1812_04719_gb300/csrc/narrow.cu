@@ -6,15 +6,16 @@
 // The triangulated grid (Sec. 3.1.2, Fig. 3) is cut into patches of 2 x 4 grid
 // quads; each primitive belongs to exactly one patch, so each primitive pair
 // is examined by exactly one patch pair.
-//   patch_pairs_kernel: per candidate vesicle pair, one warp lists the patch
+//   patch_pairs_kernel: per candidate vesicle pair, one CTA lists the patch
 //     pairs whose FP32 (outward) boxes overlap and some of whose cells (1 x 2
 //     quads) meet;
 //   narrow_kernel (stages 1-3a): per patch pair, one warp stages both patches
 //     in shared memory, finds the primitive pairs whose boxes overlap from bit
 //     masks over the vertex slots and filters them; the survivors leave as
 //     global pair descriptors;
-//   pieces_kernel (stage 3b) and fp64_kernel (stage 4) work on those lists,
-//     so that every stage runs on full warps.  The stages:
+//   roots_kernel (d_m = 0) or pieces_kernel (d_m > 0) for stage 3b and
+//     fp64_kernel (stage 4) work on those lists, so that every stage runs on
+//     full warps.  The stages:
 //     1. FP32 swept-box test (conservative: never drops an overlapping pair);
 //     2. the exact FP64 swept-box test (counts the pairs tested), decided
 //        from the FP32 boxes and their error bound, on the FP64 values only
@@ -1353,8 +1354,8 @@ __device__ __forceinline__ int tri_gid(const PatchRef& R, int s0, int s1, int s2
 // through stages 2 and 3a on full warps; survivors are compacted in place and
 // pushed together.
 //
-// Four CTAs of 4 warps an SM (139 KB of staging): bound by issue slots at 70 %
-// of them.  4096 vesicles 7.7 ms, with three CTAs 8.3, with five (registers
+// Four CTAs of 8 warps an SM (139 KB of staging): bound by issue slots, 74 %
+// of them busy.  4096 vesicles 7.7 ms, with three CTAs 8.3, with five (registers
 // spill) 8.0; 1440 of order 16 0.58, 0.62 and 0.62 ms.
 template <bool MIXED, bool DM>
 __global__ void __launch_bounds__(NW * 32, 4) narrow_kernel(narrow_args a) {

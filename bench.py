@@ -391,10 +391,10 @@ def kernel_roofline(S, sc, form: str, prec, stage_ms: dict, counts, peaks: dict,
             inst = fig["inst_per_patch_pair"] * units
             roof["work_per_launch"] = inst
             roof["work"] = "warp instructions issued (ncu smsp__inst_executed.sum per patch pair on the " \
-                           "144-vesicle piece of the lattice, times the launch's patch pairs)"
+                           "288-vesicle lattice, times the launch's patch pairs)"
             roof["achieved"] = inst / (ms * 1e-3) / 1e9
             roof["traffic"] = fig["dram_bytes_per_patch_pair"] * units
-            roof["traffic_unit"] = "bytes per launch (ncu on the 144-vesicle piece, scaled by patch pairs)"
+            roof["traffic_unit"] = "bytes per launch (ncu on the 288-vesicle lattice, scaled by patch pairs)"
     elif dom == "fp64":
         roof.update({"kernel": "fp64_kernel (stage 4)", "bound": "alu", "unit": "GFLOP/s", "peak": peaks["fp64_gflops"],
                      "peak_source": "FP64 FMA rate measured by the library's probe in this run",

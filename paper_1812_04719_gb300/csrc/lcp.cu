@@ -105,6 +105,8 @@ __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t
 constexpr int ST = 256;      // threads of a row-side CTA
 constexpr int CH = 2048;     // points sorted at a time
 constexpr int SD = 128;      // digits of the sort (7 bits)
+// dynamic shared memory of row_sides_kernel: one entry per vertex (nv), 16-bit
+constexpr size_t side_table_bytes(int nv) { return sizeof(uint16_t) * (size_t)((nv + 7) & ~7); }
 
 // Exclusive scan over an ST-thread CTA; *total = the sum.  wsum: ST / 32 ints.
 __device__ __forceinline__ int cta_scan(int v, int* wsum, int* total) {
@@ -760,29 +762,44 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   int32_t* vstart = (int32_t*)(w + o_vs);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-  STIV_PROF_N(h, st, "lcp_matrix", 11);
-  STIV_CUDA(h, cudaMemsetAsync(w, 0, clear, st));
-  bounds_kernel<<<sms * 4, 256, 0, st>>>(counts_dev, ccap, ct->pair, pstart, pend);
-  rows_kernel<<<1, RT, 0, st>>>(counts_dev, pcap, ccap, pstart, pend, V_pair_dev, rcap, lcp->row_pair, lcp->q,
-                                lcp->dims);
-  row_sides_kernel<<<sms * 6, ST, sizeof(uint16_t) * (size_t)((nv + 7) & ~7), st>>>(
-      lcp->dims, lcp->row_pair, pstart, pend, cand->i, g_ves_dev, g_vid_dev, grad_dev, nv,
-      (((uintptr_t)g_ves_dev | (uintptr_t)g_vid_dev) & 15) == 0, sbeg, scnt, ukey, ug);
-  ves_count_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vcnt);
-  ves_scan_kernel<<<1, RT, 0, st>>>(n_ves, vcnt, vstart);
-  ves_fill_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vcnt, lst);
-  ves_rank_kernel<<<sms, 256, 0, st>>>(n_ves, vstart, lst, vrow);
-  bcount_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vrow, vstart, bcnt);
-  bscan_kernel<<<1, RT, 0, st>>>(lcp->dims, bcnt, lcp->nnz_capacity, lcp->row_ptr);
   // one vertex-index table per warp: as many warps per CTA as 96 KB holds
   int nvtab = nv;
   int bw = (int)((96 * 1024) / (sizeof(int32_t) * (size_t)nvtab));
   bw = bw < 1 ? 1 : (bw > 8 ? 8 : bw);
   size_t bsmem = sizeof(int32_t) * (size_t)nvtab * bw;
-  if (bsmem > 48 * 1024)
-    STIV_CUDA(h, cudaFuncSetAttribute(bval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem));
+  // both limits before the first launch, so that no call is refused halfway (a
+  // table of order 32 beside row_sides_kernel's own arrays passes 48 KB)
+  STIV_CUDA(h, cudaFuncSetAttribute(row_sides_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)side_table_bytes(stiv_nverts(2 * STIV_MAX_P))));
+  STIV_CUDA(h, cudaFuncSetAttribute(bval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+  STIV_PROF_N(h, st, "lcp_matrix", 11);
+  STIV_CUDA(h, cudaMemsetAsync(w, 0, clear, st));
+  // every kernel reads what the ones before it wrote: none is launched after one
+  // that was refused
+  bounds_kernel<<<sms * 4, 256, 0, st>>>(counts_dev, ccap, ct->pair, pstart, pend);
+  STIV_LAUNCH(h);
+  rows_kernel<<<1, RT, 0, st>>>(counts_dev, pcap, ccap, pstart, pend, V_pair_dev, rcap, lcp->row_pair, lcp->q,
+                                lcp->dims);
+  STIV_LAUNCH(h);
+  row_sides_kernel<<<sms * 6, ST, side_table_bytes(nv), st>>>(
+      lcp->dims, lcp->row_pair, pstart, pend, cand->i, g_ves_dev, g_vid_dev, grad_dev, nv,
+      (((uintptr_t)g_ves_dev | (uintptr_t)g_vid_dev) & 15) == 0, sbeg, scnt, ukey, ug);
+  STIV_LAUNCH(h);
+  ves_count_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vcnt);
+  STIV_LAUNCH(h);
+  ves_scan_kernel<<<1, RT, 0, st>>>(n_ves, vcnt, vstart);
+  STIV_LAUNCH(h);
+  ves_fill_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vcnt, lst);
+  STIV_LAUNCH(h);
+  ves_rank_kernel<<<sms, 256, 0, st>>>(n_ves, vstart, lst, vrow);
+  STIV_LAUNCH(h);
+  bcount_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vrow, vstart, bcnt);
+  STIV_LAUNCH(h);
+  bscan_kernel<<<1, RT, 0, st>>>(lcp->dims, bcnt, lcp->nnz_capacity, lcp->row_ptr);
+  STIV_LAUNCH(h);
   bcol_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vrow, vstart, lcp->row_ptr,
                                    lcp->nnz_capacity, lcp->col, nzrow);
+  STIV_LAUNCH(h);
   bval_kernel<<<sms * 4, 32 * bw, bsmem, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, sbeg, scnt, ukey, ug,
                                                m_ves_dev, t_ves_dev, nvtab, lcp->nnz_capacity, lcp->row_ptr, lcp->col, nzrow,
                                                lcp->val);

@@ -322,18 +322,31 @@ __device__ __forceinline__ double vert_at(const fid_args& a, size_t idx) {
 
 constexpr int FRMAX = 8;   // fine ring pairs per pass at most
 
-// Pairs of fine rings (r and Pf - r) per pass for order p: as many as keep the
-// pass's point tasks (one per ring and longitude quarter) within two rounds of 256
-// threads, so that few lanes of the last warp idle.
-__host__ __device__ inline int fid_pairs(int p, int factor) {
-  int nq = factor * p + 1, r = 256 / nq;
-  return r < 1 ? 1 : (r > FRMAX ? FRMAX : r);
+// Dynamic shared memory of a CTA at most: 227 KB less the kernel's own arrays.
+constexpr size_t FID_SMEM = 226 * 1024;
+
+__host__ __device__ constexpr size_t fid_pass_bytes(int p, int pairs) {
+  return sizeof(double) * ((size_t)3 * (p + 1) * (p + 1) + (size_t)6 * pairs * ((2 * p + 1) + (4 * p) * 4));
 }
 
-__host__ __device__ inline size_t fid_smem_doubles(int p, int factor) {
-  const size_t rings = 2 * fid_pairs(p, factor);
-  return (size_t)3 * (p + 1) * (p + 1) + rings * 3 * (2 * p + 1) + rings * 3 * (4 * p) * 4;
+// Pairs of fine rings (r and Pf - r) per pass for order p: as many as keep the
+// pass's point tasks (one per ring and longitude quarter) within two rounds of 256
+// threads, so that few lanes of the last warp idle, and its rings within the shared
+// memory (factor 1 at p = 31: 7 pairs, as 8 would take 239 KB).
+__host__ __device__ constexpr int fid_pairs(int p, int factor) {
+  int nq = factor * p + 1, r = 256 / nq;
+  r = r < 1 ? 1 : (r > FRMAX ? FRMAX : r);
+  while (r > 1 && fid_pass_bytes(p, r) > FID_SMEM) --r;
+  return r;
 }
+
+constexpr bool fid_fits() {   // every order and factor that the entry point takes
+  for (int p = 1; p <= STIV_MAX_P; ++p)
+    for (int f = 1; f <= 8; ++f)
+      if (fid_pass_bytes(p, fid_pairs(p, f)) > FID_SMEM) return false;
+  return true;
+}
+static_assert(fid_fits(), "a pass of fidelity_kernel must fit the shared memory");
 
 // The mesh along one fine ring, per coordinate field and longitude cell j
 // (j1 = j + 1 mod 2P), as two lines in the cell fraction b:
@@ -569,7 +582,7 @@ extern "C" int stiv_mesh_fidelity(stiv_handle* h, void* stream, int32_t n_ves, i
   for (int p = 1; p <= p_max; ++p) {
     a.off[p] = total;
     total += fid_doubles(p, factor);
-    size_t b = sizeof(double) * fid_smem_doubles(p, factor);
+    size_t b = fid_pass_bytes(p, fid_pairs(p, factor));
     smem = b > smem ? b : smem;
   }
   STIV_PROF_N(h, st, "mesh_fidelity", 2);

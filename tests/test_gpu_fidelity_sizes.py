@@ -1,0 +1,40 @@
+"""Mesh fidelity over the factors and orders whose passes differ in shared memory:
+the largest passes are factor 1's at the largest orders, which hold the most rings.
+Against the oracle."""
+import numpy as np
+import pytest
+
+from paper_1812_04719_gb300 import scenegen as G
+from paper_1812_04719_gb300 import stiv as S
+from tests.test_gpu_fidelity import gpu_errors, oracle_errors
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("p,factor", [(30, 1), (31, 1), (32, 1), (31, 2)])
+def test_largest_passes(orc, p, factor):
+    """Factor 1 is the mesh's own grid, where the mesh meets the series up to
+    rounding; the other factors within the rounding bound of the smaller orders."""
+    sc = G.two_vesicles(p=p, seed=1)
+    got, scale = gpu_errors(sc, S.STIV_FP64, factor)
+    if factor == 1:
+        assert got.max() <= 1e-13 * scale
+    else:
+        assert np.abs(got[:1] - oracle_errors(orc, sc, [0], factor)).max() <= 1e-11 * scale
+
+
+def test_largest_order_not_present(orc):
+    """p_max = 32 with vesicles of orders 31 and 6: each order has a pass of its own."""
+    a, b = G.two_vesicles(p=31, seed=2), G.two_vesicles(p=6, seed=2)
+    sc = G._pack("31 and 6", [31, 6], [a.coef_of(0), b.coef_of(1)], np.zeros(3), a.centers)
+    eng = S.Stiv.for_scene(sc)
+    ds = S.DeviceScene.from_scene(sc)
+    ds.p_max = 32
+    eng.upsample(ds)
+    for factor in (1, 3):
+        got = eng.mesh_fidelity(ds, factor=factor).cpu().numpy()
+        scale = float(ds.verts.abs().max())
+        if factor == 1:
+            assert got.max() <= 1e-13 * scale
+        else:
+            assert np.abs(got[1:] - oracle_errors(orc, sc, [1], factor)).max() <= 1e-11 * scale

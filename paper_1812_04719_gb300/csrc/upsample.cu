@@ -577,6 +577,9 @@ extern "C" int stiv_mesh_fidelity(stiv_handle* h, void* stream, int32_t n_ves, i
     if (rc) return rc;
     a.theta[p] = h->tab[p].theta;
   }
+  // always raised, and before anything is launched or cleared: the kernel's own
+  // arrays count too, so that the line is not at 48 KB of dynamic memory
+  STIV_CUDA(h, cudaFuncSetAttribute(fidelity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FID_SMEM));
   size_t total = 0, smem = 0;
   for (int p = 0; p <= STIV_MAX_P; ++p) a.off[p] = 0;
   for (int p = 1; p <= p_max; ++p) {
@@ -607,8 +610,6 @@ extern "C" int stiv_mesh_fidelity(stiv_handle* h, void* stream, int32_t n_ves, i
     h->fid_factor = factor; h->fid_pmax = p_max; h->fid_stream = stream;
   }
   STIV_CUDA(h, cudaMemsetAsync(err_dev, 0, sizeof(double) * 2 * (size_t)n_ves, st));
-  if (smem > 48 * 1024)
-    STIV_CUDA(h, cudaFuncSetAttribute(fidelity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   // enough chunks for a dozen CTAs per SM, at most one per pass of the largest order
   const int passes = (factor * p_max + fid_pairs(p_max, factor)) / fid_pairs(p_max, factor);
   int chunks = (12 * 152 + 2 * n_ves - 1) / (2 * n_ves);

@@ -1,6 +1,10 @@
 """Mesh fidelity over the factors and orders whose passes differ in shared memory:
 the largest passes are factor 1's at the largest orders, which hold the most rings.
 Against the oracle."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -38,3 +42,23 @@ def test_largest_order_not_present(orc):
             assert got.max() <= 1e-13 * scale
         else:
             assert np.abs(got[1:] - oracle_errors(orc, sc, [1], factor)).max() <= 1e-11 * scale
+
+
+@pytest.mark.parametrize("p,factor", [(16, 5), (21, 5), (30, 6), (30, 8)])
+def test_sizes_near_48_kb(p, factor):
+    """48 to 49 KB of shared memory, as the first call of a process: the limit of a
+    launch that was raised once stays raised.  The values are checked elsewhere;
+    here they lie below those of a quarter of the order."""
+    code = f"""
+import torch
+from paper_1812_04719_gb300 import scenegen as G, stiv as S
+def worst(p):
+    sc = G.two_vesicles(p=p, seed=1)
+    eng, ds = S.Stiv.for_scene(sc), S.DeviceScene.from_scene(sc)
+    eng.upsample(ds)
+    return float(eng.mesh_fidelity(ds, factor={factor}).max())
+a = worst({p})
+assert 0 < a < worst({p} // 4), a
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)

@@ -121,9 +121,9 @@ extern "C" int stiv_profile_read(stiv_handle* h, int32_t max_names, char* names,
   std::vector<stiv_profiler::rec> keep;
   for (auto& r : P->recs) {
     if (!r.valid) { keep.push_back(r); continue; }   // captured but not replayed yet
-    if (cudaEventSynchronize(r.e) != cudaSuccess) return STIV_ERR_CUDA;
+    STIV_CUDA(h, cudaEventSynchronize(r.e));
     float ms = 0.f;
-    if (cudaEventElapsedTime(&ms, r.b, r.e) != cudaSuccess) return STIV_ERR_CUDA;
+    STIV_CUDA(h, cudaEventElapsedTime(&ms, r.b, r.e));
     size_t k = 0;
     while (k < keys.size() && keys[k] != r.name) ++k;
     if (k == keys.size()) { keys.push_back(r.name); cnt.push_back(0); tot.push_back(0.0); }
@@ -166,7 +166,7 @@ extern "C" int stiv_create(stiv_handle** out, const stiv_params* prm) {
   if (!h) return STIV_ERR_ARG;
   h->prm = *prm;
   cudaError_t e = cudaGetDevice(&h->device);
-  if (e != cudaSuccess) { free(h); return STIV_ERR_CUDA; }
+  if (e != cudaSuccess) { free(h); return stiv_cuda_failed(nullptr, e); }
   *out = h;
   return STIV_OK;
 }
@@ -207,7 +207,7 @@ extern "C" int stiv_mesh_topology(int32_t P, int32_t* tri_dev, int32_t* edge_dev
   if (P < 2 || P > STIV_MAX_PP || !tri_dev || !edge_dev) return STIV_ERR_ARG;
   int n = stiv_ntris(P);
   topology_kernel<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(P, tri_dev, edge_dev);
-  if (cudaGetLastError() != cudaSuccess) return STIV_ERR_CUDA;
+  STIV_LAUNCH(STIV_NO_HANDLE);
   return STIV_OK;
 }
 
@@ -337,11 +337,11 @@ extern "C" int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_
   auto timed = [&](float& ms) -> int {
     float best = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
-      if (cudaEventRecord(e0, st) != cudaSuccess) return STIV_ERR_CUDA;
+      STIV_CUDA(h, cudaEventRecord(e0, st));
       int rc = stiv_detect(h, stream, n_ves, p_max, p_dev, vert_off_dev, verts_dev, cand, out, counts_dev);
       if (rc) return rc;
-      if (cudaEventRecord(e1, st) != cudaSuccess) return STIV_ERR_CUDA;
-      if (cudaEventSynchronize(e1) != cudaSuccess) return STIV_ERR_CUDA;
+      STIV_CUDA(h, cudaEventRecord(e1, st));
+      STIV_CUDA(h, cudaEventSynchronize(e1));
       float t = 0.f;
       cudaEventElapsedTime(&t, e0, e1);
       if (t < best) best = t;
@@ -390,9 +390,8 @@ extern "C" int stiv_set_tuning(stiv_handle* h, const int32_t* values) {
 
 extern "C" int stiv_sync_counts(void* stream, const int64_t* counts_dev, int64_t* counts_host) {
   if (!counts_dev || !counts_host) return STIV_ERR_ARG;
-  if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return STIV_ERR_CUDA;
-  if (cudaMemcpy(counts_host, counts_dev, sizeof(int64_t) * STIV_NCOUNTS, cudaMemcpyDeviceToHost) != cudaSuccess)
-    return STIV_ERR_CUDA;
+  STIV_CUDA(STIV_NO_HANDLE, cudaStreamSynchronize((cudaStream_t)stream));
+  STIV_CUDA(STIV_NO_HANDLE, cudaMemcpy(counts_host, counts_dev, sizeof(int64_t) * STIV_NCOUNTS, cudaMemcpyDeviceToHost));
   int64_t f = counts_host[STIV_C_STATUS];
   if (f & (STIV_F_PAIRS_OVERFLOW | STIV_F_CONTACTS_OVERFLOW | STIV_F_WORK_OVERFLOW)) return STIV_ERR_CAPACITY;
   if (f & (STIV_F_BOX_TOO_SMALL | STIV_F_NONFINITE | STIV_F_BAD_ORDER)) return STIV_ERR_INPUT;
@@ -457,12 +456,11 @@ extern "C" int stiv_step(stiv_handle* h, void* stream, int32_t use_graph, int32_
   if (rc) { if (graph) cudaGraphDestroy(graph); return rc; }
   if (e != cudaSuccess || h->ws != ws_before) {
     if (graph) cudaGraphDestroy(graph);
-    h->last_cuda_error = (int)e;
-    return STIV_ERR_CUDA;
+    return stiv_cuda_failed(h, e);
   }
   e = cudaGraphInstantiate(&h->graph_exec, graph, 0);
   cudaGraphDestroy(graph);
-  if (e != cudaSuccess) { h->graph_exec = nullptr; h->last_cuda_error = (int)e; return STIV_ERR_CUDA; }
+  if (e != cudaSuccess) { h->graph_exec = nullptr; return stiv_cuda_failed(h, e); }
   h->graph_key = key;
   return STIV_OK;
 }

@@ -45,16 +45,16 @@ extern "C" int stiv_peak_probe(void* stream, int32_t kind, int64_t iters, double
   if (kind < 0 || kind > 1 || iters < 1 || iters > ((int64_t)1 << 32) || !sink_dev || !flops_out)
     return STIV_ERR_ARG;
   int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return STIV_ERR_CUDA;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-    return STIV_ERR_CUDA;
+  STIV_CUDA(STIV_NO_HANDLE, cudaGetDevice(&dev));
+  STIV_CUDA(STIV_NO_HANDLE, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (sms < 1) return STIV_ERR_CUDA;
   int blocks = sms * PROBE_BLOCKS_PER_SM;
   cudaStream_t st = (cudaStream_t)stream;
   if (kind == 0)
     fma_probe_kernel<double><<<blocks, PROBE_THREADS, 0, st>>>(iters, 0.999999, 1e-7, sink_dev);
   else
     fma_probe_kernel<float><<<blocks, PROBE_THREADS, 0, st>>>(iters, 0.999999f, 1e-7f, sink_dev);
-  if (cudaGetLastError() != cudaSuccess) return STIV_ERR_CUDA;
+  STIV_LAUNCH(STIV_NO_HANDLE);
   *flops_out = 2.0 * NCHAIN * (double)iters * (double)blocks * PROBE_THREADS;
   return STIV_OK;
 }

@@ -190,8 +190,8 @@ int stiv_sort_pairs_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_
   int passes = (key_bits + 7) / 8;
   if (passes == 0) {
     if (n > 0) {
-      if (cudaMemcpyAsync(kout, kin, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return STIV_ERR_CUDA;
-      if (cudaMemcpyAsync(vout, vin, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return STIV_ERR_CUDA;
+      STIV_CUDA(STIV_NO_HANDLE, cudaMemcpyAsync(kout, kin, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, st));
+      STIV_CUDA(STIV_NO_HANDLE, cudaMemcpyAsync(vout, vin, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, st));
     }
     return STIV_OK;
   }
@@ -211,7 +211,7 @@ int stiv_sort_pairs_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_
     hist_kernel<<<grid, kThreads, 0, st>>>(ka, n_dev, n, shift, mask, hist);
     scan_kernel<<<kRadix, kThreads, 0, st>>>(hist, n_dev, n, totals);
     scatter_kernel<<<grid, kThreads, 0, st>>>(ka, va, kb, vb, n_dev, n, shift, mask, hist, totals);
-    if (cudaGetLastError() != cudaSuccess) return STIV_ERR_CUDA;
+    STIV_LAUNCH(STIV_NO_HANDLE);
     ka = kb;
     va = vb;
   }
@@ -231,8 +231,8 @@ int stiv_sort_user_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_t
   for (int a = 0; a < 2; ++a)
     for (int b = 0; b < 2; ++b) overlap = overlap || (in[a] < out[b] + len[b] && out[b] < in[a] + len[a]);
   if (overlap && ((key_bits + 7) / 8) % 2 == 1) {
-    if (cudaMemcpyAsync(kt, kin, len[0], cudaMemcpyDeviceToDevice, st) != cudaSuccess) return STIV_ERR_CUDA;
-    if (cudaMemcpyAsync(vt, vin, len[1], cudaMemcpyDeviceToDevice, st) != cudaSuccess) return STIV_ERR_CUDA;
+    STIV_CUDA(STIV_NO_HANDLE, cudaMemcpyAsync(kt, kin, len[0], cudaMemcpyDeviceToDevice, st));
+    STIV_CUDA(STIV_NO_HANDLE, cudaMemcpyAsync(vt, vin, len[1], cudaMemcpyDeviceToDevice, st));
     kin = kt;
     vin = vt;
   }

@@ -35,7 +35,8 @@ static __device__ __align__(256) unsigned char g_sort_scratch[kScratchBytes];
 // across a device reset or a new context, where the array may move.
 int scratch_address(unsigned char** out) {
   void* p = nullptr;
-  if (cudaGetSymbolAddress(&p, g_sort_scratch) != cudaSuccess || !p) return STIV_ERR_CUDA;
+  STIV_CUDA(STIV_NO_HANDLE, cudaGetSymbolAddress(&p, g_sort_scratch));
+  if (!p) return STIV_ERR_CUDA;
   *out = (unsigned char*)p;
   return STIV_OK;
 }

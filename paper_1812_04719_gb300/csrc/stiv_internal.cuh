@@ -169,23 +169,22 @@ struct detect_ws {
 // ---------------------------------------------------------------------------
 // error handling
 // ---------------------------------------------------------------------------
-#define STIV_CUDA(h, call)                                \
-  do {                                                    \
-    cudaError_t e_ = (call);                              \
-    if (e_ != cudaSuccess) {                              \
-      if (h) (h)->last_cuda_error = (int)e_;              \
-      return STIV_ERR_CUDA;                               \
-    }                                                     \
+// A failed call: noted in the handle (if any), and taken off the thread's pending
+// error, which the check of the next good launch would report again.
+inline int stiv_cuda_failed(stiv_handle* h, cudaError_t e) {
+  if (h) h->last_cuda_error = (int)e;
+  cudaGetLastError();
+  return STIV_ERR_CUDA;
+}
+
+#define STIV_CUDA(h, call)                                        \
+  do {                                                            \
+    cudaError_t e_ = (call);                                      \
+    if (e_ != cudaSuccess) return stiv_cuda_failed((h), e_);      \
   } while (0)
 
-#define STIV_LAUNCH(h)                                    \
-  do {                                                    \
-    cudaError_t e_ = cudaGetLastError();                  \
-    if (e_ != cudaSuccess) {                              \
-      if (h) (h)->last_cuda_error = (int)e_;              \
-      return STIV_ERR_CUDA;                               \
-    }                                                     \
-  } while (0)
+#define STIV_LAUNCH(h) STIV_CUDA(h, cudaGetLastError())
+#define STIV_NO_HANDLE ((stiv_handle*)nullptr)
 
 int stiv_ensure_tables(stiv_handle* h, cudaStream_t st, int p);
 // STIV_MIXED synthesis on the tensor cores (3xTF32), FP32 vertices.

@@ -797,5 +797,6 @@ int stiv_grad_to_coef_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t
 extern "C" int stiv_wait_selftest(void* stream, int64_t limit_cycles, int32_t* status_dev) {
   if (!status_dev || limit_cycles < 0 || limit_cycles > WAIT_CYCLES) return STIV_ERR_ARG;
   wait_selftest_kernel<<<1, 32, 0, (cudaStream_t)stream>>>((long long)limit_cycles, status_dev);
-  return cudaGetLastError() == cudaSuccess ? STIV_OK : STIV_ERR_CUDA;
+  STIV_LAUNCH(STIV_NO_HANDLE);
+  return STIV_OK;
 }

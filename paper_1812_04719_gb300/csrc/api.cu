@@ -96,13 +96,19 @@ void stiv_prof_drop_graph(stiv_handle* h) {
   P->recs.swap(keep);
 }
 
+// Forget the captured step: the next stiv_step with use_graph captures again.
+void stiv_drop_graph(stiv_handle* h) {
+  if (h->graph_exec) { cudaGraphExecDestroy(h->graph_exec); h->graph_exec = nullptr; h->graph_key = 0; }
+  stiv_prof_drop_graph(h);
+}
+
 extern "C" int stiv_profile(stiv_handle* h, int32_t enable) {
   if (!h) return STIV_ERR_ARG;
   if (enable && !h->prof) h->prof = new stiv_profiler();
   if (!enable && h->prof) {
     stiv_profiler* P = (stiv_profiler*)h->prof;
     cudaDeviceSynchronize();
-    if (h->graph_exec) { cudaGraphExecDestroy(h->graph_exec); h->graph_exec = nullptr; h->graph_key = 0; }
+    stiv_drop_graph(h);
     for (auto& r : P->recs) { cudaEventDestroy(r.b); cudaEventDestroy(r.e); }
     for (auto ev : P->pool) cudaEventDestroy(ev);
     delete P;
@@ -196,6 +202,7 @@ extern "C" int stiv_destroy(stiv_handle* h) {
 
 int stiv_ws_reserve(stiv_handle* h, size_t bytes) {
   if (bytes <= h->ws_bytes) return STIV_OK;
+  stiv_drop_graph(h);
   if (h->ws) { STIV_CUDA(h, cudaFree(h->ws)); h->ws = nullptr; h->ws_bytes = 0; }
   size_t nb = bytes + bytes / 4;
   STIV_CUDA(h, cudaMalloc(&h->ws, nb));
@@ -371,8 +378,7 @@ extern "C" int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_
     for (int k = 0; k < STIV_NTUNE; ++k) h->tune[k] = saved[k];
     return rc;
   }
-  if (h->graph_exec) { cudaGraphExecDestroy(h->graph_exec); h->graph_exec = nullptr; h->graph_key = 0; }
-  stiv_prof_drop_graph(h);
+  stiv_drop_graph(h);
   if (choice_out) for (int k = 0; k < STIV_NTUNE; ++k) choice_out[k] = h->tune[k];
   if (best_ms_out) *best_ms_out = best_ms;
   return STIV_OK;
@@ -383,8 +389,7 @@ extern "C" int stiv_set_tuning(stiv_handle* h, const int32_t* values) {
   for (int k = 0; k < STIV_NTUNE; ++k)
     if (values[k] < 0 || values[k] > 64 || (k == STIV_TUNE_PIECE_LEVELS && values[k] > 6)) return STIV_ERR_ARG;
   for (int k = 0; k < STIV_NTUNE; ++k) h->tune[k] = values[k];
-  if (h->graph_exec) { cudaGraphExecDestroy(h->graph_exec); h->graph_exec = nullptr; h->graph_key = 0; }
-  stiv_prof_drop_graph(h);
+  stiv_drop_graph(h);
   return STIV_OK;
 }
 
@@ -444,8 +449,7 @@ extern "C" int stiv_step(stiv_handle* h, void* stream, int32_t use_graph, int32_
   int rc = step_eager(h, stream, n_ves, p_max, p_dev, coef_off_dev, coef_dev, vert_off_dev, verts_dev, cand, out,
                       counts_dev, V_contact_dev, V_pair_dev, grad_dev, g_ves_dev, g_vid_dev);
   if (rc) return rc;
-  if (h->graph_exec) { cudaGraphExecDestroy(h->graph_exec); h->graph_exec = nullptr; }
-  stiv_prof_drop_graph(h);
+  stiv_drop_graph(h);
   cudaStream_t st = (cudaStream_t)stream;
   STIV_CUDA(h, cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
   void* ws_before = h->ws;

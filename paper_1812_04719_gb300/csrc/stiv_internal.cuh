@@ -54,7 +54,7 @@ struct stiv_handle {
   // per-call scratch, and the device status word of its bounded waits
   float* ytab[STIV_MAX_P + 1];
   float* ytabT[STIV_MAX_P + 1];   // transposed blocks for the adjoint
-  void* tc_ws;                    // synthesis scratch (referenced by captured graphs: never reused)
+  void* tc_ws;                    // synthesis scratch (referenced by the captured step)
   size_t tc_ws_bytes;
   void* tc_ws2;                   // adjoint scratch
   size_t tc_ws2_bytes;
@@ -75,7 +75,8 @@ struct stiv_handle {
   int32_t tune[STIV_NTUNE];
   void* ws;
   size_t ws_bytes;
-  // CUDA graph of stiv_step
+  // CUDA graph of stiv_step.  Its launches hold the addresses of ws and tc_ws:
+  // whoever frees one of them drops the graph (stiv_drop_graph).
   cudaGraphExec_t graph_exec;
   unsigned long long graph_key;
   // per-kernel CUDA-event profiler (stiv_profile); null when off
@@ -196,6 +197,7 @@ int stiv_grad_to_coef_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t
                          const int64_t* coef_off_dev, const int64_t* vert_off_dev, const double* gX_dev,
                          double* gcoef_dev);
 int stiv_ws_reserve(stiv_handle* h, size_t bytes);
+void stiv_drop_graph(stiv_handle* h);
 int stiv_sort_pairs_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_t* kin, const int32_t* vin,
                          uint64_t* kout, int32_t* vout, uint64_t* ktmp, int32_t* vtmp, void* scratch,
                          size_t scratch_bytes, const int64_t* n_dev);

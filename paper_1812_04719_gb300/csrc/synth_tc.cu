@@ -719,6 +719,7 @@ int stiv_upsample_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t p_m
   size_t o_b = align256(o_ci + sizeof(tc_colinfo) * (size_t)max_ntn * TN);
   size_t total = o_b + (size_t)max_blocks * BLK_BYTES;
   if (total > h->tc_ws_bytes) {
+    stiv_drop_graph(h);
     if (h->tc_ws) { STIV_CUDA(h, cudaFree(h->tc_ws)); h->tc_ws = nullptr; h->tc_ws_bytes = 0; }
     STIV_CUDA(h, cudaMalloc(&h->tc_ws, total));
     h->tc_ws_bytes = total;

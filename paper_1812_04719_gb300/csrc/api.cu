@@ -335,7 +335,7 @@ extern "C" int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_
                              double* best_ms_out) {
   if (!h || !counts_dev) return STIV_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  static const int32_t cands[STIV_NTUNE][4] = {{2, 3, 4, 0}, {1, 2, 3, 4}, {4, 8, 16, 32}, {8, 12, 16, 0}, {2, 3, 4, 5}};
+  static const int32_t cands[STIV_NTUNE][4] = {{2, 3, 4, 0}, {1, 2, 3, 4}, {4, 8, 16, 32}, {2, 4, 8, 0}, {2, 3, 4, 0}};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   STIV_CUDA(h, cudaEventCreate(&e0));
   STIV_CUDA(h, cudaEventCreate(&e1));
@@ -361,10 +361,23 @@ extern "C" int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_
   float best_ms = 0.f;
   int rc = timed(best_ms);   // warm-up with the current shapes (sizes the workspace)
   if (!rc) rc = timed(best_ms);
+  // what a value means at launch: 0 the default, CTAs up to those that fit
+  auto shape = [&](int k, int32_t v) -> int32_t {
+    if (k == STIV_TUNE_NARROW_CTAS || k == STIV_TUNE_PIECES_CTAS) {
+      const int32_t most = h->max_ctas[k == STIV_TUNE_NARROW_CTAS ? 0 : 1];
+      return v == 0 || v > most ? most : v;
+    }
+    if (v) return v;
+    return k == STIV_TUNE_FP64_BLOCKS ? STIV_FP64_BLOCKS : (k == STIV_TUNE_PATCH_BLOCKS ? STIV_PATCH_BLOCKS : STIV_PIECE_LEVELS);
+  };
   for (int k = 0; k < STIV_NTUNE && !rc; ++k) {
+    // no effect, so nothing but noise to choose by: the pieces without the filter,
+    // their levels at d_m = 0 (the root test has none)
+    if (h->prm.exact_only && (k == STIV_TUNE_PIECES_CTAS || k == STIV_TUNE_PIECE_LEVELS)) continue;
+    if (!(h->prm.d_m > 0.0) && k == STIV_TUNE_PIECE_LEVELS) continue;
     int32_t keep = h->tune[k];
     for (int c = 0; c < 4 && !rc; ++c) {
-      if (cands[k][c] == 0 || cands[k][c] == keep) continue;
+      if (cands[k][c] == 0 || shape(k, cands[k][c]) == shape(k, keep)) continue;
       h->tune[k] = cands[k][c];
       float ms = 0.f;
       rc = timed(ms);

@@ -2093,7 +2093,7 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
   const double* L = h->prm.box_L;
   // CTAs per SM: enough to hide the phases of one pair behind those of others
   int blocks = (int)cand->capacity;
-  int pp_mult = h->tune[STIV_TUNE_PATCH_BLOCKS] > 0 ? h->tune[STIV_TUNE_PATCH_BLOCKS] : 12;
+  int pp_mult = h->tune[STIV_TUNE_PATCH_BLOCKS] > 0 ? h->tune[STIV_TUNE_PATCH_BLOCKS] : STIV_PATCH_BLOCKS;
   if (cand->capacity > (int64_t)pp_mult * num_sms) blocks = pp_mult * num_sms;
   if (blocks < 1) blocks = 1;
   int mp = stiv_npatches(2 * p_max);
@@ -2116,7 +2116,7 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
   a.dm = h->prm.d_m;
   // five levels by default: at 360 vesicles (p = 15, d_m > 0) pieces and FP64 test
   // take 1.19 ms at 2 levels, 1.06 at 4, 1.04 at 5
-  a.nlevel = h->tune[STIV_TUNE_PIECE_LEVELS] > 0 ? h->tune[STIV_TUNE_PIECE_LEVELS] : 5;
+  a.nlevel = h->tune[STIV_TUNE_PIECE_LEVELS] > 0 ? h->tune[STIV_TUNE_PIECE_LEVELS] : STIV_PIECE_LEVELS;
   if (a.nlevel > NLEVEL) a.nlevel = NLEVEL;
   if (a.nlevel < 1) a.nlevel = 1;
   a.vorg = w.vorg; a.fprep = w.fprep; a.fstride = w.fstride;
@@ -2134,6 +2134,7 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
   STIV_CUDA(h, cudaFuncSetAttribute(nk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   STIV_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nk, NW * 32, smem));
+  h->max_ctas[0] = per_sm;
   if (h->tune[STIV_TUNE_NARROW_CTAS] > 0 && h->tune[STIV_TUNE_NARROW_CTAS] < per_sm) per_sm = h->tune[STIV_TUNE_NARROW_CTAS];
   if (per_sm < 1) per_sm = 1;
   {
@@ -2148,6 +2149,7 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
     if (dmk) STIV_CUDA(h, cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm2));
     int per_sm2 = 0;
     STIV_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, pk, PW * 32, psm2));
+    h->max_ctas[1] = per_sm2;
     if (h->tune[STIV_TUNE_PIECES_CTAS] > 0 && h->tune[STIV_TUNE_PIECES_CTAS] < per_sm2)
       per_sm2 = h->tune[STIV_TUNE_PIECES_CTAS];
     if (per_sm2 < 1) per_sm2 = 1;
@@ -2159,7 +2161,7 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
     STIV_PROF(h, st, "fp64");
     auto fk = mixed ? (dmk ? fp64_kernel<true, true> : fp64_kernel<true, false>)
                     : (dmk ? fp64_kernel<false, true> : fp64_kernel<false, false>);
-    int fm = h->tune[STIV_TUNE_FP64_BLOCKS] > 0 ? h->tune[STIV_TUNE_FP64_BLOCKS] : 16;
+    int fm = h->tune[STIV_TUNE_FP64_BLOCKS] > 0 ? h->tune[STIV_TUNE_FP64_BLOCKS] : STIV_FP64_BLOCKS;
     fk<<<num_sms * fm, 128, 0, st>>>(a);
   }
   STIV_LAUNCH(h);

@@ -31,6 +31,10 @@
 #define STIV_ROW_CHUNK 512   // boxes tested per unit of a row
 #define STIV_ROW_KEEP 32     // hits kept per unit
 #define STIV_ROW_SUM 256     // units per partial sum of their hits
+// Launch shapes of the narrow phase that stiv_autotune may replace.
+#define STIV_FP64_BLOCKS 16    // FP64 contact-test blocks per SM
+#define STIV_PATCH_BLOCKS 12   // patch-pair blocks per SM
+#define STIV_PIECE_LEVELS 5    // d_m > 0: refinement levels of the piece test
 inline int stiv_row_chunks(int n) { return (n + STIV_ROW_CHUNK - 1) / STIV_ROW_CHUNK; }
 
 // ---------------------------------------------------------------------------
@@ -71,8 +75,10 @@ struct stiv_handle {
   int fid_factor, fid_pmax;
   const void* fid_stream;
   bool fid_captured;
-  // launch shapes of the narrow phase (0 = default), set by stiv_autotune
+  // launch shapes of the narrow phase (0 = default), set by stiv_autotune; and the
+  // CTAs per SM that its first two allow (their default), found by the last launch
   int32_t tune[STIV_NTUNE];
+  int32_t max_ctas[2];
   void* ws;
   size_t ws_bytes;
   // CUDA graph of stiv_step.  Its launches hold the addresses of ws and tc_ws:

@@ -193,6 +193,7 @@ extern "C" int stiv_destroy(stiv_handle* h) {
   if (h->lcp_ws) cudaFree(h->lcp_ws);
   if (h->lcp_ws2) cudaFree(h->lcp_ws2);
   if (h->fid_tab) cudaFree(h->fid_tab);
+  if (h->fid_done) cudaEventDestroy(h->fid_done);
   if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
   if (h->ws) cudaFree(h->ws);
   stiv_profile(h, 0);

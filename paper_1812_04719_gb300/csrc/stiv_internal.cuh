@@ -68,12 +68,12 @@ struct stiv_handle {
   size_t lcp_ws_bytes;
   void* lcp_ws2;
   size_t lcp_ws2_bytes;
-  // tables of the mesh-fidelity estimate, for the factor, orders and stream of
-  // the last call
+  // tables of the mesh-fidelity estimate, for the factor (0: none) and orders of
+  // the last call, and the end of that call
   double* fid_tab;
   size_t fid_tab_bytes;
   int fid_factor, fid_pmax;
-  const void* fid_stream;
+  cudaEvent_t fid_done;
   bool fid_captured;
   // launch shapes of the narrow phase (0 = default), set by stiv_autotune; and the
   // CTAs per SM that its first two allow (their default), found by the last launch

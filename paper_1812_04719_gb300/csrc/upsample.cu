@@ -589,25 +589,30 @@ extern "C" int stiv_mesh_fidelity(stiv_handle* h, void* stream, int32_t n_ves, i
     smem = b > smem ? b : smem;
   }
   STIV_PROF_N(h, st, "mesh_fidelity", 2);
-  // The tables stay valid for the same stream, factor and orders.  A table made on
-  // another stream would need waiting for: it is made again.  A captured call makes
-  // them in its graph, whose replays overwrite them at any time: from then on every
-  // call of the handle makes its own.
+  // The tables stay valid for the same factor and orders.  Every call waits for
+  // the end of the one before (an event: a stream's handle may be that of a
+  // destroyed stream, or stand for a stream of each thread), so that it finds
+  // them written, and rewrites them only once they have been read.  A captured
+  // call makes them in its graph, whose replays overwrite them at any time: from
+  // then on every call of the handle makes its own.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   STIV_CUDA(h, cudaStreamIsCapturing(st, &cap));
-  if (cap != cudaStreamCaptureStatusNone) h->fid_captured = true;
-  const bool made = h->fid_tab && !h->fid_captured && h->fid_factor == factor && h->fid_pmax == p_max &&
-                    h->fid_stream == stream;
+  const bool captured = cap != cudaStreamCaptureStatusNone;
+  if (captured) h->fid_captured = true;
+  else if (h->fid_done) STIV_CUDA(h, cudaStreamWaitEvent(st, h->fid_done, 0));
+  else STIV_CUDA(h, cudaEventCreateWithFlags(&h->fid_done, cudaEventDisableTiming));
+  const bool made = h->fid_tab && !h->fid_captured && h->fid_factor == factor && h->fid_pmax == p_max;
   if (sizeof(double) * total > h->fid_tab_bytes) {
+    h->fid_factor = 0;
     if (h->fid_tab) { STIV_CUDA(h, cudaFree(h->fid_tab)); h->fid_tab = nullptr; h->fid_tab_bytes = 0; }
     STIV_CUDA(h, cudaMalloc(&h->fid_tab, sizeof(double) * total));
     h->fid_tab_bytes = sizeof(double) * total;
   }
   a.tab = h->fid_tab;
   if (!made) {
+    h->fid_factor = 0;   // set again once all has been launched
     fid_tables_kernel<<<dim3(factor * p_max + 1, p_max), 64, 0, st>>>(a, h->fid_tab);
     STIV_LAUNCH(h);
-    h->fid_factor = factor; h->fid_pmax = p_max; h->fid_stream = stream;
   }
   STIV_CUDA(h, cudaMemsetAsync(err_dev, 0, sizeof(double) * 2 * (size_t)n_ves, st));
   // enough chunks for a dozen CTAs per SM, at most one per pass of the largest order
@@ -616,5 +621,7 @@ extern "C" int stiv_mesh_fidelity(stiv_handle* h, void* stream, int32_t n_ves, i
   chunks = chunks < 1 ? 1 : (chunks > passes ? passes : chunks);
   fidelity_kernel<<<dim3(n_ves, 2, chunks), 256, smem, st>>>(a);
   STIV_LAUNCH(h);
+  if (!captured) STIV_CUDA(h, cudaEventRecord(h->fid_done, st));
+  h->fid_factor = factor; h->fid_pmax = p_max;
   return STIV_OK;
 }

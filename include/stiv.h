@@ -357,6 +357,13 @@ int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_t p_max, co
  * STIV_TUNE_PIECE_LEVELS in [1, 6]); STIV_ERR_ARG for a value out of range. */
 int stiv_set_tuning(stiv_handle* h, const int32_t* values);
 
+/* Broad-phase changeover (not a step of the method: both ways give the same
+ * candidate pairs in the same order; for cross-checks).  Up to n_ves vesicles
+ * stiv_detect tests every pair of boxes, above that it uses the Morton grid of
+ * Alg. 1.  n_ves in [0, 8192], 8192 by default (where the quadratic test and the
+ * grid take the same time); 0: always the grid.  STIV_ERR_ARG out of range. */
+int stiv_set_all_pairs_limit(stiv_handle* h, int32_t n_ves);
+
 /* Check of the bounded device waits (not a step of the method): one thread
  * waits on a shared-memory barrier that nothing completes, giving up after
  * limit_cycles SM clocks (0 <= limit_cycles <= the bound the tensor-core

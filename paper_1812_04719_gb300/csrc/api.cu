@@ -171,6 +171,7 @@ extern "C" int stiv_create(stiv_handle** out, const stiv_params* prm) {
   stiv_handle* h = (stiv_handle*)calloc(1, sizeof(stiv_handle));
   if (!h) return STIV_ERR_ARG;
   h->prm = *prm;
+  h->all_pairs = STIV_BRUTE_MAX;
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) { free(h); return stiv_cuda_failed(nullptr, e); }
   *out = h;
@@ -222,7 +223,7 @@ extern "C" int stiv_mesh_topology(int32_t P, int32_t* tri_dev, int32_t* edge_dev
 // Scratch of stiv_detect, carved from the handle's buffer.
 static int detect_layout(stiv_handle* h, int n, int p_max, const stiv_pairs* cand, const stiv_contacts* out,
                          detect_ws& w, bool carve) {
-  const bool brute = n <= STIV_BRUTE_MAX;   // no grid records and no candidate keys
+  const bool brute = n <= h->all_pairs;   // no grid records and no candidate keys
   const size_t units = brute ? (size_t)n * stiv_row_chunks(n) : 0;
   w.R = brute ? 1 : (int64_t)n * 64 + 1024;
   w.Q = brute ? 1 : cand->capacity * 8 + 1024;
@@ -403,6 +404,13 @@ extern "C" int stiv_set_tuning(stiv_handle* h, const int32_t* values) {
   for (int k = 0; k < STIV_NTUNE; ++k)
     if (values[k] < 0 || values[k] > 64 || (k == STIV_TUNE_PIECE_LEVELS && values[k] > 6)) return STIV_ERR_ARG;
   for (int k = 0; k < STIV_NTUNE; ++k) h->tune[k] = values[k];
+  stiv_drop_graph(h);
+  return STIV_OK;
+}
+
+extern "C" int stiv_set_all_pairs_limit(stiv_handle* h, int32_t n_ves) {
+  if (!h || n_ves < 0 || n_ves > STIV_BRUTE_MAX) return STIV_ERR_ARG;
+  h->all_pairs = n_ves;
   stiv_drop_graph(h);
   return STIV_OK;
 }

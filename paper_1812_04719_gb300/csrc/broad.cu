@@ -655,7 +655,7 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   bk<<<n, BT, bsmem, st>>>(n, p_dev, voff, X, mixed, h->prm.d_m, L[0], L[1], L[2], w.vbox, w.pbox,
                                       w.pstride, w.vorg, w.fprep, w.fstride, ctr, vb_cap, p_max, w.fbox);
   }
-  if (n <= STIV_BRUTE_MAX) {
+  if (n <= h->all_pairs) {
     rows_args a;
     a.n = n; a.nchunk = stiv_row_chunks(n); a.vbox = w.vbox; a.fbox = w.fbox;
     for (int c = 0; c < 3; ++c) a.L[c] = L[c];

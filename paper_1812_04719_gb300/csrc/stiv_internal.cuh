@@ -26,7 +26,8 @@
 #define STIV_PBOX 40
 #define STIV_PBOX_CELLS 8
 // Candidate pairs by testing every pair of boxes up to this many vesicles;
-// beyond, by the Morton grid and its sorts.
+// beyond, by the Morton grid and its sorts (stiv_set_all_pairs_limit lowers it
+// for a handle).
 #define STIV_BRUTE_MAX 8192
 #define STIV_ROW_CHUNK 512   // boxes tested per unit of a row
 #define STIV_ROW_KEEP 32     // hits kept per unit
@@ -79,6 +80,7 @@ struct stiv_handle {
   // CTAs per SM that its first two allow (their default), found by the last launch
   int32_t tune[STIV_NTUNE];
   int32_t max_ctas[2];
+  int32_t all_pairs;      // most vesicles whose boxes are all tested against each other
   void* ws;
   size_t ws_bytes;
   // CUDA graph of stiv_step.  Its launches hold the addresses of ws and tc_ws:

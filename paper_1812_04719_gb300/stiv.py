@@ -37,6 +37,7 @@ EXPORTS = ["stiv_create", "stiv_destroy", "stiv_status_string", "stiv_last_cuda_
            "stiv_upsample", "stiv_detect", "stiv_stiv", "stiv_stiv_grad", "stiv_grad_scatter",
            "stiv_grad_to_coef", "stiv_step", "stiv_sync_counts", "stiv_sort_scratch_bytes", "stiv_sort_pairs",
            "stiv_profile", "stiv_profile_read", "stiv_sort_pairs_static", "stiv_autotune", "stiv_set_tuning",
+           "stiv_set_all_pairs_limit",
            "stiv_wait_selftest", "stiv_lcp_matrix", "stiv_lcp_solve",
            "stiv_mesh_fidelity", "stiv_stiv_grad_x0", "stiv_peak_probe"]
 TUNE_NAMES = ("narrow_ctas_per_sm", "pieces_ctas_per_sm", "fp64_blocks_per_sm", "patch_blocks_per_sm",
@@ -107,6 +108,7 @@ def lib() -> ctypes.CDLL:
     L.stiv_sort_pairs_static.argtypes = [vp, i64, i32, vp, vp, vp, vp]
     L.stiv_autotune.argtypes = [vp, vp, i32, i32, vp, vp, vp, P(StivPairs), P(StivContacts), vp, vp, vp]
     L.stiv_set_tuning.argtypes = [vp, vp]
+    L.stiv_set_all_pairs_limit.argtypes = [vp, i32]
     L.stiv_wait_selftest.argtypes = [vp, i64, vp]
     L.stiv_lcp_matrix.argtypes = [vp, vp, i32, i32, P(StivPairs), P(StivContacts), vp, vp, vp, vp, vp, vp, vp,
                                   P(StivLcp)]
@@ -222,6 +224,12 @@ def stiv_sort_pairs_static(stream, n, key_bits, keys_in_ptr, vals_in_ptr, keys_o
     that cannot allocate device memory; calls that overlap on the GPU race."""
     _check(lib().stiv_sort_pairs_static(stream, n, key_bits, keys_in_ptr, vals_in_ptr, keys_out_ptr,
                                         vals_out_ptr), "stiv_sort_pairs_static")
+
+
+def stiv_set_all_pairs_limit(h: int, n_ves: int):
+    """Candidate pairs by testing all pairs of boxes up to n_ves vesicles (0 to
+    8192, the default), by the Morton grid above; the same pairs either way."""
+    _check(lib().stiv_set_all_pairs_limit(h, int(n_ves)), "stiv_set_all_pairs_limit")
 
 
 def stiv_peak_probe(stream, kind: int, iters: int, sink_ptr: int) -> float:

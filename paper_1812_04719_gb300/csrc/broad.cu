@@ -164,10 +164,16 @@ __global__ void __launch_bounds__(BT) boxes_kernel(int n, const int32_t* pv, con
   if (threadIdx.x < 3) {
     int c = threadIdx.x;
     double l = vlo_s[c] - dm, u = vhi_s[c] + dm;
-    vbox[6 * v + c] = l;
-    vbox[6 * v + 3 + c] = u;
-    fbox[(size_t)c * n + v] = __double2float_rd(l);
-    fbox[(size_t)(3 + c) * n + v] = __double2float_ru(u);
+    // a box that is not finite on every axis (the vesicle is flagged) is inverted
+    // on all of them: infinite ends would meet the inverted boxes above, and the
+    // broad phase tells inverted boxes by any one axis
+    bool fin = true;
+    for (int q = 0; q < 3; ++q) fin = fin && isfinite(vlo_s[q]) && isfinite(vhi_s[q]);
+    const double bl = fin ? l : INFINITY, bu = fin ? u : -INFINITY;
+    vbox[6 * v + c] = bl;
+    vbox[6 * v + 3 + c] = bu;
+    fbox[(size_t)c * n + v] = __double2float_rd(bl);
+    fbox[(size_t)(3 + c) * n + v] = __double2float_ru(bu);
     double L = c == 0 ? Lx : c == 1 ? Ly : Lz;
     if (L > 0.0 && !(u - l < 0.5 * L)) atomicOr((unsigned long long*)&ctr[STIV_C_STATUS], STIV_F_BOX_TOO_SMALL);
     // FP32 frame of this vesicle: origin at the (float-rounded) box centre

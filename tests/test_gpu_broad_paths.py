@@ -101,6 +101,36 @@ def test_bad_order_is_left_out(limit, bad):
 
 
 @pytest.mark.parametrize("limit", [GRID, ALL_PAIRS])
+@pytest.mark.parametrize("precision", [S.STIV_FP64, S.STIV_MIXED])
+def test_boxes_that_are_not_finite_are_left_out(limit, precision):
+    """Vesicles that reach from -inf to inf on every axis or on one, or that are NaN
+    on one, beside one of an order that is left out: flagged, in no pair, and the
+    other pairs as without them."""
+    sc = SCENES["free"]()
+    X = oracle_vertices(sc)
+    kw = dict(precision=precision, pair_cap=1 << 15, contact_cap=1 << 19)
+    want = gpu_pairs_rows(run_gpu_on(sc, X, precision=precision, grad=False, eng=engine(sc, ALL_PAIRS, **kw)))
+    out = [3, 40, 41, 500, 501, 999]     # infinite on all axes, on y, on z to one side, NaN on y, on x, bad order
+    X = X.copy().reshape(sc.n, 2, 3, -1)
+    X[3, 0, :, 5], X[3, 1, :, 5] = -np.inf, np.inf
+    X[40, 0, 1, 5], X[40, 1, 1, 5] = -np.inf, np.inf
+    X[41, 0, 2, 5] = -np.inf
+    X[500, :, 1], X[501, :, 0] = np.nan, np.nan
+    eng = engine(sc, limit, **kw)
+    ds = S.DeviceScene.from_scene(sc, precision=precision)
+    ds.verts.copy_(torch.from_numpy(X.ravel()))
+    ds.p[999] = 1000
+    with pytest.raises(S.StivError) as e:
+        eng.step(ds, grad=False, upsample=False)
+    assert e.value.status == S.STIV_ERR_INPUT
+    counts = eng.buf.counts.cpu().numpy()
+    assert counts[S.C_STATUS] == S.F_NONFINITE | S.F_BAD_ORDER
+    b, n = eng.buf, int(counts[S.C_PAIRS])
+    got = gpu_pairs_rows({q: x[:n].cpu().numpy() for q, x in (("i", b.ci), ("j", b.cj), ("shift", b.cs))})
+    assert np.array_equal(got, want[~np.isin(want[:, 0], out) & ~np.isin(want[:, 1], out)])
+
+
+@pytest.mark.parametrize("limit", [GRID, ALL_PAIRS])
 def test_overflowing_lists_grow(limit):
     sc = SCENES["few_cells"]()
     X = oracle_vertices(sc)

@@ -81,7 +81,8 @@ enum stiv_count {
 enum stiv_flag {
   STIV_F_PAIRS_OVERFLOW = 1,     /* candidate pairs exceeded stiv_pairs.capacity */
   STIV_F_CONTACTS_OVERFLOW = 2,  /* contacts exceeded stiv_contacts.capacity    */
-  STIV_F_BOX_TOO_SMALL = 4,      /* a vesicle box spans >= L/2 on a periodic axis */
+  STIV_F_BOX_TOO_SMALL = 4,      /* a vesicle box spans >= L/2 on a periodic axis, or
+                                    (Morton grid) lies over 500 cells beyond the lowest */
   STIV_F_NONFINITE = 8,          /* a vertex coordinate is NaN or infinite      */
   STIV_F_WORK_OVERFLOW = 16,     /* internal work list overflow (re-run)         */
   STIV_F_TIMEOUT = 32,           /* a bounded device wait gave up (mixed-form synthesis) */

@@ -334,19 +334,26 @@ __global__ void __launch_bounds__(1024) grid_kernel(int n, const double* vbox, d
         double G = floor(L[c] / hm);
         if (G < 1.0) G = 1.0;
         if (G > 256.0) G = 256.0;
-        grid[c] = 0.0; grid[3 + c] = L[c] / G; grid[6 + c] = G; grid[9 + c] = 1.0;
+        // whole boxes below the lowest vesicle: unwrapped cells count from there
+        grid[c] = floor(slo[c][0] / L[c]) * L[c]; grid[3 + c] = L[c] / G; grid[6 + c] = G; grid[9 + c] = 1.0;
       } else {
         double ext = shi[c][0] - slo[c][0];
         double h = hm;
         if (ext / h > 255.0) h = ext / 255.0;
-        grid[c] = slo[c][0]; grid[3 + c] = h; grid[6 + c] = floor(ext / h) + 1.0; grid[9 + c] = 0.0;
+        double G = floor(ext / h) + 1.0;
+        if (!(G >= 1.0)) G = 1.0;   // an extent past the doubles
+        grid[c] = slo[c][0]; grid[3 + c] = h; grid[6 + c] = G; grid[9 + c] = 0.0;
       }
     }
     grid[12] = hm;
   }
 }
 
-__device__ __forceinline__ void cell_range(const double* grid, const double* box, int c, int& u0, int& u1) {
+// Cells u0 <= u <= u1 of a box on axis c.  Returns false when a periodic axis' cells
+// leave the range that a record holds (then clamped, as the records written are
+// those counted whatever the box).
+constexpr int UMAX = 500;
+__device__ __forceinline__ bool cell_range(const double* grid, const double* box, int c, int& u0, int& u1) {
   double o = grid[c], h = grid[3 + c];
   const double slack = 1e-6;  // cells; covers rounding of the divisions
   u0 = (int)floor((box[c] - o) / h - slack);
@@ -355,37 +362,49 @@ __device__ __forceinline__ void cell_range(const double* grid, const double* box
     int G = (int)grid[6 + c];
     u0 = max(0, min(u0, G - 1));
     u1 = max(0, min(u1, G - 1));
+    return true;
   }
-  u0 = max(u0, -500); u1 = min(u1, 500);
+  const bool fits = u0 >= -UMAX && u1 <= UMAX;
+  u0 = min(max(u0, -UMAX), UMAX);
+  u1 = min(max(u1, -UMAX), UMAX);
+  return fits;
 }
 
-__global__ void cell_count_kernel(int n, const double* vbox, const double* grid, int32_t* cnt) {
+__global__ void cell_count_kernel(int n, const double* vbox, const double* grid, int32_t* cnt, int64_t* ctr) {
   int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= n) return;
   if (!(vbox[6 * v] <= vbox[6 * v + 3])) { cnt[v] = 0; return; }   // inverted box: no cells
   int c = 1;
-  for (int a = 0; a < 3; ++a) { int u0, u1; cell_range(grid, vbox + 6 * v, a, u0, u1); c *= (u1 - u0 + 1); }
+  bool fits = true;
+  for (int a = 0; a < 3; ++a) {
+    int u0, u1;
+    fits = cell_range(grid, vbox + 6 * v, a, u0, u1) && fits;
+    c *= (u1 - u0 + 1);   // at most (2 UMAX + 1)^3 < 2^31
+  }
+  if (!fits) atomicOr((unsigned long long*)&ctr[STIV_C_STATUS], STIV_F_BOX_TOO_SMALL);
   cnt[v] = c;
 }
 
-// Exclusive scan of n+1 ints (last = total), one CTA.
+// Exclusive scan of n+1 ints (last = total), one CTA; sums above 2^31 - 1 stay there
+// (more than any list holds).
 __global__ void __launch_bounds__(1024) scan1_kernel(const int32_t* in, int n, int32_t* out) {
-  __shared__ int32_t part[1024];
+  __shared__ int64_t part[1024];
+  const int64_t top = 0x7FFFFFFF;
   int per = (n + 1023) / 1024;
   int lo = threadIdx.x * per, hi = min(lo + per, n);
-  int32_t s = 0;
+  int64_t s = 0;
   for (int i = lo; i < hi; ++i) s += in[i];
   part[threadIdx.x] = s;
   __syncthreads();
   for (int off = 1; off < 1024; off <<= 1) {
-    int32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
+    int64_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
     __syncthreads();
     part[threadIdx.x] += v;
     __syncthreads();
   }
-  int32_t run = threadIdx.x ? part[threadIdx.x - 1] : 0;
-  for (int i = lo; i < hi; ++i) { out[i] = run; run += in[i]; }
-  if (threadIdx.x == 1023) out[n] = part[1023];
+  int64_t run = threadIdx.x ? part[threadIdx.x - 1] : 0;
+  for (int i = lo; i < hi; ++i) { out[i] = (int32_t)(run < top ? run : top); run += in[i]; }
+  if (threadIdx.x == 1023) out[n] = (int32_t)(part[1023] < top ? part[1023] : top);
 }
 
 __device__ __forceinline__ uint32_t spread10(uint32_t x) {
@@ -428,7 +447,8 @@ __global__ void cell_pairs_kernel(const int64_t* nrec_dev, int64_t R, const uint
                                   const int32_t* rbox, const int32_t* rcell, const double* vbox,
                                   const double* grid, double Lx, double Ly, double Lz, int64_t Q,
                                   uint64_t* pkey, int32_t* pval, int64_t* ctr, int nb) {
-  int64_t nrec = *nrec_dev; if (nrec > R) nrec = R;
+  const int64_t nrec = *nrec_dev;
+  if (nrec > R) return;   // not all are there: flagged, to be run again
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nrec) return;
   double L[3] = {Lx, Ly, Lz};
@@ -676,7 +696,7 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   {
   STIV_PROF_N(h, st, "cells", 4);
   grid_kernel<<<1, 1024, 0, st>>>(n, w.vbox, L[0], L[1], L[2], w.grid);
-  cell_count_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, w.vbox, w.grid, w.cell_count);
+  cell_count_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, w.vbox, w.grid, w.cell_count, ctr);
   scan1_kernel<<<1, 1024, 0, st>>>(w.cell_count, n, w.cell_off);
   cell_emit_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, w.vbox, w.grid, w.cell_off, w.R, w.rec_key, w.rec_val,
                                                     w.rec_box, w.rec_cell, ctr);

@@ -130,6 +130,46 @@ def test_boxes_that_are_not_finite_are_left_out(limit, precision):
     assert np.array_equal(got, want[~np.isin(want[:, 0], out) & ~np.isin(want[:, 1], out)])
 
 
+@pytest.mark.parametrize("boxes_off", [-700, 3, 700])
+def test_suspension_far_from_the_origin(orc, boxes_off):
+    """Periodic coordinates that are never wrapped, whole boxes away."""
+    sc = spheres(300, (32, 32, 0), (1.0, 3.0), 13, side=30.0)
+    X = oracle_vertices(sc).reshape(sc.n, 2, 3, -1).copy()
+    X[:, :, :2] += boxes_off * 32.0
+    X = X.ravel()
+    pairs = orc.candidate_pairs(np.stack([orc.vesicle_box(x, 0.0) for x in verts_list(sc, X)]), sc.L)
+    assert len(pairs) > 300
+    for limit in (GRID, ALL_PAIRS):
+        g = run_gpu_on(sc, X, grad=False, eng=engine(sc, limit, pair_cap=1 << 13, contact_cap=1 << 18))
+        assert np.array_equal(gpu_pairs_rows(g), pairs), limit
+
+
+@pytest.mark.parametrize("what", ["spread", "large", "huge"])
+def test_boxes_beyond_the_records_are_flagged(what):
+    """The grid's records hold some 1000 unwrapped cells per axis.  Vesicles spread
+    over more, and boxes that cover more (their cells counted past 2^31), are
+    flagged; the next good call is right."""
+    sc = spheres(300, (60, 60, 60), (0.2, 0.4), 14)
+    X0 = oracle_vertices(sc)
+    X = X0.reshape(sc.n, 2, 3, -1).copy()
+    if what == "spread":
+        X[::2] += 1000 * 60.0
+    else:
+        X[5:40, 1] += 1e6 if what == "large" else 1e200
+    eng = engine(sc, GRID, pair_cap=1 << 12, contact_cap=1 << 16)
+    ds = S.DeviceScene.from_scene(sc)
+    ds.verts.copy_(torch.from_numpy(X.ravel()))
+    b = eng._buffers(False)
+    st = torch.cuda.current_stream().cuda_stream
+    S.stiv_detect(eng.h, st, ds.n, ds.p_max, S._ptr(ds.p), S._ptr(ds.vert_off), S._ptr(ds.verts), b.pairs_struct(),
+                  b.contacts_struct(), S._ptr(b.counts))
+    counts = S.stiv_sync_counts(st, S._ptr(b.counts))[1]
+    assert counts[S.C_STATUS] & S.F_BOX_TOO_SMALL
+    want = run_gpu_on(sc, X0, grad=False, eng=engine(sc, ALL_PAIRS, pair_cap=1 << 12, contact_cap=1 << 16))
+    got = run_gpu_on(sc, X0, grad=False, eng=eng)
+    assert got["counts"][S.C_STATUS] == 0 and np.array_equal(gpu_pairs_rows(got), gpu_pairs_rows(want))
+
+
 @pytest.mark.parametrize("limit", [GRID, ALL_PAIRS])
 def test_overflowing_lists_grow(limit):
     sc = SCENES["few_cells"]()

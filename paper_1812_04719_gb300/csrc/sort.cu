@@ -219,8 +219,8 @@ int stiv_sort_pairs_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_
 }
 
 // The sort of a caller's arrays, which may overlap (sorting in place): with an odd
-// number of passes the first one writes the output, so an overlapping input is
-// copied to the temporaries before.
+// number of passes the first one writes the output, and with none (key_bits 0) the
+// keys' copy does, so an overlapping input is copied to the temporaries before.
 int stiv_sort_user_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_t* kin, const int32_t* vin,
                         uint64_t* kout, int32_t* vout, uint64_t* kt, int32_t* vt, void* scratch, size_t scratch_bytes) {
   if (key_bits < 0 || key_bits > 64) return STIV_ERR_ARG;
@@ -230,7 +230,8 @@ int stiv_sort_user_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_t
   bool overlap = false;
   for (int a = 0; a < 2; ++a)
     for (int b = 0; b < 2; ++b) overlap = overlap || (in[a] < out[b] + len[b] && out[b] < in[a] + len[a]);
-  if (overlap && ((key_bits + 7) / 8) % 2 == 1) {
+  const int passes = (key_bits + 7) / 8;
+  if (overlap && (passes % 2 == 1 || passes == 0)) {
     STIV_CUDA(STIV_NO_HANDLE, cudaMemcpyAsync(kt, kin, len[0], cudaMemcpyDeviceToDevice, st));
     STIV_CUDA(STIV_NO_HANDLE, cudaMemcpyAsync(vt, vin, len[1], cudaMemcpyDeviceToDevice, st));
     kin = kt;

@@ -75,11 +75,26 @@ __device__ int block_scan(int v, int* sh, int& total) {
   return pre + x - v;
 }
 
+// A row of more than LONG_ROW contacts is cut into segments of SEG_C contacts for
+// row_sides_kernel; the segments after the first are listed (in any order, a row's
+// own in a run).
+constexpr int LONG_ROW = 2048;
+constexpr int SEG_C = 1024;
+struct seg_list {
+  int32_t* count;    // segments listed (cleared before)
+  int32_t* row;      // [ccap / SEG_C + 1]  the row of each
+  int32_t* first;    // [rcap]  long rows: place of the row's second segment
+  int32_t* done;     // [2 rcap]  long rows: segments finished per side (cleared before)
+  int64_t rcap;      // a listed segment's slot in sbeg and scnt: 2 (rcap + place) + side
+};
+__host__ __device__ inline int row_segments(int len) { return len > LONG_ROW ? (len + SEG_C - 1) / SEG_C : 1; }
+
 // dims: [0] rows, [1] nnz, [2] status (1: rows over capacity, 2: nonzeros
 // over capacity), [3] entries (4 x contacts), [4] 2 x rows
 __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t pcap, int64_t ccap,
                                                   const int32_t* pstart, const int32_t* pend, const double* Vp,
-                                                  int64_t rcap, int32_t* row_pair, double* q, int64_t* dims) {
+                                                  int64_t rcap, int32_t* row_pair, double* q, int64_t* dims,
+                                                  seg_list segs) {
   __shared__ int sh[RT / 32];
   int64_t np = counts[STIV_C_PAIRS] < pcap ? counts[STIV_C_PAIRS] : pcap;
   int base = 0;
@@ -91,6 +106,12 @@ __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t
     if (has && base + ex < rcap) {
       row_pair[base + ex] = (int32_t)p;
       q[base + ex] = -Vp[p];
+      const int more = row_segments(pend[p] - pstart[p]) - 1;
+      if (more) {
+        const int at = atomicAdd(segs.count, more);
+        segs.first[base + ex] = at;
+        for (int k = 0; k < more; ++k) segs.row[at + k] = base + ex;
+      }
     }
     base += tot;
   }
@@ -125,6 +146,47 @@ __device__ __forceinline__ int cta_scan(int v, int* wsum, int* total) {
   return pre + x - v;
 }
 
+// Joins the segments of a long row's side, each its vertices and sums, into one
+// list at the first one's place: segment by segment, a vertex seen before adds to
+// its entry, another one takes the next.  In place: an entry moves to no place
+// after its own, and a batch is read before it is written.  Returns the entries.
+__device__ __noinline__ int join_segments(const seg_list& segs, int64_t row, int side, int nseg, int nv, uint16_t* tab,
+                                          int* wsum, const int32_t* sbeg, const int32_t* scnt, int32_t* ukey,
+                                          double* ug) {
+  for (int q = threadIdx.x; q < nv; q += ST) tab[q] = 0xFFFF;
+  __syncthreads();
+  const int64_t base = __ldcg(&sbeg[2 * row + side]), more = segs.rcap + segs.first[row] - 1;
+  int unique = 0;
+  for (int sg = 0; sg < nseg; ++sg) {
+    const int64_t slot = 2 * (sg ? more + sg : row) + side, lo = __ldcg(&sbeg[slot]);
+    const int cnt = __ldcg(&scnt[slot]);
+    for (int i0 = 0; i0 < cnt; i0 += ST) {
+      const int i = i0 + threadIdx.x;
+      const bool in = i < cnt;
+      int v = 0;
+      double g[3] = {0.0, 0.0, 0.0};
+      if (in) {
+        v = __ldcg(&ukey[lo + i]);
+        for (int c = 0; c < 3; ++c) g[c] = __ldcg(&ug[3 * (lo + i) + c]);
+      }
+      const bool fresh = in && tab[v] == 0xFFFF;
+      int add;
+      const int u = unique + cta_scan(fresh ? 1 : 0, wsum, &add);   // barriers: all of the batch is read
+      if (fresh) {
+        tab[v] = (uint16_t)u;
+        ukey[base + u] = v;
+        for (int c = 0; c < 3; ++c) ug[3 * (base + u) + c] = g[c];
+      } else if (in) {   // a vertex once per segment: no other thread adds to its entry
+        double* d = ug + 3 * (base + tab[v]);
+        for (int c = 0; c < 3; ++c) d[c] += g[c];
+      }
+      unique += add;
+      __syncthreads();
+    }
+  }
+  return unique;
+}
+
 // The unique vertices of row r's side s and the sum of their gradient rows, at
 // [sbeg[2 r + s], + scnt[2 r + s]) of ukey and ug (a row's points start at four
 // times its first contact, side 1's after side 0's).  The points are taken in
@@ -136,44 +198,65 @@ __device__ __forceinline__ int cta_scan(int v, int* wsum, int* total) {
 // The global alternative (a keyed entry per point, a radix sort of all of them by
 // row, side and vertex, a gather and a segmented scan over all entries: 25
 // launches) took 0.42 ms of device time at 1440 vesicles (2.5M points), this
-// kernel 0.15 ms, bound by the latency of its short phases.
+// kernel 0.15 ms, bound by the latency of its short phases.  A row in one CTA takes
+// 21 ns a contact, so that a pair that interpenetrates deeply would hold the
+// assembly (55,202 contacts of two vesicles at p = 31: 1264 us, 266 in the global
+// form): a row of more than LONG_ROW contacts goes in segments to as many CTAs, and
+// the one that finishes last joins them (no CTA waits for another): 258 us, and 225
+// -> 115 for 7050 contacts (global 190); shorter rows, up to 1620 contacts at 1440
+// vesicles, are as they were (213 us).
 __global__ void __launch_bounds__(ST, 6) row_sides_kernel(const int64_t* dims, const int32_t* row_pair, const int32_t* pstart,
                                                        const int32_t* pend, const int32_t* ci, const int32_t* gves,
-                                                       const int32_t* gvid, const double* grad, int nv, bool vec, int32_t* sbeg,
-                                                       int32_t* scnt, int32_t* ukey, double* ug) {
+                                                       const int32_t* gvid, const double* grad, int nv, bool vec,
+                                                       seg_list segs, int32_t* sbeg, int32_t* scnt, int32_t* ukey,
+                                                       double* ug) {
   extern __shared__ uint16_t tab[];          // [nv rounded up to 8]
   __shared__ uint32_t item[2][CH];           // vertex << 12 | place in the chunk
   __shared__ int32_t src[CH];                // by place: gradient row
   __shared__ int32_t cnt[ST / 32][SD];
   __shared__ uint16_t start[CH + 1];         // runs
   __shared__ int wsum[ST / 32];
+  __shared__ bool last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t nitem = 2 * dims[0];
+  const int nlist = *segs.count;             // the listed segments first: their rows take longest
+  const int64_t nitem = 2 * (dims[0] + nlist);
   for (int64_t it = blockIdx.x; it < nitem; it += gridDim.x) {
-    const int side = (int)(it & 1), p = row_pair[it >> 1], vi = ci[p];
-    const int k0 = pstart[p], k1 = pend[p];
+    const int side = (int)(it & 1), unit = (int)(it >> 1);
+    const int row = unit < nlist ? segs.row[unit] : unit - nlist;
+    const int p = row_pair[row], vi = ci[p];
+    const int k0 = pstart[p], k1 = pend[p], nseg = row_segments(k1 - k0);
+    const int seg = unit < nlist ? unit - segs.first[row] + 1 : 0;
+    const int ka = nseg > 1 ? k0 + seg * SEG_C : k0, ke = nseg > 1 ? min(ka + SEG_C, k1) : k1;
     for (int q = threadIdx.x; q < nv; q += ST) tab[q] = 0xFFFF;
     int64_t base = 4 * (int64_t)k0;
-    if (side) {   // after the points of side 0
-      int c = 0, tot;
-      for (int k = k0 + threadIdx.x; k < k1; k += ST) {
+    if (side || seg) {   // after the points of side 0 (side 1) and those of earlier segments
+      int c = 0, before = 0, tot;
+#pragma unroll 4
+      for (int k = k0 + threadIdx.x; k < (side ? k1 : ka); k += ST) {
+        int m = 0;
         if (vec) {
           int4 a = ((const int4*)gves)[k];
-          c += (a.x == vi) + (a.y == vi) + (a.z == vi) + (a.w == vi);
+          m = (a.x == vi) + (a.y == vi) + (a.z == vi) + (a.w == vi);
         } else {
-          for (int q = 0; q < 4; ++q) c += gves[4 * (int64_t)k + q] == vi;
+          for (int q = 0; q < 4; ++q) m += gves[4 * (int64_t)k + q] == vi;
         }
+        c += m;
+        before += k < ka ? m : 0;
       }
       cta_scan(c, wsum, &tot);
-      base += tot;
+      base += tot;         // side 0: of the segments before; side 1: of the row
+      if (side && seg) {
+        cta_scan(before, wsum, &tot);
+        base += 4 * (int64_t)(ka - k0) - tot;
+      }
     }
     int unique = 0, n = 0;
-    for (int kb = k0; kb < k1; kb += ST) {
+    for (int kb = ka; kb < ke; kb += ST) {
       // the points of the next ST contacts on this side
       const int64_t k = kb + threadIdx.x;
       int vs[4], vd[4], c = 0, tot;
       unsigned mine = 0;
-      if (k < k1) {
+      if (k < ke) {
         if (vec) {
           int4 a = ((const int4*)gves)[k], b = ((const int4*)gvid)[k];
           vs[0] = a.x; vs[1] = a.y; vs[2] = a.z; vs[3] = a.w;
@@ -193,7 +276,7 @@ __global__ void __launch_bounds__(ST, 6) row_sides_kernel(const int64_t* dims, c
         }
       n += tot;
       __syncthreads();
-      if (kb + ST < k1 && n + 4 * ST <= CH) continue;
+      if (kb + ST < ke && n + 4 * ST <= CH) continue;
       // sort the n points by vertex
       int cur = 0;
       for (int shift = 12; shift < 26 && (nv - 1) >> (shift - 12); shift += 7) {
@@ -277,7 +360,19 @@ __global__ void __launch_bounds__(ST, 6) row_sides_kernel(const int64_t* dims, c
       n = 0;
       __syncthreads();
     }
-    if (threadIdx.x == 0) { sbeg[it] = (int32_t)base; scnt[it] = unique; }
+    const int64_t slot = 2 * (int64_t)(unit < nlist ? segs.rcap + unit : row) + side;
+    if (threadIdx.x == 0) { sbeg[slot] = (int32_t)base; scnt[slot] = unique; }
+    if (nseg > 1) {
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) last = atomicAdd(&segs.done[2 * row + side], 1) == nseg - 1;
+      __syncthreads();
+      if (last) {
+        __threadfence();
+        unique = join_segments(segs, row, side, nseg, nv, tab, wsum, sbeg, scnt, ukey, ug);
+        if (threadIdx.x == 0) scnt[2 * row + side] = unique;
+      }
+    }
     __syncthreads();
   }
 }
@@ -730,14 +825,20 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   int64_t E = 4 * ccap;
   if (E >= ((int64_t)1 << 31)) return STIV_ERR_ARG;
   const int nv = stiv_nverts(2 * p_max);
-  // scratch (handle-owned, grown on demand); pstart, pend and vcnt are cleared together
+  // scratch (handle-owned, grown on demand); pstart, pend, vcnt and the segments'
+  // counts are cleared together
   size_t o = 0;
   size_t o_ps = o; o = al256(o + sizeof(int32_t) * pcap);
   size_t o_pe = o; o = al256(o + sizeof(int32_t) * pcap);
   size_t o_vc = o; o = al256(o + sizeof(int32_t) * n_ves);
+  size_t o_sn = o; o = al256(o + sizeof(int32_t));
+  size_t o_sd = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
   const size_t clear = o;
-  size_t o_sb = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
-  size_t o_sc = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
+  const int64_t scap = ccap / SEG_C + 1;   // listed segments: a long row has less than its contacts / SEG_C
+  size_t o_sr = o; o = al256(o + sizeof(int32_t) * scap);
+  size_t o_sf = o; o = al256(o + sizeof(int32_t) * rcap);
+  size_t o_sb = o; o = al256(o + sizeof(int32_t) * 2 * (rcap + scap));
+  size_t o_sc = o; o = al256(o + sizeof(int32_t) * 2 * (rcap + scap));
   size_t o_bc = o; o = al256(o + sizeof(int32_t) * rcap);
   size_t o_nr = o; o = al256(o + sizeof(int32_t) * lcp->nnz_capacity);
   size_t o_uk = o; o = al256(o + sizeof(int32_t) * E);
@@ -753,6 +854,9 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   char* w = (char*)h->lcp_ws;
   int32_t* pstart = (int32_t*)(w + o_ps); int32_t* pend = (int32_t*)(w + o_pe);
   int32_t* vcnt = (int32_t*)(w + o_vc);
+  seg_list segs;
+  segs.count = (int32_t*)(w + o_sn); segs.row = (int32_t*)(w + o_sr); segs.first = (int32_t*)(w + o_sf);
+  segs.done = (int32_t*)(w + o_sd); segs.rcap = rcap;
   int32_t* sbeg = (int32_t*)(w + o_sb); int32_t* scnt = (int32_t*)(w + o_sc);
   int32_t* bcnt = (int32_t*)(w + o_bc);
   int32_t* nzrow = (int32_t*)(w + o_nr);
@@ -779,11 +883,11 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   bounds_kernel<<<sms * 4, 256, 0, st>>>(counts_dev, ccap, ct->pair, pstart, pend);
   STIV_LAUNCH(h);
   rows_kernel<<<1, RT, 0, st>>>(counts_dev, pcap, ccap, pstart, pend, V_pair_dev, rcap, lcp->row_pair, lcp->q,
-                                lcp->dims);
+                                lcp->dims, segs);
   STIV_LAUNCH(h);
   row_sides_kernel<<<sms * 6, ST, side_table_bytes(nv), st>>>(
       lcp->dims, lcp->row_pair, pstart, pend, cand->i, g_ves_dev, g_vid_dev, grad_dev, nv,
-      (((uintptr_t)g_ves_dev | (uintptr_t)g_vid_dev) & 15) == 0, sbeg, scnt, ukey, ug);
+      (((uintptr_t)g_ves_dev | (uintptr_t)g_vid_dev) & 15) == 0, segs, sbeg, scnt, ukey, ug);
   STIV_LAUNCH(h);
   ves_count_kernel<<<sms, 256, 0, st>>>(lcp->dims, lcp->row_pair, cand->i, cand->j, vcnt);
   STIV_LAUNCH(h);

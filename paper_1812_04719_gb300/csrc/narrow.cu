@@ -741,9 +741,10 @@ __device__ __forceinline__ bool df_of_unit(double m, dflt& r) {
   return true;
 }
 
-// FP64 operations of the procedure, counted as executed (+ - * / sqrt = 1,
-// fma = 2, negations and comparisons 0): the algorithmic work of the exact
-// contact test, reported for the roofline.
+// FP64 operations of the procedure (+ - * / sqrt = 1, fma = 2, negations and
+// comparisons 0): the algorithmic work of the exact contact test.  Halvings and
+// critical points that are decided without their values count all the same, so
+// that the count over the time is no fraction of the FP64 rate.
 //
 // The bisection takes exactly the FP64 path: every midpoint is the FP64
 // midpoint (mid_rn), and every sign is the sign of the FP64 Horner value.

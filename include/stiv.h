@@ -85,7 +85,11 @@ enum stiv_flag {
   STIV_F_BOX_TOO_SMALL = 4,      /* a vesicle box spans >= L/2 on a periodic axis, or
                                     (Morton grid) lies over 500 cells beyond the lowest */
   STIV_F_NONFINITE = 8,          /* a vertex coordinate is NaN or infinite      */
-  STIV_F_WORK_OVERFLOW = 16,     /* internal work list overflow (re-run)         */
+  STIV_F_WORK_OVERFLOW = 16,     /* the work limit of the capacities: an internal list
+                                    overflowed, or the primitive pairs that the sign
+                                    test leaves (a cubic that may vanish) exceed 16
+                                    stiv_contacts.capacity + 4096 (re-run with larger
+                                    capacities)                                  */
   STIV_F_TIMEOUT = 32,           /* a bounded device wait gave up (mixed-form synthesis) */
   STIV_F_BAD_ORDER = 64          /* a vesicle's p_dev entry lies outside [1, p_max]: that
                                     vesicle is left out of synthesis, boxes and contacts */

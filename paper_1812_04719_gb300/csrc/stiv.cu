@@ -300,9 +300,10 @@ __global__ void vpair_kernel(const int32_t* pair, const int64_t* counts, int64_t
 
 // Exclusive scan of the per-pair counts (one CTA); counts pairs with contacts and
 // writes the detection's counts (every counter is final here).  The work limit of a
-// contact capacity (Q3 primitive pairs) is held against the pairs that the sign
-// test leaves, as callers' buffers have grown by it, although the separation test
-// keeps most of those off the list.
+// contact capacity (Q3 primitive pairs left by the sign test) is part of the
+// interface (STIV_F_WORK_OVERFLOW in stiv.h): capacities that were refused stay
+// refused, and callers that grow by it keep the sizes they had, although the
+// separation test keeps most of those pairs off the list.
 __global__ void __launch_bounds__(1024) pair_scan_kernel(int64_t* ctr, int64_t pcap, int64_t C, int64_t Q3,
                                                          const int32_t* cnt,
                                                          int32_t* off, int64_t* counts, int* tc_status) {

@@ -70,6 +70,7 @@ __device__ __forceinline__ float d2f_dir(double x, bool up) {
 // instead of eight barriers, two lanes per patch (a column half each): 0.176 ->
 // 0.158 ms.
 constexpr int BT = 512;
+constexpr size_t VB_SMEM = 96 * 1024;   // per-vertex boxes kept in shared memory at most
 template <bool MIXED>
 __global__ void __launch_bounds__(BT) boxes_kernel(int n, const int32_t* pv, const int64_t* voff, const void* X,
                                                     int mixed, double dm, double Lx, double Ly, double Lz,
@@ -674,13 +675,14 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   STIV_PROF(h, st, "boxes");
   // per-vertex boxes in shared memory up to 96 KB (orders up to P = 44)
   size_t nv_max = (size_t)(w.fstride / 8);
-  size_t vb_cap = 6 * nv_max * sizeof(float) <= 96 * 1024 ? 6 * nv_max : 0;
+  size_t vb_cap = 6 * nv_max * sizeof(float) <= VB_SMEM ? 6 * nv_max : 0;
   size_t bsmem = vb_cap * sizeof(float);
   auto bk = mixed ? boxes_kernel<true> : boxes_kernel<false>;
-  STIV_CUDA(h, cudaFuncSetAttribute(bk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem));
+  STIV_CUDA(h, cudaFuncSetAttribute(bk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VB_SMEM));
   bk<<<n, BT, bsmem, st>>>(n, p_dev, voff, X, mixed, h->prm.d_m, L[0], L[1], L[2], w.vbox, w.pbox,
                                       w.pstride, w.vorg, w.fprep, w.fstride, ctr, vb_cap, p_max, w.fbox);
   }
+  STIV_LAUNCH(h);
   if (n <= h->all_pairs) {
     rows_args a;
     a.n = n; a.nchunk = stiv_row_chunks(n); a.vbox = w.vbox; a.fbox = w.fbox;
@@ -689,6 +691,7 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
     unsigned blocks = (unsigned)(((int64_t)n * a.nchunk + 7) / 8);
     STIV_PROF_N(h, st, "pairs", 2);
     row_pairs_kernel<<<blocks, 256, 0, st>>>(a);
+    STIV_LAUNCH(h);
     emit_pairs_kernel<<<blocks, 256, 0, st>>>(a, cand->capacity, cand->i, cand->j, cand->shift, ctr);
     STIV_LAUNCH(h);
     return STIV_OK;
@@ -696,8 +699,11 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   {
   STIV_PROF_N(h, st, "cells", 4);
   grid_kernel<<<1, 1024, 0, st>>>(n, w.vbox, L[0], L[1], L[2], w.grid);
+  STIV_LAUNCH(h);
   cell_count_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, w.vbox, w.grid, w.cell_count, ctr);
+  STIV_LAUNCH(h);
   scan1_kernel<<<1, 1024, 0, st>>>(w.cell_count, n, w.cell_off);
+  STIV_LAUNCH(h);
   cell_emit_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, w.vbox, w.grid, w.cell_off, w.R, w.rec_key, w.rec_val,
                                                     w.rec_box, w.rec_cell, ctr);
   }

@@ -209,7 +209,9 @@ int stiv_sort_pairs_impl(cudaStream_t st, int64_t n, int key_bits, const uint64_
     uint64_t* kb = (passes - 1 - ps) % 2 == 0 ? kout : ktmp;
     int32_t* vb = (passes - 1 - ps) % 2 == 0 ? vout : vtmp;
     hist_kernel<<<grid, kThreads, 0, st>>>(ka, n_dev, n, shift, mask, hist);
+    STIV_LAUNCH(STIV_NO_HANDLE);
     scan_kernel<<<kRadix, kThreads, 0, st>>>(hist, n_dev, n, totals);
+    STIV_LAUNCH(STIV_NO_HANDLE);
     scatter_kernel<<<grid, kThreads, 0, st>>>(ka, va, kb, vb, n_dev, n, shift, mask, hist, totals);
     STIV_LAUNCH(STIV_NO_HANDLE);
     ka = kb;

@@ -587,7 +587,9 @@ int stiv_contact_order(stiv_handle* h, cudaStream_t st, const stiv_pairs* cand, 
   int blocks = (int)((C + 255) / 256); if (blocks > 4096) blocks = 4096; if (blocks < 1) blocks = 1;
   STIV_PROF_N(h, st, "contact_order", 3);
   pair_scan_kernel<<<1, 1024, 0, st>>>(w.ctr, pcap, C, w.Q3, w.pair_cnt, w.pair_off, counts, h->tc_status);
+  STIV_LAUNCH(h);
   pair_scatter_kernel<<<blocks, 256, 0, st>>>(w.ctr, C, rp, rt, ra, rb, w.pair_off, w.pair_fill, w.seg);
+  STIV_LAUNCH(h);
   const int smem = (int)sizeof(unsigned long long) * 2 * SEG;
   STIV_CUDA(h, cudaFuncSetAttribute(pair_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   int sblocks = (int)(pcap < 5 * 152 ? pcap : 5 * 152);
@@ -698,8 +700,9 @@ extern "C" int stiv_grad_to_coef(stiv_handle* h, void* stream, int32_t n_ves, in
     a.leg[p] = h->tab[p].leg; a.trig[p] = h->tab[p].trig;
   }
   int Pm = 2 * p_max;
-  size_t smem = sizeof(double) * ((size_t)(Pm + 1) * (2 * p_max + 1) + (size_t)(Pm + 1) * 4 * (Pm / 2 + 1));
-  STIV_CUDA(h, cudaFuncSetAttribute(adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  auto bytes = [](int P) { return sizeof(double) * ((size_t)(P + 1) * (P + 1) + (size_t)(P + 1) * 4 * (P / 2 + 1)); };
+  size_t smem = bytes(Pm);
+  STIV_CUDA(h, cudaFuncSetAttribute(adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(STIV_MAX_PP)));
   STIV_PROF(h, st, "grad_to_coef");
   adjoint_kernel<<<dim3(n_ves, 3), 256, smem, st>>>(a);
   STIV_LAUNCH(h);

@@ -192,6 +192,13 @@ inline int stiv_cuda_failed(stiv_handle* h, cudaError_t e) {
     if (e_ != cudaSuccess) return stiv_cuda_failed((h), e_);      \
   } while (0)
 
+// After every launch whose output the next one reads: none runs on what a refused
+// one did not write.
+//
+// A kernel's limit of dynamic shared memory (cudaFuncSetAttribute) is set to the
+// most that any call of it takes, never to the call's own size: it belongs to the
+// device, and another thread's call with a smaller size would take it back between
+// this one's setting and its launch.
 #define STIV_LAUNCH(h) STIV_CUDA(h, cudaGetLastError())
 #define STIV_NO_HANDLE ((stiv_handle*)nullptr)
 

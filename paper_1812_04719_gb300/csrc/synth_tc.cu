@@ -735,8 +735,10 @@ int stiv_upsample_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t p_m
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   STIV_PROF_N(h, st, "synth", 3);
   group_kernel<<<1, 1024, 0, st>>>(n_ves, p_max, p_dev, g, tiles, list, 0, sms);
+  STIV_LAUNCH(h);
   prep_kernel<false><<<prep_grid(sms, max_blocks), PREP_THREADS, 0, st>>>(p_max, g, tiles, list, coef_off_dev, vert_off_dev,
                                                                          coef_dev, bblk, ci);
+  STIV_LAUNCH(h);
   gemm_args A;
   A.g = g; A.tiles = tiles; A.bblk = bblk; A.ci = ci; A.X = verts_dev; A.status = status; A.p_max = p_max;
   for (int p = 0; p <= STIV_MAX_P; ++p) A.ytab[p] = p >= 1 && p <= p_max ? h->ytab[p] : nullptr;
@@ -782,8 +784,10 @@ int stiv_grad_to_coef_tc(stiv_handle* h, cudaStream_t st, int32_t n_ves, int32_t
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   STIV_PROF_N(h, st, "grad_to_coef", 3);
   group_kernel<<<1, 1024, 0, st>>>(n_ves, p_max, p_dev, g, tiles, list, 1, sms);
+  STIV_LAUNCH(h);
   prep_kernel<true><<<prep_grid(sms, max_blocks), PREP_THREADS, 0, st>>>(p_max, g, tiles, list, coef_off_dev, vert_off_dev,
                                                                         gX_dev, bblk, ci);
+  STIV_LAUNCH(h);
   gemm_args A;
   A.g = g; A.tiles = tiles; A.bblk = bblk; A.ci = ci; A.X = gcoef_dev; A.status = status; A.p_max = p_max;
   for (int p = 0; p <= STIV_MAX_P; ++p) A.ytab[p] = p >= 1 && p <= p_max ? h->ytabT[p] : nullptr;

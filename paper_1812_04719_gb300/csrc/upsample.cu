@@ -551,10 +551,12 @@ extern "C" int stiv_upsample(stiv_handle* h, void* stream, int32_t n_ves, int32_
   size_t smem = synth_smem(p_max, split ? 1 : 3);
   STIV_PROF(h, st, "synth");
   if (split) {
-    STIV_CUDA(h, cudaFuncSetAttribute(synth_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    STIV_CUDA(h, cudaFuncSetAttribute(synth_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)synth_smem(STIV_MAX_P, 1)));
     synth_kernel<1><<<dim3(n_ves, 2, 3), 256, smem, st>>>(a);
   } else {
-    STIV_CUDA(h, cudaFuncSetAttribute(synth_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    STIV_CUDA(h, cudaFuncSetAttribute(synth_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)synth_smem(STIV_MAX_P, 3)));
     synth_kernel<3><<<dim3(n_ves, 2), 256, smem, st>>>(a);
   }
   STIV_LAUNCH(h);

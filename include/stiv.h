@@ -306,7 +306,8 @@ typedef struct {
   int32_t* col;           /* [nnz_capacity]                                       */
   double* val;            /* [nnz_capacity]                                       */
   int64_t* dims;          /* [8]: rows, nonzeros, status (1 rows over capacity, 2
-                             nonzeros over capacity), internal counts             */
+                             nonzeros over capacity), contact points (4 per
+                             contact), row sides (2 per row); the rest is not used */
 } stiv_lcp;
 /* Forms B (Alg. 3) and q from the outputs of stiv_detect (cand, contacts,
  * counts) and stiv_stiv_grad (V_pair, grad, g_ves, g_vid) of the same step,

@@ -74,14 +74,9 @@ struct WarpSm {
 };
 
 struct narrow_args {
-  const int32_t* pv;
-  const int64_t* voff;
   const void* X;
   int mixed;
   double L[3];
-  const int32_t* ci;
-  const int32_t* cj;
-  const int32_t* cs;
   const uint64_t* work;
   int64_t W;
   int include_ee;
@@ -2110,10 +2105,9 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
   STIV_LAUNCH(h);
   narrow_args a;
   bool mixed = h->prm.precision == STIV_MIXED;
-  a.pv = p_dev; a.voff = voff; a.X = X; a.mixed = mixed;
+  a.X = X; a.mixed = mixed;
   a.pinfo = w.pinfo;
   a.L[0] = L[0]; a.L[1] = L[1]; a.L[2] = L[2];
-  a.ci = cand->i; a.cj = cand->j; a.cs = cand->shift;
   a.work = w.work; a.W = w.W; a.include_ee = h->prm.include_ee; a.exact_only = w.exact_only;
   a.dm = h->prm.d_m;
   // five levels by default: at 360 vesicles (p = 15, d_m > 0) pieces and FP64 test

@@ -1885,7 +1885,9 @@ __global__ void __launch_bounds__(128, DM ? 8 : 6) fp64_kernel(narrow_args a) {
 //
 // Bound by latency: with one warp per vesicle pair a few deep pairs held the stage
 // (a hundred by a hundred patches, 32 at a time); a CTA's warps share them.  1440
-// vesicles 0.25 -> 0.14 ms, 4096 1.15 -> 0.52, 64 at 30% 0.13 -> 0.04.
+// vesicles 0.25 -> 0.14 ms, 4096 1.15 -> 0.52, 64 at 30% 0.13 -> 0.04.  Small orders,
+// whose patches fill less than a CTA, pay for it: 9216 vesicles of order 3 (9
+// patches) 0.13 -> 0.37 ms.
 constexpr int PPT = 128;   // threads of a CTA
 
 struct patch_list {

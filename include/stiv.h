@@ -25,6 +25,10 @@
  *     found by the kernels themselves (capacity overflow, invalid periodic
  *     box, non-finite input) are flags in counts[STIV_C_STATUS].
  *   - Scratch memory is owned by the handle (grown on demand with cudaMalloc).
+ *     Calls of one handle share it: on different streams the caller orders
+ *     them.  A stream capture of the caller's own holds its addresses, and is
+ *     good until a larger call of the handle (stiv_step's graph follows by
+ *     itself).
  *
  * Layouts (N = number of vesicles, p_v = SH order of vesicle v, P_v = 2 p_v):
  *   coef:  per vesicle [2 time][3 coord][(p_v+1)^2] doubles at coef_off[v];
@@ -354,7 +358,7 @@ enum stiv_tune_param {
   STIV_TUNE_PIECES_CTAS = 1,   /* piece-test CTAs per SM                          */
   STIV_TUNE_FP64_BLOCKS = 2,   /* FP64 contact-test blocks per SM                 */
   STIV_TUNE_PATCH_BLOCKS = 3,  /* patch-pair blocks per SM                        */
-  STIV_TUNE_PIECE_LEVELS = 4,  /* d_m > 0: refinement levels of the FP32 piece test (2-6) */
+  STIV_TUNE_PIECE_LEVELS = 4,  /* d_m > 0: refinement levels of the FP32 piece test (1-6) */
   STIV_NTUNE = 5
 };
 int stiv_autotune(stiv_handle* h, void* stream, int32_t n_ves, int32_t p_max, const int32_t* p_dev,

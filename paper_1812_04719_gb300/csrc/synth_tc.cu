@@ -37,10 +37,10 @@
 //                 K = 8, kind::tf32) into one of two TMEM accumulators, and
 //                 warps 2-5 read the other accumulator (tcgen05.ld 32x32b) and
 //                 write the FP32 vertices while the next tile accumulates.
-// 4096 vesicles of orders 8, 12 and 16: the synthesis products take 72 us (87
-// with every column's address and degree-0 term loaded and shuffled between
-// its stores), the adjoint's 58 us (71 with the tiles in ascending order,
-// whose last round held the longest).
+// 4096 vesicles of orders 8, 12 and 16: the synthesis products take 71 us (87
+// with single tiles, and every column's address and degree-0 term loaded and
+// shuffled between its stores), the adjoint's 57 us (71 with the tiles in
+// ascending order, whose last round held the longest).
 // Every wait on an mbarrier is bounded; a wait that gives up sets a status
 // word (reported as STIV_F_TIMEOUT) and the tile is abandoned.
 #include "stiv_internal.cuh"
@@ -158,10 +158,10 @@ struct tc_group {
 // blocks are copied and read from shared memory once for both (the products
 // are bound by shared memory's bandwidth: 8 KB read per N = 128 instruction
 // beside the copies into it).  It pays while the units still fill the SMs
-// evenly, from four rounds of single tiles on: synthesis of 4096 vesicles of
-// orders 8, 12 and 16 (13 rounds) 115 us in single tiles and 108 us in pairs,
-// of 1440 of order 16 (7.6 rounds) 78 and 73; but the adjoint of the same 4096
-// (1.3 rounds) 139 and 170, of the 1440 (0.7 rounds) 95 and 134.
+// evenly, from four rounds of single tiles on.  The products alone: synthesis of
+// 4096 vesicles of orders 8, 12 and 16 (13 rounds) 78 us in single tiles and 71 in
+// pairs, of 1440 of order 16 (7.6 rounds) 52 and 47; but the adjoint of the same
+// 4096 (1.3 rounds) 57 and 86, of the 1440 (0.7 rounds) 49 and 87.
 constexpr int WIDE_ROUNDS = 4;
 constexpr int GROUP_V = 4;              // vesicles per thread and round of the grouping
 

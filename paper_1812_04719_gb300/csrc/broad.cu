@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(BT) boxes_kernel(int n, const int32_t* pv, con
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr((unsigned long long*)&ctr[STIV_C_STATUS], STIV_F_NONFINITE);
   __shared__ float sorg[4];
   __shared__ double vlo_s[3], vhi_s[3];
+  int fin = 1;
   if (threadIdx.x < 3) {
     int c = threadIdx.x;
     long long a = red[0][c], b = red[0][3 + c];
@@ -161,16 +162,16 @@ __global__ void __launch_bounds__(BT) boxes_kernel(int n, const int32_t* pv, con
     }
     vlo_s[c] = okey_val(a);
     vhi_s[c] = okey_val(b);
+    fin = (~__double_as_longlong(vlo_s[c]) & 0x7FF0000000000000ll) != 0 &&
+          (~__double_as_longlong(vhi_s[c]) & 0x7FF0000000000000ll) != 0;
   }
-  __syncthreads();
+  // a box that is not finite on every axis (the vesicle is flagged) is inverted on
+  // all of them: infinite ends would meet the inverted boxes above, and the broad
+  // phase tells inverted boxes by any one axis
+  fin = __syncthreads_and(fin);
   if (threadIdx.x < 3) {
     int c = threadIdx.x;
     double l = vlo_s[c] - dm, u = vhi_s[c] + dm;
-    // a box that is not finite on every axis (the vesicle is flagged) is inverted
-    // on all of them: infinite ends would meet the inverted boxes above, and the
-    // broad phase tells inverted boxes by any one axis
-    bool fin = true;
-    for (int q = 0; q < 3; ++q) fin = fin && isfinite(vlo_s[q]) && isfinite(vhi_s[q]);
     const double bl = fin ? l : INFINITY, bu = fin ? u : -INFINITY;
     vbox[6 * v + c] = bl;
     vbox[6 * v + 3 + c] = bu;
@@ -679,7 +680,7 @@ int stiv_broad_phase(stiv_handle* h, cudaStream_t st, int n, int p_max, const in
   size_t vb_cap = 6 * nv_max * sizeof(float) <= VB_SMEM ? 6 * nv_max : 0;
   size_t bsmem = vb_cap * sizeof(float);
   auto bk = mixed ? boxes_kernel<true> : boxes_kernel<false>;
-  STIV_CUDA(h, cudaFuncSetAttribute(bk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VB_SMEM));
+  STIV_SMEM(h, bk, bsmem, 4096, VB_SMEM);
   bk<<<n, BT, bsmem, st>>>(n, p_dev, voff, X, mixed, h->prm.d_m, L[0], L[1], L[2], w.vbox, w.pbox,
                                       w.pstride, w.vorg, w.fprep, w.fstride, ctr, vb_cap, p_max, w.fbox);
   }

@@ -84,7 +84,7 @@ struct seg_list {
   int32_t* count;    // segments listed (cleared before)
   int32_t* row;      // [ccap / SEG_C + 1]  the row of each
   int32_t* first;    // [rcap]  long rows: place of the row's second segment
-  int32_t* done;     // [2 rcap]  long rows: segments finished per side (cleared before)
+  int32_t* done;     // [2 rcap]  long rows: segments finished per side
   int64_t rcap;      // a listed segment's slot in sbeg and scnt: 2 (rcap + place) + side
 };
 __host__ __device__ inline int row_segments(int len) { return len > LONG_ROW ? (len + SEG_C - 1) / SEG_C : 1; }
@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t
       if (more) {
         const int at = atomicAdd(segs.count, more);
         segs.first[base + ex] = at;
+        segs.done[2 * (base + ex)] = 0;
+        segs.done[2 * (base + ex) + 1] = 0;
         for (int k = 0; k < more; ++k) segs.row[at + k] = base + ex;
       }
     }
@@ -126,7 +128,9 @@ __global__ void __launch_bounds__(RT) rows_kernel(const int64_t* counts, int64_t
 constexpr int ST = 256;      // threads of a row-side CTA
 constexpr int CH = 2048;     // points sorted at a time
 constexpr int SD = 128;      // digits of the sort (7 bits)
-// dynamic shared memory of row_sides_kernel: one entry per vertex (nv), 16-bit
+// shared memory of row_sides_kernel: its own arrays (33 KB at most) and one 16-bit
+// entry per vertex (nv)
+constexpr size_t SIDE_SMEM = 2 * 4 * CH + 4 * CH + 4 * (ST / 32) * SD + 2 * (CH + 1) + 256;
 constexpr size_t side_table_bytes(int nv) { return sizeof(uint16_t) * (size_t)((nv + 7) & ~7); }
 
 // Exclusive scan over an ST-thread CTA; *total = the sum.  wsum: ST / 32 ints.
@@ -826,14 +830,13 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   if (E >= ((int64_t)1 << 31)) return STIV_ERR_ARG;
   const int nv = stiv_nverts(2 * p_max);
   // scratch (handle-owned, grown on demand); pstart, pend, vcnt and the segments'
-  // counts are cleared together
+  // count (after vcnt) are cleared together
   size_t o = 0;
   size_t o_ps = o; o = al256(o + sizeof(int32_t) * pcap);
   size_t o_pe = o; o = al256(o + sizeof(int32_t) * pcap);
-  size_t o_vc = o; o = al256(o + sizeof(int32_t) * n_ves);
-  size_t o_sn = o; o = al256(o + sizeof(int32_t));
-  size_t o_sd = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
+  size_t o_vc = o; o = al256(o + sizeof(int32_t) * ((size_t)n_ves + 1));
   const size_t clear = o;
+  size_t o_sd = o; o = al256(o + sizeof(int32_t) * 2 * rcap);
   const int64_t scap = ccap / SEG_C + 1;   // listed segments: a long row has less than its contacts / SEG_C
   size_t o_sr = o; o = al256(o + sizeof(int32_t) * scap);
   size_t o_sf = o; o = al256(o + sizeof(int32_t) * rcap);
@@ -855,7 +858,7 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   int32_t* pstart = (int32_t*)(w + o_ps); int32_t* pend = (int32_t*)(w + o_pe);
   int32_t* vcnt = (int32_t*)(w + o_vc);
   seg_list segs;
-  segs.count = (int32_t*)(w + o_sn); segs.row = (int32_t*)(w + o_sr); segs.first = (int32_t*)(w + o_sf);
+  segs.count = vcnt + n_ves; segs.row = (int32_t*)(w + o_sr); segs.first = (int32_t*)(w + o_sf);
   segs.done = (int32_t*)(w + o_sd); segs.rcap = rcap;
   int32_t* sbeg = (int32_t*)(w + o_sb); int32_t* scnt = (int32_t*)(w + o_sc);
   int32_t* bcnt = (int32_t*)(w + o_bc);
@@ -873,9 +876,8 @@ extern "C" int stiv_lcp_matrix(stiv_handle* h, void* stream, int32_t n_ves, int3
   size_t bsmem = sizeof(int32_t) * (size_t)nvtab * bw;
   // both limits before the first launch, so that no call is refused halfway (a
   // table of order 32 beside row_sides_kernel's own arrays passes 48 KB)
-  STIV_CUDA(h, cudaFuncSetAttribute(row_sides_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)side_table_bytes(stiv_nverts(2 * STIV_MAX_P))));
-  STIV_CUDA(h, cudaFuncSetAttribute(bval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+  STIV_SMEM(h, row_sides_kernel, side_table_bytes(nv), SIDE_SMEM, side_table_bytes(stiv_nverts(2 * STIV_MAX_P)));
+  STIV_SMEM(h, bval_kernel, bsmem, 0, 96 * 1024);
   STIV_PROF_N(h, st, "lcp_matrix", 11);
   STIV_CUDA(h, cudaMemsetAsync(w, 0, clear, st));
   // every kernel reads what the ones before it wrote: none is launched after one

@@ -2096,8 +2096,7 @@ int stiv_narrow_phase(stiv_handle* h, cudaStream_t st, const int32_t* p_dev, con
   if (blocks < 1) blocks = 1;
   int mp = stiv_npatches(2 * p_max);
   size_t psmem = (size_t)4 * mp * sizeof(float4);
-  STIV_CUDA(h, cudaFuncSetAttribute(patch_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(4 * stiv_npatches(STIV_MAX_PP) * sizeof(float4))));
+  STIV_SMEM(h, patch_pairs_kernel, psmem, 1024, 4 * stiv_npatches(STIV_MAX_PP) * sizeof(float4));
   {
     STIV_PROF(h, st, "patch_pairs");
     patch_pairs_kernel<<<blocks, PPT, psmem, st>>>(p_dev, w.vbox, w.pbox, L[0], L[1], L[2], cand->i, cand->j,

@@ -702,7 +702,7 @@ extern "C" int stiv_grad_to_coef(stiv_handle* h, void* stream, int32_t n_ves, in
   int Pm = 2 * p_max;
   auto bytes = [](int P) { return sizeof(double) * ((size_t)(P + 1) * (P + 1) + (size_t)(P + 1) * 4 * (P / 2 + 1)); };
   size_t smem = bytes(Pm);
-  STIV_CUDA(h, cudaFuncSetAttribute(adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(STIV_MAX_PP)));
+  STIV_SMEM(h, adjoint_kernel, smem, 0, bytes(STIV_MAX_PP));
   STIV_PROF(h, st, "grad_to_coef");
   adjoint_kernel<<<dim3(n_ves, 3), 256, smem, st>>>(a);
   STIV_LAUNCH(h);

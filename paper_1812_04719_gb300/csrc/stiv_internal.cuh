@@ -194,13 +194,26 @@ inline int stiv_cuda_failed(stiv_handle* h, cudaError_t e) {
 
 // After every launch whose output the next one reads: none runs on what a refused
 // one did not write.
-//
-// A kernel's limit of dynamic shared memory (cudaFuncSetAttribute) is set to the
-// most that any call of it takes, never to the call's own size: it belongs to the
-// device, and another thread's call with a smaller size would take it back between
-// this one's setting and its launch.
 #define STIV_LAUNCH(h) STIV_CUDA(h, cudaGetLastError())
 #define STIV_NO_HANDLE ((stiv_handle*)nullptr)
+
+// A kernel's limit of dynamic shared memory, for a call that takes `bytes` of it
+// beside the kernel's own arrays: raised to the most that any call takes, never set
+// to the call's own size (it belongs to the device, and another thread's smaller
+// call would take it back between this one's setting and its launch).  Calls of up
+// to 48 KB in all need none.  (A raised limit can cost a small kernel that needs
+// none: patch_pairs_kernel 11.8 -> 12.5 us for two vesicles.)
+template <class K>
+inline int stiv_smem_limit(stiv_handle* h, K kernel, size_t bytes, size_t own, size_t most) {
+  if (bytes + own <= 48 * 1024) return STIV_OK;
+  STIV_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  return STIV_OK;
+}
+#define STIV_SMEM(h, kernel, bytes, own, most)                   \
+  do {                                                            \
+    int rc_ = stiv_smem_limit((h), (kernel), (bytes), (own), (most)); \
+    if (rc_) return rc_;                                          \
+  } while (0)
 
 int stiv_ensure_tables(stiv_handle* h, cudaStream_t st, int p);
 // STIV_MIXED synthesis on the tensor cores (3xTF32), FP32 vertices.

@@ -2067,8 +2067,11 @@ __global__ void __launch_bounds__(PPT) patch_pairs_kernel(const int32_t* pv, con
       if (m) {
         unsigned long long base = 0;
         const int nm = __popc(m);
-        if (lane == 0)
+        if (lane == 0) {
           base = atomicAdd((unsigned long long*)&ctr[STIV_C_PATCH], (unsigned long long)(nm * sa * sb));
+          // the further items, which the reported count leaves out
+          if (sa * sb > 1) atomicAdd((unsigned long long*)&ctr[18], (unsigned long long)(nm * (sa * sb - 1)));
+        }
         base = __shfl_sync(0xffffffffu, base, 0);
         if (hit)
           for (int z = 0; z < sa * sb; ++z) {

@@ -338,6 +338,7 @@ __global__ void __launch_bounds__(1024) pair_scan_kernel(int64_t* ctr, int64_t p
     if (ctr[17] > Q3) ctr[STIV_C_STATUS] |= STIV_F_WORK_OVERFLOW;
     if (tc_status && *tc_status) { ctr[STIV_C_STATUS] |= STIV_F_TIMEOUT; *tc_status = 0; }
     for (int k = 0; k < 8; ++k) counts[k] = ctr[k];
+    counts[STIV_C_PATCH] -= ctr[18];   // patch pairs, not their work items
     counts[STIV_C_FLOPS] = ctr[12];
     counts[STIV_C_EXACT] = ctr[13];
     counts[STIV_C_PIECE] = ctr[14];

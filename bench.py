@@ -49,11 +49,11 @@ NARROW_SRC = os.path.join(ROOT, "paper_1812_04719_gb300", "csrc", "narrow.cu")
 # csrc/narrow.cu differs from the captured source (SHA-256 prefix), the
 # instruction roofline and the traffic are reported as null.
 NARROW_NCU = {
-    "src_sha256": "a7e0872c208ba59d",
-    # 110966655 inst, 15174400 + 162048 B over 71040 patch pairs
-    "fp64": {"inst_per_patch_pair": 1562.03, "dram_bytes_per_patch_pair": 215.88},
-    # 111735635 inst, 15186944 + 162048 B over 71037 patch pairs
-    "mixed": {"inst_per_patch_pair": 1572.92, "dram_bytes_per_patch_pair": 216.07},
+    "src_sha256": "46270546bbc7eaaa",
+    # 110966655 inst, 15155712 + 151808 B over 71040 patch pairs
+    "fp64": {"inst_per_patch_pair": 1562.03, "dram_bytes_per_patch_pair": 215.48},
+    # 111735635 inst, 15160832 + 158976 B over 71037 patch pairs
+    "mixed": {"inst_per_patch_pair": 1572.92, "dram_bytes_per_patch_pair": 215.66},
 }
 FP64_WORK = ("FP64 operations of the contact test's procedure, counted by the kernel; halvings whose sign is proved "
              "without a value are counted and not computed, so this rate is no fraction of the peak (ncu: the FP64 "
